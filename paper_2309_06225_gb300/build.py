@@ -18,7 +18,9 @@ SOURCES = ["grf_api.cu", "grf_stage.cu", "grf_stage_dec.cu", "grf_stage_fold.cu"
            "grf_batch.cu", "grf_batch_persistent.cu", "grf_patches.cu", "grf_noalloc.cu", "grf_tlm.cu", "grf_adjoint.cu"]
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INC, "-I" + CSRC]
+# -fmad=false: products and sums fuse only where the source writes fma, so that every instantiation of
+# the pointwise equations (coupling kinds, batched boxes, tangents) gives the same bits.
+FLAGS = ["-O3", "-lineinfo", "-fmad=false", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INC, "-I" + CSRC]
 # Per-source ptxas flags. The dual-number (tangent) kernels are very large functions on which
 # ptxas -O2/-O3 settles for 32 registers and an 87 KB stack; -O1 keeps 255 registers and a
 # 36 KB stack. The reverse-mode stage (about 4,300 recording calls) takes ptxas 10 minutes at

@@ -46,7 +46,7 @@ using grf_rev::Rev;
 // leaves of the pointwise map: values, first derivatives (24 slots x 3), second derivatives
 // (12 slots x 6), KO sums, u_n, acc, lambda, g2
 enum : int { kLV = 0, kLD1 = 27, kLD2 = 99, kLKO = 171, kLUN = 198, kLACC = 225, kLLAM = 252, kLG2 = 253, kNLeaf = 254 };
-// tape entries per point and stage: the pointwise RHS records about 4,220, the stage update and
+// tape entries per point and stage: the pointwise RHS records about 2,250, the stage update and
 // enforcement about 130 more; an overflow is detected and reported
 constexpr int kTapeCap = 5120;
 constexpr int kAdjThreads = 128;
@@ -81,10 +81,10 @@ __device__ __forceinline__ void enforce_point_t(T u[NFIELDS], double min_chi, do
 #pragma unroll
     for (int m = 0; m < 6; ++m) hh[m] = u[F_H + m];
     sym3_inv(hh, hi, id);
-    const T tr = hi[0] * u[F_A] + hi[3] * u[F_A + 3] + hi[5] * u[F_A + 5]
-                 + 2.0 * (hi[1] * u[F_A + 1] + hi[2] * u[F_A + 2] + hi[4] * u[F_A + 4]);
+    const T off = dot3(hi[1], u[F_A + 1], hi[2], u[F_A + 2], hi[4], u[F_A + 4]);
+    const T tr3 = fma(T(2.0), off, dot3(hi[0], u[F_A], hi[3], u[F_A + 3], hi[5], u[F_A + 5])) * (1.0 / 3.0);
 #pragma unroll
-    for (int m = 0; m < 6; ++m) u[F_A + m] = u[F_A + m] - hh[m] * tr * (1.0 / 3.0);
+    for (int m = 0; m < 6; ++m) u[F_A + m] = fnma(hh[m], tr3, u[F_A + m]);
     u[F_CHI] = fmax(u[F_CHI], T(min_chi));
     u[F_LAPSE] = fmax(u[F_LAPSE], T(min_lapse));
 }
@@ -113,8 +113,8 @@ __device__ __forceinline__ void rev_sweep(int entries, long long col) {
         const double g = adj[node];
         if (g == 0.0) continue;
         adj[node] = 0.0;
-        if (oc.x != grf_rev::kNone) adj[(long long)oc.x * S + col] += pc.x * g;
-        if (oc.y != grf_rev::kNone) adj[(long long)oc.y * S + col] += pc.y * g;
+        if (oc.x != grf_rev::kNone) adj[(long long)oc.x * S + col] = fma(pc.x, g, adj[(long long)oc.x * S + col]);
+        if (oc.y != grf_rev::kNone) adj[(long long)oc.y * S + col] = fma(pc.y, g, adj[(long long)oc.y * S + col]);
         if (oc.z != grf_rev::kNone) adj[(long long)oc.z * S + col] += g;
     }
 }
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) adj_tape_kernel(Geom g, Coeffs
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
         const long long o = f * g.fstride + p;
-        const Rev kf = r[f] + a.ko * Rev(kos[f], kLKO + f);
+        const Rev kf = fma(Rev(a.ko), Rev(kos[f], kLKO + f), r[f]);
         knode[f] = kf.i;
         const Rev unf = (STAGE == 0) ? ir.v[f] : Rev(a.un[o], kLUN + f);
         out[f] = (STAGE == 3) ? fma(Rev(cs), Rev(a.acc[o], kLACC + f) + kf, unf) : fma(Rev(cs), kf, unf);

@@ -17,7 +17,7 @@ __global__ void ko_kernel(Geom g, const double* __restrict__ s, double* __restri
     int i, j, k;
     if (!interior_thread(g, i, j, k)) return;
     const long long p = gidx(g, i + NG, j + NG, k + NG);
-    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] += ko * ko6(s + f * g.fstride, p, g.pitch, g.plane);
+    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, ko6(s + f * g.fstride, p, g.pitch, g.plane), rhs[f * g.fstride + p]);
 }
 
 // The 6th-order scheme's dissipation: rhs += ko sum_d Delta^8_d u (ko = -sigma / (256 dx)).
@@ -25,7 +25,7 @@ __global__ void ko8_kernel(Geom g, const double* __restrict__ s, double* __restr
     int i, j, k;
     if (!interior_thread(g, i, j, k)) return;
     const long long p = gidx(g, i + NG6, j + NG6, k + NG6);
-    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] += ko * ko8(s + f * g.fstride, p, g.pitch, g.plane);
+    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, ko8(s + f * g.fstride, p, g.pitch, g.plane), rhs[f * g.fstride + p]);
 }
 
 // Periodic ghost fill: one thread per ghosted (i, j) column and field; walks k.

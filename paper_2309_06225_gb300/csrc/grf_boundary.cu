@@ -90,8 +90,8 @@ __device__ __forceinline__ double sommerfeld_rhs(const Geom& g, const Sommerfeld
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         double du;
-        if (q.side[d] > 0) du = (3.0 * u0 - 4.0 * u[p - st[d]] + u[p - 2 * st[d]]) * i2dx;
-        else if (q.side[d] < 0) du = (-3.0 * u0 + 4.0 * u[p + st[d]] - u[p + 2 * st[d]]) * i2dx;
+        if (q.side[d] > 0) du = fma(3.0, u0, fma(-4.0, u[p - st[d]], u[p - 2 * st[d]])) * i2dx;
+        else if (q.side[d] < 0) du = fma(-3.0, u0, fma(4.0, u[p + st[d]], -u[p + 2 * st[d]])) * i2dx;
         else du = (u[p + st[d]] - u[p - st[d]]) * i2dx;
         adv = fma(q.xr[d], du, adv);
     }

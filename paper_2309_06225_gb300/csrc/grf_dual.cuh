@@ -34,7 +34,7 @@ GRF_DHD D3 operator*(double a, const D3& b) { return D3(a * b.v, a * b.d0, a * b
 GRF_DHD D3 operator/(const D3& a, const D3& b) {
     const double ib = 1.0 / b.v;
     const double q = a.v * ib;
-    return D3(q, (a.d0 - q * b.d0) * ib, (a.d1 - q * b.d1) * ib, (a.d2 - q * b.d2) * ib);
+    return D3(q, ::fma(-q, b.d0, a.d0) * ib, ::fma(-q, b.d1, a.d1) * ib, ::fma(-q, b.d2, a.d2) * ib);
 }
 GRF_DHD D3 operator/(const D3& a, double b) { return a * (1.0 / b); }
 GRF_DHD D3 exp(const D3& a) {
@@ -43,7 +43,7 @@ GRF_DHD D3 exp(const D3& a) {
 }
 GRF_DHD D3 operator/(double a, const D3& b) {
     const double q = a / b.v;
-    const double r = -q / b.v;
+    const double r = a == 1.0 ? -(q * q) : -q / b.v;  // 1/b, the common case, without a second division
     return D3(q, r * b.d0, r * b.d1, r * b.d2);
 }
 GRF_DHD D3& operator+=(D3& a, const D3& b) { a = a + b; return a; }
@@ -67,6 +67,11 @@ GRF_DHD D3 fma(const D3& a, const D3& b, double c) {
 GRF_DHD D3 fma(double a, double b, const D3& c) { return D3(::fma(a, b, c.v), c.d0, c.d1, c.d2); }
 GRF_DHD D3 fma(double a, const D3& b, double c) { return D3(::fma(a, b.v, c), a * b.d0, a * b.d1, a * b.d2); }
 GRF_DHD D3 fma(const D3& a, double b, double c) { return fma(b, a, c); }
+// c - a * b
+GRF_DHD D3 fnma(const D3& a, const D3& b, const D3& c) {
+    return D3(::fma(-a.v, b.v, c.v), ::fma(-a.v, b.d0, ::fma(-a.d0, b.v, c.d0)), ::fma(-a.v, b.d1, ::fma(-a.d1, b.v, c.d1)),
+              ::fma(-a.v, b.d2, ::fma(-a.d2, b.v, c.d2)));
+}
 GRF_DHD D3 fabs(const D3& a) { return a.v < 0.0 ? -a : a; }
 GRF_DHD D3 fmax(const D3& a, const D3& b) { return a.v >= b.v ? a : b; }
 GRF_DHD D3 fmax(const D3& a, double b) { return a.v >= b ? a : D3(b); }

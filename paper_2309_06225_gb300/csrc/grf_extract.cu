@@ -78,8 +78,7 @@ __device__ __forceinline__ double interp4(const Geom& g, const double* __restric
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const double* row = f + gidx(g, i0[0] - 1, i0[1] - 1 + b, i0[2] - 1 + c);
-            const double va = L[0][0] * __ldg(row) + L[0][1] * __ldg(row + 1) + L[0][2] * __ldg(row + 2) +
-                              L[0][3] * __ldg(row + 3);
+            const double va = fma(L[0][3], __ldg(row + 3), dot3(L[0][0], __ldg(row), L[0][1], __ldg(row + 1), L[0][2], __ldg(row + 2)));
             vb = fma(L[1][b], va, vb);
         }
         v = fma(L[2][c], vb, v);

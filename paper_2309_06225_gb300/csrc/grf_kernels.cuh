@@ -42,10 +42,10 @@ __device__ __forceinline__ long long gidx(const Geom& g, int i, int j, int k) { 
 // Mixed derivatives (tensor product of the first-derivative weights) are formed below as the
 // first-derivative stencil applied to rounded first derivatives.
 __device__ __forceinline__ double fd1(const double* __restrict__ u, long long p, long long s, double i12) {
-    return ((GRF_LDG(u + p - 2 * s) - GRF_LDG(u + p + 2 * s)) + 8.0 * (GRF_LDG(u + p + s) - GRF_LDG(u + p - s))) * i12;
+    return fma(8.0, GRF_LDG(u + p + s) - GRF_LDG(u + p - s), GRF_LDG(u + p - 2 * s) - GRF_LDG(u + p + 2 * s)) * i12;
 }
 __device__ __forceinline__ double fd2(const double* __restrict__ u, long long p, long long s, double u0, double i12s) {
-    return (16.0 * (GRF_LDG(u + p + s) + GRF_LDG(u + p - s)) - (GRF_LDG(u + p + 2 * s) + GRF_LDG(u + p - 2 * s)) - 30.0 * u0) * i12s;
+    return fma(-30.0, u0, fma(16.0, GRF_LDG(u + p + s) + GRF_LDG(u + p - s), -(GRF_LDG(u + p + 2 * s) + GRF_LDG(u + p - 2 * s)))) * i12s;
 }
 
 __device__ __forceinline__ bool has_d2(int f) {
@@ -97,20 +97,18 @@ __device__ __forceinline__ double mixed_x_warp(const WarpRow& wr, int b, int t, 
     const double m1 = wr.lane < 1 ? hB : vm1;
     const double p1 = wr.lane > 30 ? hB : vp1;
     const double p2 = wr.lane > 29 ? hA : vp2;
-    return __dmul_rn((m2 - p2) + 8.0 * (p1 - m1), i12);
+    return fma(8.0, p1 - m1, m2 - p2) * i12;
 }
 
 // d_s d_t u with the four t-derivatives at the s-neighbours evaluated here (s = x or y). The
-// scalings are explicitly rounded (__dmul_rn, never fused into a neighbouring add), so the sums
-// are those of the shuffle and shared-memory paths, whose neighbour values arrive rounded.
-__device__ __forceinline__ double fd1_rounded(const double* __restrict__ u, long long p, long long s, double i12) {
-    return __dmul_rn((GRF_LDG(u + p - 2 * s) - GRF_LDG(u + p + 2 * s)) + 8.0 * (GRF_LDG(u + p + s) - GRF_LDG(u + p - s)), i12);
-}
+// scalings are rounded (the library is built with -fmad=false: nothing is fused that is not written
+// as fma), so the sums are those of the shuffle and shared-memory paths, whose neighbour values
+// arrive rounded.
 __device__ __forceinline__ double mixed_local(const double* __restrict__ u, long long p, long long so, long long t,
                                               double i12) {
-    const double m2 = fd1_rounded(u, p - 2 * so, t, i12), m1 = fd1_rounded(u, p - so, t, i12);
-    const double p1 = fd1_rounded(u, p + so, t, i12), p2 = fd1_rounded(u, p + 2 * so, t, i12);
-    return __dmul_rn((m2 - p2) + 8.0 * (p1 - m1), i12);
+    const double m2 = fd1(u, p - 2 * so, t, i12), m1 = fd1(u, p - so, t, i12);
+    const double p1 = fd1(u, p + so, t, i12), p2 = fd1(u, p + 2 * so, t, i12);
+    return fma(8.0, p1 - m1, m2 - p2) * i12;
 }
 
 // d_y d_z in blocks of 32 x 4 threads (every warp one x-row, the 4 warps consecutive y-rows):
@@ -134,8 +132,8 @@ __device__ __forceinline__ void yz_rows_fill(const Geom& g, const double* __rest
 #pragma unroll
     for (int b = 0; b < 12; ++b) {
         const double* u = s + (long long)d2field(b) * g.fstride;
-        sh.dz[b][wy + 2][lane] = fd1_rounded(u, po, g.plane, i12);
-        sh.dz[b][rh][lane] = fd1_rounded(u, ph, g.plane, i12);
+        sh.dz[b][wy + 2][lane] = fd1(u, po, g.plane, i12);
+        sh.dz[b][rh][lane] = fd1(u, ph, g.plane, i12);
     }
 }
 
@@ -182,28 +180,24 @@ __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__
                 const double x = fma(18.0, a1, fma(-6.0, a2, a3)) - fma(3.0, b1, 10.0 * u0);
                 av = fma(fabs(bet[d]), x * i12, av);
             }
-            if (d == 2 && has_d2(f)) {  // rounded: shared with the neighbours' d_y d_z
-                d1[d] = sh ? sh->dz[d2slot(f)][wy + 2][lane] : __dmul_rn((m2 - q2) + 8.0 * (q1 - m1), i12);
-            } else {
-                d1[d] = ((m2 - q2) + 8.0 * (q1 - m1)) * i12;
-            }
+            d1[d] = (sh && d == 2 && has_d2(f)) ? sh->dz[d2slot(f)][wy + 2][lane] : fma(8.0, q1 - m1, m2 - q2) * i12;
             if (!(f >= F_B && f < F_B + 3)) in.d1[d1slot(f)][d] = d1[d];
             p1[d] = q1 + m1;
             p2[d] = q2 + m2;
         }
         if (has_d2(f)) {
             const int b = d2slot(f);
-            in.d2[b][0] = (16.0 * p1[0] - p2[0] - 30.0 * u0) * i12s;
+            in.d2[b][0] = fma(-30.0, u0, fma(16.0, p1[0], -p2[0])) * i12s;
             in.d2[b][1] = wr ? mixed_x_warp(*wr, b, 0, d1[1], i12) : mixed_local(u, p, st[0], st[1], i12);
             in.d2[b][2] = wr ? mixed_x_warp(*wr, b, 1, d1[2], i12) : mixed_local(u, p, st[0], st[2], i12);
-            in.d2[b][3] = (16.0 * p1[1] - p2[1] - 30.0 * u0) * i12s;
+            in.d2[b][3] = fma(-30.0, u0, fma(16.0, p1[1], -p2[1])) * i12s;
             if (sh) {
                 const double(*r)[32] = sh->dz[b];
-                in.d2[b][4] = __dmul_rn((r[wy][lane] - r[wy + 4][lane]) + 8.0 * (r[wy + 3][lane] - r[wy + 1][lane]), i12);
+                in.d2[b][4] = fma(8.0, r[wy + 3][lane] - r[wy + 1][lane], r[wy][lane] - r[wy + 4][lane]) * i12;
             } else {
                 in.d2[b][4] = mixed_local(u, p, st[1], st[2], i12);
             }
-            in.d2[b][5] = (16.0 * p1[2] - p2[2] - 30.0 * u0) * i12s;
+            in.d2[b][5] = fma(-30.0, u0, fma(16.0, p1[2], -p2[2])) * i12s;
         }
         if (LOP) adv[f] = av;
         const double t3 = LOP ? (p3[0] + p3[1]) + p3[2]
@@ -212,7 +206,7 @@ __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__
                                     (GRF_LDG(u + p - 3 * st[2]) + GRF_LDG(u + p + 3 * st[2]));
         const double t2 = (p2[0] + p2[1]) + p2[2];
         const double t1 = (p1[0] + p1[1]) + p1[2];
-        kos[f] = t3 - 6.0 * t2 + 15.0 * t1 - 60.0 * u0;
+        kos[f] = fma(-60.0, u0, fma(15.0, t1, fma(-6.0, t2, t3)));
     }
 }
 
@@ -224,7 +218,7 @@ __device__ __forceinline__ double ko6(const double* __restrict__ u, long long p,
     for (int r = 1; r <= 3; ++r)
         t[r] = ((GRF_LDG(u + p - r * st[0]) + GRF_LDG(u + p + r * st[0])) + (GRF_LDG(u + p - r * st[1]) + GRF_LDG(u + p + r * st[1]))) +
                (GRF_LDG(u + p - r * st[2]) + GRF_LDG(u + p + r * st[2]));
-    return t[3] - 6.0 * t[2] + 15.0 * t[1] - 60.0 * GRF_LDG(u + p);
+    return fma(-60.0, GRF_LDG(u + p), fma(15.0, t[1], fma(-6.0, t[2], t[3])));
 }
 
 __device__ __forceinline__ bool interior_thread(const Geom& g, int& i, int& j, int& k) {
@@ -294,10 +288,10 @@ __device__ __forceinline__ void enforce_point(double u[NFIELDS], double min_chi,
 #pragma unroll
     for (int m = 0; m < 6; ++m) hh[m] = u[F_H + m];
     sym3_inv(hh, hi, id);
-    const double tr = hi[0] * u[F_A] + hi[3] * u[F_A + 3] + hi[5] * u[F_A + 5]
-                      + 2.0 * (hi[1] * u[F_A + 1] + hi[2] * u[F_A + 2] + hi[4] * u[F_A + 4]);
+    const double off = dot3(hi[1], u[F_A + 1], hi[2], u[F_A + 2], hi[4], u[F_A + 4]);
+    const double tr3 = fma(2.0, off, dot3(hi[0], u[F_A], hi[3], u[F_A + 3], hi[5], u[F_A + 5])) * (1.0 / 3.0);
 #pragma unroll
-    for (int m = 0; m < 6; ++m) u[F_A + m] -= hh[m] * tr * (1.0 / 3.0);
+    for (int m = 0; m < 6; ++m) u[F_A + m] = fnma(hh[m], tr3, u[F_A + m]);
     u[F_CHI] = fmax(u[F_CHI], min_chi);
     u[F_LAPSE] = fmax(u[F_LAPSE], min_lapse);
 }
@@ -328,7 +322,7 @@ __device__ __forceinline__ double rk4_value(const StageArgs& a, long long q, dou
     double accf;
     if (STAGE == 0) accf = kf;
     else if (STAGE == 3) accf = a.acc[q] + kf;
-    else accf = a.acc[q] + 2.0 * kf;
+    else accf = fma(2.0, kf, a.acc[q]);
     if (STAGE < 3) a.acc[q] = accf;
     const double cs = (STAGE == 0 || STAGE == 1) ? 0.5 * a.dt : (STAGE == 2 ? a.dt : a.dt * (1.0 / 6.0));
     return (STAGE == 3) ? fma(cs, accf, unf) : fma(cs, kf, unf);
@@ -371,7 +365,7 @@ __device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, cons
     double out[NFIELDS];
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
-        const double kf = r[f] + a.ko * kos[f];
+        const double kf = fma(a.ko, kos[f], r[f]);
         const double unf = (STAGE == 0) ? in.v[f] : a.un[f * g.fstride + p];
         out[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
     }

@@ -82,7 +82,7 @@ __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict_
         }
 #pragma unroll
         for (int r = 1; r <= 4; ++r) t[r] = (pr[0][r] + pr[1][r]) + pr[2][r];
-        kos[f] = fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))) + 210.0 * u0;
+        kos[f] = fma(210.0, u0, fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
     }
 }
 
@@ -229,7 +229,7 @@ __device__ __forceinline__ void gather6_block(const Geom& g, const double* __res
         double t[5];
 #pragma unroll
         for (int r = 1; r <= 4; ++r) t[r] = (pr[0][r] + pr[1][r]) + pr[2][r];
-        kos[f] = fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))) + 210.0 * u0;
+        kos[f] = fma(210.0, u0, fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
     }
 }
 
@@ -253,7 +253,7 @@ __device__ __forceinline__ void stage_point6(const Geom& g, const Coeffs& c, con
     double out[NFIELDS];
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
-        const double kf = r[f] + a.ko * kos[f];
+        const double kf = fma(a.ko, kos[f], r[f]);
         const double unf = (STAGE == 0) ? in.v[f] : a.un[f * g.fstride + p];
         out[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
     }
@@ -284,7 +284,7 @@ __device__ __forceinline__ double ko8(const double* __restrict__ u, long long p,
     for (int r = 1; r <= 4; ++r)
         t[r] = ((__ldg(u + p - r * st[0]) + __ldg(u + p + r * st[0])) + (__ldg(u + p - r * st[1]) + __ldg(u + p + r * st[1]))) +
                (__ldg(u + p - r * st[2]) + __ldg(u + p + r * st[2]));
-    return fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))) + 210.0 * __ldg(u + p);
+    return fma(210.0, __ldg(u + p), fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
 }
 
 }  // namespace grf

@@ -17,8 +17,17 @@
 //     8 pi S_ij = S1_ij - 4 [G_S ij Phi_nn + Y_ij + Q_ij(C)]
 // where Phi_ab = nabla_a nabla_b beta(phi) and the first-order (X, X^2) parts rho1, S1 are
 // those of (1/16 pi)(X + g2 X^2). C_ij (through d_t K_ij) and Phi_nn (through d_t Pi) are
-// the only places the unknowns enter, affinely: the 7x7 system M v = r for v = (d_t K_ij, d_t Pi)
-// is assembled from these expressions and solved by LU with partial pivoting.
+// the only places the unknowns enter, affinely: the 7x7 system M v = r for v = (C_ij, H_nn), which hold
+// d_t K_ij and d_t Pi, is assembled from these expressions and solved by LU with partial pivoting.
+//
+// What bounds it: the FP64 pipe (2 lanes per SM and clock), one instruction at a time, so the formulas are
+// chosen by their instruction count. The curvature goes through the six components of the 3D Riemann
+// tensor (its double dual is the raised Einstein tensor), the derivatives of Gt^k that cancel between
+// R_ij and D_(i Z_j) are never formed, and C_ij and H_nn are the unknowns, in which the lapse's
+// derivatives and the shift terms cancel. About 2,100 FP64 instructions where the forms through
+// d_m (h^ij Gt_lij) and d_t K_ij took 2,900: 256^3 step 506 -> 412 ms, 36 x 32 x 30 gradient (whose tape
+// has one entry per operation) 76.9 -> 52.7 ms, 72^2 x 60 diagnostics 6.57 -> 4.97 ms.
+// Products and sums are fused only where fma is written (-fmad=false), so all instantiations round alike.
 //
 // The cubic Horndeski term (1/16 pi) g3 X box(phi) (general instantiation, COUP = 1) adds, with
 // H = nabla nabla phi in the same basis (H_nn holding d_t Pi, H_ni, H_ij = D_i D_j phi + K_ij Pi),
@@ -120,26 +129,51 @@ struct PointExtraT {
 };
 using PointExtra = PointExtraT<double>;
 
+// a0 b0 + a1 b1 + a2 b2, and c - a b
+template <typename T>
+GRF_HD T dot3(const T& a0, const T& b0, const T& a1, const T& b1, const T& a2, const T& b2) {
+    return fma(a2, b2, fma(a1, b1, a0 * b0));
+}
+template <typename T>
+GRF_HD T fnma(const T& a, const T& b, const T& c) { return fma(-a, b, c); }
+
+// x / 2 and 2 x. For doubles on the device these step the exponent on the integer pipe, which runs
+// beside the FP64 pipe (2 lanes per SM and clock against 64); zeros, infinities, NaNs and the ends of
+// the exponent range pass through unchanged.
+template <typename T>
+GRF_HD T half_of(const T& x) { return 0.5 * x; }
+template <typename T>
+GRF_HD T twice_of(const T& x) { return 2.0 * x; }
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ double exponent_step(double x, int step) {
+    const int hi = __double2hiint(x);
+    const unsigned e = ((unsigned)hi << 1) - (2u << 21);
+    return __hiloint2double(e < (0x7fcu << 21) ? hi + step : hi, __double2loint(x));
+}
+__device__ __forceinline__ double half_of(const double& x) { return exponent_step(x, -(1 << 20)); }
+__device__ __forceinline__ double twice_of(const double& x) { return exponent_step(x, 1 << 20); }
+#endif
+
 template <typename T>
 GRF_HD T sym3_det(const T h[6]) {
-    return h[0] * (h[3] * h[5] - h[4] * h[4]) - h[1] * (h[1] * h[5] - h[4] * h[2])
-           + h[2] * (h[1] * h[4] - h[3] * h[2]);
+    const T a = fnma(h[4], h[4], h[3] * h[5]), b = fnma(h[1], h[5], h[4] * h[2]), d = fnma(h[3], h[2], h[1] * h[4]);
+    return dot3(h[0], a, h[1], b, h[2], d);
 }
 
 // symmetric inverse; returns determinant
 template <typename T>
 GRF_HD T sym3_inv(const T h[6], T hi[6], T& id) {
-    const T c00 = h[3] * h[5] - h[4] * h[4];
-    const T c01 = h[2] * h[4] - h[1] * h[5];
-    const T c02 = h[1] * h[4] - h[2] * h[3];
-    const T det = h[0] * c00 + h[1] * c01 + h[2] * c02;
+    const T c00 = fnma(h[4], h[4], h[3] * h[5]);
+    const T c01 = fnma(h[1], h[5], h[2] * h[4]);
+    const T c02 = fnma(h[2], h[3], h[1] * h[4]);
+    const T det = dot3(h[0], c00, h[1], c01, h[2], c02);
     id = 1.0 / det;
     hi[0] = c00 * id;
     hi[1] = c01 * id;
     hi[2] = c02 * id;
-    hi[3] = (h[0] * h[5] - h[2] * h[2]) * id;
-    hi[4] = (h[1] * h[2] - h[0] * h[4]) * id;
-    hi[5] = (h[0] * h[3] - h[1] * h[1]) * id;
+    hi[3] = fnma(h[2], h[2], h[0] * h[5]) * id;
+    hi[4] = fnma(h[0], h[4], h[1] * h[2]) * id;
+    hi[5] = fnma(h[1], h[1], h[0] * h[3]) * id;
     return det;
 }
 
@@ -197,7 +231,7 @@ GRF_HD double det7(const double M[7][8], double* ratio) {
         det *= A[k][k];
         for (int i = k + 1; i < 7; ++i) {
             const double f = A[i][k] / A[k][k];
-            for (int j = k + 1; j < 7; ++j) A[i][j] -= f * A[k][j];
+            for (int j = k + 1; j < 7; ++j) A[i][j] = fma(-f, A[k][j], A[i][j]);
         }
     }
     *ratio = mx > 0.0 ? mn / mx : 0.0;
@@ -251,7 +285,7 @@ GRF_HD bool solve7(T M[7][8]) {
 // off-diagonal components pre-multiplied by 2.
 template <typename T>
 GRF_HD T sdotw(const T a[6], const T bw[6]) {
-    return a[0] * bw[0] + a[1] * bw[1] + a[2] * bw[2] + a[3] * bw[3] + a[4] * bw[4] + a[5] * bw[5];
+    return fma(a[5], bw[5], fma(a[4], bw[4], fma(a[3], bw[3], dot3(a[0], bw[0], a[1], bw[1], a[2], bw[2]))));
 }
 
 // Levi-Civita bookkeeping of the Codazzi block: B_kij (antisymmetric in ij) is stored through
@@ -266,17 +300,19 @@ GRF_HD void q_of(const T X[6], const T gd[6], const T gw[6], const T Phd[6], con
                  T out[6]) {
     const T XP = sdotw(X, Phuw);
     const T trX = sdotw(X, gw);
+    const T sx = fnma(trX, trP, XP);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
-            T pu = Phm[i][0] * X[sidx(0, j)];
-            pu = fma(Phm[i][1], X[sidx(1, j)], pu);
-            pu = fma(Phm[i][2], X[sidx(2, j)], pu);
-            pu = fma(Phm[j][0], X[sidx(i, 0)], pu);
-            pu = fma(Phm[j][1], X[sidx(i, 1)], pu);
-            pu = fma(Phm[j][2], X[sidx(i, 2)], pu);
-            out[sidx(i, j)] = gd[sidx(i, j)] * (XP - trX * trP) - pu + trP * X[sidx(i, j)] + trX * Phd[sidx(i, j)];
+            T q = fma(gd[sidx(i, j)], sx, fma(trP, X[sidx(i, j)], trX * Phd[sidx(i, j)]));
+            if (i == j) {
+                q = fma(-2.0, dot3(Phm[i][0], X[sidx(0, j)], Phm[i][1], X[sidx(1, j)], Phm[i][2], X[sidx(2, j)]), q);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) q = fnma(Phm[i][k], X[sidx(k, j)], fnma(Phm[j][k], X[sidx(i, k)], q));
+            }
+            out[sidx(i, j)] = q;
         }
 }
 
@@ -299,15 +335,14 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     T hi[6], ideth;
     sym3_inv(h, hi, ideth);
     const T ichi = 1.0 / chi;
-    const T ial = 1.0 / al;
     // weighted inverses (off-diagonals doubled) for symmetric contractions; gamma^ij = chi h^ij
     T hw[6], gu[6], gw[6], gd[6];
 #pragma unroll
     for (int m = 0; m < 6; ++m) {
         const bool off = (m == 1 || m == 2 || m == 4);
-        hw[m] = off ? 2.0 * hi[m] : hi[m];
+        hw[m] = off ? twice_of(hi[m]) : hi[m];
         gu[m] = chi * hi[m];
-        gw[m] = chi * hw[m];
+        gw[m] = off ? twice_of(gu[m]) : gu[m];
         gd[m] = h[m] * ichi;
     }
 
@@ -332,10 +367,11 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         for (int i = 0; i < 3; ++i) db[j][i] = D1(F_SHIFT + i, j);
     const T divb = db[0][0] + db[1][1] + db[2][2];
     const T bx = v[F_SHIFT], by = v[F_SHIFT + 1], bz = v[F_SHIFT + 2];
-#define ADV(f) (LOP ? adv[f] : (bx * D1(f, 0) + by * D1(f, 1) + bz * D1(f, 2)))
+#define ADV(f) (LOP ? adv[f] : dot3(bx, D1(f, 0), by, D1(f, 1), bz, D1(f, 2)))
 
     // ---- conformal Christoffels: G1[l][ij] = Gt_{l ij}, G2[k][ij] = Gt^k_ij,
-    //      Gl_l = h^ij Gt_lij (= h_lk Gt^k), Gtc^k = h^kl Gl_l
+    //      Gl_l = h^ij Gt_lij (= h_lk Gt^k), Gtc^k = h^kl Gl_l. Where two of the indices of Gt_lij agree
+    //      two of its three derivatives cancel: Gt_llj = d_j h_ll / 2, Gt_lii = d_i h_li - d_l h_ii / 2.
     GRF_SECTION(2);
     T G1[3][6], G2[3][6], Gl[3], Gtc[3];
 #pragma unroll
@@ -343,65 +379,56 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = i; j < 3; ++j)
-                G1[l][sidx(i, j)] = 0.5 * (dh[i][sidx(l, j)] + dh[j][sidx(l, i)] - dh[l][sidx(i, j)]);
+            for (int j = i; j < 3; ++j) {
+                const int m = sidx(i, j);
+                if (i == l || j == l) G1[l][m] = half_of(dh[i == l ? j : i][sidx(l, l)]);
+                else if (i == j) G1[l][m] = fma(-0.5, dh[l][m], dh[i][sidx(l, i)]);
+                else G1[l][m] = half_of(dh[i][sidx(l, j)] + dh[j][sidx(l, i)] - dh[l][m]);
+            }
 #pragma unroll
     for (int l = 0; l < 3; ++l) Gl[l] = sdotw(G1[l], hw);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        Gtc[k] = hi[sidx(k, 0)] * Gl[0] + hi[sidx(k, 1)] * Gl[1] + hi[sidx(k, 2)] * Gl[2];
+        Gtc[k] = dot3(hi[sidx(k, 0)], Gl[0], hi[sidx(k, 1)], Gl[1], hi[sidx(k, 2)], Gl[2]);
 #pragma unroll
         for (int m = 0; m < 6; ++m)
-            G2[k][m] = hi[sidx(k, 0)] * G1[0][m] + hi[sidx(k, 1)] * G1[1][m] + hi[sidx(k, 2)] * G1[2][m];
+            G2[k][m] = dot3(hi[sidx(k, 0)], G1[0][m], hi[sidx(k, 1)], G1[1][m], hi[sidx(k, 2)], G1[2][m]);
     }
 
-    // ---- dGl[m][l] = d_m Gl_l = d_m h^ij Gt_lij + h^ij d_m d_i h_lj - h^ij d_m d_l h_ij / 2
+    // ---- the six components of the conformal Riemann tensor (1212, 1213, 1223, 1313, 1323, 2323)
+    //   Rt_iklm = (d_k d_l h_im + d_i d_m h_kl - d_k d_m h_il - d_i d_l h_km)/2 + Gt^n_kl Gt_nim - Gt^n_km Gt_nil.
+    // In three dimensions they hold the whole curvature: its contraction takes 21 products, where the
+    // Ricci tensor written through d_m (h^ij Gt_lij) differentiates h^ij and takes about 300 more.
     GRF_SECTION(3);
-    T dGl[3][3];
-    T hdd[6];  // h^pq d_m d_l h_pq, symmetric in (m, l)
+#define DH(a, b, c, d) D2(F_H + sidx(a, b), sidx(c, d)) /* d_c d_d h_ab */
+    T Rm[6];
+    {
+        auto riem = [&](int i, int k, int l, int m) -> T {
+            T x = (i == l && k == m) ? twice_of(DH(i, k, i, k)) - (DH(i, i, k, k) + DH(k, k, i, i))
+                                     : (DH(i, m, k, l) + DH(k, l, i, m)) - (DH(i, l, k, m) + DH(k, m, i, l));
+            x = half_of(x);
 #pragma unroll
-    for (int ml = 0; ml < 6; ++ml) {
-        T b = hw[0] * D2(F_H + 0, ml);
-#pragma unroll
-        for (int q = 1; q < 6; ++q) b = fma(hw[q], D2(F_H + q, ml), b);
-        hdd[ml] = b;
-    }
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-        T Tm[3][3];  // h^ac d_m h_cd
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                Tm[a][d] = hi[sidx(a, 0)] * dh[m][sidx(0, d)] + hi[sidx(a, 1)] * dh[m][sidx(1, d)]
-                           + hi[sidx(a, 2)] * dh[m][sidx(2, d)];
-        T dhiw[6];  // -(h^-1 d_m h h^-1), off-diagonals doubled
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = a; b < 3; ++b) {
-                const T x = Tm[a][0] * hi[sidx(0, b)] + Tm[a][1] * hi[sidx(1, b)] + Tm[a][2] * hi[sidx(2, b)];
-                dhiw[sidx(a, b)] = (a == b) ? -x : -2.0 * x;
-            }
-#pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            T s = sdotw(G1[l], dhiw);
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) s = fma(hi[sidx(i, j)], D2(F_H + sidx(l, j), sidx(m, i)), s);
-            dGl[m][l] = fma(-0.5, hdd[sidx(m, l)], s);
-        }
+            for (int n = 0; n < 3; ++n)
+                x = fma(G2[n][sidx(k, l)], G1[n][sidx(i, m)], fnma(G2[n][sidx(k, m)], G1[n][sidx(i, l)], x));
+            return x;
+        };
+        Rm[0] = riem(0, 1, 0, 1);
+        Rm[1] = riem(0, 1, 0, 2);
+        Rm[2] = riem(0, 1, 1, 2);
+        Rm[3] = riem(0, 2, 0, 2);
+        Rm[4] = riem(0, 2, 1, 2);
+        Rm[5] = riem(1, 2, 1, 2);
     }
 
     // ---- physical Christoffels Gp^k_ij = Gt^k_ij - (delta^k_i d_j chi + delta^k_j d_i chi - h_ij h^kl d_l chi)/(2 chi)
     GRF_SECTION(4);
+    const T hichi = half_of(ichi);
     T hidchi[3], c1[3], c2[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        hidchi[k] = hi[sidx(k, 0)] * dchi[0] + hi[sidx(k, 1)] * dchi[1] + hi[sidx(k, 2)] * dchi[2];
-        c1[k] = (0.5 * ichi) * dchi[k];
-        c2[k] = (0.5 * ichi) * hidchi[k];
+        hidchi[k] = dot3(hi[sidx(k, 0)], dchi[0], hi[sidx(k, 1)], dchi[1], hi[sidx(k, 2)], dchi[2]);
+        c1[k] = hichi * dchi[k];
+        c2[k] = hichi * hidchi[k];
     }
     T Gp[3][6];
 #pragma unroll
@@ -416,11 +443,70 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
                 Gp[k][sidx(i, j)] = t;
             }
 
-    // ---- plain Ricci tensor of gamma = h/chi:
-    // R_ij = -1/2 h^lm d_l d_m h_ij + d_(i Gl_j) - Gt^k Gt_kij
-    //        + h^lm (Gt^k_li Gt_jkm + Gt^k_lj Gt_ikm + Gt^k_im Gt_klj) + chi part
+    // ---- the chi part of the curvature of gamma = h/chi: with
+    //   T_ij = D~_i D~_j chi/(2 chi) - d_i chi d_j chi/(4 chi^2) - h_ij |d chi|^2/(8 chi^2) = Pc_ij + ch8 h_ij
+    // chi Riem_iklm = Rt_iklm + h_il T_km + h_km T_il - h_im T_kl - h_kl T_im.
     GRF_SECTION(5);
-    T Ric[6];
+    T Pc[6], chiLap, dchi2;
+    const T qichi2 = -(hichi * hichi);
+    {
+        T DDchi[6];
+#pragma unroll
+        for (int m = 0; m < 6; ++m)
+            DDchi[m] = fnma(G2[0][m], dchi[0], fnma(G2[1][m], dchi[1], fnma(G2[2][m], dchi[2], D2(F_CHI, m))));
+        chiLap = sdotw(DDchi, hw);
+        dchi2 = dot3(dchi[0], hidchi[0], dchi[1], hidchi[1], dchi[2], hidchi[2]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const T qd = qichi2 * dchi[i];
+#pragma unroll
+            for (int j = i; j < 3; ++j) Pc[sidx(i, j)] = fma(hichi, DDchi[sidx(i, j)], qd * dchi[j]);
+        }
+        const T ch8 = half_of(qichi2 * dchi2);
+        T Tc[6];
+#pragma unroll
+        for (int m = 0; m < 6; ++m) Tc[m] = fma(ch8, h[m], Pc[m]);
+        auto wedge = [&](int i, int k, int l, int m, T x) -> T {
+            if (i == l && k == m)
+                return fma(h[sidx(i, i)], Tc[sidx(k, k)], fma(h[sidx(k, k)], Tc[sidx(i, i)],
+                           fnma(twice_of(h[sidx(i, k)]), Tc[sidx(i, k)], x)));
+            x = fma(h[sidx(i, l)], Tc[sidx(k, m)], fma(h[sidx(k, m)], Tc[sidx(i, l)], x));
+            return fnma(h[sidx(i, m)], Tc[sidx(k, l)], fnma(h[sidx(k, l)], Tc[sidx(i, m)], x));
+        };
+        Rm[0] = wedge(0, 1, 0, 1, Rm[0]);
+        Rm[1] = wedge(0, 1, 0, 2, Rm[1]);
+        Rm[2] = wedge(0, 1, 1, 2, Rm[2]);
+        Rm[3] = wedge(0, 2, 0, 2, Rm[3]);
+        Rm[4] = wedge(0, 2, 1, 2, Rm[4]);
+        Rm[5] = wedge(1, 2, 1, 2, Rm[5]);
+    }
+    // the Einstein tensor is minus the double dual of Riemann, G^11 = -Riem_2323/det gamma and so on, so
+    // the scalar curvature -2 gamma_ij G^ij is (Rm holds chi Riem)
+    const T chidet = chi * ideth;
+    T Rs;
+    {
+        T dg = dot3(h[0], Rm[5], h[3], Rm[3], h[5], Rm[0]);
+        const T off = fnma(h[1], Rm[4], fnma(h[4], Rm[1], h[2] * Rm[2]));
+        dg = fma(2.0, off, dg);
+        Rs = twice_of(chidet) * dg;
+    }
+
+    // ---- Z terms: Zl_i = h_ik (Gamma-hat^k - Gt^k)/2, R^Z_ij = R_ij + D_i Z_j + D_j Z_i. Written out, the
+    // derivatives of Gt^k in R_ij and in D_(i Z_j) cancel, as do the Gt_kij Gt^k and Gt_kij Gamma-hat^k terms:
+    //   R^Z_ij = -1/2 h^lm d_l d_m h_ij + U^km_i d_m h_jk + U^km_j Gt_ikm + Gamma-hat^k d_k h_ij/2
+    //            + h_k(i d_j) Gamma-hat^k + chi part, U^km_i = h^lm Gt^k_li
+    GRF_SECTION(6);
+    T dG[3], Zl[3];
+    const T Gh[3] = {v[F_GAM], v[F_GAM + 1], v[F_GAM + 2]};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dG[k] = Gh[k] - Gtc[k];
+    {
+        const T hdG[3] = {half_of(dG[0]), half_of(dG[1]), half_of(dG[2])};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            Zl[i] = dot3(h[sidx(i, 0)], hdG[0], h[sidx(i, 1)], hdG[1], h[sidx(i, 2)], hdG[2]);
+    }
+    T RZ[6];
     {
         T U[3][3][3];  // U[k][m][i] = h^lm Gt^k_li
 #pragma unroll
@@ -429,79 +515,45 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             for (int m = 0; m < 3; ++m)
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
-                    U[k][m][i] = hi[sidx(0, m)] * G2[k][sidx(0, i)] + hi[sidx(1, m)] * G2[k][sidx(1, i)]
-                                 + hi[sidx(2, m)] * G2[k][sidx(2, i)];
-        T Q1[3][3];
+                    U[k][m][i] = dot3(hi[sidx(0, m)], G2[k][sidx(0, i)], hi[sidx(1, m)], G2[k][sidx(1, i)],
+                                      hi[sidx(2, m)], G2[k][sidx(2, i)]);
+        T mhw[6];
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+        for (int q = 0; q < 6; ++q) mhw[q] = half_of(hw[q]);
+        const T hGh[3] = {half_of(Gh[0]), half_of(Gh[1]), half_of(Gh[2])};
+        const T dGd = dot3(dG[0], dchi[0], dG[1], dchi[1], dG[2], dchi[2]);
+        const T chz = fma(hichi, chiLap - dGd, 3.0 * (qichi2 * dchi2));
+        const T dci[3] = {twice_of(c1[0]), twice_of(c1[1]), twice_of(c1[2])};  // d_i chi / chi
+        T hdGam[3][3];  // d_j Gamma-hat^k / 2
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                T s = 0.0;
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) hdGam[k][j] = half_of(D1(F_GAM + k, j));
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const T us01 = U[0][1][j] + U[1][0][j], us02 = U[0][2][j] + U[2][0][j], us12 = U[1][2][j] + U[2][1][j];
+#pragma unroll
+            for (int i = 0; i <= j; ++i) {
+                const int ij = sidx(i, j);
+                T r = fma(chz, h[ij], Pc[ij]);
+                r = fma(dci[i], Zl[j], fma(dci[j], Zl[i], r));
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    r = fma(hGh[k], dh[k][ij], r);
+                    if (i == j) r = fma(h[sidx(i, k)], D1(F_GAM + k, i), r);
+                    else r = fma(h[sidx(i, k)], hdGam[k][j], fma(h[sidx(j, k)], hdGam[k][i], r));
+                }
+                r = fma(U[0][0][j], G1[i][0], fma(us01, G1[i][1], fma(us02, G1[i][2], r)));
+                r = fma(U[1][1][j], G1[i][3], fma(us12, G1[i][4], fma(U[2][2][j], G1[i][5], r)));
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
 #pragma unroll
-                    for (int m = 0; m < 3; ++m)
-                        s = (k == 0 && m == 0) ? U[0][0][i] * G1[j][0] : fma(U[k][m][i], G1[j][sidx(k, m)], s);
-                Q1[i][j] = s;
+                    for (int m = 0; m < 3; ++m) r = fma(U[k][m][i], dh[m][sidx(j, k)], r);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) r = fnma(mhw[q], D2(F_H + ij, q), r);
+                RZ[ij] = r;
             }
-        T DDchi[6];
-#pragma unroll
-        for (int m = 0; m < 6; ++m)
-            DDchi[m] = D2(F_CHI, m) - G2[0][m] * dchi[0] - G2[1][m] * dchi[1] - G2[2][m] * dchi[2];
-        const T lapchi = sdotw(DDchi, hw);
-        const T dchi2 = dchi[0] * hidchi[0] + dchi[1] * hidchi[1] + dchi[2] * hidchi[2];
-        const T hichi = 0.5 * ichi, qichi2 = -0.25 * ichi * ichi;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) {
-                T r = Q1[i][j] + Q1[j][i] + 0.5 * (dGl[j][i] + dGl[i][j]);
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-#pragma unroll
-                    for (int l = 0; l < 3; ++l) r = fma(U[k][l][i], G1[k][sidx(l, j)], r);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) r = fma(-Gtc[k], G1[k][sidx(i, j)], r);
-#pragma unroll
-                for (int q = 0; q < 6; ++q) r = fma(-0.5 * hw[q], D2(F_H + sidx(i, j), q), r);
-                r = fma(hichi, fma(h[sidx(i, j)], lapchi, DDchi[sidx(i, j)]), r);
-                r = fma(qichi2, fma(3.0 * h[sidx(i, j)], dchi2, dchi[i] * dchi[j]), r);
-                Ric[sidx(i, j)] = r;
-            }
-    }
-    const T Rs = sdotw(Ric, gw);
-
-    // ---- Z terms: Zl_i = (h_ik Gamma-hat^k - Gl_i)/2, R^Z_ij = R_ij + D_i Z_j + D_j Z_i
-    GRF_SECTION(6);
-    T dG[3], Zl[3], Zu[3];
-    const T Gh[3] = {v[F_GAM], v[F_GAM + 1], v[F_GAM + 2]};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        dG[k] = Gh[k] - Gtc[k];
-        Zu[k] = (0.5 * chi) * dG[k];
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-        Zl[i] = 0.5 * (h[sidx(i, 0)] * Gh[0] + h[sidx(i, 1)] * Gh[1] + h[sidx(i, 2)] * Gh[2] - Gl[i]);
-    T RZ[6];
-    {
-        T dZ[3][3];  // dZ[j][i] = d_j Zl_i
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                T s = -dGl[j][i];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) s = fma(dh[j][sidx(i, k)], Gh[k], fma(h[sidx(i, k)], D1(F_GAM + k, j), s));
-                dZ[j][i] = 0.5 * s;
-            }
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) {
-                const T gz = Gp[0][sidx(i, j)] * Zl[0] + Gp[1][sidx(i, j)] * Zl[1] + Gp[2][sidx(i, j)] * Zl[2];
-                RZ[sidx(i, j)] = fma(-2.0, gz, Ric[sidx(i, j)] + (dZ[i][j] + dZ[j][i]));
-            }
+        }
     }
     const T RZs = sdotw(RZ, gw);
 
@@ -510,113 +562,109 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     T DDa[6], DDp[6];
 #pragma unroll
     for (int m = 0; m < 6; ++m) {
-        DDa[m] = D2(F_LAPSE, m) - Gp[0][m] * dal[0] - Gp[1][m] * dal[1] - Gp[2][m] * dal[2];
-        DDp[m] = D2(F_PHI, m) - Gp[0][m] * dphi[0] - Gp[1][m] * dphi[1] - Gp[2][m] * dphi[2];
+        DDa[m] = fnma(Gp[0][m], dal[0], fnma(Gp[1][m], dal[1], fnma(Gp[2][m], dal[2], D2(F_LAPSE, m))));
+        DDp[m] = fnma(Gp[0][m], dphi[0], fnma(Gp[1][m], dphi[1], fnma(Gp[2][m], dphi[2], D2(F_PHI, m))));
     }
     const T lapal = sdotw(DDa, gw);
 
-    // ---- extrinsic curvature K_ij = (A_ij + h_ij K/3)/chi and friends
+    // ---- extrinsic curvature K_ij = Ah_ij/chi, Ah_ij = A_ij + h_ij K/3, and friends
     GRF_SECTION(8);
     const T K3 = K * (1.0 / 3.0);
-    T Kp[6], Aud[3][3];
+    T Ah[6], Kp[6], Aud[3][3];
 #pragma unroll
-    for (int m = 0; m < 6; ++m) Kp[m] = fma(h[m], K3, A[m]) * ichi;
+    for (int m = 0; m < 6; ++m) {
+        Ah[m] = fma(h[m], K3, A[m]);
+        Kp[m] = Ah[m] * ichi;
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j)
-            Aud[i][j] = hi[sidx(i, 0)] * A[sidx(0, j)] + hi[sidx(i, 1)] * A[sidx(1, j)] + hi[sidx(i, 2)] * A[sidx(2, j)];
+            Aud[i][j] = dot3(hi[sidx(i, 0)], A[sidx(0, j)], hi[sidx(i, 1)], A[sidx(1, j)], hi[sidx(i, 2)], A[sidx(2, j)]);
     // K^i_j = A^i_j + delta^i_j K/3
-    auto Kud = [&](int i, int j) -> T { return i == j ? Aud[i][j] + K3 : Aud[i][j]; };
-    const T trK = K + Aud[0][0] + Aud[1][1] + Aud[2][2];
-    T Au[6];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j)
-            Au[sidx(i, j)] = Aud[i][0] * hi[sidx(0, j)] + Aud[i][1] * hi[sidx(1, j)] + Aud[i][2] * hi[sidx(2, j)];
-    const T AA = A[0] * Au[0] + A[3] * Au[3] + A[5] * Au[5] + 2.0 * (A[1] * Au[1] + A[2] * Au[2] + A[4] * Au[4]);
-    T KK[6];  // K_ik K^k_j
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j)
-            KK[sidx(i, j)] = Kp[sidx(i, 0)] * Kud(0, j) + Kp[sidx(i, 1)] * Kud(1, j) + Kp[sidx(i, 2)] * Kud(2, j);
-    T dKp[3][6];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const T dK3 = dK[k] * (1.0 / 3.0);
-#pragma unroll
-        for (int m = 0; m < 6; ++m)
-            dKp[k][m] = fma(-Kp[m], dchi[k], fma(dh[k][m], K3, fma(h[m], dK3, D1(F_A + m, k)))) * ichi;
-    }
-    T LbK[6];
+    const T Kdg[3] = {Aud[0][0] + K3, Aud[1][1] + K3, Aud[2][2] + K3};
+    auto Kud = [&](int i, int j) -> T { return i == j ? Kdg[i] : Aud[i][j]; };
+    T Au[6], Auw[6], AAud[6];  // A^ij, with off-diagonals doubled, A_ik A^k_j
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
             const int m = sidx(i, j);
-            T s = LOP ? fma(-Kp[m], adv[F_CHI], fma(adv[F_H + m], K3, fma(h[m], adv[F_K] * (1.0 / 3.0), adv[F_A + m]))) * ichi
-                      : bx * dKp[0][m] + by * dKp[1][m] + bz * dKp[2][m];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) s = fma(Kp[sidx(k, j)], db[i][k], fma(Kp[sidx(i, k)], db[j][k], s));
-            LbK[sidx(i, j)] = s;
+            Au[m] = dot3(Aud[i][0], hi[sidx(0, j)], Aud[i][1], hi[sidx(1, j)], Aud[i][2], hi[sidx(2, j)]);
+            Auw[m] = (i == j) ? Au[m] : twice_of(Au[m]);
+            AAud[m] = dot3(A[sidx(i, 0)], Aud[0][j], A[sidx(i, 1)], Aud[1][j], A[sidx(i, 2)], Aud[2][j]);
         }
+    const T AA = sdotw(A, Auw);
     // Codazzi block through its dual: bb[k][m] = B_{k,(m+1),(m+2)} = D_a K_kb - D_b K_ka with
-    // (a, b) = (m+1, m+2). The Gp^l_ab K_kl parts of the two covariant derivatives cancel (the
-    // connection is symmetric), leaving d_a K_kb - d_b K_ka - Gp^l_ak K_lb + Gp^l_bk K_la.
-    T bb[3][3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const int a = (m + 1) % 3, b = (m + 2) % 3;
-            T s = dKp[a][sidx(k, b)] - dKp[b][sidx(k, a)];
-#pragma unroll
-            for (int l = 0; l < 3; ++l)
-                s = fma(-Gp[l][sidx(a, k)], Kp[sidx(l, b)], fma(Gp[l][sidx(b, k)], Kp[sidx(l, a)], s));
-            bb[k][m] = s;
-        }
+    // (a, b) = (m+1, m+2). The connection's symmetric part cancels between the two covariant
+    // derivatives, and with K_ij = (A_ij + h_ij K/3)/chi (D~_a h_kb = 0) so do the derivatives of h:
+    //   chi B_kab = d_a A_kb - d_b A_ka - Gt^l_ak A_lb + Gt^l_bk A_la + h_kb e_a - h_ka e_b - q_a A_kb + q_b A_ka,
+    //   q_a = d_a chi/(2 chi), e_a = d_a K/3 + h^lm q_m A_la;
+    // the q terms are carried by the l = k Christoffels.
+    T bb[3][3], Bv[3];  // Bv_j = B_j = gamma^ab B_abj
 #define BC(k, i, j) (cyclic(i, j) ? bb[k][third(i, j)] : -bb[k][third(i, j)])
-    T Bv[3];  // B_j = gamma^ab B_abj
+#define BCFMA(B, k, i, j, x, s) (cyclic(i, j) ? fma(B[k][third(i, j)], x, s) : fnma(B[k][third(i, j)], x, s))
+    {
+        T ev[3], Gk[3][3], bx3[3][3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        T s = 0.0;
-        bool first = true;
+        for (int a = 0; a < 3; ++a) {
+            ev[a] = fma(c2[0], A[sidx(0, a)], fma(c2[1], A[sidx(1, a)], fma(c2[2], A[sidx(2, a)], dK[a] * (1.0 / 3.0))));
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+            for (int k = 0; k < 3; ++k) Gk[k][a] = G2[k][sidx(a, k)] + c1[a];
+        }
 #pragma unroll
-            for (int b = 0; b < 3; ++b)
-                if (b != j) {
-                    s = first ? gu[sidx(a, b)] * BC(a, b, j) : fma(gu[sidx(a, b)], BC(a, b, j), s);
-                    first = false;
-                }
-        Bv[j] = s;
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const int a = (m + 1) % 3, b = (m + 2) % 3;
+                T s = D1(F_A + sidx(k, b), a) - D1(F_A + sidx(k, a), b);
+                s = fma(h[sidx(k, b)], ev[a], fnma(h[sidx(k, a)], ev[b], s));
+#pragma unroll
+                for (int l = 0; l < 3; ++l)
+                    s = fnma(l == k ? Gk[k][a] : G2[l][sidx(a, k)], A[sidx(l, b)],
+                             fma(l == k ? Gk[k][b] : G2[l][sidx(b, k)], A[sidx(l, a)], s));
+                bx3[k][m] = s;
+                bb[k][m] = s * ichi;
+            }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int p = (j + 1) % 3, q = (j + 2) % 3;
+            T s = fnma(hi[sidx(j, p)], bx3[j][q], hi[sidx(j, q)] * bx3[j][p]);
+            s = fma(hi[sidx(q, q)], bx3[q][p], fnma(hi[sidx(p, p)], bx3[p][q], s));
+            s = fma(hi[sidx(p, q)], bx3[p][p], fnma(hi[sidx(p, q)], bx3[q][q], s));
+            Bv[j] = s;
+        }
     }
 
-    // ---- Gauss block S_ij and its Einstein tensor G_S
+    // ---- Gauss block S_iklm = Riem_iklm + K_il K_km - K_im K_kl: its contraction S_ij and the double
+    // dual G_S^ij (the raised Einstein tensor), both from the six components
     GRF_SECTION(9);
-    T S[6];
-#pragma unroll
-    for (int m = 0; m < 6; ++m) S[m] = fma(trK, Kp[m], Ric[m] - KK[m]);
+    Rm[0] = fma(Kp[0], Ah[3], fnma(Kp[1], Ah[1], Rm[0]));
+    Rm[1] = fma(Kp[0], Ah[4], fnma(Kp[2], Ah[1], Rm[1]));
+    Rm[2] = fma(Kp[1], Ah[4], fnma(Kp[2], Ah[3], Rm[2]));
+    Rm[3] = fma(Kp[0], Ah[5], fnma(Kp[2], Ah[2], Rm[3]));
+    Rm[4] = fma(Kp[1], Ah[5], fnma(Kp[2], Ah[4], Rm[4]));
+    Rm[5] = fma(Kp[3], Ah[5], fnma(Kp[4], Ah[4], Rm[5]));
+    T S[6], GSuw[6];
+    S[0] = dot3(hi[3], Rm[0], hw[4], Rm[1], hi[5], Rm[3]);
+    S[3] = fma(hi[0], Rm[0], fnma(hw[2], Rm[2], hi[5] * Rm[5]));
+    S[5] = dot3(hi[0], Rm[3], hw[1], Rm[4], hi[3], Rm[5]);
+    S[1] = fnma(hi[1], Rm[0], fnma(hi[2], Rm[1], fma(hi[4], Rm[2], hi[5] * Rm[4])));
+    S[2] = fnma(hi[1], Rm[1], fnma(hi[3], Rm[2], fnma(hi[2], Rm[3], fnma(hi[4], Rm[4], T(0.0)))));
+    S[4] = fnma(hi[2], Rm[4], fnma(hi[4], Rm[5], fma(hi[0], Rm[1], hi[1] * Rm[2])));
     const T Ss = sdotw(S, gw);
-    T GS[6], GSuw[6];
+    T GS[6];
+    const T hSs = half_of(Ss);
 #pragma unroll
-    for (int m = 0; m < 6; ++m) GS[m] = fma(-0.5 * Ss, gd[m], S[m]);
+    for (int m = 0; m < 6; ++m) GS[m] = fnma(hSs, gd[m], S[m]);
     {
-        T M1[3][3];  // gamma^ia G_S ab
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-                M1[i][b] = gu[sidx(i, 0)] * GS[sidx(0, b)] + gu[sidx(i, 1)] * GS[sidx(1, b)] + gu[sidx(i, 2)] * GS[sidx(2, b)];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) {
-                const T x = M1[i][0] * gu[sidx(0, j)] + M1[i][1] * gu[sidx(1, j)] + M1[i][2] * gu[sidx(2, j)];
-                GSuw[sidx(i, j)] = (i == j) ? x : 2.0 * x;  // G_S^ij, off-diagonals doubled
-            }
+        const T cd = chi * chidet, cd2 = twice_of(cd);  // off-diagonals doubled
+        GSuw[0] = fnma(cd, Rm[5], T(0.0));
+        GSuw[3] = fnma(cd, Rm[3], T(0.0));
+        GSuw[5] = fnma(cd, Rm[0], T(0.0));
+        GSuw[1] = cd2 * Rm[4];
+        GSuw[2] = fnma(cd2, Rm[2], T(0.0));
+        GSuw[4] = cd2 * Rm[1];
     }
 
     // ---- scalar: nabla nabla phi blocks, Phi = nabla nabla beta(phi)
@@ -636,15 +684,18 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     }
     T dphiu[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) dphiu[i] = gu[sidx(i, 0)] * dphi[0] + gu[sidx(i, 1)] * dphi[1] + gu[sidx(i, 2)] * dphi[2];
-    const T dphi2 = dphi[0] * dphiu[0] + dphi[1] * dphiu[1] + dphi[2] * dphiu[2];
-    const T X = 0.5 * (Pi * Pi - dphi2);
+    for (int i = 0; i < 3; ++i)
+        dphiu[i] = dot3(gu[sidx(i, 0)], dphi[0], gu[sidx(i, 1)], dphi[1], gu[sidx(i, 2)], dphi[2]);
+    const T dphi2 = dot3(dphi[0], dphiu[0], dphi[1], dphiu[1], dphi[2], dphiu[2]);
+    const T Pi2 = Pi * Pi;
+    const T X = half_of(Pi2 - dphi2);
     const T g2 = c.g2;
     T Hij[6], Hn[3];
 #pragma unroll
     for (int m = 0; m < 6; ++m) Hij[m] = fma(Kp[m], Pi, DDp[m]);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) Hn[i] = dPi[i] + Kud(0, i) * dphi[0] + Kud(1, i) * dphi[1] + Kud(2, i) * dphi[2];
+    for (int i = 0; i < 3; ++i)
+        Hn[i] = fma(Kud(0, i), dphi[0], fma(Kud(1, i), dphi[1], fma(Kud(2, i), dphi[2], dPi[i])));
     T Phd[6], Phn[3];
     const T b2Pi = b2 * Pi;
 #pragma unroll
@@ -659,15 +710,15 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            Phm[i][k] = Phd[sidx(i, 0)] * gu[sidx(0, k)] + Phd[sidx(i, 1)] * gu[sidx(1, k)] + Phd[sidx(i, 2)] * gu[sidx(2, k)];
+            Phm[i][k] = dot3(Phd[sidx(i, 0)], gu[sidx(0, k)], Phd[sidx(i, 1)], gu[sidx(1, k)], Phd[sidx(i, 2)], gu[sidx(2, k)]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
 #pragma unroll
         for (int j = i; j < 3; ++j) {
-            const T x = gu[sidx(i, 0)] * Phm[0][j] + gu[sidx(i, 1)] * Phm[1][j] + gu[sidx(i, 2)] * Phm[2][j];
-            Phuw[sidx(i, j)] = (i == j) ? x : 2.0 * x;
+            const T x = dot3(gu[sidx(i, 0)], Phm[0][j], gu[sidx(i, 1)], Phm[1][j], gu[sidx(i, 2)], Phm[2][j]);
+            Phuw[sidx(i, j)] = (i == j) ? x : twice_of(x);
         }
-        Phnu[i] = gu[sidx(i, 0)] * Phn[0] + gu[sidx(i, 1)] * Phn[1] + gu[sidx(i, 2)] * Phn[2];
+        Phnu[i] = dot3(gu[sidx(i, 0)], Phn[0], gu[sidx(i, 1)], Phn[1], gu[sidx(i, 2)], Phn[2]);
     }
     const T trP = Phm[0][0] + Phm[1][1] + Phm[2][2];
 
@@ -678,68 +729,63 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     // decoupled mode: the scalar's stress-energy is left out of the metric equations (rho, S_i,
     // S_ij and their coupling to d_t K_ij); the scalar equation below is unchanged
     const bool dec = (DEC < 0) ? (c.decoupled != 0) : (DEC == 1);
-    T rho8 = dec ? T(0.0) : fma(0.5 * fX, Pi * Pi, fma(-4.0, sdotw(GS, Phuw), -0.5 * XX));
+    const T fXh = half_of(fX), XXh = half_of(XX);
+    T rho8 = dec ? T(0.0) : fma(fXh, Pi2, fma(-4.0, sdotw(GS, Phuw), -XXh));
     T S8[3];
-    const T BPn = Bv[0] * Phnu[0] + Bv[1] * Phnu[1] + Bv[2] * Phnu[2];
+    const T BPn = dot3(Bv[0], Phnu[0], Bv[1], Phnu[1], Bv[2], Phnu[2]);
+    T Phuh[6];  // Phi^ij
+#pragma unroll
+    for (int m = 0; m < 6; ++m) Phuh[m] = (m == 1 || m == 2 || m == 4) ? half_of(Phuw[m]) : Phuw[m];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        T s = GS[sidx(i, 0)] * Phnu[0] + GS[sidx(i, 1)] * Phnu[1] + GS[sidx(i, 2)] * Phnu[2];
-        s = fma(trP, Bv[i], s - (Phm[i][0] * Bv[0] + Phm[i][1] * Bv[1] + Phm[i][2] * Bv[2]));
+        T s = dot3(GS[sidx(i, 0)], Phnu[0], GS[sidx(i, 1)], Phnu[1], GS[sidx(i, 2)], Phnu[2]);
+        s = fma(trP, Bv[i], fnma(Phm[i][0], Bv[0], fnma(Phm[i][1], Bv[1], fnma(Phm[i][2], Bv[2], s))));
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int l = 0; l < 3; ++l)
-                if (l != i) {
-                    const T pkl = (k == l) ? Phuw[sidx(k, l)] : 0.5 * Phuw[sidx(k, l)];
-                    s = fma(BC(k, i, l), pkl, s);
-                }
-        S8[i] = dec ? T(0.0) : fma(-0.5 * fX * Pi, dphi[i], 4.0 * s);
+                if (l != i) s = BCFMA(bb, k, i, l, Phuh[sidx(k, l)], s);
+        S8[i] = dec ? T(0.0) : fnma(fXh * Pi, dphi[i], 4.0 * s);
     }
     // cubic term: the n-n and n-i parts of its stress tensor (no unknown in them)
     const bool cub = COUP && c.g3 != 0.0;
     T trH3 = 0.0, Hnd3 = 0.0, Hdd3 = 0.0, Hdv3[3];
     if (cub) {
         trH3 = sdotw(Hij, gw);
-        Hnd3 = dphiu[0] * Hn[0] + dphiu[1] * Hn[1] + dphiu[2] * Hn[2];
+        Hnd3 = dot3(dphiu[0], Hn[0], dphiu[1], Hn[1], dphiu[2], Hn[2]);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            Hdv3[i] = Hij[sidx(i, 0)] * dphiu[0] + Hij[sidx(i, 1)] * dphiu[1] + Hij[sidx(i, 2)] * dphiu[2];
-        Hdd3 = dphiu[0] * Hdv3[0] + dphiu[1] * Hdv3[1] + dphiu[2] * Hdv3[2];
+            Hdv3[i] = dot3(Hij[sidx(i, 0)], dphiu[0], Hij[sidx(i, 1)], dphiu[1], Hij[sidx(i, 2)], dphiu[2]);
+        Hdd3 = dot3(dphiu[0], Hdv3[0], dphiu[1], Hdv3[1], dphiu[2], Hdv3[2]);
         if (!dec) {
             const double g3h = 0.5 * c.g3;
-            rho8 = fma(g3h, fma(Pi * Pi, trH3, -Hdd3), rho8);
+            rho8 = fma(g3h, fma(Pi2, trH3, -Hdd3), rho8);
             const T a3 = fma(Pi, trH3, -Hnd3);
 #pragma unroll
             for (int i = 0; i < 3; ++i) S8[i] = fma(-g3h, fma(a3, dphi[i], Pi * fma(Pi, Hn[i], -Hdv3[i])), S8[i]);
         }
     }
     T S1[6], Y[6];
-    const T fXh = 0.5 * fX, XXh = 0.5 * XX;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
             S1[sidx(i, j)] = dec ? T(0.0) : fma(fXh * dphi[i], dphi[j], XXh * gd[sidx(i, j)]);
             T y = fma(Bv[j], Phn[i], Bv[i] * Phn[j]);
-            y = fma(-2.0 * BPn, gd[sidx(i, j)], y);
+            y = fnma(twice_of(BPn), gd[sidx(i, j)], y);
 #pragma unroll
             for (int l = 0; l < 3; ++l) {
-                if (l != j) y = fma(BC(i, j, l), Phnu[l], y);
-                if (l != i) y = fma(BC(j, i, l), Phnu[l], y);
+                if (l != j) y = BCFMA(bb, i, j, l, Phnu[l], y);
+                if (l != i) y = BCFMA(bb, j, i, l, Phnu[l], y);
             }
             Y[sidx(i, j)] = dec ? T(0.0) : y;
         }
 
-    // C0 = C at d_t K_ij = 0
     GRF_SECTION(12);
-    T C0[6];
-#pragma unroll
-    for (int m = 0; m < 6; ++m) C0[m] = fma(DDa[m] - LbK[m], ial, KK[m]);
-    const T bdPi = LOP ? adv[F_PI] : bx * dPi[0] + by * dPi[1] + bz * dPi[2];
-    const T dadp = dal[0] * dphiu[0] + dal[1] * dphiu[1] + dal[2] * dphiu[2];
-    const T Phnn0 = fma(b1 * ial, -(bdPi + dadp), b2Pi * Pi);
+    const T bdPi = LOP ? adv[F_PI] : dot3(bx, dPi[0], by, dPi[1], bz, dPi[2]);
+    const T dadp = dot3(dal[0], dphiu[0], dal[1], dphiu[1], dal[2], dphiu[2]);
 
-    // L_GB at d_t K_ij = 0: 8 G_S^ij C_ij - 4 B_kij B^kij + 8 B_i B^i, with
+    // L_GB without its 8 G_S^ij C_ij: -4 B_kij B^kij + 8 B_i B^i, with
     // B_kij B^kij = 2 chi^3 / det(h) h^kk' h_mm' bb[k][m] bb[k'][m']
     GRF_SECTION(13);
     T L0;
@@ -749,156 +795,165 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int q = 0; q < 3; ++q)
-                N[k][q] = h[sidx(0, q)] * bb[k][0] + h[sidx(1, q)] * bb[k][1] + h[sidx(2, q)] * bb[k][2];
+                N[k][q] = dot3(h[sidx(0, q)], bb[k][0], h[sidx(1, q)], bb[k][1], h[sidx(2, q)], bb[k][2]);
         T tt[6];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
-            for (int kk = k; kk < 3; ++kk) tt[sidx(k, kk)] = N[k][0] * bb[kk][0] + N[k][1] * bb[kk][1] + N[k][2] * bb[kk][2];
-        const T BB = (2.0 * chi * chi * chi * ideth) * sdotw(tt, hw);
-        const T Bvu0 = gu[0] * Bv[0] + gu[1] * Bv[1] + gu[2] * Bv[2];
-        const T Bvu1 = gu[1] * Bv[0] + gu[3] * Bv[1] + gu[4] * Bv[2];
-        const T Bvu2 = gu[2] * Bv[0] + gu[4] * Bv[1] + gu[5] * Bv[2];
-        const T BvBv = Bv[0] * Bvu0 + Bv[1] * Bvu1 + Bv[2] * Bvu2;
-        L0 = fma(8.0, sdotw(C0, GSuw), fma(-4.0, BB, 8.0 * BvBv));
+            for (int kk = k; kk < 3; ++kk)
+                tt[sidx(k, kk)] = dot3(N[k][0], bb[kk][0], N[k][1], bb[kk][1], N[k][2], bb[kk][2]);
+        const T BB = (chi * (chi * chidet)) * sdotw(tt, hw);  // half of B_kij B^kij
+        const T Bvu0 = dot3(gu[0], Bv[0], gu[1], Bv[1], gu[2], Bv[2]);
+        const T Bvu1 = dot3(gu[1], Bv[0], gu[3], Bv[1], gu[4], Bv[2]);
+        const T Bvu2 = dot3(gu[2], Bv[0], gu[4], Bv[1], gu[5], Bv[2]);
+        const T BvBv = dot3(Bv[0], Bvu0, Bv[1], Bvu1, Bv[2], Bvu2);
+        L0 = 8.0 * (BvBv - BB);
     }
 
     // ---- CCZ4 right-hand sides without S_ij (rho and S_i included)
     GRF_SECTION(14);
-    rhs[F_CHI] = fma((2.0 / 3.0) * chi, al * K - divb, ADV(F_CHI));
+    rhs[F_CHI] = fma((2.0 / 3.0) * chi, fma(al, K, -divb), ADV(F_CHI));
     const T divb23 = (2.0 / 3.0) * divb;
-    const T al2 = 2.0 * al;
+    const T al2 = twice_of(al);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
-            T x = fma(-h[sidx(i, j)], divb23, fma(-al2, A[sidx(i, j)], ADV(F_H + sidx(i, j))));
+            T x = fnma(h[sidx(i, j)], divb23, fnma(al2, A[sidx(i, j)], ADV(F_H + sidx(i, j))));
+            if (i == j) {
+                x = fma(2.0, dot3(h[sidx(i, 0)], db[i][0], h[sidx(i, 1)], db[i][1], h[sidx(i, 2)], db[i][2]), x);
+            } else {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) x = fma(h[sidx(i, k)], db[j][k], fma(h[sidx(j, k)], db[i][k], x));
+                for (int k = 0; k < 3; ++k) x = fma(h[sidx(i, k)], db[j][k], fma(h[sidx(j, k)], db[i][k], x));
+            }
             rhs[F_H + sidx(i, j)] = x;
         }
-    const T K2Th = K - 2.0 * Th;
+    const T K2Th = K - twice_of(Th);
     // b(x) of the modified gauge enters through the auxiliary metric g^ab - b n^a n^b of the Z terms
     // of the covariant equation; its 3+1 projection is carried by Hb = H - 16 pi rho
     // - 2 kappa1 (2 + kappa2) Theta (plain H = R - A_ij A^ij + 2/3 K^2) in d_t K and d_t Theta, and
     // by the momentum-constraint combination in d_t Gamma-hat below.
-    const T Hb = fma(-2.0 * c.kappa1 * (2.0 + c.kappa2), Th, Rs - AA + (2.0 / 3.0) * K * K - 2.0 * rho8);
-    const T Kdot0 = ADV(F_K) + al * fma(K, K2Th, RZs) - (3.0 * c.kappa1 * (1.0 + c.kappa2)) * al * Th - lapal
-                    - 1.5 * al * rho8 - (c.bK * al) * Hb;
+    const T Hb = fma(-2.0 * c.kappa1 * (2.0 + c.kappa2), Th, fma(-2.0, rho8, fma((2.0 / 3.0) * K, K, Rs - AA)));
+    // kS: (d_t K without advection, the lapse's Laplacian, alpha R^Z and S_ij) / alpha
+    const T kS = fma(K, K2Th, fma(-3.0 * c.kappa1 * (1.0 + c.kappa2), Th, fma(-1.5, rho8, -c.bK * Hb)));
+    const T Kdot0 = fma(al, kS + RZs, ADV(F_K) - lapal);
     T Adot0[6];
     {
         T Xa[6];
 #pragma unroll
         for (int m = 0; m < 6; ++m) Xa[m] = fma(al, RZ[m], -DDa[m]);
         const T trX3 = sdotw(Xa, hw) * (1.0 / 3.0);
-        const T alK2Th = al * K2Th;
+        const T aA = fma(al, K2Th, -divb23);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = i; j < 3; ++j) {
-                T x = fma(chi, fma(-h[sidx(i, j)], trX3, Xa[sidx(i, j)]), ADV(F_A + sidx(i, j)));
-                x = fma(alK2Th - divb23, A[sidx(i, j)], x);
+                const int m = sidx(i, j);
+                T x = fma(chi, fnma(h[m], trX3, Xa[m]), ADV(F_A + m));
+                x = fma(aA, A[m], fnma(al2, AAud[m], x));
+                if (i == j) {
+                    x = fma(2.0, dot3(A[sidx(i, 0)], db[i][0], A[sidx(i, 1)], db[i][1], A[sidx(i, 2)], db[i][2]), x);
+                } else {
 #pragma unroll
-                for (int k = 0; k < 3; ++k)
-                    x = fma(A[sidx(i, k)], fma(-al2, Aud[k][j], db[j][k]), fma(A[sidx(j, k)], db[i][k], x));
-                Adot0[sidx(i, j)] = x;
+                    for (int k = 0; k < 3; ++k) x = fma(A[sidx(i, k)], db[j][k], fma(A[sidx(j, k)], db[i][k], x));
+                }
+                Adot0[m] = x;
             }
     }
     // d_t Theta = beta.dTheta + alpha (D_i Z^i - Theta K) - Z^i d_i alpha + alpha Hb / (2 (1 + b)),
-    // with 2 D_i Z^i = RZs - Rs
-    rhs[F_TH] = ADV(F_TH) + al * fma(0.5, RZs - Rs, -Th * K) - (Zu[0] * dal[0] + Zu[1] * dal[1] + Zu[2] * dal[2])
-                + (c.bTh * al) * Hb;
+    // with 2 D_i Z^i = RZs - Rs and Z^i = chi (Gamma-hat^i - Gt^i)/2
     {
-        T hZ[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) hZ[i] = hi[sidx(i, 0)] * Zl[0] + hi[sidx(i, 1)] * Zl[1] + hi[sidx(i, 2)] * Zl[2];
-        T ddbk[3];  // sum_k d_j d_k beta^k
-#pragma unroll
-        for (int j = 0; j < 3; ++j) ddbk[j] = D2(F_SHIFT, sidx(j, 0)) + D2(F_SHIFT + 1, sidx(j, 1)) + D2(F_SHIFT + 2, sidx(j, 2));
-        T Auw[6];
-#pragma unroll
-        for (int m = 0; m < 6; ++m) Auw[m] = (m == 1 || m == 2 || m == 4) ? 2.0 * Au[m] : Au[m];
-        T tk[3];  // 2 (al d_k Theta - Theta d_k al - 2/3 al K Z_k)
-        const T alK23 = (2.0 / 3.0) * al * K;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) tk[k] = 2.0 * fma(al, dTh[k], fma(-Th, dal[k], -alK23 * Zl[k]));
-        const T k3div = (4.0 / 3.0) * c.kappa3 * divb;
-        const T ak1 = 2.0 * al * c.kappa1;
-        // b(x) part of d_t Z_j: -(b/(1+b)) alpha wb_j, wb_j = M_j + d_j Theta - K^k_j Z_k - kappa1 Z_j with
-        // the momentum constraint M_j = B_j - 8 pi S_j; Gamma-hat^i carries 2 h^ij Z_j, so d_t Gamma-hat^i
-        // gains -(2b/(1+b)) alpha h^ij wb_j (2b/(1+b) = 2 - 4 bTh)
-        T wb[3];
+        const T Zda = half_of(chi) * dot3(dG[0], dal[0], dG[1], dal[1], dG[2], dal[2]);
+        rhs[F_TH] = fma(al, fma(c.bTh, Hb, fnma(Th, K, half_of(RZs - Rs))), ADV(F_TH) - Zda);
+    }
+    {
+        // d_t Gamma-hat^i with everything contracted with h^ij in one covector V_j, with A^ij in va_j and
+        // with d_k beta^i in Gk: h^ij Z_j = (Gamma-hat^i - Gt^i)/2. The b(x) part of d_t Z_j is
+        // -(b/(1+b)) alpha wb_j, wb_j = M_j + d_j Theta - K^k_j Z_k - kappa1 Z_j with the momentum constraint
+        // M_j = B_j - 8 pi S_j; Gamma-hat^i carries 2 h^ij Z_j, so d_t Gamma-hat^i gains
+        // -(2b/(1+b)) alpha h^ij wb_j (2b/(1+b) = 2 - 4 bTh)
+        const T abG = (2.0 - 4.0 * c.bTh) * al;
+        const T m3 = -3.0 * (al * ichi), alK43 = (4.0 / 3.0) * (al * K), al43 = (4.0 / 3.0) * al, Th2 = twice_of(Th);
+        const T cTh = al2 - abG, cZ = fma(abG, c.kappa1, -alK43);
+        T va[3], V[3], Gk[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            T s = (Bv[j] - S8[j]) + dTh[j];
-            s = fma(-c.kappa1, Zl[j], s);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) s = fma(-Kud(k, j), Zl[k], s);
-            wb[j] = s;
+            va[j] = fma(m3, dchi[j], -2.0 * dal[j]);
+            Gk[j] = fma(c.kappa3, dG[j], Gtc[j]);
+            const T ddbk = D2(F_SHIFT, sidx(j, 0)) + D2(F_SHIFT + 1, sidx(j, 1)) + D2(F_SHIFT + 2, sidx(j, 2));
+            const T kz = dot3(Kud(0, j), Zl[0], Kud(1, j), Zl[1], Kud(2, j), Zl[2]);
+            T x = fma(1.0 / 3.0, ddbk, fma(cTh, dTh[j] - S8[j], cZ * Zl[j]));
+            x = fnma(Th2, dal[j], fnma(al43, dK[j], x));
+            V[j] = fma(abG, kz - Bv[j], x);
         }
-        const T abG = (2.0 - 4.0 * c.bTh) * al;
+        const T kz2 = fma((2.0 / 3.0) * c.kappa3, divb, -(c.kappa1 * al));
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const T t1 = sdotw(G2[i], Auw);
-            const T t2 = Au[sidx(i, 0)] * dchi[0] + Au[sidx(i, 1)] * dchi[1] + Au[sidx(i, 2)] * dchi[2];
-            const T t3 = hi[sidx(i, 0)] * dK[0] + hi[sidx(i, 1)] * dK[1] + hi[sidx(i, 2)] * dK[2];
-            const T t4 = Au[sidx(i, 0)] * dal[0] + Au[sidx(i, 1)] * dal[1] + Au[sidx(i, 2)] * dal[2];
-            T t5 = 0.0;
-#pragma unroll
-            for (int q = 0; q < 6; ++q) t5 = (q == 0) ? hw[0] * D2(F_SHIFT + i, 0) : fma(hw[q], D2(F_SHIFT + i, q), t5);
-            const T t6 = hZ[0] * db[0][i] + hZ[1] * db[1][i] + hZ[2] * db[2][i];
-            T x = ADV(F_GAM + i) + al2 * (t1 - (1.5 * ichi) * t2 - (2.0 / 3.0) * t3) - 2.0 * t4 + t5;
+            T x = fma(al2, sdotw(G2[i], Auw), ADV(F_GAM + i));
+            x = fma(kz2, dG[i], fma(divb23, Gtc[i], x));
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                x = fma(hi[sidx(k, i)], fma(1.0 / 3.0, ddbk[k], tk[k]), x);
-                x = fma(-Gtc[k], db[k][i], x);
+                x = fma(Au[sidx(i, k)], va[k], x);
+                x = fma(hi[sidx(i, k)], V[k], x);
+                x = fnma(Gk[k], db[k][i], x);
             }
-            x = fma((2.0 / 3.0) * divb, Gtc[i], x);
-            x = fma(k3div - ak1, hZ[i], x);
-            x = fma(-2.0 * c.kappa3, t6, x);
-            x = fma(-al2, hi[sidx(i, 0)] * S8[0] + hi[sidx(i, 1)] * S8[1] + hi[sidx(i, 2)] * S8[2], x);
-            x = fma(-abG, hi[sidx(i, 0)] * wb[0] + hi[sidx(i, 1)] * wb[1] + hi[sidx(i, 2)] * wb[2], x);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) x = fma(hw[q], D2(F_SHIFT + i, q), x);
             rhs[F_GAM + i] = x;
             rhs[F_B + i] = fma(-c.eta, v[F_B + i], x);
             rhs[F_SHIFT + i] = fma(c.shift_F * c.inv_1pa, v[F_B + i],
-                                   -(c.a_1pa * al * chi) * (hi[sidx(i, 0)] * dal[0] + hi[sidx(i, 1)] * dal[1] + hi[sidx(i, 2)] * dal[2]));
+                                   -((c.a_1pa * al * chi) * dot3(hi[sidx(i, 0)], dal[0], hi[sidx(i, 1)], dal[1],
+                                                                 hi[sidx(i, 2)], dal[2])));
         }
     }
     rhs[F_LAPSE] = fma(-2.0 * c.inv_1pa * al, K2Th, ADV(F_LAPSE));
     rhs[F_PHI] = fma(al, Pi, ADV(F_PHI));
 
-    // ---- coupled system for v = (d_t K_ij, d_t Pi):
-    //   u - 4 L(Q(u)) - 4 b1 L(G_S) w = r,   w - (8 b1 / D) G_S^ij u_ij = r_w,   L(X) = X - gamma tr(X)/2
+    // ---- coupled system, in the curvature components that hold the unknowns: C_ij = R_ninj (d_t K_ij) and
+    // N = H_nn = (d_t Pi - beta^k d_k Pi - d^k alpha d_k phi)/alpha (d_t Pi):
+    //   C - 4 L(Q(C)) - 4 b1 L(G_S) N = r,   N - (8 b1 / D) G_S^ij C_ij = r_N,   L(X) = X - gamma tr(X)/2.
+    // Without S_ij, C = R^Z + (K - 2 Theta) K_ij - K_ik K^k_j + a trace: the lapse's derivatives and every
+    // shift term of d_t K_ij cancel in it.
     GRF_SECTION(15);
     T Msys[7][8];
-    T S3[6], PPc[6], HnnSol0 = 0.0;  // cubic term: 8 pi S3_ij without d_t Pi, Pi^2 gamma^ij - d^i phi d^j phi
-    T QC0[6];
-    q_of(C0, gd, gw, Phd, Phuw, Phm, trP, QC0);
+    T S3[6], PPc[6];  // cubic term: 8 pi S3_ij without N, Pi^2 gamma^ij - d^i phi d^j phi
     {
-        const T chid = rhs[F_CHI];
-        const T trS1h = 0.5 * sdotw(S1, gw), trYh = 0.5 * sdotw(Y, gw), trQh = 0.5 * sdotw(QC0, gw);
+        const T a1 = fma(-2.0 / 3.0, K, K2Th);
+        const T a0 = (1.0 / 3.0) * fma((-1.0 / 3.0) * K, K, kS);
+        const T trS1h = half_of(sdotw(S1, gw)), trYh = half_of(sdotw(Y, gw));
         const T Ss4 = 0.25 * Ss;
-        const T al4 = 4.0 * al;
-        const T four_b1 = 4.0 * b1;
+        const T four_b1 = 4.0 * b1, b2Pi2x4 = 4.0 * (b2Pi * Pi);
 #pragma unroll
         for (int m = 0; m < 6; ++m) {
-            const T LGS = fma(-Ss4, gd[m], S[m]);
-            const T U0 = fma(-Kp[m], chid, fma(rhs[F_H + m], K3, fma(h[m], Kdot0 * (1.0 / 3.0), Adot0[m]))) * ichi;
-            const T lin = dec ? T(0.0) : fma(LGS, Phnn0, (Y[m] + QC0[m]) - gd[m] * (trYh + trQh));
-            Msys[m][7] = fma(al4, lin, fma(-al, fma(-trS1h, gd[m], S1[m]), U0));
-            Msys[m][6] = dec ? T(0.0) : -four_b1 * LGS;
+            T r = fma(ichi, fma(a1, A[m], fma(a0, h[m], -AAud[m])), RZ[m]);
+            T w6 = T(0.0);
+            if (!dec) {
+                const T LGS = fnma(Ss4, gd[m], S[m]);
+                r = r - fnma(trS1h, gd[m], S1[m]);
+                r = fma(4.0, fnma(trYh, gd[m], Y[m]), fma(b2Pi2x4, LGS, r));
+                w6 = fnma(four_b1, LGS, T(0.0));
+            }
+            Msys[m][7] = r;
+            Msys[m][6] = w6;
         }
         // 6x6 block, column (a,b): -4 L(Q(E_ab)) with E_ab the unit symmetric matrix
         //   = -2 gamma_ij w_ab (Phi^ab - gamma^ab tr Phi) - 4 w_ab gamma^ab Phi_ij + 4 P_ij,ab - 4 tr(Phi) [ij == ab]
         //   P_ij,ab = Phi_i^k E_kj + Phi_j^k E_ik
         const T one4P = fma(-4.0, trP, 1.0);
+        T gd2[6], Ph4[3][3];
+#pragma unroll
+        for (int m = 0; m < 6; ++m) gd2[m] = twice_of(gd[m]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) Ph4[i][k] = twice_of(twice_of(Phm[i][k]));
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int b = a; b < 3; ++b) {
                 const int col = sidx(a, b);
-                const T sab = Phuw[col] - gw[col] * trP;   // w_ab (Phi^ab - gamma^ab trP)
-                const T tab = -4.0 * gw[col];               // -4 w_ab gamma^ab
+                const T sab = fnma(gw[col], trP, Phuw[col]);    // w_ab (Phi^ab - gamma^ab trP)
+                const T tab = twice_of(twice_of(gw[col]));      // 4 w_ab gamma^ab
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -906,28 +961,33 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
                         const int row = sidx(i, j);
                         T p = 0.0;
                         bool any = false;
-                        // Phi_i^k E_kj: E_kj = [k==a][j==b] + [k==b][j==a] (single term when a == b)
-                        if (j == b) { p = any ? p + Phm[i][a] : Phm[i][a]; any = true; }
-                        if (a != b && j == a) { p = any ? p + Phm[i][b] : Phm[i][b]; any = true; }
-                        if (i == b) { p = any ? p + Phm[j][a] : Phm[j][a]; any = true; }
-                        if (a != b && i == a) { p = any ? p + Phm[j][b] : Phm[j][b]; any = true; }
-                        T e = fma(-2.0 * gd[row], sab, tab * Phd[row]);
-                        if (any) e = fma(4.0, p, e);
-                        if (row == col) e = e + one4P;
+                        // 4 Phi_i^k E_kj: E_kj = [k==a][j==b] + [k==b][j==a] (single term when a == b)
+                        if (j == b && i == j) { p = twice_of(Ph4[i][a]); any = true; }
+                        else {
+                            if (j == b) { p = Ph4[i][a]; any = true; }
+                            if (i == b) { p = any ? p + Ph4[j][a] : Ph4[j][a]; any = true; }
+                        }
+                        if (a != b && j == a && i == j) { p = any ? p + twice_of(Ph4[i][b]) : twice_of(Ph4[i][b]); any = true; }
+                        else if (a != b) {
+                            if (j == a) { p = any ? p + Ph4[i][b] : Ph4[i][b]; any = true; }
+                            if (i == a) { p = any ? p + Ph4[j][b] : Ph4[j][b]; any = true; }
+                        }
+                        if (row == col) { p = any ? p + one4P : one4P; any = true; }
+                        T e = any ? fnma(tab, Phd[row], p) : fnma(tab, Phd[row], T(0.0));
+                        e = fnma(gd2[row], sab, e);
                         Msys[row][col] = dec ? T(row == col ? 1.0 : 0.0) : e;
                     }
             }
-        T Dphi = fma(2.0 * g2, Pi * Pi, fX);
-        T E3 = 0.0;  // the cubic term's share of the scalar equation without H_nn and d_t K_ij
+        T Dphi = fma(2.0 * g2, Pi2, fX);
+        T E3 = 0.0;  // the cubic term's share of the scalar equation without N and C
         if (cub) {
             Dphi = fma(2.0 * c.g3, trH3, Dphi);
-            const T Hnn0 = -(bdPi + dadp) * ial;
             T Hm[3][3], ppw[6], PPuw[6];  // H_i^k, d^i phi d^j phi and Pi^2 gamma^ij - d^i phi d^j phi (weighted)
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
-                    Hm[i][k] = Hij[sidx(i, 0)] * gu[sidx(0, k)] + Hij[sidx(i, 1)] * gu[sidx(1, k)] + Hij[sidx(i, 2)] * gu[sidx(2, k)];
+                    Hm[i][k] = dot3(Hij[sidx(i, 0)], gu[sidx(0, k)], Hij[sidx(i, 1)], gu[sidx(1, k)], Hij[sidx(i, 2)], gu[sidx(2, k)]);
             T HH = 0.0;
 #pragma unroll
             for (int i = 0; i < 3; ++i)
@@ -936,53 +996,51 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             T HnHn = 0.0, BdP = 0.0;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const T hnu = gu[sidx(i, 0)] * Hn[0] + gu[sidx(i, 1)] * Hn[1] + gu[sidx(i, 2)] * Hn[2];
+                const T hnu = dot3(gu[sidx(i, 0)], Hn[0], gu[sidx(i, 1)], Hn[1], gu[sidx(i, 2)], Hn[2]);
                 HnHn = fma(Hn[i], hnu, HnHn);
                 BdP = fma(Bv[i], dphiu[i], BdP);
             }
-            const T Pi2 = Pi * Pi;
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
                 for (int j = i; j < 3; ++j) {
                     const T pp = dphiu[i] * dphiu[j];
-                    ppw[sidx(i, j)] = (i == j) ? pp : 2.0 * pp;
+                    ppw[sidx(i, j)] = (i == j) ? pp : twice_of(pp);
                     PPuw[sidx(i, j)] = fma(Pi2, gw[sidx(i, j)], -ppw[sidx(i, j)]);
                 }
             T e3 = fma(trH3, trH3, fma(2.0, HnHn, -HH));
             e3 = fma(-2.0 * Pi, BdP, e3);
-            e3 = e3 - sdotw(S, ppw) - sdotw(C0, PPuw);
+            e3 = e3 - sdotw(S, ppw);
             E3 = c.g3 * e3;
             if (!dec) {
-                // 8 pi S3_ij without its d_t Pi part, and that part's coefficient in the metric rows:
-                // S3_ij = S3_0 + g3 w / (2 alpha) (Pi^2 gamma_ij - d_i phi d_j phi)
-                const T pcoef = 0.5 * (trH3 - Hnn0);                               // of d_i phi d_j phi
-                const T gcoef = fma(0.5 * Hnn0, Pi2, fma(0.5, Hdd3, -Pi * Hnd3));  // of gamma_ij
+                // 8 pi S3_ij without its N part, and that part's coefficient in the metric rows:
+                // S3_ij = S3_0 + g3 N / 2 (Pi^2 gamma_ij - d_i phi d_j phi)
+                const T pcoef = half_of(trH3);                        // of d_i phi d_j phi
+                const T gcoef = fma(0.5, Hdd3, -(Pi * Hnd3));         // of gamma_ij
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
 #pragma unroll
                     for (int j = i; j < 3; ++j) {
                         T x = fma(gcoef, gd[sidx(i, j)], pcoef * (dphi[i] * dphi[j]));
-                        x = fma(0.5 * Pi, fma(Hn[i], dphi[j], Hn[j] * dphi[i]), x);
+                        x = fma(half_of(Pi), fma(Hn[i], dphi[j], Hn[j] * dphi[i]), x);
                         x = fma(-0.5, fma(Hdv3[i], dphi[j], Hdv3[j] * dphi[i]), x);
                         S3[sidx(i, j)] = c.g3 * x;
                     }
-                const T trS3h = 0.5 * sdotw(S3, gw);
-                const T wc = 0.5 * (dphi2 - Pi2);
+                const T trS3h = half_of(sdotw(S3, gw));
+                const T wc = half_of(dphi2 - Pi2);
 #pragma unroll
                 for (int m = 0; m < 6; ++m) {
                     const int i = (m < 3) ? 0 : (m < 5 ? 1 : 2);
                     const int j = (m < 3) ? m : (m < 5 ? m - 2 : 2);
-                    Msys[m][7] = fma(-al, fma(-trS3h, gd[m], S3[m]), Msys[m][7]);
-                    Msys[m][6] = fma(0.5 * c.g3, fma(wc, gd[m], -dphi[i] * dphi[j]), Msys[m][6]);
+                    Msys[m][7] = Msys[m][7] - fnma(trS3h, gd[m], S3[m]);
+                    Msys[m][6] = fma(0.5 * c.g3, fma(wc, gd[m], -(dphi[i] * dphi[j])), Msys[m][6]);
                 }
             }
 #pragma unroll
             for (int col = 0; col < 6; ++col) PPc[col] = PPuw[col];
-            HnnSol0 = Hnn0;
         }
         const T iD = 1.0 / Dphi;
-        const T c8 = -8.0 * b1 * iD;
+        const T c8 = -8.0 * (b1 * iD);
 #pragma unroll
         for (int col = 0; col < 6; ++col) Msys[6][col] = c8 * GSuw[col];
         if (cub) {
@@ -991,16 +1049,16 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         }
         Msys[6][6] = 1.0;
         const T trH = sdotw(Hij, gw);
-        const T Hnd = dphiu[0] * Hn[0] + dphiu[1] * Hn[1] + dphiu[2] * Hn[2];
+        const T Hnd = dot3(dphiu[0], Hn[0], dphiu[1], Hn[1], dphiu[2], Hn[2]);
         T Hdd = 0.0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const T t = Hij[sidx(i, 0)] * dphiu[0] + Hij[sidx(i, 1)] * dphiu[1] + Hij[sidx(i, 2)] * dphiu[2];
+            const T t = dot3(Hij[sidx(i, 0)], dphiu[0], Hij[sidx(i, 1)], dphiu[1], Hij[sidx(i, 2)], dphiu[2]);
             Hdd = (i == 0) ? dphiu[0] * t : fma(dphiu[i], t, Hdd);
         }
-        T src = fma(fX, trH, fma(4.0 * g2 * Pi, Hnd, fma(-2.0 * g2, Hdd, b1 * L0)));
+        T src = fma(fX, trH, fma(4.0 * (g2 * Pi), Hnd, fma(-2.0 * g2, Hdd, b1 * L0)));
         if (cub) src = src + E3;
-        Msys[6][7] = fma(al * iD, src, bdPi + dadp);
+        Msys[6][7] = iD * src;
         if constexpr (std::is_same<T, double>::value) {
             if (extra && extra->want_hyp) {
                 extra->hyp[0] = det7(Msys, &extra->hyp[3]);
@@ -1011,10 +1069,10 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     }
     GRF_SECTION(16);
     ok = solve7(Msys);
-    T u[6];
+    T C[6];
 #pragma unroll
-    for (int m = 0; m < 6; ++m) u[m] = Msys[m][7];
-    const T w = Msys[6][7];
+    for (int m = 0; m < 6; ++m) C[m] = Msys[m][7];
+    const T Hnn = Msys[6][7];
     if constexpr (std::is_same<T, double>::value) {
         if (cub && extra && extra->want_hyp) {
             // g_eff in the basis (n, e_i) at the solution: g_eff^nn = -D (stored above),
@@ -1022,7 +1080,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             // - 2 g2 d^i phi d^j phi + 2 g3 (box(phi) gamma^ij - H^ij); by the Schur complement on the
             // n-n entry, det g_eff / det g = D det(g_eff^ij + g_eff^ni g_eff^nj / D) det(gamma_ij)
             const double D = extra->hyp[2];
-            const double box = trH3 - fma(w, ial, HnnSol0);
+            const double box = trH3 - Hnn;
             double e0[3], Hu[3][3], Sc[6];
             for (int i = 0; i < 3; ++i) {
                 const double hnu = gu[sidx(i, 0)] * Hn[0] + gu[sidx(i, 1)] * Hn[1] + gu[sidx(i, 2)] * Hn[2];
@@ -1044,29 +1102,27 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     // ---- full S_ij at the solution and the final K, A_ij, Pi right-hand sides
     GRF_SECTION(17);
     {
-        T Qu[6];
-        q_of(u, gd, gw, Phd, Phuw, Phm, trP, Qu);
-        const T Phnn = fma(b1 * ial, w, Phnn0);
-        T S8ij[6];
+        T QC[6], S8ij[6];
+        if (!dec) q_of(C, gd, gw, Phd, Phuw, Phm, trP, QC);
+        const T Phnn = fma(b1, Hnn, b2Pi * Pi);
 #pragma unroll
-        for (int m = 0; m < 6; ++m)
-            S8ij[m] = dec ? T(0.0) : fma(-4.0, fma(GS[m], Phnn, Y[m] + fma(Qu[m], ial, QC0[m])), S1[m]);
+        for (int m = 0; m < 6; ++m) S8ij[m] = dec ? T(0.0) : fma(-4.0, fma(GS[m], Phnn, Y[m] + QC[m]), S1[m]);
         if (cub && !dec) {
-            const T gw2 = (0.5 * c.g3) * (w * ial);
+            const T gw2 = (0.5 * c.g3) * Hnn;
 #pragma unroll
             for (int m = 0; m < 6; ++m) {
                 const int i = (m < 3) ? 0 : (m < 5 ? 1 : 2);
                 const int j = (m < 3) ? m : (m < 5 ? m - 2 : 2);
-                S8ij[m] = S8ij[m] + fma(gw2, fma(Pi * Pi, gd[m], -dphi[i] * dphi[j]), S3[m]);
+                S8ij[m] = S8ij[m] + fma(gw2, fma(Pi2, gd[m], -(dphi[i] * dphi[j])), S3[m]);
             }
         }
         const T Ss8 = sdotw(S8ij, gw);
-        rhs[F_K] = fma(0.5 * al, Ss8, Kdot0);
+        rhs[F_K] = fma(half_of(al), Ss8, Kdot0);
         const T trh3 = sdotw(S8ij, hw) * (1.0 / 3.0);
         const T alchi = al * chi;
 #pragma unroll
-        for (int m = 0; m < 6; ++m) rhs[F_A + m] = fma(-alchi, fma(-h[m], trh3, S8ij[m]), Adot0[m]);
-        rhs[F_PI] = w;
+        for (int m = 0; m < 6; ++m) rhs[F_A + m] = fnma(alchi, fnma(h[m], trh3, S8ij[m]), Adot0[m]);
+        rhs[F_PI] = fma(al, Hnn, bdPi + dadp);
     }
     if (extra) {
         extra->ham = fma(-2.0, rho8, Ss);
@@ -1083,7 +1139,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
                 // so with the Riemann blocks (Ricci equation, Codazzi, Gauss)
                 //   Psi_4 = 1/2 R_ninj mbar^i mbar^j - R_nikj mbar^i e_r^k mbar^j + 1/2 R_kilj e_r^k mbar^i e_r^l mbar^j,
                 //   R_ninj = (d_t K_ij - L_beta K_ij + D_i D_j alpha)/alpha + K_ik K^k_j,
-                //   R_nikj = D_k K_ij - D_j K_ik,  R_kilj e_r e_r = R_ij + K_rr K_ij - K_ri K_rj (3D: Ricci form).
+                //   R_nikj = D_k K_ij - D_j K_ik,  R_kilj = S_kilj (the Gauss block).
                 const double x = extra->xyz[0], y = extra->xyz[1], z = extra->xyz[2];
                 double pr = 0.0, pim = 0.0;
                 if (x * x + y * y != 0.0) {
@@ -1117,16 +1173,11 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
                             for (int j = 0; j < 3; ++j) q = fma(S6[sidx(i, j)] * a[i], b[j], q);
                         return q;
                     };
-                    double Rn[6];
-#pragma unroll
-                    for (int m = 0; m < 6; ++m) Rn[m] = fma(u[m] - LbK[m] + DDa[m], ial, KK[m]);
-                    const double E1r = 0.5 * (form(Rn, e[1], e[1]) - form(Rn, e[2], e[2]));
-                    const double E1i = -form(Rn, e[1], e[2]);
-                    const double Krr = form(Kp, e[0], e[0]), Krt = form(Kp, e[0], e[1]), Krp = form(Kp, e[0], e[2]);
-                    const double E3r = 0.5 * (form(Ric, e[1], e[1]) - form(Ric, e[2], e[2]))
-                                       + Krr * 0.5 * (form(Kp, e[1], e[1]) - form(Kp, e[2], e[2]))
-                                       - 0.5 * (Krt * Krt - Krp * Krp);
-                    const double E3i = -form(Ric, e[1], e[2]) - Krr * form(Kp, e[1], e[2]) + Krt * Krp;
+                    const double E1r = 0.5 * (form(C, e[1], e[1]) - form(C, e[2], e[2]));
+                    const double E1i = -form(C, e[1], e[2]);
+                    // S_kilj e_r^k e_r^l on (e_theta, e_phi) is S_ij there up to a multiple of the metric
+                    const double E3r = 0.5 * (form(S, e[1], e[1]) - form(S, e[2], e[2]));
+                    const double E3i = -form(S, e[1], e[2]);
                     // E2 = sum_i mbar^i W_i, W_i = sum_{k != j} R_nikj e_r^k mbar^j, mbar = (e_t - i e_p)/sqrt2
                     double E2r = 0.0, E2i = 0.0;
 #pragma unroll
@@ -1154,6 +1205,8 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         }
     }
 #undef BC
+#undef BCFMA
+#undef DH
 #undef D1
 #undef D2
 #undef ADV

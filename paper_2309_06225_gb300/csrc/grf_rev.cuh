@@ -118,6 +118,13 @@ GRF_RHD Rev fma(const Rev& a, const Rev& b, const Rev& c) {
     if (ia < 0 && ib < 0) return Rev(v, c.i);
     return Rev(v, GRF_REV_RECORD(ia, b.v, ib, a.v, c.i));
 }
+// c - a * b as one entry
+GRF_RHD Rev fnma(const Rev& a, const Rev& b, const Rev& c) {
+    const double v = ::fma(-a.v, b.v, c.v);
+    const int ia = b.v == 0.0 ? -1 : a.i, ib = a.v == 0.0 ? -1 : b.i;
+    if (ia < 0 && ib < 0) return Rev(v, c.i);
+    return Rev(v, GRF_REV_RECORD(ia, -b.v, ib, -a.v, c.i));
+}
 GRF_RHD Rev exp(const Rev& a) {
     const double e = ::exp(a.v);
     if (a.i < 0) return Rev(e);

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(128) rhs_kernel(Geom g, Coeffs c, const double
     point_rhs<double, double, -1, LOP>(c, in, r, nullptr, ok, adv);
     if (!ok) atomicOr(status, 1);
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = r[f] + ko * kos[f];
+    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, kos[f], r[f]);
 }
 
 void launch_rhs(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,

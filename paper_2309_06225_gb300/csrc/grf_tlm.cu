@@ -15,6 +15,16 @@
 #include "grf_launch.h"
 #include "grf_sphere.cuh"
 
+namespace grf_dual {
+// halves and doubles of all four components (exponent steps on the integer pipe)
+__device__ __forceinline__ D3 half_of(const D3& x) {
+    return D3(grf::half_of(x.v), grf::half_of(x.d0), grf::half_of(x.d1), grf::half_of(x.d2));
+}
+__device__ __forceinline__ D3 twice_of(const D3& x) {
+    return D3(grf::twice_of(x.v), grf::twice_of(x.d0), grf::twice_of(x.d1), grf::twice_of(x.d2));
+}
+}  // namespace grf_dual
+
 namespace grf {
 
 using grf_dual::D3;
@@ -44,7 +54,7 @@ __device__ __forceinline__ void gather_d3(const Geom& g, const double* const* s,
             if (first) {
                 d1[c][0] = fd1(u, p, sx, i12);
                 d1[c][1] = fd1(u, p, sy, i12);
-                d1[c][2] = second ? fd1_rounded(u, p, sz, i12) : fd1(u, p, sz, i12);  // as in gather()
+                d1[c][2] = fd1(u, p, sz, i12);
             }
             if (second) {
                 d2[c][0] = fd2(u, p, sx, v[c], i12s);
@@ -74,10 +84,10 @@ __device__ __forceinline__ void enforce_point_d3(D3 u[NFIELDS], double min_chi, 
 #pragma unroll
     for (int m = 0; m < 6; ++m) hh[m] = u[F_H + m];
     sym3_inv(hh, hi, id);
-    const D3 tr = hi[0] * u[F_A] + hi[3] * u[F_A + 3] + hi[5] * u[F_A + 5]
-                  + 2.0 * (hi[1] * u[F_A + 1] + hi[2] * u[F_A + 2] + hi[4] * u[F_A + 4]);
+    const D3 off = dot3(hi[1], u[F_A + 1], hi[2], u[F_A + 2], hi[4], u[F_A + 4]);
+    const D3 tr3 = fma(D3(2.0), off, dot3(hi[0], u[F_A], hi[3], u[F_A + 3], hi[5], u[F_A + 5])) * (1.0 / 3.0);
 #pragma unroll
-    for (int m = 0; m < 6; ++m) u[F_A + m] = u[F_A + m] - hh[m] * tr * (1.0 / 3.0);
+    for (int m = 0; m < 6; ++m) u[F_A + m] = fnma(hh[m], tr3, u[F_A + m]);
     u[F_CHI] = grf_dual::fmax(u[F_CHI], min_chi);
     u[F_LAPSE] = grf_dual::fmax(u[F_LAPSE], min_lapse);
 }
@@ -101,11 +111,11 @@ __global__ void __launch_bounds__(128) tlm_stage_kernel(Geom g, CoeffsT<D3> c, T
         const double inv[4] = {in.v[f].v, in.v[f].d0, in.v[f].d1, in.v[f].d2};
 #pragma unroll
         for (int cmp = 0; cmp < 4; ++cmp) {
-            kf[cmp] = rv[cmp] + a.ko * ko6(a.src[cmp] + f * g.fstride, p, g.pitch, g.plane);
+            kf[cmp] = fma(a.ko, ko6(a.src[cmp] + f * g.fstride, p, g.pitch, g.plane), rv[cmp]);
             unf[cmp] = (STAGE == 0) ? inv[cmp] : a.un[cmp][f * g.fstride + p];
             if (STAGE == 0) accf[cmp] = kf[cmp];
             else if (STAGE == 3) accf[cmp] = a.acc[cmp][f * g.fstride + p] + kf[cmp];
-            else accf[cmp] = a.acc[cmp][f * g.fstride + p] + 2.0 * kf[cmp];
+            else accf[cmp] = fma(2.0, kf[cmp], a.acc[cmp][f * g.fstride + p]);
             if (STAGE < 3) a.acc[cmp][f * g.fstride + p] = accf[cmp];
         }
         const double cs = (STAGE == 0 || STAGE == 1) ? 0.5 * a.dt : (STAGE == 2 ? a.dt : a.dt * (1.0 / 6.0));
