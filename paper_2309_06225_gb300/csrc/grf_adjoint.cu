@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) adj_tape_kernel(Geom g, Coeffs
     const long long p = gidx(g, i + NG, j + NG, k + NG);
     PointIn in;
     double kos[NFIELDS];
-    gather<0>(g, a.src, p, in, kos, nullptr, nullptr, 0);
+    gather<0>(g, a.src, p, in, kos);
     grf_rev::s_count[threadIdx.x] = 0;
     PointInT<Rev> ir;
 #pragma unroll 1
@@ -389,7 +389,7 @@ Geom adj_geom(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    g.dx = b->dx;
+    set_spacing(g, b->dx);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;
     return g;
@@ -473,17 +473,14 @@ int recompute_stages(const grf_box* box, const Geom& g, const Coeffs& c, const g
     a.min_lapse = p->min_lapse;
     a.enforce = p->enforce_algebraic;
     a.status = status;
-    a.k0 = 0;
-    a.fold = 32;
     a.un = un;
     a.acc = ACC;
-    const dim3 blk(32, 4, 1), grd((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
     a.src = un; a.dst = U1;
-    launch_stage(0, grd, blk, st, g, c, a);
+    launch_stage(0, 0, g.nz, st, g, c, a);
     a.src = U1; a.dst = U2;
-    launch_stage(1, grd, blk, st, g, c, a);
+    launch_stage(1, 0, g.nz, st, g, c, a);
     a.src = U2; a.dst = U3;
-    launch_stage(2, grd, blk, st, g, c, a);
+    launch_stage(2, 0, g.nz, st, g, c, a);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GRF_OK : fail(e);
 }

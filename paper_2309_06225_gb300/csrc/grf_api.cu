@@ -13,11 +13,16 @@ namespace grf {
 
 char g_cuda_msg[256] = "";
 
-__global__ void ko_kernel(Geom g, const double* __restrict__ s, double* __restrict__ rhs, double ko) {
+// One thread per interior point and field (grid.y).
+__global__ void __launch_bounds__(128) ko_kernel(Geom g, const double* __restrict__ s, double* __restrict__ rhs, double ko) {
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long long)g.nx * g.ny * g.nz) return;
     int i, j, k;
-    if (!interior_thread(g, i, j, k)) return;
-    const long long p = gidx(g, i + NG, j + NG, k + NG);
-    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, ko6(s + f * g.fstride, p, g.pitch, g.plane), rhs[f * g.fstride + p]);
+    point_of(g, q, i, j, k);
+    const long long p = (long long)blockIdx.y * g.fstride + gidx(g, i + NG, j + NG, k + NG);
+    FieldDiffs r;
+    field_diffs<0>(g, s + p, false, false, nullptr, r);
+    rhs[p] = fma(ko, r.ko, rhs[p]);
 }
 
 // The 6th-order scheme's dissipation: rhs += ko sum_d Delta^8_d u (ko = -sigma / (256 dx)).
@@ -208,7 +213,7 @@ Geom make_geom(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    g.dx = b->dx;
+    set_spacing(g, b->dx);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = (b->bc == GRF_BC_REFLECT_LOW || b->bc == GRF_BC_REFLECT_LOW_SOMMERFELD);
     return g;
@@ -235,40 +240,6 @@ const dim3 kBlock(32, 4, 1);
 
 dim3 interior_grid(const Geom& g) {
     return dim3((g.nx + kBlock.x - 1) / kBlock.x, (g.ny + kBlock.y - 1) / kBlock.y, (g.nz + kBlock.z - 1) / kBlock.z);
-}
-
-// x-points per warp row of the stage launch: 32 (one row per warp, the block gather), or a
-// folded 16 / 8 when that fills enough more lanes of a box whose x-extent is not a multiple of 32
-// to pay for the per-thread gather, whose extra FP64 work and less coalesced loads cost about
-// 15% with rows of 16 and 35% with rows of 8 (measured: 48^3 folded to rows of 16 runs 17%
-// faster; 100^3 folded to rows of 4 ran 3% slower than unfolded).
-// Folding also cuts the number of blocks, so it is used only when the folded grid still fills
-// at least one wave of resident blocks (3 per SM); a smaller box ran 10% slower folded (13^3).
-int fold_width(const Geom& g, const grf_params* p) {
-    const int nx = g.nx;
-    // the folded kernel: 4th order, centred advection, linear or quadratic coupling
-    if (nx % 32 == 0 || g.ng != NG || p->advection || p->beta_kind == GRF_BETA_EXPONENTIAL) return 32;
-    int sms = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 32;
-    }
-    int best = 32;
-    double best_eff = (double)nx / (32.0 * ((nx + 31) / 32));
-    for (int w : {16, 8}) {
-        const double cost = (w == 16) ? 1.15 : 1.35;
-        const double eff = (double)nx / ((double)w * ((nx + w - 1) / w)) / cost;
-        const int rows = 4 * (32 / w);
-        const long long blocks = (long long)((nx + w - 1) / w) * ((g.ny + rows - 1) / rows) * g.nz;
-        if (eff > best_eff + 1e-12 && blocks >= 3LL * sms) { best = w; best_eff = eff; }
-    }
-    return best;
-}
-
-// Stage launch grid for `planes` z-planes with row width w (blocks of 32 x 4 x 1 threads).
-dim3 stage_grid(const Geom& g, int planes, int w) {
-    const int rows = 4 * (32 / w);
-    return dim3((unsigned)((g.nx + w - 1) / w), (unsigned)((g.ny + rows - 1) / rows), (unsigned)planes);
 }
 
 size_t state_bytes(const Geom& g) { return sizeof(double) * (size_t)NFIELDS * (size_t)g.fstride; }
@@ -299,8 +270,7 @@ int fill_ghosts(const Geom& g, int bc, double* s, cudaStream_t st) {
 }
 
 size_t constraint_partials(const Geom& g) {
-    dim3 grd = interior_grid(g);
-    return (size_t)grd.x * grd.y * grd.z;
+    return constraint_blocks(g);
 }
 
 // ---- host-to-host stepping (grf_rk4_step_host): per-device copy stream and events
@@ -460,7 +430,7 @@ int grf_rhs(const grf_box* box, const grf_params* params, double* state, double*
     cudaStream_t st = (cudaStream_t)stream;
     int r = fill_ghosts(g, box->bc, state, st);
     if (r) return r;
-    launch_rhs(interior_grid(g), kBlock, st, g, make_coeffs(params), state, rhs, ko_factor(g, params->sigma_ko),
+    launch_rhs(st, g, make_coeffs(params), state, rhs, ko_factor(g, params->sigma_ko),
                status_ptr());
     if (box->bc == GRF_BC_SOMMERFELD || box->bc == GRF_BC_REFLECT_LOW_SOMMERFELD) {  // evolved ghosts' RHS
         StageArgs a{};
@@ -476,7 +446,8 @@ int grf_ko_dissipation(const grf_box* box, double sigma, const double* state, do
     if (g.ng == NG6)
         ko8_kernel<<<interior_grid(g), kBlock, 0, (cudaStream_t)stream>>>(g, state, rhs_accum, ko_factor(g, sigma));
     else
-        ko_kernel<<<interior_grid(g), kBlock, 0, (cudaStream_t)stream>>>(g, state, rhs_accum, ko_factor(g, sigma));
+        ko_kernel<<<dim3(point_blocks((long long)g.nx * g.ny * g.nz, 128), NFIELDS), 128, 0, (cudaStream_t)stream>>>(
+            g, state, rhs_accum, ko_factor(g, sigma));
     return check_launch();
 }
 
@@ -506,11 +477,8 @@ int grf_rk4_step(const grf_box* box, const grf_params* params, double* state, do
     a.min_lapse = params->min_lapse;
     a.enforce = params->enforce_algebraic;
     a.status = status_ptr();
-    a.k0 = 0;
-    a.fold = fold_width(g, params);
     a.un = state;
     a.acc = acc;
-    const dim3 grd = stage_grid(g, g.nz, a.fold);
     // outer boundaries after each stage: Sommerfeld ghosts take the same stage update, extrapolated
     // ghosts are refilled from the stage's new interior; behind mirror planes the images of the
     // evolved high-face ghosts follow their update
@@ -524,16 +492,16 @@ int grf_rk4_step(const grf_box* box, const grf_params* params, double* state, do
     };
     for (int n = 0; n < nsteps; ++n) {
         a.src = state; a.dst = A;
-        launch_stage(0, grd, kBlock, st, g, c, a);
+        launch_stage(0, 0, g.nz, st, g, c, a);
         boundary(0);
         a.src = A; a.dst = B;
-        launch_stage(1, grd, kBlock, st, g, c, a);
+        launch_stage(1, 0, g.nz, st, g, c, a);
         boundary(1);
         a.src = B; a.dst = A;
-        launch_stage(2, grd, kBlock, st, g, c, a);
+        launch_stage(2, 0, g.nz, st, g, c, a);
         boundary(2);
         a.src = A; a.dst = state;
-        launch_stage(3, grd, kBlock, st, g, c, a);
+        launch_stage(3, 0, g.nz, st, g, c, a);
         boundary(3);
         r = check_launch();
         if (r) return r;
@@ -612,9 +580,6 @@ int grf_rk4_step_host(const grf_box* box, const grf_params* params, const double
     a.status = status_ptr();
     a.un = state;
     a.acc = acc;
-    a.fold = fold_width(g, params);
-    const dim3 full = stage_grid(g, g.nz, a.fold);
-    auto slab_grid = [&](int s) { return stage_grid(g, hi(s) - lo(s), a.fold); };
     const dim3 gblk(32, 8, 1), ggrd((g.NX + 31) / 32, (g.NY + 7) / 8, NFIELDS);
 
     for (int s = 0; s < S && e == cudaSuccess; ++s) {
@@ -634,26 +599,22 @@ int grf_rk4_step_host(const grf_box* box, const grf_params* params, const double
                     slab_ghost_kernel<<<ggrd, gblk, 0, st>>>(g, state, A, B, clo(s), chi(s));
                 }
                 if (s >= 1) {
-                    a.k0 = lo(s - 1);
-                    launch_stage(0, slab_grid(s - 1), kBlock, st, g, c, a);
+                    launch_stage(0, lo(s - 1), hi(s - 1) - lo(s - 1), st, g, c, a);
                 }
             }
         } else {
-            a.k0 = 0;
-            launch_stage(0, full, kBlock, st, g, c, a);
+            launch_stage(0, 0, g.nz, st, g, c, a);
         }
-        a.k0 = 0;
         a.src = A; a.dst = B;
-        launch_stage(1, full, kBlock, st, g, c, a);
+        launch_stage(1, 0, g.nz, st, g, c, a);
         a.src = B; a.dst = A;
-        launch_stage(2, full, kBlock, st, g, c, a);
+        launch_stage(2, 0, g.nz, st, g, c, a);
         a.src = A; a.dst = state;
         if (n < nsteps - 1) {
-            launch_stage(3, full, kBlock, st, g, c, a);
+            launch_stage(3, 0, g.nz, st, g, c, a);
         } else {  // last stage, slab by slab, each finished slab copied out behind the next
             for (int s = 0; s < S; ++s) {
-                a.k0 = lo(s);
-                launch_stage(3, slab_grid(s), kBlock, st, g, c, a);
+                launch_stage(3, lo(s), hi(s) - lo(s), st, g, c, a);
                 e = cudaEventRecord(P.s4[s], st);
                 if (e == cudaSuccess) e = cudaStreamWaitEvent(P.copy, P.s4[s], 0);
                 plane_runs(g, lo(s) + NG, hi(s) + NG, false, runs);
@@ -686,7 +647,7 @@ int grf_constraints(const grf_box* box, const grf_params* params, double* state,
     int r = fill_ghosts(g, box->bc, state, st);
     if (r) return r;
     double* part = norms_host ? (double*)ws : nullptr;
-    launch_constraints(interior_grid(g), kBlock, st, g, make_coeffs(params), state, out4, part, nullptr, nullptr,
+    launch_constraints(st, g, make_coeffs(params), state, out4, part, nullptr, nullptr,
                        make_double3(0.0, 0.0, 0.0));
     r = check_launch();
     if (r || !norms_host) return r;
@@ -706,7 +667,7 @@ int grf_energy_densities(const grf_box* box, const grf_params* params, double* s
     cudaStream_t st = (cudaStream_t)stream;
     int r = fill_ghosts(g, box->bc, state, st);
     if (r) return r;
-    launch_constraints(interior_grid(g), kBlock, st, g, make_coeffs(params), state, nullptr, nullptr, out3, nullptr,
+    launch_constraints(st, g, make_coeffs(params), state, nullptr, nullptr, out3, nullptr,
                        make_double3(0.0, 0.0, 0.0));
     return check_launch();
 }
@@ -717,7 +678,7 @@ int grf_weyl_psi4(const grf_box* box, const grf_params* params, double* state, d
     cudaStream_t st = (cudaStream_t)stream;
     int r = fill_ghosts(g, box->bc, state, st);
     if (r) return r;
-    launch_constraints(interior_grid(g), kBlock, st, g, make_coeffs(params), state, nullptr, nullptr, nullptr, out2,
+    launch_constraints(st, g, make_coeffs(params), state, nullptr, nullptr, nullptr, out2,
                        make_double3(box->x0, box->y0, box->z0));
     return check_launch();
 }
@@ -728,7 +689,7 @@ int grf_hyperbolicity(const grf_box* box, const grf_params* params, double* stat
     cudaStream_t st = (cudaStream_t)stream;
     int r = fill_ghosts(g, box->bc, state, st);
     if (r) return r;
-    launch_constraints(interior_grid(g), kBlock, st, g, make_coeffs(params), state, nullptr, nullptr, nullptr, nullptr,
+    launch_constraints(st, g, make_coeffs(params), state, nullptr, nullptr, nullptr, nullptr,
                        make_double3(0.0, 0.0, 0.0), out4);
     return check_launch();
 }

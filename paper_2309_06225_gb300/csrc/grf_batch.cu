@@ -25,16 +25,15 @@ namespace grf {
 template <int STAGE>
 __global__ void __launch_bounds__(128, 3) batch_stage_kernel(const BoxDesc* __restrict__ boxes,
                                                           const TileDesc* __restrict__ tiles, int ntiles, int* status) {
-    __shared__ YzRows sh;
     const int t = blockIdx.x;
     if (t >= ntiles) return;
     const TileDesc td = tiles[t];
     // the decoupled mode and lopsided advection are compile-time instantiations (as in the single-box
     // kernels, whose bits these must match); the full theory with centred advection stays inlined
     const Coeffs& c = boxes[td.box].c;
-    if (c.advection) batch_tile_call<STAGE, -1, 1>(boxes, td, status, sh);
-    else if (c.decoupled) batch_tile_call<STAGE, 1, 0>(boxes, td, status, sh);
-    else batch_tile<STAGE, 0, 0>(boxes, td, status, sh);
+    if (c.advection) batch_tile_call<STAGE, -1, 1>(boxes, td, status);
+    else if (c.decoupled) batch_tile_call<STAGE, 1, 0>(boxes, td, status);
+    else batch_tile<STAGE, 0, 0>(boxes, td, status);
 }
 
 __global__ void batch_ghost_fill_kernel(const BoxDesc* __restrict__ boxes, int box) {
@@ -72,7 +71,7 @@ void batch_box_desc(BoxDesc& d, const grf_box* b, const grf_params* p, double dt
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    g.dx = b->dx;
+    set_spacing(g, b->dx);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;  // mirror boxes are not accepted here
     d.c = make_coeffs(p);
@@ -83,18 +82,9 @@ void batch_box_desc(BoxDesc& d, const grf_box* b, const grf_params* p, double dt
     d.enforce = p->enforce_algebraic;
 }
 
-// A box whose x-extent is not a multiple of 32 would leave lanes idle through the whole stage;
-// its tiles are folded instead, each warp covering 32 / w rows of w = 8 or 16 points, whichever
-// fills the most lanes (the folded tiles take the per-thread gather).
-int batch_row_width(int nx) {
-    if (nx % 32 == 0) return 32;
-    int best = 32;
-    double best_eff = (double)nx / (32.0 * ((nx + 31) / 32));
-    for (int w : {16, 8}) {
-        const double eff = (double)nx / ((double)w * ((nx + w - 1) / w));
-        if (eff > best_eff + 1e-12) { best = w; best_eff = eff; }
-    }
-    return best;
+void batch_append_tiles(std::vector<TileDesc>& tiles, int box, const Geom& g, int points) {
+    const long long n = (long long)g.nx * g.ny * g.nz;
+    for (long long q = 0; q < n; q += points) tiles.push_back(TileDesc{box, 0, q});
 }
 
 void launch_batch_stage(int stage, long long ntiles, dim3 block, cudaStream_t st, const BoxDesc* boxes,
@@ -143,18 +133,7 @@ Geom geom_of(const grf_box* b) {
 
 size_t state_bytes_of(const Geom& g) { return sizeof(double) * (size_t)NFIELDS * (size_t)g.fstride; }
 
-// x-points per tile row for a box: folded rows (batch_row_width) with 32 x 4 x 1 tiles, else the
-// tile's width.
-int row_width(const grf_box* b, const grf_batch_config* c) {
-    if (!(c->tile_x == 32 && c->tile_y == 4 && c->tile_z == 1)) return c->tile_x;
-    return batch_row_width(b->nx);
-}
-
-long long tiles_of(const grf_box* b, const grf_batch_config* c) {
-    const int w = row_width(b, c);
-    const int rows = c->tile_y * (c->tile_x / w);
-    return (long long)((b->nx + w - 1) / w) * ((b->ny + rows - 1) / rows) * ((b->nz + c->tile_z - 1) / c->tile_z);
-}
+int tile_points(const grf_batch_config* c) { return c->tile_x * c->tile_y * c->tile_z; }
 
 struct Layout {
     size_t ctrl, boxes, tiles, bufs, total;
@@ -166,8 +145,9 @@ Layout layout(const grf_batch_item* items, int n, const grf_batch_config* c) {
     L.ntiles = 0;
     size_t bufs = 0;
     for (int i = 0; i < n; ++i) {
-        L.ntiles += tiles_of(&items[i].box, c);
-        bufs += 3 * align_up(state_bytes_of(geom_of(&items[i].box)));
+        const Geom g = geom_of(&items[i].box);
+        L.ntiles += batch_tiles(g, tile_points(c));
+        bufs += 3 * align_up(state_bytes_of(g));
     }
     L.ctrl = 0;
     L.boxes = kAlign;
@@ -293,11 +273,7 @@ int grf_batched_rk4(const grf_batch_item* items, int nitems, const grf_params* p
         d.B = (double*)(base + off + sb);
         d.acc = (double*)(base + off + 2 * sb);
         off += 3 * sb;
-        const int w = row_width(&it.box, cfg);
-        const int rows = cfg->tile_y * (cfg->tile_x / w);
-        for (int k = 0; k < it.box.nz; k += cfg->tile_z)
-            for (int j = 0; j < it.box.ny; j += rows)
-                for (int i = 0; i < it.box.nx; i += w) ht.push_back(TileDesc{b, i, j, k, w});
+        batch_append_tiles(ht, b, d.g, tile_points(cfg));
     }
     cudaError_t e = cudaMemcpyAsync(dboxes, hb.data(), sizeof(BoxDesc) * nitems, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)

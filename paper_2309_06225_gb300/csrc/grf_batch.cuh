@@ -3,6 +3,8 @@
 // compiled in separate translation units so that the library builds in parallel.
 #pragma once
 
+#include <vector>
+
 #include "grf.h"
 #include "grf_kernels.cuh"
 
@@ -21,28 +23,19 @@ struct BoxDesc {
 };
 
 struct TileDesc {
-    int box, i0, j0, k0;
-    int w;  // x-points per row: blockDim.x (one row per warp), or 8 / 16 (a folded 32-wide tile:
-            // each warp covers 32 / w rows of a narrow box)
+    int box, pad_;
+    long long q0;  // the tile's first interior point (x-fastest order); one point per thread of the block
 };
 
 // DEC: 0 full theory, 1 without backreaction, -1 read from the box's coefficients; LOP: lopsided
 // advection.
 template <int STAGE, int DEC, int LOP>
-__device__ __forceinline__ void batch_tile(const BoxDesc* __restrict__ boxes, const TileDesc& td, int* status,
-                                           YzRows& sh) {
+__device__ __forceinline__ void batch_tile(const BoxDesc* __restrict__ boxes, const TileDesc& td, int* status) {
     const BoxDesc& d = boxes[td.box];
-    const bool folded = td.w != (int)blockDim.x;
-    const int i = td.i0 + (folded ? (int)threadIdx.x % td.w : (int)threadIdx.x);
-    const int j = td.j0 + (folded ? (int)threadIdx.y * ((int)blockDim.x / td.w) + (int)threadIdx.x / td.w : (int)threadIdx.y);
-    const int k = td.k0 + threadIdx.z;
-    // Tile shape -> gather mode (all modes give the same bits):
-    //   32 x 4 x 1: block mode, d_y d_z through the shared rows; every thread stays to the barrier.
-    //   width a multiple of 32: warp mode; whole warps stay for the shuffles.
-    //   folded tiles and other shapes: per-thread mode.
-    const int mode = folded ? GATHER_LOCAL
-                     : ((blockDim.x == 32 && blockDim.y == 4 && blockDim.z == 1) ? GATHER_BLOCK
-                        : ((blockDim.x & 31) == 0 ? GATHER_WARP : GATHER_LOCAL));
+    const long long q = td.q0 + threadIdx.x + (int)blockDim.x * ((int)threadIdx.y + (int)blockDim.y * (int)threadIdx.z);
+    if (q >= (long long)d.g.nx * d.g.ny * d.g.nz) return;
+    int i, j, k;
+    point_of(d.g, q, i, j, k);
     StageArgs a;
     a.un = d.un;
     a.acc = d.acc;
@@ -52,36 +45,26 @@ __device__ __forceinline__ void batch_tile(const BoxDesc* __restrict__ boxes, co
     a.min_lapse = d.min_lapse;
     a.enforce = d.enforce;
     a.status = status;
-    a.k0 = 0;
-    a.fold = 32;
     a.src = (STAGE == 0) ? d.un : (STAGE == 1 ? d.A : (STAGE == 2 ? d.B : d.A));
     a.dst = (STAGE == 0) ? d.A : (STAGE == 1 ? d.B : (STAGE == 2 ? d.A : d.un));
-    if (mode == GATHER_BLOCK) {
-        if (k >= d.g.nz) return;  // the whole block (k = td.k0)
-        __syncthreads();          // readers of the previous tile's rows are done
-        yz_rows_fill(d.g, a.src, i, td.j0, threadIdx.y, k, threadIdx.x, sh);
-        __syncthreads();
-    } else if (j >= d.g.ny || k >= d.g.nz || (mode == GATHER_LOCAL && i >= d.g.nx)) {
-        return;
-    }
-    stage_point<STAGE, DEC, LOP>(d.g, d.c, a, i, j, k, mode, &sh);
+    stage_point<STAGE, DEC, LOP>(d.g, d.c, a, i, j, k);
 }
 
 // Out-of-line copy of batch_tile for the persistent kernel: with the four stages inlined into one
 // kernel, ptxas spilled 52 KB per thread; called, each stage is allocated on its own (13 KB).
 template <int STAGE, int DEC, int LOP>
-__device__ __noinline__ void batch_tile_call(const BoxDesc* __restrict__ boxes, const TileDesc& td, int* status,
-                                             YzRows& sh) {
-    batch_tile<STAGE, DEC, LOP>(boxes, td, status, sh);
+__device__ __noinline__ void batch_tile_call(const BoxDesc* __restrict__ boxes, const TileDesc& td, int* status) {
+    batch_tile<STAGE, DEC, LOP>(boxes, td, status);
 }
 
 // Shared with the split-box evolution (grf_patches.cu), in grf_batch.cu: the couplings check of
 // one parameter set; a box descriptor (geometry, coefficients, dissipation, floors and dt; the
-// buffers are left null); the x-points per row of a box's 32 x 4 x 1 tiles (32, or a folded 16 or 8);
-// one stage launch over a tile list.
+// buffers are left null); the tiles of a box in a work list and their number; one stage launch over
+// a tile list.
 bool batch_params_ok(const grf_params* p);
 void batch_box_desc(BoxDesc& d, const grf_box* b, const grf_params* p, double dt);
-int batch_row_width(int nx);
+inline long long batch_tiles(const Geom& g, int points) { return ((long long)g.nx * g.ny * g.nz + points - 1) / points; }
+void batch_append_tiles(std::vector<TileDesc>& tiles, int box, const Geom& g, int points);
 void launch_batch_stage(int stage, long long ntiles, dim3 block, cudaStream_t st, const BoxDesc* boxes,
                         const TileDesc* tiles, int* status);
 

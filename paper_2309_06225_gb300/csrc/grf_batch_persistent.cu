@@ -47,7 +47,6 @@ __global__ void __launch_bounds__(128, 3) batch_persistent_kernel(const BoxDesc*
                                                                const TileDesc* __restrict__ tiles, int ntiles,
                                                                int nsteps, unsigned* bar, int* status,
                                                                long long timeout) {
-    __shared__ YzRows sh;
     for (int n = 0; n < nsteps; ++n) {
 #pragma unroll 1
         for (int s = 0; s < 4; ++s) {
@@ -56,14 +55,14 @@ __global__ void __launch_bounds__(128, 3) batch_persistent_kernel(const BoxDesc*
                 const bool dec = boxes[td.box].c.decoupled != 0;
                 const bool lop = boxes[td.box].c.advection != 0;
                 switch (s) {
-                    case 0: lop ? batch_tile_call<0, -1, 1>(boxes, td, status, sh)
-                                : (dec ? batch_tile_call<0, 1, 0>(boxes, td, status, sh) : batch_tile_call<0, 0, 0>(boxes, td, status, sh)); break;
-                    case 1: lop ? batch_tile_call<1, -1, 1>(boxes, td, status, sh)
-                                : (dec ? batch_tile_call<1, 1, 0>(boxes, td, status, sh) : batch_tile_call<1, 0, 0>(boxes, td, status, sh)); break;
-                    case 2: lop ? batch_tile_call<2, -1, 1>(boxes, td, status, sh)
-                                : (dec ? batch_tile_call<2, 1, 0>(boxes, td, status, sh) : batch_tile_call<2, 0, 0>(boxes, td, status, sh)); break;
-                    default: lop ? batch_tile_call<3, -1, 1>(boxes, td, status, sh)
-                                 : (dec ? batch_tile_call<3, 1, 0>(boxes, td, status, sh) : batch_tile_call<3, 0, 0>(boxes, td, status, sh)); break;
+                    case 0: lop ? batch_tile_call<0, -1, 1>(boxes, td, status)
+                                : (dec ? batch_tile_call<0, 1, 0>(boxes, td, status) : batch_tile_call<0, 0, 0>(boxes, td, status)); break;
+                    case 1: lop ? batch_tile_call<1, -1, 1>(boxes, td, status)
+                                : (dec ? batch_tile_call<1, 1, 0>(boxes, td, status) : batch_tile_call<1, 0, 0>(boxes, td, status)); break;
+                    case 2: lop ? batch_tile_call<2, -1, 1>(boxes, td, status)
+                                : (dec ? batch_tile_call<2, 1, 0>(boxes, td, status) : batch_tile_call<2, 0, 0>(boxes, td, status)); break;
+                    default: lop ? batch_tile_call<3, -1, 1>(boxes, td, status)
+                                 : (dec ? batch_tile_call<3, 1, 0>(boxes, td, status) : batch_tile_call<3, 0, 0>(boxes, td, status)); break;
                 }
             }
             if (!grid_barrier(bar, gridDim.x, timeout, status)) return;

@@ -9,7 +9,7 @@ namespace grf {
 // part[block][8] = {sum H^2, max|H|, sum M1^2, max|M1|, ...}
 // out4 (H, M_i; with the per-block norm partials in `part`) and dens (the energy densities of the
 // three scalar terms) are each written when non-null.
-// ORD = 4: block gather mode (as rhs_kernel); ORD = 6: the 6th-order per-thread gather.
+// ORD = 4: as rhs_kernel; ORD = 6: the 6th-order per-thread gather.
 // psi4 (2 fields, re and im) receives the Weyl scalar with the triad about the origin; o = the
 // coordinates of interior point (0, 0, 0); hyp (4 fields) the hyperbolicity diagnostics of the
 // coupled system (PointExtraT::hyp). PSI4 = 1 compiles those outputs in (they need the assembled
@@ -20,28 +20,21 @@ __global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, cons
                                                           double* __restrict__ out4, double* __restrict__ part,
                                                           double* __restrict__ dens, double* __restrict__ psi4,
                                                           double3 o, double* __restrict__ hyp) {
-    // blocks of (32, 4, 1); every thread stays to the reduction
+    // 128 consecutive points a block; every thread stays to the reduction
     __shared__ double red[8][128];
-    const int lane = threadIdx.x;
-    const int i = blockIdx.x * 32 + lane;
-    const int j = blockIdx.y * 4 + threadIdx.y;
-    const int k = blockIdx.z;
-    const bool live = i < g.nx && j < g.ny;
-    long long p;
+    const long long q = (long long)blockIdx.x * 128 + threadIdx.x;
+    const bool live = q < (long long)g.nx * g.ny * g.nz;
+    int i = 0, j = 0, k = 0;
+    long long p = 0;
     PointIn in;
     double kos[NFIELDS];
-    if constexpr (ORD == 4) {
-        __shared__ YzRows sh;
-        yz_rows_fill(g, s, i, blockIdx.y * 4, threadIdx.y, k, lane, sh);
-        __syncthreads();
-        const int jc = min(j, g.ny + 2);
-        p = gidx(g, min(i, g.nx + 2) + NG, jc + NG, k + NG);
-        WarpRow wr;
-        warp_row_halo(g, s, i - lane, jc, k, lane, wr);
-        gather(g, s, p, in, kos, &wr, &sh, threadIdx.y);
-    } else {
-        p = gidx(g, min(i, g.nx - 1) + NG6, min(j, g.ny - 1) + NG6, k + NG6);
-        if (live) gather6<0>(g, s, p, in, kos, nullptr);
+    if (live) {
+        point_of(g, q, i, j, k);
+        p = gidx(g, i + g.ng, j + g.ng, k + g.ng);
+        // H, M_i and the densities take no derivative of Theta, Gamma-hat, the lapse, the shift or B
+        constexpr unsigned kMetricScalar = ((1u << F_TH) - 1) | 1u << F_PHI | 1u << F_PI;
+        if constexpr (ORD == 4) gather<0>(g, s, p, in, kos, nullptr, PSI4 ? (1u << NFIELDS) - 1 : kMetricScalar);
+        else gather6<0>(g, s, p, in, kos, nullptr);
     }
     double vals[4] = {0.0, 0.0, 0.0, 0.0};
     if (live) {
@@ -71,7 +64,7 @@ __global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, cons
         if (PSI4 && hyp)
             for (int m = 0; m < 4; ++m) hyp[m * g.fstride + p] = ex.hyp[m];
     }
-    const int t = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+    const int t = threadIdx.x;
     for (int m = 0; m < 4; ++m) {
         red[2 * m][t] = vals[m] * vals[m];
         red[2 * m + 1][t] = fabs(vals[m]);
@@ -86,8 +79,7 @@ __global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, cons
         __syncthreads();
     }
     if (t == 0 && part) {
-        const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-        for (int m = 0; m < 8; ++m) part[b * 8 + m] = red[m][0];
+        for (int m = 0; m < 8; ++m) part[(long long)blockIdx.x * 8 + m] = red[m][0];
     }
 }
 

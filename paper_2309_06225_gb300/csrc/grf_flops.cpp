@@ -80,6 +80,7 @@ inline void opaque(double&) {}
 
 #define GRF_SECTION(id) (grfc::g_sec = (id))
 #define GRF_OPAQUE(x) grfc::opaque(x)
+#include "grf_fixed.cuh"
 #include "grf_point.cuh"
 #include "grf.h"
 
@@ -184,6 +185,17 @@ int grf_host_point_hyp(const grf_params* p, const double* v, const double* d1, c
     grf::point_rhs(c, in, rhs, &ex, ok);
     for (int m = 0; m < 4; ++m) out4[m] = ex.hyp[m];
     return ok ? 0 : -5;
+}
+
+// sum_i w[i] x[i] in block fixed point with `guard` (1 or 2) guard bits, times c when c > 0.
+double grf_host_fixed_sum(const double* x, const int* w, int n, int guard, double c) {
+    int mag = 0;
+    for (int i = 0; i < n; ++i) mag = grf::fx_max(mag, grf::fx_mag(x[i]));
+    const int e = grf::fx_exponent(mag);
+    long long s = 0;
+    for (int i = 0; i < n; ++i) s += w[i] * (guard == 1 ? grf::fx_int<1>(x[i], e) : grf::fx_int<2>(x[i], e));
+    if (c > 0.0) return guard == 1 ? grf::fx_value<1>(s, e, grf::fx_scale_of(c)) : grf::fx_value<2>(s, e, grf::fx_scale_of(c));
+    return guard == 1 ? grf::fx_value<1>(s, e) : grf::fx_value<2>(s, e);
 }
 
 }  // extern "C"

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include "grf_fixed.cuh"
 #include "grf_point.cuh"
 
 // Loads of stencil sources. By default the read-only, non-coherent path (__ldg): every kernel
@@ -29,81 +30,34 @@ struct Geom {
     int periodic;            // ghosts are periodic images (written by the owner of each value)
     int reflect;             // the three low faces are mirror planes (images written by the owner)
     int ng;                  // ghost layers: 3 (4th-order scheme) or 4 (6th-order scheme)
+    FxScale i12, i12s, i144s;  // 1/(12 dx), 1/(12 dx^2), 1/(144 dx^2) (4th-order scheme)
 };
 
+inline void set_spacing(Geom& g, double dx) {
+    g.dx = dx;
+    g.i12 = fx_scale_of(1.0 / (12.0 * dx));
+    g.i12s = fx_scale_of(1.0 / (12.0 * dx * dx));
+    g.i144s = fx_scale_of(1.0 / (144.0 * dx * dx));
+}
+
 constexpr int NG = 3;        // ghost layers of the 4th-order kernels (those of this header)
+
+// Blocks (of 128 points) of the constraint kernel, each with one set of partial norms.
+inline unsigned constraint_blocks(const Geom& g) { return (unsigned)(((long long)g.nx * g.ny * g.nz + 127) / 128); }
 
 __device__ __forceinline__ long long gidx(const Geom& g, int i, int j, int k) {  // ghosted indices
     return (long long)k * g.plane + (long long)j * g.pitch + i;
 }
 
-// Centred 4th-order first and second derivatives at ghosted offset p.
+// Centred 4th-order differences at ghosted offset p in FP64 (the adjoint's transposed stencils).
 // first: (u_-2 - 8 u_-1 + 8 u_+1 - u_+2)/(12 dx) ; second: (-u_-2 + 16 u_-1 - 30 u_0 + 16 u_+1 - u_+2)/(12 dx^2)
-// Mixed derivatives (tensor product of the first-derivative weights) are formed below as the
-// first-derivative stencil applied to rounded first derivatives.
+// mixed: the first-derivative stencil along s applied to first derivatives along t.
 __device__ __forceinline__ double fd1(const double* __restrict__ u, long long p, long long s, double i12) {
     return fma(8.0, GRF_LDG(u + p + s) - GRF_LDG(u + p - s), GRF_LDG(u + p - 2 * s) - GRF_LDG(u + p + 2 * s)) * i12;
 }
 __device__ __forceinline__ double fd2(const double* __restrict__ u, long long p, long long s, double u0, double i12s) {
     return fma(-30.0, u0, fma(16.0, GRF_LDG(u + p + s) + GRF_LDG(u + p - s), -(GRF_LDG(u + p + 2 * s) + GRF_LDG(u + p - 2 * s)))) * i12s;
 }
-
-__device__ __forceinline__ bool has_d2(int f) {
-    return f == F_CHI || (f >= F_H && f < F_H + 6) || f == F_LAPSE || (f >= F_SHIFT && f < F_SHIFT + 3) || f == F_PHI;
-}
-
-// Field index of d2 slot b (inverse of d2slot).
-__host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? F_LAPSE : (b < 11 ? b + 11 : F_PHI)); }
-
-// Mixed derivatives d_x d_t u (t = y or z) are the x-stencil applied to the scaled first
-// t-derivatives at x-2, x-1, x+1, x+2:  ((D(x-2) - D(x+2)) + 8 (D(x+1) - D(x-1))) / (12 dx),
-// D = fd1 along t. Where a warp is one x-row of 32 consecutive points, the four D values come
-// from the neighbouring lanes by shuffles (the lanes computed them as their own first
-// derivatives), and the 4 points beyond the row ends from a halo computed once per warp.
-// Elsewhere each thread evaluates the four D itself. Both give bit-identical results.
-struct WarpRow {
-    int lane;      // lane = x offset in the row
-    int selA, selB;  // halo slot for the x-2 / x+2 (A) and x-1 / x+1 (B) neighbours of end lanes
-    double hv[3];  // this lane's share of the halo: 12 d2 slots x {y, z} x 4 points, 3 per lane
-};
-
-// Halo of the warp's row: the first t-derivatives (t = y, z) of the 12 fields with second
-// derivatives at x0-2, x0-1, x0+32, x0+33 (clamped to the last ghost column; values beyond
-// nx+1 are never used by an interior point). Value (b, t, q) lives in lane 8 (b % 4) + 4 t + q,
-// register b / 4. Every lane of the warp must call this.
-__device__ __forceinline__ void warp_row_halo(const Geom& g, const double* __restrict__ s, int x0, int j, int k,
-                                              int lane, WarpRow& wr) {
-    const double i12 = 1.0 / (12.0 * g.dx);
-    const int q = lane & 3, t = (lane >> 2) & 1, bq = lane >> 3;
-    const int hx = min(q < 2 ? x0 - 2 + q : x0 + 30 + q, g.nx + 2);
-    const long long ph = gidx(g, hx + NG, j + NG, k + NG);
-    const long long sd = t ? g.plane : g.pitch;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) wr.hv[r] = fd1(s + (long long)d2field(4 * r + bq) * g.fstride, ph, sd, i12);
-    wr.lane = lane;
-    wr.selA = lane == 0 ? 0 : (lane == 1 ? 1 : (lane == 30 ? 2 : 3));
-    wr.selB = lane == 0 ? 1 : 2;
-}
-
-// d_x d_t u for d2 slot b from this lane's own D = fd1_t(u) and the neighbours' (warp path).
-__device__ __forceinline__ double mixed_x_warp(const WarpRow& wr, int b, int t, double own, double i12) {
-    const unsigned full = 0xffffffffu;
-    const int base = 8 * (b & 3) + 4 * t;
-    const double hA = __shfl_sync(full, wr.hv[b >> 2], base + wr.selA);
-    const double hB = __shfl_sync(full, wr.hv[b >> 2], base + wr.selB);
-    const double vm2 = __shfl_up_sync(full, own, 2), vm1 = __shfl_up_sync(full, own, 1);
-    const double vp1 = __shfl_down_sync(full, own, 1), vp2 = __shfl_down_sync(full, own, 2);
-    const double m2 = wr.lane < 2 ? hA : vm2;
-    const double m1 = wr.lane < 1 ? hB : vm1;
-    const double p1 = wr.lane > 30 ? hB : vp1;
-    const double p2 = wr.lane > 29 ? hA : vp2;
-    return fma(8.0, p1 - m1, m2 - p2) * i12;
-}
-
-// d_s d_t u with the four t-derivatives at the s-neighbours evaluated here (s = x or y). The
-// scalings are rounded (the library is built with -fmad=false: nothing is fused that is not written
-// as fma), so the sums are those of the shuffle and shared-memory paths, whose neighbour values
-// arrive rounded.
 __device__ __forceinline__ double mixed_local(const double* __restrict__ u, long long p, long long so, long long t,
                                               double i12) {
     const double m2 = fd1(u, p - 2 * so, t, i12), m1 = fd1(u, p - so, t, i12);
@@ -111,102 +65,116 @@ __device__ __forceinline__ double mixed_local(const double* __restrict__ u, long
     return fma(8.0, p1 - m1, m2 - p2) * i12;
 }
 
-// d_y d_z in blocks of 32 x 4 threads (every warp one x-row, the 4 warps consecutive y-rows):
-// the rounded first z-derivatives of the 12 fields with second derivatives on rows y0-2 .. y0+5
-// (row index y - y0 + 2) are shared through shared memory; each warp adds one halo row.
-struct YzRows {
-    double dz[12][8][32];
+__device__ __forceinline__ bool has_d2(int f) {
+    return f == F_CHI || (f >= F_H && f < F_H + 6) || f == F_LAPSE || (f >= F_SHIFT && f < F_SHIFT + 3) || f == F_PHI;
+}
+__device__ __forceinline__ bool has_d1(int f) { return !(f >= F_B && f < F_B + 3); }
+
+// Differences of one field at one point (weights above; sums in block fixed point, grf_fixed.cuh).
+struct FieldDiffs {
+    double v, d1[3], d2[6], ko;  // value, first and second derivatives, Kreiss-Oliger sum
+    double up[3];                // lopsided first differences (LOP)
 };
 
-// Every thread of the block calls this, then __syncthreads(). x, y0 + wy: the thread's point
-// (clamped to the last ghost column / row: values there are only read by points outside the
-// interior); k: an interior plane.
-__device__ __forceinline__ void yz_rows_fill(const Geom& g, const double* __restrict__ s, int x, int y0, int wy,
-                                             int k, int lane, YzRows& sh) {
-    const double i12 = 1.0 / (12.0 * g.dx);
-    const int xc = min(x, g.nx + 2);
-    const int yo = min(y0 + wy, g.ny + 2);
-    const int yh = min(wy < 2 ? y0 - 2 + wy : y0 + 2 + wy, g.ny + 2);  // rows y0-2, y0-1, y0+4, y0+5
-    const int rh = wy < 2 ? wy : wy + 4;
-    const long long po = gidx(g, xc + NG, yo + NG, k + NG), ph = gidx(g, xc + NG, yh + NG, k + NG);
+// The mixed derivative along strides sa, sb: the tensor product of the first-difference weights
+// (1, -8, 8, -1) on 16 points. Weights of total magnitude 18^2 leave room for one guard bit.
+__device__ __forceinline__ double fx_mixed(const double* __restrict__ u, long long sa, long long sb, const FxScale& c) {
+    double x[4][4];
+    int mag = 0;
 #pragma unroll
-    for (int b = 0; b < 12; ++b) {
-        const double* u = s + (long long)d2field(b) * g.fstride;
-        sh.dz[b][wy + 2][lane] = fd1(u, po, g.plane, i12);
-        sh.dz[b][rh][lane] = fd1(u, ph, g.plane, i12);
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            x[a][b] = GRF_LDG(u + (a < 2 ? a - 2 : a - 1) * sa + (b < 2 ? b - 2 : b - 1) * sb);
+            mag = fx_max(mag, fx_mag(x[a][b]));
+        }
+    const int e = fx_exponent(mag);
+    long long d[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        d[a] = ((fx_int<1>(x[a][2], e) - fx_int<1>(x[a][1], e)) << 3) + (fx_int<1>(x[a][0], e) - fx_int<1>(x[a][3], e));
+    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, c);
+}
+
+// All differences of the field at u (pointing at the point). Integer sums: the 19 points of the axes
+// take one block exponent (weights up to 192: two guard bits), each mixed derivative its own.
+//   LOP = 1: also the differences biased towards the side the shift component bet[d] points to (offsets
+//   -1..3, mirrored for bet[d] < 0): (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx) with a_n = u at n
+//   points towards that side, b1 = u one point away from it.
+template <int LOP>
+__device__ __forceinline__ void field_diffs(const Geom& g, const double* __restrict__ u, bool first, bool second,
+                                            const double* bet, FieldDiffs& r) {
+    const long long st[3] = {1, g.pitch, g.plane};
+    const double u0 = GRF_LDG(u);
+    double m[3][3], q[3][3];
+    int mag = fx_mag(u0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            m[d][k] = GRF_LDG(u - (k + 1) * st[d]);
+            q[d][k] = GRF_LDG(u + (k + 1) * st[d]);
+            mag = fx_max(mag, fx_max(fx_mag(m[d][k]), fx_mag(q[d][k])));
+        }
+    const int e = fx_exponent(mag);
+    const long long c0 = fx_int<2>(u0, e), c2 = c0 + c0;
+    long long t1 = 0, t2 = 0, t3 = 0;
+    r.v = u0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const long long m1 = fx_int<2>(m[d][0], e), q1 = fx_int<2>(q[d][0], e);
+        const long long m2 = fx_int<2>(m[d][1], e), q2 = fx_int<2>(q[d][1], e);
+        const long long m3 = fx_int<2>(m[d][2], e), q3 = fx_int<2>(q[d][2], e);
+        const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2;  // pair sums less 2 u0
+        if (first) r.d1[d] = fx_value<2>(((q1 - m1) << 3) + (m2 - q2), e, g.i12);
+        if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<2>((p1 << 4) - p2, e, g.i12s);
+        if (LOP) {
+            const bool fw = bet[d] >= 0.0;
+            const long long a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, b1 = fw ? m1 : q1;
+            r.up[d] = fx_value<2>(18 * a1 - 6 * a2 + a3 - 3 * b1 - 5 * c2, e, g.i12);
+        }
+        t1 += p1;
+        t2 += p2;
+        t3 += q3 + m3 - c2;
+    }
+    r.ko = fx_value<2>((t1 << 4) - t1 - 6 * t2 + t3, e);
+    if (second) {
+        r.d2[1] = fx_mixed(u, st[0], st[1], g.i144s);
+        r.d2[2] = fx_mixed(u, st[0], st[2], g.i144s);
+        r.d2[4] = fx_mixed(u, st[1], st[2], g.i144s);
     }
 }
 
-// Values, first derivatives and second derivatives of all fields at ghosted offset p, and each
-// field's Kreiss-Oliger sum (as ko6 below, same order of additions), the pair sums at distances
-// 1 and 2 shared with the second derivatives.
-//   wr != nullptr: the warp is one x-row; d_x d_y and d_x d_z come from the neighbouring lanes
-//                  (every lane of the warp must call this).
-//   sh != nullptr: d_y d_z (and the first z-derivatives of the 12 fields with second
-//                  derivatives) come from the block's shared rows; wy = the thread's row.
-// Every combination gives the same bits.
-//   LOP = 1: also the lopsided advection terms adv[f] = sum_d beta^d D_d u_f, D_d the 4th-order
-//            stencil on offsets -1..3 biased towards the side beta^d points to (mirrored for
-//            beta^d < 0): beta^d D_d u = |beta^d| (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx),
-//            a_n = u at n points towards that side, b1 = u one point away from it. The points
-//            are those the centred and Kreiss-Oliger stencils load anyway.
+// Values, first derivatives and second derivatives of all fields at ghosted offset p, and each field's
+// Kreiss-Oliger sum sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3).
+//   LOP = 1: also the lopsided advection terms adv[f] = sum_d |beta^d| D_d u_f.
+// The fields are a rolled loop: the integer code of one field is about 1,500 instructions.
+// fields: bit f set for the fields to take (the others are left alone).
 template <int LOP = 0>
 __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                       double kos[NFIELDS], const WarpRow* wr, const YzRows* sh, int wy,
-                                       double* adv = nullptr) {
-    const double i12 = 1.0 / (12.0 * g.dx), i12s = 1.0 / (12.0 * g.dx * g.dx);
-    const long long st[3] = {1, g.pitch, g.plane};
-    const int lane = threadIdx.x & 31;
+                                       double kos[NFIELDS], double* adv = nullptr, unsigned fields = (1u << NFIELDS) - 1) {
     double bet[3] = {0.0, 0.0, 0.0};
     if (LOP) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) bet[d] = GRF_LDG(s + (F_SHIFT + d) * g.fstride + p);
     }
-#pragma unroll
+#pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
-        const double* u = s + f * g.fstride;
-        const double u0 = GRF_LDG(u + p);
-        in.v[f] = u0;
-        double p1[3], p2[3], d1[3], p3[3], av = 0.0;
+        if (!(fields >> f & 1u)) continue;
+        const bool first = has_d1(f), second = has_d2(f);
+        FieldDiffs r;
+        field_diffs<LOP>(g, s + f * g.fstride + p, first, second, bet, r);
+        in.v[f] = r.v;
+        kos[f] = r.ko;
+        if (first) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const double m1 = GRF_LDG(u + p - st[d]), q1 = GRF_LDG(u + p + st[d]);
-            const double m2 = GRF_LDG(u + p - 2 * st[d]), q2 = GRF_LDG(u + p + 2 * st[d]);
-            if (LOP) {
-                const double m3 = GRF_LDG(u + p - 3 * st[d]), q3 = GRF_LDG(u + p + 3 * st[d]);
-                p3[d] = m3 + q3;
-                const bool fw = bet[d] >= 0.0;
-                const double a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, b1 = fw ? m1 : q1;
-                const double x = fma(18.0, a1, fma(-6.0, a2, a3)) - fma(3.0, b1, 10.0 * u0);
-                av = fma(fabs(bet[d]), x * i12, av);
-            }
-            d1[d] = (sh && d == 2 && has_d2(f)) ? sh->dz[d2slot(f)][wy + 2][lane] : fma(8.0, q1 - m1, m2 - q2) * i12;
-            if (!(f >= F_B && f < F_B + 3)) in.d1[d1slot(f)][d] = d1[d];
-            p1[d] = q1 + m1;
-            p2[d] = q2 + m2;
+            for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
         }
-        if (has_d2(f)) {
-            const int b = d2slot(f);
-            in.d2[b][0] = fma(-30.0, u0, fma(16.0, p1[0], -p2[0])) * i12s;
-            in.d2[b][1] = wr ? mixed_x_warp(*wr, b, 0, d1[1], i12) : mixed_local(u, p, st[0], st[1], i12);
-            in.d2[b][2] = wr ? mixed_x_warp(*wr, b, 1, d1[2], i12) : mixed_local(u, p, st[0], st[2], i12);
-            in.d2[b][3] = fma(-30.0, u0, fma(16.0, p1[1], -p2[1])) * i12s;
-            if (sh) {
-                const double(*r)[32] = sh->dz[b];
-                in.d2[b][4] = fma(8.0, r[wy + 3][lane] - r[wy + 1][lane], r[wy][lane] - r[wy + 4][lane]) * i12;
-            } else {
-                in.d2[b][4] = mixed_local(u, p, st[1], st[2], i12);
-            }
-            in.d2[b][5] = fma(-30.0, u0, fma(16.0, p1[2], -p2[2])) * i12s;
+        if (second) {
+#pragma unroll
+            for (int m = 0; m < 6; ++m) in.d2[d2slot(f)][m] = r.d2[m];
         }
-        if (LOP) adv[f] = av;
-        const double t3 = LOP ? (p3[0] + p3[1]) + p3[2]
-                              : ((GRF_LDG(u + p - 3 * st[0]) + GRF_LDG(u + p + 3 * st[0])) +
-                                 (GRF_LDG(u + p - 3 * st[1]) + GRF_LDG(u + p + 3 * st[1]))) +
-                                    (GRF_LDG(u + p - 3 * st[2]) + GRF_LDG(u + p + 3 * st[2]));
-        const double t2 = (p2[0] + p2[1]) + p2[2];
-        const double t1 = (p1[0] + p1[1]) + p1[2];
-        kos[f] = fma(-60.0, u0, fma(15.0, t1, fma(-6.0, t2, t3)));
+        if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
     }
 }
 
@@ -306,8 +274,7 @@ struct StageArgs {
     double min_chi, min_lapse;
     int enforce;
     int* status;
-    int k0;              // first interior z-plane of the launch (grid.z covers planes k0, k0+1, ...)
-    int fold;            // x-points per warp row: 32, or 16 / 8 / 4 for rk4_stage_fold_kernel
+    long long q0, q1;    // the launch's interior points in x-fastest order: [q0, q1)
 };
 
 // Lopsided advection: the ADV terms of point_rhs come from in.adv (filled by the gather).
@@ -328,36 +295,24 @@ __device__ __forceinline__ double rk4_value(const StageArgs& a, long long q, dou
     return (STAGE == 3) ? fma(cs, accf, unf) : fma(cs, kf, unf);
 }
 
-// How a stage's gather takes its mixed derivatives (all modes give the same bits).
-enum GatherMode {
-    GATHER_LOCAL = 0,  // per thread
-    GATHER_WARP = 1,   // warps are x-rows: d_x d_y, d_x d_z by shuffles
-    GATHER_BLOCK = 2,  // blocks of 32 x 4 (x-rows stacked in y): also d_y d_z through shared memory
-};
+// Interior point q (x fastest) as (i, j, k).
+__device__ __forceinline__ void point_of(const Geom& g, long long q, int& i, int& j, int& k) {
+    const long long nxy = (long long)g.nx * g.ny;
+    k = (int)(q / nxy);
+    const unsigned r = (unsigned)(q - (long long)k * nxy);
+    j = (int)(r / (unsigned)g.nx);
+    i = (int)(r - (unsigned)j * (unsigned)g.nx);
+}
 
 // One RK4 stage at one point, fused: gather -> pointwise RHS -> + KO -> stage update ->
-// enforcement -> store (with periodic images). STAGE 0..3. In the warp and block modes the
-// threads past the interior (i >= nx, and j >= ny in block mode) take part in the gather, at the
-// last ghost column / row at most, and then write nothing. sh: the block's rows (block mode,
-// already filled and synchronised).
+// enforcement -> store (with periodic images). STAGE 0..3.
 template <int STAGE, int DEC = -1, int LOP = 0, int COUP = 1>
-__device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, const StageArgs& a, int i, int j, int k,
-                                            int mode, const YzRows* sh) {
-    const bool live = i < g.nx && j < g.ny;
-    const int ic = min(i, g.nx + 2), jc = min(j, g.ny + 2);
-    const long long p = gidx(g, ic + NG, jc + NG, k + NG);
+__device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, const StageArgs& a, int i, int j, int k) {
+    const long long p = gidx(g, i + NG, j + NG, k + NG);
     PointIn in;
     double kos[NFIELDS];
     double adv[LOP ? NFIELDS : 1];
-    if (mode != GATHER_LOCAL) {
-        WarpRow wr;
-        const int lane = threadIdx.x & 31;
-        warp_row_halo(g, a.src, i - lane, jc, k, lane, wr);
-        gather<LOP>(g, a.src, p, in, kos, &wr, mode == GATHER_BLOCK ? sh : nullptr, threadIdx.y, adv);
-    } else {
-        gather<LOP>(g, a.src, p, in, kos, nullptr, nullptr, 0, adv);
-    }
-    if (!live) return;
+    gather<LOP>(g, a.src, p, in, kos, adv);
     double r[NFIELDS];
     bool ok = true;
     point_rhs<double, double, DEC, LOP, COUP>(c, in, r, nullptr, ok, adv);
@@ -374,35 +329,21 @@ __device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, cons
     for (int f = 0; f < NFIELDS; ++f) store_with_images(g, a.dst, f, i, j, k, out[f]);
 }
 
-// Launched with blocks of (32, 4, 1) threads (block gather mode). Planes k0, k0+1, ...
-// 3 resident blocks of 128 threads per SM (168 registers a thread): the extra warps hide more
-// FP64 dependency latency than the added spills cost (measured 2% faster than 2 blocks).
+// One thread per interior point of [q0, q1), consecutive threads consecutive points in x-fastest order,
+// so that every lane of every warp but the last works whatever the box's extents (no derivative is
+// exchanged between lanes, so the mapping is free). Blocks of stage_threads() threads.
+// 12 resident warps per SM (168 registers a thread): more warps hide more FP64 dependency latency than
+// the added spills cost (measured 2% faster than 8 warps at 255 registers).
 // DEC: 0 full theory, 1 without backreaction (a separate instantiation each, so the full
 // theory's kernel carries no test of the mode), -1 the mode read from c. LOP: lopsided advection.
 // COUP = 0: the linear and quadratic couplings only.
 template <int STAGE, int DEC = 0, int LOP = 0, int COUP = 1>
 __global__ void __launch_bounds__(128, 3) rk4_stage_kernel(Geom g, Coeffs c, StageArgs a) {
-    __shared__ YzRows sh;
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    const int j = blockIdx.y * 4 + threadIdx.y;
-    const int k = blockIdx.z + a.k0;
-    if (k >= g.nz) return;  // whole block
-    yz_rows_fill(g, a.src, i, blockIdx.y * 4, threadIdx.y, k, threadIdx.x, sh);
-    __syncthreads();
-    stage_point<STAGE, DEC, LOP, COUP>(g, c, a, i, j, k, GATHER_BLOCK, &sh);
-}
-
-// Folded variant for boxes whose x-extent is not a multiple of 32, chosen by the host when it
-// fills more lanes: blocks of (32, 4, 1), each warp covering 32 / w rows of w = a.fold x-points,
-// with the per-thread gather. It gives the same bits as rk4_stage_kernel.
-template <int STAGE, int DEC>
-__global__ void __launch_bounds__(128, 3) rk4_stage_fold_kernel(Geom g, Coeffs c, StageArgs a) {
-    const int w = a.fold, per = 32 / a.fold;
-    const int i = blockIdx.x * w + (int)threadIdx.x % w;
-    const int j = blockIdx.y * (4 * per) + (int)threadIdx.y * per + (int)threadIdx.x / w;
-    const int k = blockIdx.z + a.k0;
-    if (i >= g.nx || j >= g.ny || k >= g.nz) return;
-    stage_point<STAGE, DEC>(g, c, a, i, j, k, GATHER_LOCAL, nullptr);
+    const long long q = a.q0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= a.q1) return;
+    int i, j, k;
+    point_of(g, q, i, j, k);
+    stage_point<STAGE, DEC, LOP, COUP>(g, c, a, i, j, k);
 }
 
 }  // namespace grf

@@ -10,6 +10,9 @@ namespace grf {
 
 constexpr int NG6 = 4;  // ghost layers of the 6th-order scheme
 
+// Field index of d2 slot b (inverse of d2slot).
+__host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? F_LAPSE : (b < 11 ? b + 11 : F_PHI)); }
+
 // 6th-order centred first difference times 60 dx at offset p along stride t:
 //   (u_3 - u_-3) - 9 (u_2 - u_-2) + 45 (u_1 - u_-1)
 __device__ __forceinline__ double fd1_6(const double* __restrict__ u, long long p, long long t) {
@@ -262,15 +265,14 @@ __device__ __forceinline__ void stage_point6(const Geom& g, const Coeffs& c, con
     for (int f = 0; f < NFIELDS; ++f) store_with_images<NG6>(g, a.dst, f, i, j, k, out[f]);
 }
 
-// Blocks of (32, 4, 1) threads (block gather); planes k0, k0+1, ... The decoupled mode is read
+// Blocks of (32, 4, 1) threads (block gather); one plane per grid.z. The decoupled mode is read
 // from c at run time.
 template <int STAGE, int LOP>
 __global__ void __launch_bounds__(128, 3) rk4_stage6_kernel(Geom g, Coeffs c, StageArgs a) {
     __shared__ YzRows6 sh;
     const int i = blockIdx.x * 32 + threadIdx.x;
     const int j = blockIdx.y * 4 + threadIdx.y;
-    const int k = blockIdx.z + a.k0;
-    if (k >= g.nz) return;  // whole block
+    const int k = blockIdx.z;
     yz_rows_fill6(g, a.src, i, blockIdx.y * 4, threadIdx.y, k, threadIdx.x, sh);
     __syncthreads();
     stage_point6<STAGE, LOP>(g, c, a, i, j, k, sh);

@@ -27,29 +27,32 @@ inline Coeffs make_coeffs(const grf_params* p) {
     return c;
 }
 
-void launch_stage(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a);
-void launch_stage_decoupled(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
+// One stage on the interior z-planes [k0, k0 + planes) of a box: picks the instantiation and the launch
+// shape (grf_stage.cu).
+void launch_stage(int stage, int k0, int planes, cudaStream_t st, const Geom& g, const Coeffs& c, StageArgs a);
+// Its instantiations, each in its own translation unit: without backreaction; lopsided advection; every
+// coupling (both decoupled modes compiled in); the 6th-order scheme, centred and lopsided.
+void launch_stage_decoupled(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                             const StageArgs& a);
-void launch_stage_folded(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
-                         const StageArgs& a);
-// 4th-order scheme with lopsided advection; 6th-order scheme (centred / lopsided advection)
-void launch_stage_lopsided(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
+void launch_stage_lopsided(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                            const StageArgs& a);
-// 4th-order scheme, centred advection, every coupling (both decoupled modes compiled in)
-void launch_stage_general(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
+void launch_stage_general(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                           const StageArgs& a);
-void launch_stage6(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
-                   const StageArgs& a);
+void launch_stage6(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a);
 void launch_stage6_lopsided(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
                             const StageArgs& a);
-void launch_rhs6(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
+// Threads per block of a launch with one thread per point: 128, or 32 while a whole launch is less than
+// one wave of warps (12 a SM), where single-warp blocks spread evenly over the SMs.
+inline unsigned point_threads(long long npts) { return npts <= 152LL * 12 * 32 ? 32u : 128u; }
+inline unsigned point_blocks(long long npts, unsigned threads) { return (unsigned)((npts + threads - 1) / threads); }
+void launch_rhs6(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
                  double ko, int* status);
-void launch_constraints6(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
+void launch_constraints6(dim3 grid, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
                          double* out4, double* part, double* dens, double* psi4, double3 origin,
                          double* hyp = nullptr);
-void launch_rhs(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
+void launch_rhs(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
                 double ko, int* status);
-void launch_constraints(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
+void launch_constraints(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
                         double* out4, double* part, double* dens, double* psi4, double3 origin,
                          double* hyp = nullptr);
 // Outer boundaries (grf_boundary.cu): the extrapolation fill of all ghosts of s, and the

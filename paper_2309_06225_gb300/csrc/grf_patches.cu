@@ -40,7 +40,8 @@ __host__ __device__ __forceinline__ Geom patch_geom(const PatchTable& t, int a, 
     g.pitch = patch_pitch(g.nx);
     g.plane = g.pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    g.dx = 0.0;  // not used by the copies
+    g.dx = 0.0;  // the spacing is not used by the copies
+    g.i12 = g.i12s = g.i144s = FxScale{0, 0};
     g.periodic = 0;
     g.reflect = 0;
     return g;
@@ -107,6 +108,7 @@ using namespace grf;
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int kTilePoints = 128;  // points (threads) per tile of a stage launch
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 bool level_ok(const grf_patch_level* L) {
@@ -166,9 +168,7 @@ PatchLayout patch_layout(const PatchTable& t, int np) {
     size_t bufs = 0;
     for (int q = 0; q < np; ++q) {
         const Geom g = geom_at(t, q);
-        const int w = batch_row_width(g.nx);
-        const int rows = 4 * (32 / w);
-        L.ntiles += (long long)((g.nx + w - 1) / w) * ((g.ny + rows - 1) / rows) * g.nz;
+        L.ntiles += batch_tiles(g, kTilePoints);
         bufs += 3 * align_up(patch_state_bytes(g));
     }
     L.boxes = kAlign;  // the status word lives at the start
@@ -215,7 +215,7 @@ int grf_patch_copy(const grf_patch_level* level, double* box_state, double* cons
     box.pitch = B.pitch;
     box.plane = B.pitch * box.NY;
     box.fstride = box.plane * box.NZ;
-    box.dx = B.dx;
+    set_spacing(box, B.dx);
     box.periodic = 1;
     box.reflect = 0;
     const int h = direction == 0 ? 2 * NG : 0;
@@ -341,11 +341,7 @@ int grf_patches_rk4(const grf_patch_level* level, const grf_params* params, doub
         d.B = bufB[q] = (double*)(base + off + sb);
         d.acc = (double*)(base + off + 2 * sb);
         off += 3 * sb;
-        const int w = batch_row_width(pb.nx);
-        const int rows = 4 * (32 / w);
-        for (int k = 0; k < pb.nz; ++k)
-            for (int j = 0; j < pb.ny; j += rows)
-                for (int i = 0; i < pb.nx; i += w) ht.push_back(TileDesc{q, i, j, k, w});
+        batch_append_tiles(ht, q, d.g, kTilePoints);
     }
     cudaError_t e = cudaMemcpyAsync(dboxes, hb.data(), sizeof(BoxDesc) * np, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
@@ -364,7 +360,7 @@ int grf_patches_rk4(const grf_patch_level* level, const grf_params* params, doub
         return exchange ? exchange(exchange_ctx, level, bufs.data(), stream)
                         : grf_halo_exchange(level, bufs.data(), stream);
     };
-    const dim3 block(32, 4, 1);
+    const dim3 block(kTilePoints, 1, 1);
     int r = halo(un);
     if (r) return r;
     for (int n = 0; n < nsteps; ++n) {

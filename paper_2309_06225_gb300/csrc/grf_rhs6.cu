@@ -31,16 +31,16 @@ __global__ void __launch_bounds__(128) rhs6_kernel(Geom g, Coeffs c, const doubl
     for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, kos[f], r[f]);
 }
 
-void launch_rhs6(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
-                 double ko, int* status) {
+void launch_rhs6(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs, double ko, int* status) {
+    const dim3 block(32, 4, 1), grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
     if (c.advection) rhs6_kernel<kLopsided><<<grid, block, 0, st>>>(g, c, s, rhs, ko, status);
     else rhs6_kernel<0><<<grid, block, 0, st>>>(g, c, s, rhs, ko, status);
 }
 
-void launch_constraints6(dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
-                         double* out4, double* part, double* dens, double* psi4, double3 origin, double* hyp) {
-    if (psi4 || hyp) constraints_kernel<6, 1><<<grid, block, 0, st>>>(g, c, s, out4, part, dens, psi4, origin, hyp);
-    else constraints_kernel<6, 0><<<grid, block, 0, st>>>(g, c, s, out4, part, dens, psi4, origin, hyp);
+void launch_constraints6(dim3 grid, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* out4,
+                         double* part, double* dens, double* psi4, double3 origin, double* hyp) {
+    if (psi4 || hyp) constraints_kernel<6, 1><<<grid, 128, 0, st>>>(g, c, s, out4, part, dens, psi4, origin, hyp);
+    else constraints_kernel<6, 0><<<grid, 128, 0, st>>>(g, c, s, out4, part, dens, psi4, origin, hyp);
 }
 
 }  // namespace grf

@@ -4,8 +4,8 @@
 #include "grf_launch.h"
 
 namespace grf {
-void launch_stage6(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
-                   const StageArgs& a) {
+void launch_stage6(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a) {
+    const dim3 block(32, 4, 1), grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
     if (c.advection) {
         launch_stage6_lopsided(stage, grid, block, st, g, c, a);
         return;

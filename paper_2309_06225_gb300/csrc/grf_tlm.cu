@@ -39,42 +39,28 @@ struct TlmArgs {
     int* status;
 };
 
-__device__ __forceinline__ void gather_d3(const Geom& g, const double* const* s, long long p, PointInT<D3>& in) {
-    const double i12 = 1.0 / (12.0 * g.dx), i12s = 1.0 / (12.0 * g.dx * g.dx);
-    const long long sx = 1, sy = g.pitch, sz = g.plane;
+__device__ __forceinline__ double& comp(D3& x, int c) { return (&x.v)[c]; }
+
+// gather() for the value and its three tangents: each component is a field of its own state.
+__device__ __forceinline__ void gather_d3(const Geom& g, const double* const* s, long long p, PointInT<D3>& in,
+                                          D3 kos[NFIELDS]) {
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
-        double v[4], d1[4][3], d2[4][6];
-        const bool first = !(f >= F_B && f < F_B + 3);
-        const bool second = has_d2(f);
-#pragma unroll
+        const bool first = has_d1(f), second = has_d2(f);
+#pragma unroll 1
         for (int c = 0; c < 4; ++c) {
-            const double* u = s[c] + f * g.fstride;
-            v[c] = __ldg(u + p);
+            FieldDiffs r;
+            field_diffs<0>(g, s[c] + f * g.fstride + p, first, second, nullptr, r);
+            comp(in.v[f], c) = r.v;
+            comp(kos[f], c) = r.ko;
             if (first) {
-                d1[c][0] = fd1(u, p, sx, i12);
-                d1[c][1] = fd1(u, p, sy, i12);
-                d1[c][2] = fd1(u, p, sz, i12);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) comp(in.d1[d1slot(f)][d], c) = r.d1[d];
             }
             if (second) {
-                d2[c][0] = fd2(u, p, sx, v[c], i12s);
-                d2[c][1] = mixed_local(u, p, sx, sy, i12);
-                d2[c][2] = mixed_local(u, p, sx, sz, i12);
-                d2[c][3] = fd2(u, p, sy, v[c], i12s);
-                d2[c][4] = mixed_local(u, p, sy, sz, i12);
-                d2[c][5] = fd2(u, p, sz, v[c], i12s);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) comp(in.d2[d2slot(f)][m], c) = r.d2[m];
             }
-        }
-        in.v[f] = D3(v[0], v[1], v[2], v[3]);
-        if (first) {
-            const int a = d1slot(f);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) in.d1[a][d] = D3(d1[0][d], d1[1][d], d1[2][d], d1[3][d]);
-        }
-        if (second) {
-            const int b = d2slot(f);
-#pragma unroll
-            for (int m = 0; m < 6; ++m) in.d2[b][m] = D3(d2[0][m], d2[1][m], d2[2][m], d2[3][m]);
         }
     }
 }
@@ -94,11 +80,14 @@ __device__ __forceinline__ void enforce_point_d3(D3 u[NFIELDS], double min_chi, 
 
 template <int STAGE>
 __global__ void __launch_bounds__(128) tlm_stage_kernel(Geom g, CoeffsT<D3> c, TlmArgs a) {
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long long)g.nx * g.ny * g.nz) return;
     int i, j, k;
-    if (!interior_thread(g, i, j, k)) return;
+    point_of(g, q, i, j, k);
     const long long p = gidx(g, i + NG, j + NG, k + NG);
     PointInT<D3> in;
-    gather_d3(g, a.src, p, in);
+    D3 kos[NFIELDS];
+    gather_d3(g, a.src, p, in, kos);
     D3 r[NFIELDS];
     bool ok = true;
     point_rhs<D3, D3>(c, in, r, nullptr, ok);
@@ -109,9 +98,10 @@ __global__ void __launch_bounds__(128) tlm_stage_kernel(Geom g, CoeffsT<D3> c, T
         double kf[4], unf[4], accf[4];
         const double rv[4] = {r[f].v, r[f].d0, r[f].d1, r[f].d2};
         const double inv[4] = {in.v[f].v, in.v[f].d0, in.v[f].d1, in.v[f].d2};
+        const double kov[4] = {kos[f].v, kos[f].d0, kos[f].d1, kos[f].d2};
 #pragma unroll
         for (int cmp = 0; cmp < 4; ++cmp) {
-            kf[cmp] = fma(a.ko, ko6(a.src[cmp] + f * g.fstride, p, g.pitch, g.plane), rv[cmp]);
+            kf[cmp] = fma(a.ko, kov[cmp], rv[cmp]);
             unf[cmp] = (STAGE == 0) ? inv[cmp] : a.un[cmp][f * g.fstride + p];
             if (STAGE == 0) accf[cmp] = kf[cmp];
             else if (STAGE == 3) accf[cmp] = a.acc[cmp][f * g.fstride + p] + kf[cmp];
@@ -204,7 +194,7 @@ Geom geom_from(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    g.dx = b->dx;
+    set_spacing(g, b->dx);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;  // mirror boxes are not accepted here
     return g;
@@ -292,8 +282,8 @@ int grf_tlm_rk4(const grf_box* box, const grf_params* params, const double* dpar
     a.enforce = params->enforce_algebraic;
     a.status = status;
     for (int cc = 0; cc < 4; ++cc) { a.un[cc] = un[cc]; a.acc[cc] = buf(2, cc); }
-    const dim3 blk(32, 4, 1);
-    const dim3 grd((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+    const long long npts = (long long)g.nx * g.ny * g.nz;
+    const unsigned blk = point_threads(npts), grd = point_blocks(npts, blk);
     for (int n = 0; n < nsteps; ++n) {
         for (int s = 0; s < 4; ++s) {
             for (int cc = 0; cc < 4; ++cc) {

@@ -1,0 +1,70 @@
+"""Block fixed point (csrc/grf_fixed.cuh, host build): stencil sums against exact rational arithmetic.
+
+Bound, from the representation: each value is kept to one unit of 2^-(52 + guard) of the largest one's
+leading bit (exactly, when it is within 2^guard of the largest), the integer sum is exact, and the result is
+rounded once (the scaled one after a product kept to 63 bits).
+"""
+import ctypes as C
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+KO6 = [1, -6, 15, -20, 15, -6, 1]
+MIXED = [a * b for a in (1, -8, 8, -1) for b in (1, -8, 8, -1)]
+
+
+@pytest.fixture(scope="module")
+def fixed_sum():
+    from paper_2309_06225_gb300 import build
+    L = C.CDLL(build.build_flops())
+    L.grf_host_fixed_sum.restype = C.c_double
+    L.grf_host_fixed_sum.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_int), C.c_int, C.c_int, C.c_double]
+
+    def f(x, w, guard, c=0.0):
+        x, w = np.ascontiguousarray(x, dtype=np.float64), np.ascontiguousarray(w, dtype=np.int32)
+        return L.grf_host_fixed_sum(x.ctypes.data_as(C.POINTER(C.c_double)), w.ctypes.data_as(C.POINTER(C.c_int)),
+                                    len(x), guard, c)
+    return f
+
+
+@pytest.mark.parametrize("spread", [0, 2, 12, 70, 400])
+@pytest.mark.parametrize("weights,guard", [(KO6 * 3, 2), (MIXED, 1), ([1, -1], 2), ([1], 2)])
+def test_sums_against_exact(fixed_sum, weights, guard, spread):
+    rng = np.random.default_rng(spread + len(weights))
+    for t in range(300):
+        n = len(weights)
+        x = rng.uniform(1.0, 2.0, n) * rng.choice([-1.0, 1.0], n) * 2.0 ** rng.integers(-spread, 1, n)
+        if t % 3 == 0:
+            x[rng.integers(n)] = rng.choice([0.0, -0.0])
+        if t % 7 == 0:
+            x[:] = x[0] * (1.0 + 2.0 ** -52 * rng.integers(0, 3, n))  # nearly equal: massive cancellation
+        x *= 2.0 ** int(rng.integers(-300, 300))
+        top = Fraction(2) ** (int(np.frexp(np.max(np.abs(x)))[1]) - 1)
+        unit = top / 2 ** (52 + guard)
+        for c in (0.0, 1.0 / 12.0, 7.3e5, 3.1e-9):
+            exact = sum(Fraction(int(w)) * Fraction(float(v)) for w, v in zip(weights, x)) * (Fraction(c) if c else 1)
+            got = Fraction(fixed_sum(x, weights, guard, c))
+            small = [abs(int(w)) for w, v in zip(weights, x) if v != 0 and abs(Fraction(float(v))) * 2 ** guard < top]
+            bound = sum(small) * unit * (Fraction(c) if c else 1)
+            bound += abs(exact) * Fraction(1, 2 ** 53) * (1 + Fraction(1, 2 ** 8)) + bound / 2 ** 52
+            assert abs(got - exact) <= bound, (x, c, float(got), float(exact))
+
+
+@pytest.mark.parametrize("guard", [1, 2])
+def test_special_values(fixed_sum, guard):
+    w = MIXED
+    assert fixed_sum(np.zeros(16), w, guard) == 0.0 and fixed_sum(-np.zeros(16), w, guard, 0.25) == 0.0
+    assert fixed_sum(np.full(16, -0.1), w, guard, 12.5) == 0.0          # weights sum to zero
+    assert fixed_sum(np.full(16, 1e-310), w, guard) == 0.0              # below the representation's floor
+    for bad in (np.nan, np.inf, -np.inf):
+        x = np.ones(16)
+        x[3] = bad
+        assert np.isnan(fixed_sum(x, w, guard)) and np.isnan(fixed_sum(x, w, guard, 2.0))
+        assert np.isnan(fixed_sum(np.full(16, bad), w, guard, 1e-30))
+    big = np.zeros(16)
+    big[5] = 1e308                                                      # weight 64: overflows
+    assert np.isinf(fixed_sum(big, w, guard))
+    assert fixed_sum(big, w, guard, 2.0 ** -20) == 64 * (1e308 * 2.0 ** -20)  # scaled back into range
+    x = np.array([1.7976931348623157e308, -1.7976931348623157e308])
+    assert fixed_sum(x, [1, 1], guard) == 0.0
