@@ -20,8 +20,10 @@ __global__ void __launch_bounds__(128) ko_kernel(Geom g, const double* __restric
     int i, j, k;
     point_of(g, q, i, j, k);
     const long long p = (long long)blockIdx.y * g.fstride + gidx(g, i + NG, j + NG, k + NG);
+    AxisValues v;
+    load_axes(g, s + p, v);
     FieldDiffs r;
-    field_diffs<0>(g, s + p, false, false, nullptr, r);
+    if (axis_diffs<0>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko6(s + p, 0, g.pitch, g.plane);
     rhs[p] = fma(ko, r.ko, rhs[p]);
 }
 

@@ -31,9 +31,7 @@ __global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, cons
     if (live) {
         point_of(g, q, i, j, k);
         p = gidx(g, i + g.ng, j + g.ng, k + g.ng);
-        // H, M_i and the densities take no derivative of Theta, Gamma-hat, the lapse, the shift or B
-        constexpr unsigned kMetricScalar = ((1u << F_TH) - 1) | 1u << F_PHI | 1u << F_PI;
-        if constexpr (ORD == 4) gather<0>(g, s, p, in, kos, nullptr, PSI4 ? (1u << NFIELDS) - 1 : kMetricScalar);
+        if constexpr (ORD == 4) gather<0, PSI4>(g, s, p, in, kos);
         else gather6<0>(g, s, p, in, kos, nullptr);
     }
     double vals[4] = {0.0, 0.0, 0.0, 0.0};

@@ -13,8 +13,9 @@
 //     independent of their order, so every caller gets the same bits;
 //   * the sum times a positive constant (the grid-spacing factor, as a 64-bit mantissa) is rounded once to
 //     double.
-// A block whose values are all below 2^-959 counts as zeros below 2^-1013. An infinity or NaN among the
-// block's values gives a NaN.
+// Range: the caller bounds the block exponent (FxRange), so that no result leaves the normal doubles and no
+// result has to be checked: blocks below the range count as their values' multiples of a tiny unit (2^-1000
+// and less at common spacings), blocks above it, with infinities and NaNs among them, take the FP64 sums.
 // The functions compile for the host too, where tests compare them with exact arithmetic.
 #pragma once
 
@@ -39,6 +40,20 @@ inline FxScale fx_scale_of(double c) {
     return s;
 }
 
+// Block exponents whose results (sums of magnitude 2^0 .. 2^63 units, times constants of exponents lo .. hi
+// or 1) are normal doubles.
+struct FxRange {
+    int emin, emax;
+};
+
+inline FxRange fx_range(int lo, int hi) {
+    FxRange r;
+    r.emin = 66 - (lo < 0 ? lo : 0);
+    r.emax = 2046 - 13 - (hi > 0 ? hi : 0);
+    if (r.emin > r.emax) r.emax = -1;  // no block qualifies
+    return r;
+}
+
 GRF_HD unsigned long long fx_bits(double x) {
 #ifdef __CUDA_ARCH__
     return (unsigned long long)__double_as_longlong(x);
@@ -53,72 +68,89 @@ GRF_HD unsigned long long fx_bits(double x) {
 GRF_HD int fx_mag(double x) { return (int)(fx_bits(x) >> 32) & 0x7fffffff; }
 GRF_HD int fx_max(int a, int b) { return a > b ? a : b; }
 
-constexpr int kFxNan = 1 << 20;  // "exponent" of a block that holds an infinity or a NaN
-
-GRF_HD int fx_exponent(int mag) {
-    const int e = mag >> 20;
-    return e >= 2047 ? kFxNan : fx_max(e, 64);
-}
-
-// x in units of 2^(emax - 1075 - G), truncated towards zero; |result| < 2^(53 + G).
+// x in units of 2^(emax - 1075 - G), truncated towards zero, |result| < 2^(53 + G), for |x| of exponent at
+// most emax; lim = fx_lim<G>(emax) is the exponent's word the shift is counted from.
 template <int G>
-GRF_HD long long fx_int(double x, int emax) {
+GRF_HD int fx_lim(int emax) { return (int)((unsigned)(emax + 11 - G) << 20 | 0xfffffu); }
+
+GRF_HD long long fx_int(double x, int lim) {
+#ifdef __CUDA_ARCH__
+    // 12 instructions: the shift count, the mantissa at the top of 64 bits, the shift (by 64 and more: to
+    // zero), the sign
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned s = (unsigned)(lim - (hi & 0x7fffffff)) >> 20;
+    const unsigned uh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ul = (unsigned)lo << 11;
+    long long r;
+    asm("{\n\t.reg .pred p;\n\t.reg .b64 u;\n\t"
+        "mov.b64 u, {%2, %1};\n\tshr.u64 %0, u, %3;\n\tsetp.lt.s32 p, %4, 0;\n\t@p neg.s64 %0, %0;\n\t}"
+        : "=&l"(r)
+        : "r"(uh), "r"(ul), "r"(s), "r"(hi));
+    return r;
+#else
     const unsigned long long b = fx_bits(x);
-    const int hi = (int)(b >> 32);
-    int s = emax - ((hi & 0x7fffffff) >> 20);
-    s = s < 63 ? s : 63;
-    const unsigned long long m = (((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << G) >> s;
-    return hi < 0 ? -(long long)m : (long long)m;
+    const unsigned s = (unsigned)(lim - ((int)(b >> 32) & 0x7fffffff)) >> 20;
+    const unsigned long long u = (b << 11) | 0x8000000000000000ull;
+    const long long r = s > 63 ? 0 : (long long)(u >> s);
+    return (long long)b < 0 ? -r : r;
+#endif
 }
 
-// 2^E (1.f) with 64-bit mantissa p (top bit set) and biased exponent E, rounded to nearest; the sign of I.
-GRF_HD double fx_pack(unsigned long long p, int E, long long I) {
-    unsigned long long b = (p >> 11) + ((p >> 10) & 1ull) + ((unsigned long long)(unsigned)(E - 1) << 52);
-    if (!((unsigned)(E - 1) < 2046u && I != 0)) {
-        if (E > (kFxNan >> 1)) b = 0x7ff8000000000000ull;
-        else b = (E > 0 && I != 0) ? 0x7ff0000000000000ull : 0ull;
-    }
-    b |= (unsigned long long)I & 0x8000000000000000ull;
+// |I| 2^z with the top bit set, and z (64 and 0 for I = 0).
+GRF_HD unsigned long long fx_normal(long long I, int& z) {
 #ifdef __CUDA_ARCH__
-    return __longlong_as_double((long long)b);
+    unsigned long long u = (unsigned long long)I, r;
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.s64 p, %0, 0;\n\t@p neg.s64 %0, %0;\n\t}" : "+l"(u));
+    z = __clzll((long long)u);
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(u), "r"(z));
+    return r;
 #else
+    const unsigned long long u = (unsigned long long)(I < 0 ? -I : I);
+    z = u ? __builtin_clzll(u) : 64;
+    return u ? u << z : 0;
+#endif
+}
+
+// The double of mantissa p (64 bits, top bit set; rounded to nearest) and biased exponent E in the normal
+// range, with the sign of I; 0 where z = 64.
+GRF_HD double fx_pack(unsigned long long p, int E, int z, long long I) {
+    const unsigned long long r = (p >> 11) + ((p >> 10) & 1ull);
+    const unsigned eh = z == 64 ? 0u : (unsigned)(E - 1) << 20;
+    const unsigned hi = (unsigned)(r >> 32) + eh;
+    const unsigned sg = (unsigned)((unsigned long long)I >> 32) & 0x80000000u;
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)(hi | sg), (int)(unsigned)r);
+#else
+    const unsigned long long b = ((unsigned long long)(hi | sg) << 32) | (unsigned)r;
     double x;
     std::memcpy(&x, &b, sizeof x);
     return x;
 #endif
 }
 
-GRF_HD int fx_clz(unsigned long long u) {
-#ifdef __CUDA_ARCH__
-    return __clzll((long long)u) & 63;
-#else
-    return u ? __builtin_clzll(u) : 0;
-#endif
-}
-
 // I 2^(emax - 1075 - G), rounded to double.
 template <int G>
 GRF_HD double fx_value(long long I, int emax) {
-    unsigned long long u = (unsigned long long)(I < 0 ? -I : I);
-    const int z = fx_clz(u);
-    u <<= z;
-    return fx_pack(u, emax - z + 11 - G, I);
+    int z;
+    const unsigned long long u = fx_normal(I, z);
+    return fx_pack(u, emax - z + 11 - G, z, I);
 }
 
 // I 2^(emax - 1075 - G) times the constant c, rounded once to double.
 template <int G>
 GRF_HD double fx_value(long long I, int emax, const FxScale& c) {
-    unsigned long long u = (unsigned long long)(I < 0 ? -I : I);
-    const int z = fx_clz(u);
-    u <<= z;
+    int z;
+    const unsigned long long u = fx_normal(I, z);
 #ifdef __CUDA_ARCH__
     unsigned long long p = __umul64hi(u, c.m);
 #else
     unsigned long long p = (unsigned long long)(((unsigned __int128)u * c.m) >> 64);
 #endif
-    const int q = 1 - (int)(p >> 63);
-    p <<= q;
-    return fx_pack(p, emax + c.e - z - q + 12 - G, I);
+    int E = emax + c.e - z + 12 - G;
+    if (!(p >> 63)) {
+        p += p;
+        --E;
+    }
+    return fx_pack(p, E, z, I);
 }
 
 }  // namespace grf

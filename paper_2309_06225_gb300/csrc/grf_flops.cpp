@@ -187,14 +187,18 @@ int grf_host_point_hyp(const grf_params* p, const double* v, const double* d1, c
     return ok ? 0 : -5;
 }
 
-// sum_i w[i] x[i] in block fixed point with `guard` (1 or 2) guard bits, times c when c > 0.
+// sum_i w[i] x[i] in block fixed point with `guard` (1 or 2) guard bits, times c when c > 0; NaN above the range.
 double grf_host_fixed_sum(const double* x, const int* w, int n, int guard, double c) {
     int mag = 0;
     for (int i = 0; i < n; ++i) mag = grf::fx_max(mag, grf::fx_mag(x[i]));
-    const int e = grf::fx_exponent(mag);
+    const grf::FxScale k = grf::fx_scale_of(c > 0.0 ? c : 1.0);
+    const grf::FxRange range = grf::fx_range(k.e, k.e);
+    const int e = grf::fx_max(mag >> 20, range.emin);
+    if (e > range.emax) return std::nan("");  // the kernels take such a block's sums in FP64
+    const int lim = guard == 1 ? grf::fx_lim<1>(e) : grf::fx_lim<2>(e);
     long long s = 0;
-    for (int i = 0; i < n; ++i) s += w[i] * (guard == 1 ? grf::fx_int<1>(x[i], e) : grf::fx_int<2>(x[i], e));
-    if (c > 0.0) return guard == 1 ? grf::fx_value<1>(s, e, grf::fx_scale_of(c)) : grf::fx_value<2>(s, e, grf::fx_scale_of(c));
+    for (int i = 0; i < n; ++i) s += w[i] * grf::fx_int(x[i], lim);
+    if (c > 0.0) return guard == 1 ? grf::fx_value<1>(s, e, k) : grf::fx_value<2>(s, e, k);
     return guard == 1 ? grf::fx_value<1>(s, e) : grf::fx_value<2>(s, e);
 }
 

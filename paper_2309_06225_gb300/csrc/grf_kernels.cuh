@@ -31,6 +31,7 @@ struct Geom {
     int reflect;             // the three low faces are mirror planes (images written by the owner)
     int ng;                  // ghost layers: 3 (4th-order scheme) or 4 (6th-order scheme)
     FxScale i12, i12s, i144s;  // 1/(12 dx), 1/(12 dx^2), 1/(144 dx^2) (4th-order scheme)
+    FxRange fx;                // block exponents of the fixed-point sums
 };
 
 inline void set_spacing(Geom& g, double dx) {
@@ -38,6 +39,8 @@ inline void set_spacing(Geom& g, double dx) {
     g.i12 = fx_scale_of(1.0 / (12.0 * dx));
     g.i12s = fx_scale_of(1.0 / (12.0 * dx * dx));
     g.i144s = fx_scale_of(1.0 / (144.0 * dx * dx));
+    const int lo = g.i144s.e < g.i12.e ? g.i144s.e : g.i12.e, hi = g.i12s.e > g.i12.e ? g.i12s.e : g.i12.e;
+    g.fx = fx_range(lo, hi);
 }
 
 constexpr int NG = 3;        // ghost layers of the 4th-order kernels (those of this header)
@@ -65,66 +68,79 @@ __device__ __forceinline__ double mixed_local(const double* __restrict__ u, long
     return fma(8.0, p1 - m1, m2 - p2) * i12;
 }
 
+// sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3), pair sums added x, y, z
+__device__ __forceinline__ double ko6(const double* __restrict__ u, long long p, long long sy, long long sz) {
+    const long long st[3] = {1, sy, sz};
+    double t[4];
+#pragma unroll
+    for (int r = 1; r <= 3; ++r)
+        t[r] = ((GRF_LDG(u + p - r * st[0]) + GRF_LDG(u + p + r * st[0])) + (GRF_LDG(u + p - r * st[1]) + GRF_LDG(u + p + r * st[1]))) +
+               (GRF_LDG(u + p - r * st[2]) + GRF_LDG(u + p + r * st[2]));
+    return fma(-60.0, GRF_LDG(u + p), fma(15.0, t[1], fma(-6.0, t[2], t[3])));
+}
+
 __device__ __forceinline__ bool has_d2(int f) {
     return f == F_CHI || (f >= F_H && f < F_H + 6) || f == F_LAPSE || (f >= F_SHIFT && f < F_SHIFT + 3) || f == F_PHI;
 }
 __device__ __forceinline__ bool has_d1(int f) { return !(f >= F_B && f < F_B + 3); }
 
-// Differences of one field at one point (weights above; sums in block fixed point, grf_fixed.cuh).
-struct FieldDiffs {
-    double v, d1[3], d2[6], ko;  // value, first and second derivatives, Kreiss-Oliger sum
-    double up[3];                // lopsided first differences (LOP)
+// ---- the gather: differences of the fields at one point, the sums in block fixed point (grf_fixed.cuh)
+
+// One field on the three axes through the point (19 values), and on one coordinate plane (16).
+struct AxisValues {
+    double c, m[3][3], q[3][3];  // the point; at -(k+1) and +(k+1) along axis d
+};
+struct PlaneValues {
+    double x[4][4];  // at offsets -2, -1, 1, 2 along both axes
 };
 
-// The mixed derivative along strides sa, sb: the tensor product of the first-difference weights
-// (1, -8, 8, -1) on 16 points. Weights of total magnitude 18^2 leave room for one guard bit.
-__device__ __forceinline__ double fx_mixed(const double* __restrict__ u, long long sa, long long sb, const FxScale& c) {
-    double x[4][4];
-    int mag = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            x[a][b] = GRF_LDG(u + (a < 2 ? a - 2 : a - 1) * sa + (b < 2 ? b - 2 : b - 1) * sb);
-            mag = fx_max(mag, fx_mag(x[a][b]));
-        }
-    const int e = fx_exponent(mag);
-    long long d[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-        d[a] = ((fx_int<1>(x[a][2], e) - fx_int<1>(x[a][1], e)) << 3) + (fx_int<1>(x[a][0], e) - fx_int<1>(x[a][3], e));
-    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, c);
-}
-
-// All differences of the field at u (pointing at the point). Integer sums: the 19 points of the axes
-// take one block exponent (weights up to 192: two guard bits), each mixed derivative its own.
-//   LOP = 1: also the differences biased towards the side the shift component bet[d] points to (offsets
-//   -1..3, mirrored for bet[d] < 0): (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx) with a_n = u at n
-//   points towards that side, b1 = u one point away from it.
-template <int LOP>
-__device__ __forceinline__ void field_diffs(const Geom& g, const double* __restrict__ u, bool first, bool second,
-                                            const double* bet, FieldDiffs& r) {
+__device__ __forceinline__ void load_axes(const Geom& g, const double* __restrict__ u, AxisValues& v) {
     const long long st[3] = {1, g.pitch, g.plane};
-    const double u0 = GRF_LDG(u);
-    double m[3][3], q[3][3];
-    int mag = fx_mag(u0);
+    v.c = GRF_LDG(u);
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            m[d][k] = GRF_LDG(u - (k + 1) * st[d]);
-            q[d][k] = GRF_LDG(u + (k + 1) * st[d]);
-            mag = fx_max(mag, fx_max(fx_mag(m[d][k]), fx_mag(q[d][k])));
+            v.m[d][k] = GRF_LDG(u - (k + 1) * st[d]);
+            v.q[d][k] = GRF_LDG(u + (k + 1) * st[d]);
         }
-    const int e = fx_exponent(mag);
-    const long long c0 = fx_int<2>(u0, e), c2 = c0 + c0;
+}
+__device__ __forceinline__ void load_plane(const double* __restrict__ u, long long sa, long long sb, PlaneValues& v) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            v.x[a][b] = GRF_LDG(u + (a < 2 ? a - 2 : a - 1) * sa + (b < 2 ? b - 2 : b - 1) * sb);
+}
+
+// Differences of one field at one point.
+struct FieldDiffs {
+    double d1[3], d2[6], ko;  // first and second derivatives, Kreiss-Oliger sum
+    double up[3];             // lopsided first differences (LOP)
+};
+
+// The axis part: first derivatives, unmixed second derivatives and the Kreiss-Oliger sum. The 19 points take
+// one block exponent; weights of total magnitude up to 192 leave room for two guard bits. Returns the
+// block's largest magnitude word.
+//   LOP = 1: also the differences biased towards the side the shift component bet[d] points to (offsets
+//   -1..3, mirrored for bet[d] < 0): (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx) with a_n = u at n
+//   points towards that side, b1 = u one point away from it.
+template <int LOP>
+__device__ __forceinline__ int axis_diffs(const Geom& g, const AxisValues& v, bool first, bool second, const double* bet,
+                                          FieldDiffs& r) {
+    int mag = fx_mag(v.c);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) mag = fx_max(mag, fx_max(fx_mag(v.m[d][k]), fx_mag(v.q[d][k])));
+    const int e = fx_max(mag >> 20, g.fx.emin), lim = fx_lim<2>(e);
+    const long long c0 = fx_int(v.c, lim), c2 = c0 + c0;
     long long t1 = 0, t2 = 0, t3 = 0;
-    r.v = u0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const long long m1 = fx_int<2>(m[d][0], e), q1 = fx_int<2>(q[d][0], e);
-        const long long m2 = fx_int<2>(m[d][1], e), q2 = fx_int<2>(q[d][1], e);
-        const long long m3 = fx_int<2>(m[d][2], e), q3 = fx_int<2>(q[d][2], e);
+        const long long m1 = fx_int(v.m[d][0], lim), q1 = fx_int(v.q[d][0], lim);
+        const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
+        const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
         const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2;  // pair sums less 2 u0
         if (first) r.d1[d] = fx_value<2>(((q1 - m1) << 3) + (m2 - q2), e, g.i12);
         if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<2>((p1 << 4) - p2, e, g.i12s);
@@ -138,55 +154,128 @@ __device__ __forceinline__ void field_diffs(const Geom& g, const double* __restr
         t3 += q3 + m3 - c2;
     }
     r.ko = fx_value<2>((t1 << 4) - t1 - 6 * t2 + t3, e);
-    if (second) {
-        r.d2[1] = fx_mixed(u, st[0], st[1], g.i144s);
-        r.d2[2] = fx_mixed(u, st[0], st[2], g.i144s);
-        r.d2[4] = fx_mixed(u, st[1], st[2], g.i144s);
+    return mag;
+}
+
+// A mixed derivative: the tensor product of the first-difference weights (1, -8, 8, -1) on its 16 points,
+// with their own block exponent. Weights of total magnitude 18^2 leave room for one guard bit. mag collects
+// the largest magnitude word.
+__device__ __forceinline__ double plane_diff(const Geom& g, const PlaneValues& v, int& mag) {
+    int top = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) top = fx_max(top, fx_mag(v.x[a][b]));
+    mag = fx_max(mag, top);
+    const int e = fx_max(top >> 20, g.fx.emin), lim = fx_lim<1>(e);
+    long long d[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        d[a] = ((fx_int(v.x[a][2], lim) - fx_int(v.x[a][1], lim)) << 3) + (fx_int(v.x[a][0], lim) - fx_int(v.x[a][3], lim));
+    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, g.i144s);
+}
+
+// The differences in FP64, for a point whose fields leave the fixed-point range (values near overflow,
+// infinities, NaNs): rewrites what gather() took.
+template <int LOP>
+__device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
+                                         double* kos, double* adv, unsigned fields) {
+    const double i12 = 1.0 / (12.0 * g.dx), i12s = 1.0 / (12.0 * g.dx * g.dx);
+    const long long st[3] = {1, g.pitch, g.plane};
+#pragma unroll 1
+    for (int f = 0; f < NFIELDS; ++f) {
+        if (!(fields >> f & 1u)) continue;
+        const double* u = s + f * g.fstride + p;
+        const double u0 = GRF_LDG(u);
+        double av = 0.0;
+        kos[f] = ko6(u, 0, g.pitch, g.plane);
+#pragma unroll 1
+        for (int d = 0; d < 3; ++d) {
+            if (has_d1(f)) in.d1[d1slot(f)][d] = fd1(u, 0, st[d], i12);
+            if (has_d2(f)) {
+                in.d2[d2slot(f)][d == 0 ? 0 : (d == 1 ? 3 : 5)] = fd2(u, 0, st[d], u0, i12s);
+                in.d2[d2slot(f)][d == 2 ? 4 : d + 1] = mixed_local(u, 0, st[d == 2], st[d == 0 ? 1 : 2], i12);
+            }
+            if (LOP) {
+                const double b = GRF_LDG(s + (F_SHIFT + d) * g.fstride + p);
+                const long long t = b >= 0.0 ? st[d] : -st[d];
+                const double x = fma(18.0, GRF_LDG(u + t), fma(-6.0, GRF_LDG(u + 2 * t), GRF_LDG(u + 3 * t))) -
+                                 fma(3.0, GRF_LDG(u - t), 10.0 * u0);
+                av = fma(fabs(b), x * i12, av);
+            }
+        }
+        if (LOP) adv[f] = av;
     }
 }
+
+// The 15 fields without second derivatives, in their order: K, A, Theta, Gamma-hat, B, Pi.
+__host__ __device__ constexpr int plainfield(int b) { return b < 11 ? b + 7 : (b < 14 ? b + 11 : F_PI); }
+// Field index of d2 slot b (inverse of d2slot).
+__host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? F_LAPSE : (b < 11 ? b + 11 : F_PHI)); }
 
 // Values, first derivatives and second derivatives of all fields at ghosted offset p, and each field's
 // Kreiss-Oliger sum sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3).
 //   LOP = 1: also the lopsided advection terms adv[f] = sum_d |beta^d| D_d u_f.
-// The fields are a rolled loop: the integer code of one field is about 1,500 instructions.
-// fields: bit f set for the fields to take (the others are left alone).
-template <int LOP = 0>
+//   ALL = 0: only the fields that the constraints take derivatives of (all but Theta, Gamma-hat, the lapse,
+//   the shift and B; the others' entries are left alone).
+// Two rolled loops (the 12 fields with second derivatives, the 15 without): unrolled threefold, the integer
+// code of a field no longer stays in the instruction cache (128^3 step 44 -> 50 ms). Each block's values are
+// loaded one block ahead of their use, so that the loads' latency lies under the previous block's arithmetic.
+template <int LOP = 0, int ALL = 1>
 __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                       double kos[NFIELDS], double* adv = nullptr, unsigned fields = (1u << NFIELDS) - 1) {
+                                       double kos[NFIELDS], double* adv = nullptr) {
+    const long long st[3] = {1, g.pitch, g.plane};
     double bet[3] = {0.0, 0.0, 0.0};
     if (LOP) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) bet[d] = GRF_LDG(s + (F_SHIFT + d) * g.fstride + p);
     }
+    // slots 0..6 (chi, h) and phi; with ALL also lapse and shift (slots 7..10); K, A; with ALL the rest
+    constexpr int kLastSecond = ALL ? 10 : 6, kLastPlain = ALL ? 13 : 6;
+    const double* u = s + p;
+    AxisValues ax;
+    load_axes(g, u, ax);
+    int mag = 0;
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) {
-        if (!(fields >> f & 1u)) continue;
-        const bool first = has_d1(f), second = has_d2(f);
+    for (int b = 0; b < 12; b = (b == kLastSecond ? 11 : b + 1)) {
         FieldDiffs r;
-        field_diffs<LOP>(g, s + f * g.fstride + p, first, second, bet, r);
-        in.v[f] = r.v;
+        const int f = d2field(b);
+        in.v[f] = ax.c;
+        mag = fx_max(mag, axis_diffs<LOP>(g, ax, true, true, bet, r));
+        in.d2[b][0] = r.d2[0]; in.d2[b][3] = r.d2[3]; in.d2[b][5] = r.d2[5];
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) {
+            PlaneValues pl;
+            load_plane(u, c < 2 ? 1 : st[1], c == 0 ? st[1] : st[2], pl);
+            in.d2[b][c < 2 ? c + 1 : 4] = plane_diff(g, pl, mag);
+        }
+        const int next = b == 11 ? F_K : d2field(b == kLastSecond ? 11 : b + 1);
+        u = s + next * g.fstride + p;
+        load_axes(g, u, ax);
         kos[f] = r.ko;
-        if (first) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
+        if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
+    }
+#pragma unroll 1
+    for (int b = 0; b < 15; b = (b == kLastPlain ? 14 : b + 1)) {
+        FieldDiffs r;
+        const AxisValues now = ax;
+        if (b < 14) load_axes(g, s + plainfield(b == kLastPlain ? 14 : b + 1) * g.fstride + p, ax);
+        const int f = plainfield(b);
+        in.v[f] = now.c;
+        mag = fx_max(mag, axis_diffs<LOP>(g, now, has_d1(f), false, bet, r));
+        kos[f] = r.ko;
+        if (has_d1(f)) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
         }
-        if (second) {
-#pragma unroll
-            for (int m = 0; m < 6; ++m) in.d2[d2slot(f)][m] = r.d2[m];
-        }
         if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
     }
-}
-
-// sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3), pair sums added x, y, z
-__device__ __forceinline__ double ko6(const double* __restrict__ u, long long p, long long sy, long long sz) {
-    const long long st[3] = {1, sy, sz};
-    double t[4];
-#pragma unroll
-    for (int r = 1; r <= 3; ++r)
-        t[r] = ((GRF_LDG(u + p - r * st[0]) + GRF_LDG(u + p + r * st[0])) + (GRF_LDG(u + p - r * st[1]) + GRF_LDG(u + p + r * st[1]))) +
-               (GRF_LDG(u + p - r * st[2]) + GRF_LDG(u + p + r * st[2]));
-    return fma(-60.0, GRF_LDG(u + p), fma(15.0, t[1], fma(-6.0, t[2], t[3])));
+    if (mag >> 20 > g.fx.emax) {
+        constexpr unsigned kMetricScalar = ((1u << F_TH) - 1) | 1u << F_PHI | 1u << F_PI;
+        gather_fp64<LOP>(g, s, p, in, kos, adv, ALL ? (1u << NFIELDS) - 1 : kMetricScalar);
+    }
 }
 
 __device__ __forceinline__ bool interior_thread(const Geom& g, int& i, int& j, int& k) {
@@ -295,13 +384,15 @@ __device__ __forceinline__ double rk4_value(const StageArgs& a, long long q, dou
     return (STAGE == 3) ? fma(cs, accf, unf) : fma(cs, kf, unf);
 }
 
-// Interior point q (x fastest) as (i, j, k).
+// Interior point q (x fastest) as (i, j, k); 32-bit divisions where the box allows them.
 __device__ __forceinline__ void point_of(const Geom& g, long long q, int& i, int& j, int& k) {
-    const long long nxy = (long long)g.nx * g.ny;
-    k = (int)(q / nxy);
-    const unsigned r = (unsigned)(q - (long long)k * nxy);
-    j = (int)(r / (unsigned)g.nx);
-    i = (int)(r - (unsigned)j * (unsigned)g.nx);
+    const unsigned nx = (unsigned)g.nx, ny = (unsigned)g.ny;
+    long long row;  // q / nx
+    if (q < (1LL << 32)) row = (unsigned)q / nx;
+    else row = q / nx;
+    i = (int)(q - row * nx);
+    k = (int)((unsigned)row / ny);  // rows of a box that fits the device are below 2^32
+    j = (int)((unsigned)row - (unsigned)k * ny);
 }
 
 // One RK4 stage at one point, fused: gather -> pointwise RHS -> + KO -> stage update ->
@@ -317,16 +408,15 @@ __device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, cons
     bool ok = true;
     point_rhs<double, double, DEC, LOP, COUP>(c, in, r, nullptr, ok, adv);
     if (!ok) atomicOr(a.status, 1);
-    double out[NFIELDS];
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) {
+    for (int f = 0; f < NFIELDS; ++f) {  // r becomes the stage's output values
         const double kf = fma(a.ko, kos[f], r[f]);
         const double unf = (STAGE == 0) ? in.v[f] : a.un[f * g.fstride + p];
-        out[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
+        r[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
     }
-    if (a.enforce) enforce_point(out, a.min_chi, a.min_lapse);
+    if (a.enforce) enforce_point(r, a.min_chi, a.min_lapse);
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) store_with_images(g, a.dst, f, i, j, k, out[f]);
+    for (int f = 0; f < NFIELDS; ++f) store_with_images(g, a.dst, f, i, j, k, r[f]);
 }
 
 // One thread per interior point of [q0, q1), consecutive threads consecutive points in x-fastest order,

@@ -10,9 +10,6 @@ namespace grf {
 
 constexpr int NG6 = 4;  // ghost layers of the 6th-order scheme
 
-// Field index of d2 slot b (inverse of d2slot).
-__host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? F_LAPSE : (b < 11 ? b + 11 : F_PHI)); }
-
 // 6th-order centred first difference times 60 dx at offset p along stride t:
 //   (u_3 - u_-3) - 9 (u_2 - u_-2) + 45 (u_1 - u_-1)
 __device__ __forceinline__ double fd1_6(const double* __restrict__ u, long long p, long long t) {

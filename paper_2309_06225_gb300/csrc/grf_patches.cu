@@ -42,6 +42,7 @@ __host__ __device__ __forceinline__ Geom patch_geom(const PatchTable& t, int a, 
     g.fstride = g.plane * g.NZ;
     g.dx = 0.0;  // the spacing is not used by the copies
     g.i12 = g.i12s = g.i144s = FxScale{0, 0};
+    g.fx = FxRange{0, -1};
     g.periodic = 0;
     g.reflect = 0;
     return g;

@@ -41,26 +41,23 @@ struct TlmArgs {
 
 __device__ __forceinline__ double& comp(D3& x, int c) { return (&x.v)[c]; }
 
-// gather() for the value and its three tangents: each component is a field of its own state.
+// gather() for the value and its three tangents, each a state of its own.
 __device__ __forceinline__ void gather_d3(const Geom& g, const double* const* s, long long p, PointInT<D3>& in,
                                           D3 kos[NFIELDS]) {
+    PointIn one;
+    double ko[NFIELDS];
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) {
-        const bool first = has_d1(f), second = has_d2(f);
+    for (int c = 0; c < 4; ++c) {
+        gather<0>(g, s[c], p, one, ko);
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-            FieldDiffs r;
-            field_diffs<0>(g, s[c] + f * g.fstride + p, first, second, nullptr, r);
-            comp(in.v[f], c) = r.v;
-            comp(kos[f], c) = r.ko;
-            if (first) {
-#pragma unroll
-                for (int d = 0; d < 3; ++d) comp(in.d1[d1slot(f)][d], c) = r.d1[d];
-            }
-            if (second) {
-#pragma unroll
-                for (int m = 0; m < 6; ++m) comp(in.d2[d2slot(f)][m], c) = r.d2[m];
-            }
+        for (int f = 0; f < NFIELDS; ++f) {
+            comp(in.v[f], c) = one.v[f];
+            comp(kos[f], c) = ko[f];
+        }
+#pragma unroll 1
+        for (int m = 0; m < 72; ++m) {
+            comp((&in.d1[0][0])[m], c) = (&one.d1[0][0])[m];
+            comp((&in.d2[0][0])[m], c) = (&one.d2[0][0])[m];
         }
     }
 }

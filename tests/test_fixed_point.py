@@ -1,5 +1,7 @@
 """Block fixed point (csrc/grf_fixed.cuh, host build): stencil sums against exact rational arithmetic.
 
+(The kernels take blocks outside its range in FP64: test_ko_of_extreme_values below, on a GPU.)
+
 Bound, from the representation: each value is kept to one unit of 2^-(52 + guard) of the largest one's
 leading bit (exactly, when it is within 2^guard of the largest), the integer sum is exact, and the result is
 rounded once (the scaled one after a product kept to 63 bits).
@@ -63,8 +65,50 @@ def test_special_values(fixed_sum, guard):
         assert np.isnan(fixed_sum(x, w, guard)) and np.isnan(fixed_sum(x, w, guard, 2.0))
         assert np.isnan(fixed_sum(np.full(16, bad), w, guard, 1e-30))
     big = np.zeros(16)
-    big[5] = 1e308                                                      # weight 64: overflows
-    assert np.isinf(fixed_sum(big, w, guard))
-    assert fixed_sum(big, w, guard, 2.0 ** -20) == 64 * (1e308 * 2.0 ** -20)  # scaled back into range
-    x = np.array([1.7976931348623157e308, -1.7976931348623157e308])
-    assert fixed_sum(x, [1, 1], guard) == 0.0
+    big[5] = 1e308                                                      # beyond the range: the FP64 sums'
+    assert np.isnan(fixed_sum(big, w, guard))
+    assert fixed_sum(big * 2.0 ** -20, w, guard) == 64 * (1e308 * 2.0 ** -20)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["ordinary", "tiny", "huge", "special"])
+def test_ko_of_extreme_values(fixed_sum, kind):
+    """grf_ko_dissipation on fields of any magnitude: the kernel gives the bits of the host build of the sums
+    (checked against exact arithmetic above) or, for a stencil whose largest value is out of the fixed-point
+    range, the FP64 sum, whose non-finite values it keeps."""
+    torch = pytest.importorskip("torch")
+    assert torch.cuda.is_available()
+    import paper_2309_06225_gb300 as g
+    rng = np.random.default_rng(5)
+    dx = 1.0 / 12.0                                     # the spacing constants are 1, 12, 1
+    assert (64.0 / 12.0) / (64.0 * dx) == 1.0
+    box = g.make_box(11, 7, 5, dx, bc=g.GRF_BC_FROZEN)
+    u = rng.normal(size=(27, 11, 13, 17))
+    if kind == "tiny":
+        u *= 10.0 ** rng.uniform(-320, -200, u.shape)
+    elif kind == "huge":
+        u *= 10.0 ** rng.uniform(290, 305, (27, 1, 1, 1))
+    elif kind == "special":
+        u[rng.random(u.shape) < 0.01] = np.nan
+        u[rng.random(u.shape) < 0.01] = np.inf
+        u[rng.random(u.shape) < 0.05] = 0.0
+    t, out = g.to_device(u, box), g.alloc_state(box)
+    g.grf_ko_dissipation(box, 64.0 / 12.0, t, out)
+    got = g.to_host(out, box)[:, 3:-3, 3:-3, 3:-3]
+    st = [(1, 0, 0), (0, 1, 0), (0, 0, 1)]
+    weights = [-60] + [w for _ in st for w in (15, 15, -6, -6, 1, 1)]
+    top = 2046 - 13 - 3                                 # biased exponents above this take the FP64 sum
+    fixed = 0
+    for f in range(27):
+        for k, j, i in np.ndindex(got.shape[1:]):
+            at = lambda d, r: u[f, k + 3 + r * d[2], j + 3 + r * d[1], i + 3 + r * d[0]]
+            x = [u[f, k + 3, j + 3, i + 3]] + [at(d, s * r) for d in st for r in (1, 2, 3) for s in (-1, 1)]
+            e = int(np.max(np.array(x).view(np.int64) >> 52 & 2047))
+            if e <= top:
+                fixed += 1
+                assert got[f, k, j, i] == fixed_sum(x, weights, 2), (f, k, j, i)
+            else:
+                with np.errstate(invalid="ignore", over="ignore"):
+                    ref = sum(np.longdouble(w) * v for w, v in zip(weights, x))
+                assert np.isfinite(ref) or not np.isfinite(got[f, k, j, i])
+    assert fixed > 0
