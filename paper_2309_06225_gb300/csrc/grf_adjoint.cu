@@ -39,6 +39,13 @@
 #include "grf_rev.cuh"
 #include "grf_sphere.cuh"
 
+namespace grf_rev {
+__device__ __forceinline__ Rev recip(const Rev& x) {
+    const double q = grf::recip(x.v);
+    return x.i < 0 ? Rev(q) : Rev(q, GRF_REV_RECORD(x.i, -(q * q), -1, 0.0, -1));
+}
+}  // namespace grf_rev
+
 namespace grf {
 
 using grf_rev::Rev;

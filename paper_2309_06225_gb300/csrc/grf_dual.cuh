@@ -43,7 +43,7 @@ GRF_DHD D3 exp(const D3& a) {
 }
 GRF_DHD D3 operator/(double a, const D3& b) {
     const double q = a / b.v;
-    const double r = a == 1.0 ? -(q * q) : -q / b.v;  // 1/b, the common case, without a second division
+    const double r = -q / b.v;
     return D3(q, r * b.d0, r * b.d1, r * b.d2);
 }
 GRF_DHD D3& operator+=(D3& a, const D3& b) { a = a + b; return a; }

@@ -144,7 +144,19 @@ template <typename T>
 GRF_HD T half_of(const T& x) { return 0.5 * x; }
 template <typename T>
 GRF_HD T twice_of(const T& x) { return 2.0 * x; }
+// 1 / x. For doubles on the device: the approximate reciprocal (20 bits) and two Newton-Raphson steps
+// y <- y + y (1 - x y), 4 FP64 instructions in place of a division's 9 and its branch for special cases. The
+// second step's remainder is below 2^-70, so the result is rounded as a correctly rounded one is but within
+// about 2^-17 of a rounding boundary. Zeros and infinities give NaN.
+template <typename T>
+GRF_HD T recip(const T& x) { return 1.0 / x; }
 #ifdef __CUDA_ARCH__
+__device__ __forceinline__ double recip(const double& x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
 __device__ __forceinline__ double exponent_step(double x, int step) {
     const int hi = __double2hiint(x);
     const unsigned e = ((unsigned)hi << 1) - (2u << 21);
@@ -160,6 +172,14 @@ GRF_HD T sym3_det(const T h[6]) {
     return dot3(h[0], a, h[1], b, h[2], d);
 }
 
+// A value of the point's data, read where it is used. For doubles on the device the read is volatile: kept in
+// registers from an early read, the 198 values of a point would only be spilled and read back from there.
+template <typename T>
+GRF_HD T at_use(const T& x) { return x; }
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ double at_use(const double& x) { return *(const volatile double*)&x; }
+#endif
+
 // symmetric inverse; returns determinant
 template <typename T>
 GRF_HD T sym3_inv(const T h[6], T hi[6], T& id) {
@@ -167,7 +187,7 @@ GRF_HD T sym3_inv(const T h[6], T hi[6], T& id) {
     const T c01 = fnma(h[1], h[5], h[2] * h[4]);
     const T c02 = fnma(h[2], h[3], h[1] * h[4]);
     const T det = dot3(h[0], c00, h[1], c01, h[2], c02);
-    id = 1.0 / det;
+    id = recip(det);
     hi[0] = c00 * id;
     hi[1] = c01 * id;
     hi[2] = c02 * id;
@@ -262,7 +282,7 @@ GRF_HD bool solve7(T M[7][8]) {
             }
         }
         ok = ok && abs_gt(M[k][k], thr);
-        const T ip = 1.0 / M[k][k];
+        const T ip = recip(M[k][k]);
         ipv[k] = ip;
 #pragma unroll
         for (int i = k + 1; i < 7; ++i) {
@@ -293,29 +313,6 @@ GRF_HD T sdotw(const T a[6], const T bw[6]) {
 __host__ __device__ constexpr int third(int i, int j) { return 3 - i - j; }
 __host__ __device__ constexpr bool cyclic(int i, int j) { return (j - i + 3) % 3 == 1; }
 
-// Q_ij(X) = P_ikjl X^kl-type contraction: the Gauss-Bonnet S_ij is -4 [... + Q_ij(C)] with
-//   Q_ij(X) = gamma_ij (X.Phi) - Phi_i^k X_kj - Phi_j^k X_ik + tr(Phi) X_ij - tr(X)(gamma_ij tr(Phi) - Phi_ij)
-template <typename T>
-GRF_HD void q_of(const T X[6], const T gd[6], const T gw[6], const T Phd[6], const T Phuw[6], const T Phm[3][3], T trP,
-                 T out[6]) {
-    const T XP = sdotw(X, Phuw);
-    const T trX = sdotw(X, gw);
-    const T sx = fnma(trX, trP, XP);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j) {
-            T q = fma(gd[sidx(i, j)], sx, fma(trP, X[sidx(i, j)], trX * Phd[sidx(i, j)]));
-            if (i == j) {
-                q = fma(-2.0, dot3(Phm[i][0], X[sidx(0, j)], Phm[i][1], X[sidx(1, j)], Phm[i][2], X[sidx(2, j)]), q);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) q = fnma(Phm[i][k], X[sidx(k, j)], fnma(Phm[j][k], X[sidx(i, k)], q));
-            }
-            out[sidx(i, j)] = q;
-        }
-}
-
 // DEC: the decoupled mode as a compile-time constant (0: full theory, 1: no backreaction), or -1
 // to read c.decoupled at run time.
 // LOP = 1: every advection term beta^k d_k u of an evolved field (the CCZ4 advection terms and
@@ -334,7 +331,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     for (int m = 0; m < 6; ++m) { h[m] = v[F_H + m]; A[m] = v[F_A + m]; }
     T hi[6], ideth;
     sym3_inv(h, hi, ideth);
-    const T ichi = 1.0 / chi;
+    const T ichi = recip(chi);
     // weighted inverses (off-diagonals doubled) for symmetric contractions; gamma^ij = chi h^ij
     T hw[6], gu[6], gw[6], gd[6];
 #pragma unroll
@@ -347,27 +344,50 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     }
 
     GRF_SECTION(1);
-#define D1(f, k) in.d1[d1slot(f)][k]
-#define D2(f, m) in.d2[d2slot(f)][m]
-    T dh[3][6];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int m = 0; m < 6; ++m) dh[k][m] = D1(F_H + m, k);
-    T dchi[3], dal[3], dK[3], dTh[3], dphi[3], dPi[3];
+#define D1(f, k) at_use(in.d1[d1slot(f)][k])
+#define D2(f, m) at_use(in.d2[d2slot(f)][m])
+#define DH1(k, m) D1(F_H + (m), k) /* d_k h_m */
+    T dchi[3], dphi[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        dchi[k] = D1(F_CHI, k); dal[k] = D1(F_LAPSE, k); dK[k] = D1(F_K, k);
-        dTh[k] = D1(F_TH, k); dphi[k] = D1(F_PHI, k); dPi[k] = D1(F_PI, k);
+        dchi[k] = D1(F_CHI, k); dphi[k] = D1(F_PHI, k);
     }
-    T db[3][3];  // db[j][i] = d_j beta^i
+    const T divb = D1(F_SHIFT, 0) + D1(F_SHIFT + 1, 1) + D1(F_SHIFT + 2, 2);
+    
+#define ADV(f) (LOP ? adv[f] : dot3(at_use(v[F_SHIFT]), D1(f, 0), at_use(v[F_SHIFT + 1]), D1(f, 1), at_use(v[F_SHIFT + 2]), D1(f, 2)))
+
+    // ---- the right-hand sides that need no curvature
+    {
+        const T divb23 = (2.0 / 3.0) * divb, al2 = twice_of(al);
+        rhs[F_CHI] = fma((2.0 / 3.0) * chi, fma(al, K, -divb), ADV(F_CHI));
+        T db[3][3];  // db[j][i] = d_j beta^i
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
+        for (int j = 0; j < 3; ++j)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) db[j][i] = D1(F_SHIFT + i, j);
-    const T divb = db[0][0] + db[1][1] + db[2][2];
-    const T bx = v[F_SHIFT], by = v[F_SHIFT + 1], bz = v[F_SHIFT + 2];
-#define ADV(f) (LOP ? adv[f] : dot3(bx, D1(f, 0), by, D1(f, 1), bz, D1(f, 2)))
+            for (int i = 0; i < 3; ++i) db[j][i] = D1(F_SHIFT + i, j);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) {
+                T x = fnma(h[sidx(i, j)], divb23, fnma(al2, A[sidx(i, j)], ADV(F_H + sidx(i, j))));
+                if (i == j) {
+                    x = fma(2.0, dot3(h[sidx(i, 0)], db[i][0], h[sidx(i, 1)], db[i][1], h[sidx(i, 2)], db[i][2]), x);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) x = fma(h[sidx(i, k)], db[j][k], fma(h[sidx(j, k)], db[i][k], x));
+                }
+                rhs[F_H + sidx(i, j)] = x;
+            }
+        const T dal[3] = {D1(F_LAPSE, 0), D1(F_LAPSE, 1), D1(F_LAPSE, 2)};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            rhs[F_SHIFT + i] = fma(c.shift_F * c.inv_1pa, v[F_B + i],
+                                   -((c.a_1pa * al * chi) * dot3(hi[sidx(i, 0)], dal[0], hi[sidx(i, 1)], dal[1],
+                                                                 hi[sidx(i, 2)], dal[2])));
+    }
+    const T K2Th = K - twice_of(Th);
+    rhs[F_LAPSE] = fma(-2.0 * c.inv_1pa * al, K2Th, ADV(F_LAPSE));
+    rhs[F_PHI] = fma(al, Pi, ADV(F_PHI));
 
     // ---- conformal Christoffels: G1[l][ij] = Gt_{l ij}, G2[k][ij] = Gt^k_ij,
     //      Gl_l = h^ij Gt_lij (= h_lk Gt^k), Gtc^k = h^kl Gl_l. Where two of the indices of Gt_lij agree
@@ -381,9 +401,9 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
 #pragma unroll
             for (int j = i; j < 3; ++j) {
                 const int m = sidx(i, j);
-                if (i == l || j == l) G1[l][m] = half_of(dh[i == l ? j : i][sidx(l, l)]);
-                else if (i == j) G1[l][m] = fma(-0.5, dh[l][m], dh[i][sidx(l, i)]);
-                else G1[l][m] = half_of(dh[i][sidx(l, j)] + dh[j][sidx(l, i)] - dh[l][m]);
+                if (i == l || j == l) G1[l][m] = half_of(DH1(i == l ? j : i, sidx(l, l)));
+                else if (i == j) G1[l][m] = fma(-0.5, DH1(l, m), DH1(i, sidx(l, i)));
+                else G1[l][m] = half_of(DH1(i, sidx(l, j)) + DH1(j, sidx(l, i)) - DH1(l, m));
             }
 #pragma unroll
     for (int l = 0; l < 3; ++l) Gl[l] = sdotw(G1[l], hw);
@@ -508,6 +528,11 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     }
     T RZ[6];
     {
+        T dh[3][6];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int m = 0; m < 6; ++m) dh[k][m] = DH1(k, m);
         T U[3][3][3];  // U[k][m][i] = h^lm Gt^k_li
 #pragma unroll
         for (int k = 0; k < 3; ++k)
@@ -562,7 +587,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     T DDa[6], DDp[6];
 #pragma unroll
     for (int m = 0; m < 6; ++m) {
-        DDa[m] = fnma(Gp[0][m], dal[0], fnma(Gp[1][m], dal[1], fnma(Gp[2][m], dal[2], D2(F_LAPSE, m))));
+        DDa[m] = fnma(Gp[0][m], D1(F_LAPSE, 0), fnma(Gp[1][m], D1(F_LAPSE, 1), fnma(Gp[2][m], D1(F_LAPSE, 2), D2(F_LAPSE, m))));
         DDp[m] = fnma(Gp[0][m], dphi[0], fnma(Gp[1][m], dphi[1], fnma(Gp[2][m], dphi[2], D2(F_PHI, m))));
     }
     const T lapal = sdotw(DDa, gw);
@@ -595,6 +620,82 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             AAud[m] = dot3(A[sidx(i, 0)], Aud[0][j], A[sidx(i, 1)], Aud[1][j], A[sidx(i, 2)], Aud[2][j]);
         }
     const T AA = sdotw(A, Auw);
+    // ---- the sources' share apart (rho, S_i and C_ij come below): d_t K, d_t A_ij, d_t Theta, d_t Gamma-hat and
+    // the right-hand side of C_ij, formed where their inputs are at hand, since values kept for later are
+    // spilled. C_ij holds all of (d_t K_ij - L_beta K_ij + D_i D_j alpha)/alpha + K_ik K^k_j, S_ij included:
+    //   d_t K = beta.dK - D^2 alpha + alpha (tr C + K_ij K^ij), and d_t A_ij from the trace-free part of
+    //   alpha C_ij - D_i D_j alpha. The damping and Theta terms, and a non-zero tr A, are those of C's own
+    //   right-hand side (a1: the coefficient of A_ij in it).
+    T Cr[6];  // R^Z_ij + (a1 A_ij - A_ik A^k_j)/chi
+    {
+        const T divb23 = (2.0 / 3.0) * divb, al2 = twice_of(al);
+        const T a1 = fma(-2.0 / 3.0, K, K2Th);
+        const T trA = Aud[0][0] + Aud[1][1] + Aud[2][2], AAt = fnma(a1, trA, AA);
+        rhs[F_K] = fma(al, fma(K, K3, AAt), ADV(F_K) - lapal);
+        // h_ij's coefficient: minus a third of the traces of -chi DDa and of the K_ij K^ij terms
+        const T hc = (1.0 / 3.0) * fma(chi, sdotw(DDa, hw), -(al * AAt));
+        const T aA = fma(al, K2Th - a1, -divb23);  // 2/3 (alpha K - div beta)
+        T db[3][3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) db[j][i] = D1(F_SHIFT + i, j);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) {
+                const int m = sidx(i, j);
+                Cr[m] = fma(ichi, fma(a1, A[m], -AAud[m]), RZ[m]);
+                T x = fnma(chi, DDa[m], fma(h[m], hc, ADV(F_A + m)));
+                x = fma(aA, A[m], fnma(al, AAud[m], x));
+                if (i == j) {
+                    x = fma(2.0, dot3(A[sidx(i, 0)], db[i][0], A[sidx(i, 1)], db[i][1], A[sidx(i, 2)], db[i][2]), x);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) x = fma(A[sidx(i, k)], db[j][k], fma(A[sidx(j, k)], db[i][k], x));
+                }
+                rhs[F_A + m] = x;
+            }
+        // d_t Theta = beta.dTheta + alpha (D_i Z^i - Theta K) - Z^i d_i alpha + alpha Hb / (2 (1 + b)),
+        // with 2 D_i Z^i = RZs - Rs and Z^i = chi (Gamma-hat^i - Gt^i)/2; Hb is added below
+        const T dal[3] = {D1(F_LAPSE, 0), D1(F_LAPSE, 1), D1(F_LAPSE, 2)};
+        const T Zda = half_of(chi) * dot3(dG[0], dal[0], dG[1], dal[1], dG[2], dal[2]);
+        rhs[F_TH] = fma(al, fnma(Th, K, half_of(RZs - Rs)), ADV(F_TH) - Zda);
+        // d_t Gamma-hat^i with everything contracted with h^ij in one covector V_j, with A^ij in va_j and
+        // with d_k beta^i in Gk: h^ij Z_j = (Gamma-hat^i - Gt^i)/2. The b(x) part of d_t Z_j is
+        // -(b/(1+b)) alpha wb_j, wb_j = M_j + d_j Theta - K^k_j Z_k - kappa1 Z_j with the momentum constraint
+        // M_j = B_j - 8 pi S_j (added below); Gamma-hat^i carries 2 h^ij Z_j, so d_t Gamma-hat^i gains
+        // -(2b/(1+b)) alpha h^ij wb_j (2b/(1+b) = 2 - 4 bTh)
+        const T abG = (2.0 - 4.0 * c.bTh) * al;
+        const T m3 = -3.0 * (al * ichi), alK43 = (4.0 / 3.0) * (al * K), al43 = (4.0 / 3.0) * al, Th2 = twice_of(Th);
+        const T cTh = al2 - abG, cZ = fma(abG, c.kappa1, -alK43);
+        T va[3], V[3], Gk[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            va[j] = fma(m3, dchi[j], -2.0 * dal[j]);
+            Gk[j] = fma(c.kappa3, dG[j], Gtc[j]);
+            const T ddbk = D2(F_SHIFT, sidx(j, 0)) + D2(F_SHIFT + 1, sidx(j, 1)) + D2(F_SHIFT + 2, sidx(j, 2));
+            const T kz = dot3(Kud(0, j), Zl[0], Kud(1, j), Zl[1], Kud(2, j), Zl[2]);
+            T x = fma(1.0 / 3.0, ddbk, fma(cTh, D1(F_TH, j), cZ * Zl[j]));
+            x = fnma(Th2, dal[j], fnma(al43, D1(F_K, j), x));
+            V[j] = fma(abG, kz, x);
+        }
+        const T kz2 = fma((2.0 / 3.0) * c.kappa3, divb, -(c.kappa1 * al));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            T x = fma(al2, sdotw(G2[i], Auw), ADV(F_GAM + i));
+            x = fma(kz2, dG[i], fma(divb23, Gtc[i], x));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                x = fma(Au[sidx(i, k)], va[k], x);
+                x = fma(hi[sidx(i, k)], V[k], x);
+                x = fnma(Gk[k], db[k][i], x);
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) x = fma(hw[q], D2(F_SHIFT + i, q), x);
+            rhs[F_GAM + i] = x;
+        }
+    }
     // Codazzi block through its dual: bb[k][m] = B_{k,(m+1),(m+2)} = D_a K_kb - D_b K_ka with
     // (a, b) = (m+1, m+2). The connection's symmetric part cancels between the two covariant
     // derivatives, and with K_ij = (A_ij + h_ij K/3)/chi (D~_a h_kb = 0) so do the derivatives of h:
@@ -608,7 +709,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         T ev[3], Gk[3][3], bx3[3][3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            ev[a] = fma(c2[0], A[sidx(0, a)], fma(c2[1], A[sidx(1, a)], fma(c2[2], A[sidx(2, a)], dK[a] * (1.0 / 3.0))));
+            ev[a] = fma(c2[0], A[sidx(0, a)], fma(c2[1], A[sidx(1, a)], fma(c2[2], A[sidx(2, a)], D1(F_K, a) * (1.0 / 3.0))));
 #pragma unroll
             for (int k = 0; k < 3; ++k) Gk[k][a] = G2[k][sidx(a, k)] + c1[a];
         }
@@ -695,7 +796,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     for (int m = 0; m < 6; ++m) Hij[m] = fma(Kp[m], Pi, DDp[m]);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        Hn[i] = fma(Kud(0, i), dphi[0], fma(Kud(1, i), dphi[1], fma(Kud(2, i), dphi[2], dPi[i])));
+        Hn[i] = fma(Kud(0, i), dphi[0], fma(Kud(1, i), dphi[1], fma(Kud(2, i), dphi[2], D1(F_PI, i))));
     T Phd[6], Phn[3];
     const T b2Pi = b2 * Pi;
 #pragma unroll
@@ -765,25 +866,35 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             for (int i = 0; i < 3; ++i) S8[i] = fma(-g3h, fma(a3, dphi[i], Pi * fma(Pi, Hn[i], -Hdv3[i])), S8[i]);
         }
     }
-    T S1[6], Y[6];
+    // LS_ij = L(8 pi S_ij) without its C and N parts, L(X) = X - gamma tr(X)/2, from the X terms
+    // fX d_i phi d_j phi/2 + XX gamma_ij/2 and -4 Y_ij; the traces are known (gamma^ij B_ijl = B_l, so
+    // tr Y = -2 B_l Phi_n^l):
+    //   L(Y)_ij = B_i Phi_nj + B_j Phi_ni + B_ijl Phi_n^l + B_jil Phi_n^l - gamma_ij B_l Phi_n^l
+    T LS[6];
+    if (dec) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+        for (int m = 0; m < 6; ++m) LS[m] = T(0.0);
+    } else {
+        const T tg = half_of(fma(fXh, dphi2, XXh));
 #pragma unroll
-        for (int j = i; j < 3; ++j) {
-            S1[sidx(i, j)] = dec ? T(0.0) : fma(fXh * dphi[i], dphi[j], XXh * gd[sidx(i, j)]);
-            T y = fma(Bv[j], Phn[i], Bv[i] * Phn[j]);
-            y = fnma(twice_of(BPn), gd[sidx(i, j)], y);
+        for (int i = 0; i < 3; ++i) {
+            const T fd = fXh * dphi[i];
 #pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                if (l != j) y = BCFMA(bb, i, j, l, Phnu[l], y);
-                if (l != i) y = BCFMA(bb, j, i, l, Phnu[l], y);
+            for (int j = i; j < 3; ++j) {
+                T y = fma(Bv[j], Phn[i], fnma(BPn, gd[sidx(i, j)], Bv[i] * Phn[j]));
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
+                    if (l != j) y = BCFMA(bb, i, j, l, Phnu[l], y);
+                    if (l != i) y = BCFMA(bb, j, i, l, Phnu[l], y);
+                }
+                LS[sidx(i, j)] = fma(-4.0, y, fnma(tg, gd[sidx(i, j)], fd * dphi[j]));
             }
-            Y[sidx(i, j)] = dec ? T(0.0) : y;
         }
+    }
 
     GRF_SECTION(12);
-    const T bdPi = LOP ? adv[F_PI] : dot3(bx, dPi[0], by, dPi[1], bz, dPi[2]);
-    const T dadp = dot3(dal[0], dphiu[0], dal[1], dphiu[1], dal[2], dphiu[2]);
+    const T bdPi = LOP ? adv[F_PI] : dot3(at_use(v[F_SHIFT]), D1(F_PI, 0), at_use(v[F_SHIFT + 1]), D1(F_PI, 1), at_use(v[F_SHIFT + 2]), D1(F_PI, 2));
+    const T dadp = dot3(D1(F_LAPSE, 0), dphiu[0], D1(F_LAPSE, 1), dphiu[1], D1(F_LAPSE, 2), dphiu[2]);
 
     // L_GB without its 8 G_S^ij C_ij: -4 B_kij B^kij + 8 B_i B^i, with
     // B_kij B^kij = 2 chi^3 / det(h) h^kk' h_mm' bb[k][m] bb[k'][m']
@@ -810,104 +921,28 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         L0 = 8.0 * (BvBv - BB);
     }
 
-    // ---- CCZ4 right-hand sides without S_ij (rho and S_i included)
+    // ---- rho and S_i in d_t Theta and d_t Gamma-hat
     GRF_SECTION(14);
-    rhs[F_CHI] = fma((2.0 / 3.0) * chi, fma(al, K, -divb), ADV(F_CHI));
-    const T divb23 = (2.0 / 3.0) * divb;
-    const T al2 = twice_of(al);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j) {
-            T x = fnma(h[sidx(i, j)], divb23, fnma(al2, A[sidx(i, j)], ADV(F_H + sidx(i, j))));
-            if (i == j) {
-                x = fma(2.0, dot3(h[sidx(i, 0)], db[i][0], h[sidx(i, 1)], db[i][1], h[sidx(i, 2)], db[i][2]), x);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) x = fma(h[sidx(i, k)], db[j][k], fma(h[sidx(j, k)], db[i][k], x));
-            }
-            rhs[F_H + sidx(i, j)] = x;
-        }
-    const T K2Th = K - twice_of(Th);
     // b(x) of the modified gauge enters through the auxiliary metric g^ab - b n^a n^b of the Z terms
     // of the covariant equation; its 3+1 projection is carried by Hb = H - 16 pi rho
     // - 2 kappa1 (2 + kappa2) Theta (plain H = R - A_ij A^ij + 2/3 K^2) in d_t K and d_t Theta, and
-    // by the momentum-constraint combination in d_t Gamma-hat below.
+    // by the momentum-constraint combination in d_t Gamma-hat.
     const T Hb = fma(-2.0 * c.kappa1 * (2.0 + c.kappa2), Th, fma(-2.0, rho8, fma((2.0 / 3.0) * K, K, Rs - AA)));
-    // kS: (d_t K without advection, the lapse's Laplacian, alpha R^Z and S_ij) / alpha
+    // (d_t K without advection, the lapse's Laplacian, alpha R^Z and S_ij) / alpha
     const T kS = fma(K, K2Th, fma(-3.0 * c.kappa1 * (1.0 + c.kappa2), Th, fma(-1.5, rho8, -c.bK * Hb)));
-    const T Kdot0 = fma(al, kS + RZs, ADV(F_K) - lapal);
-    T Adot0[6];
+    rhs[F_TH] = fma(c.bTh * al, Hb, rhs[F_TH]);
     {
-        T Xa[6];
+        const T abG = (2.0 - 4.0 * c.bTh) * al, cTh = twice_of(al) - abG;
+        T V[3];
 #pragma unroll
-        for (int m = 0; m < 6; ++m) Xa[m] = fma(al, RZ[m], -DDa[m]);
-        const T trX3 = sdotw(Xa, hw) * (1.0 / 3.0);
-        const T aA = fma(al, K2Th, -divb23);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) {
-                const int m = sidx(i, j);
-                T x = fma(chi, fnma(h[m], trX3, Xa[m]), ADV(F_A + m));
-                x = fma(aA, A[m], fnma(al2, AAud[m], x));
-                if (i == j) {
-                    x = fma(2.0, dot3(A[sidx(i, 0)], db[i][0], A[sidx(i, 1)], db[i][1], A[sidx(i, 2)], db[i][2]), x);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) x = fma(A[sidx(i, k)], db[j][k], fma(A[sidx(j, k)], db[i][k], x));
-                }
-                Adot0[m] = x;
-            }
-    }
-    // d_t Theta = beta.dTheta + alpha (D_i Z^i - Theta K) - Z^i d_i alpha + alpha Hb / (2 (1 + b)),
-    // with 2 D_i Z^i = RZs - Rs and Z^i = chi (Gamma-hat^i - Gt^i)/2
-    {
-        const T Zda = half_of(chi) * dot3(dG[0], dal[0], dG[1], dal[1], dG[2], dal[2]);
-        rhs[F_TH] = fma(al, fma(c.bTh, Hb, fnma(Th, K, half_of(RZs - Rs))), ADV(F_TH) - Zda);
-    }
-    {
-        // d_t Gamma-hat^i with everything contracted with h^ij in one covector V_j, with A^ij in va_j and
-        // with d_k beta^i in Gk: h^ij Z_j = (Gamma-hat^i - Gt^i)/2. The b(x) part of d_t Z_j is
-        // -(b/(1+b)) alpha wb_j, wb_j = M_j + d_j Theta - K^k_j Z_k - kappa1 Z_j with the momentum constraint
-        // M_j = B_j - 8 pi S_j; Gamma-hat^i carries 2 h^ij Z_j, so d_t Gamma-hat^i gains
-        // -(2b/(1+b)) alpha h^ij wb_j (2b/(1+b) = 2 - 4 bTh)
-        const T abG = (2.0 - 4.0 * c.bTh) * al;
-        const T m3 = -3.0 * (al * ichi), alK43 = (4.0 / 3.0) * (al * K), al43 = (4.0 / 3.0) * al, Th2 = twice_of(Th);
-        const T cTh = al2 - abG, cZ = fma(abG, c.kappa1, -alK43);
-        T va[3], V[3], Gk[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            va[j] = fma(m3, dchi[j], -2.0 * dal[j]);
-            Gk[j] = fma(c.kappa3, dG[j], Gtc[j]);
-            const T ddbk = D2(F_SHIFT, sidx(j, 0)) + D2(F_SHIFT + 1, sidx(j, 1)) + D2(F_SHIFT + 2, sidx(j, 2));
-            const T kz = dot3(Kud(0, j), Zl[0], Kud(1, j), Zl[1], Kud(2, j), Zl[2]);
-            T x = fma(1.0 / 3.0, ddbk, fma(cTh, dTh[j] - S8[j], cZ * Zl[j]));
-            x = fnma(Th2, dal[j], fnma(al43, dK[j], x));
-            V[j] = fma(abG, kz - Bv[j], x);
-        }
-        const T kz2 = fma((2.0 / 3.0) * c.kappa3, divb, -(c.kappa1 * al));
+        for (int j = 0; j < 3; ++j) V[j] = fma(cTh, S8[j], abG * Bv[j]);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            T x = fma(al2, sdotw(G2[i], Auw), ADV(F_GAM + i));
-            x = fma(kz2, dG[i], fma(divb23, Gtc[i], x));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                x = fma(Au[sidx(i, k)], va[k], x);
-                x = fma(hi[sidx(i, k)], V[k], x);
-                x = fnma(Gk[k], db[k][i], x);
-            }
-#pragma unroll
-            for (int q = 0; q < 6; ++q) x = fma(hw[q], D2(F_SHIFT + i, q), x);
+            T x = fnma(hi[sidx(i, 0)], V[0], fnma(hi[sidx(i, 1)], V[1], fnma(hi[sidx(i, 2)], V[2], rhs[F_GAM + i])));
             rhs[F_GAM + i] = x;
             rhs[F_B + i] = fma(-c.eta, v[F_B + i], x);
-            rhs[F_SHIFT + i] = fma(c.shift_F * c.inv_1pa, v[F_B + i],
-                                   -((c.a_1pa * al * chi) * dot3(hi[sidx(i, 0)], dal[0], hi[sidx(i, 1)], dal[1],
-                                                                 hi[sidx(i, 2)], dal[2])));
         }
     }
-    rhs[F_LAPSE] = fma(-2.0 * c.inv_1pa * al, K2Th, ADV(F_LAPSE));
-    rhs[F_PHI] = fma(al, Pi, ADV(F_PHI));
 
     // ---- coupled system, in the curvature components that hold the unknowns: C_ij = R_ninj (d_t K_ij) and
     // N = H_nn = (d_t Pi - beta^k d_k Pi - d^k alpha d_k phi)/alpha (d_t Pi):
@@ -916,27 +951,25 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
     // shift term of d_t K_ij cancel in it.
     GRF_SECTION(15);
     T Msys[7][8];
-    T S3[6], PPc[6];  // cubic term: 8 pi S3_ij without N, Pi^2 gamma^ij - d^i phi d^j phi
+    T PPc[6];  // cubic term: Pi^2 gamma^ij - d^i phi d^j phi
     {
-        const T a1 = fma(-2.0 / 3.0, K, K2Th);
-        const T a0 = (1.0 / 3.0) * fma((-1.0 / 3.0) * K, K, kS);
-        const T trS1h = half_of(sdotw(S1, gw)), trYh = half_of(sdotw(Y, gw));
+        const T a0 = ((1.0 / 3.0) * ichi) * fma((-1.0 / 3.0) * K, K, kS);
         const T Ss4 = 0.25 * Ss;
         const T four_b1 = 4.0 * b1, b2Pi2x4 = 4.0 * (b2Pi * Pi);
 #pragma unroll
         for (int m = 0; m < 6; ++m) {
-            T r = fma(ichi, fma(a1, A[m], fma(a0, h[m], -AAud[m])), RZ[m]);
+            T r = fma(a0, h[m], Cr[m]);
             T w6 = T(0.0);
             if (!dec) {
                 const T LGS = fnma(Ss4, gd[m], S[m]);
-                r = r - fnma(trS1h, gd[m], S1[m]);
-                r = fma(4.0, fnma(trYh, gd[m], Y[m]), fma(b2Pi2x4, LGS, r));
+                r = fma(b2Pi2x4, LGS, r - LS[m]);
                 w6 = fnma(four_b1, LGS, T(0.0));
             }
             Msys[m][7] = r;
             Msys[m][6] = w6;
         }
-        // 6x6 block, column (a,b): -4 L(Q(E_ab)) with E_ab the unit symmetric matrix
+        // 6x6 block, column (a,b): -4 L(Q(E_ab)) with E_ab the unit symmetric matrix and
+        //   Q_ij(X) = gamma_ij (X.Phi) - Phi_i^k X_kj - Phi_j^k X_ik + tr(Phi) X_ij - tr(X)(gamma_ij tr(Phi) - Phi_ij)
         //   = -2 gamma_ij w_ab (Phi^ab - gamma^ab tr Phi) - 4 w_ab gamma^ab Phi_ij + 4 P_ij,ab - 4 tr(Phi) [ij == ab]
         //   P_ij,ab = Phi_i^k E_kj + Phi_j^k E_ik
         const T one4P = fma(-4.0, trP, 1.0);
@@ -1015,6 +1048,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
             if (!dec) {
                 // 8 pi S3_ij without its N part, and that part's coefficient in the metric rows:
                 // S3_ij = S3_0 + g3 N / 2 (Pi^2 gamma_ij - d_i phi d_j phi)
+                T S3[6];
                 const T pcoef = half_of(trH3);                        // of d_i phi d_j phi
                 const T gcoef = fma(0.5, Hdd3, -(Pi * Hnd3));         // of gamma_ij
 #pragma unroll
@@ -1039,7 +1073,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
 #pragma unroll
             for (int col = 0; col < 6; ++col) PPc[col] = PPuw[col];
         }
-        const T iD = 1.0 / Dphi;
+        const T iD = recip(Dphi);
         const T c8 = -8.0 * (b1 * iD);
 #pragma unroll
         for (int col = 0; col < 6; ++col) Msys[6][col] = c8 * GSuw[col];
@@ -1099,29 +1133,13 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
         }
     }
 
-    // ---- full S_ij at the solution and the final K, A_ij, Pi right-hand sides
+    // ---- the final K, A_ij, Pi right-hand sides
     GRF_SECTION(17);
     {
-        T QC[6], S8ij[6];
-        if (!dec) q_of(C, gd, gw, Phd, Phuw, Phm, trP, QC);
-        const T Phnn = fma(b1, Hnn, b2Pi * Pi);
+        rhs[F_K] = fma(al, sdotw(C, gw), rhs[F_K]);
+        const T trC3 = (1.0 / 3.0) * sdotw(C, hw), alchi = al * chi;
 #pragma unroll
-        for (int m = 0; m < 6; ++m) S8ij[m] = dec ? T(0.0) : fma(-4.0, fma(GS[m], Phnn, Y[m] + QC[m]), S1[m]);
-        if (cub && !dec) {
-            const T gw2 = (0.5 * c.g3) * Hnn;
-#pragma unroll
-            for (int m = 0; m < 6; ++m) {
-                const int i = (m < 3) ? 0 : (m < 5 ? 1 : 2);
-                const int j = (m < 3) ? m : (m < 5 ? m - 2 : 2);
-                S8ij[m] = S8ij[m] + fma(gw2, fma(Pi2, gd[m], -(dphi[i] * dphi[j])), S3[m]);
-            }
-        }
-        const T Ss8 = sdotw(S8ij, gw);
-        rhs[F_K] = fma(half_of(al), Ss8, Kdot0);
-        const T trh3 = sdotw(S8ij, hw) * (1.0 / 3.0);
-        const T alchi = al * chi;
-#pragma unroll
-        for (int m = 0; m < 6; ++m) rhs[F_A + m] = fnma(alchi, fnma(h[m], trh3, S8ij[m]), Adot0[m]);
+        for (int m = 0; m < 6; ++m) rhs[F_A + m] = fma(alchi, fnma(h[m], trC3, C[m]), rhs[F_A + m]);
         rhs[F_PI] = fma(al, Hnn, bdPi + dadp);
     }
     if (extra) {
@@ -1207,6 +1225,7 @@ GRF_HD void point_rhs(const CoeffsT<P>& c, const PointInT<T>& in, T rhs[NFIELDS]
 #undef BC
 #undef BCFMA
 #undef DH
+#undef DH1
 #undef D1
 #undef D2
 #undef ADV

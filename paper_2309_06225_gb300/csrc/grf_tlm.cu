@@ -23,6 +23,10 @@ __device__ __forceinline__ D3 half_of(const D3& x) {
 __device__ __forceinline__ D3 twice_of(const D3& x) {
     return D3(grf::twice_of(x.v), grf::twice_of(x.d0), grf::twice_of(x.d1), grf::twice_of(x.d2));
 }
+__device__ __forceinline__ D3 recip(const D3& x) {
+    const double q = grf::recip(x.v), r = -(q * q);
+    return D3(q, r * x.d0, r * x.d1, r * x.d2);
+}
 }  // namespace grf_dual
 
 namespace grf {
