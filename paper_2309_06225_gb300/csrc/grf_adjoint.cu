@@ -34,9 +34,9 @@
 #include <cstring>
 
 #include "grf.h"
+#include "grf_adjoint.cuh"
 #include "grf_kernels.cuh"
 #include "grf_launch.h"
-#include "grf_rev.cuh"
 #include "grf_sphere.cuh"
 
 namespace grf_rev {
@@ -50,38 +50,6 @@ namespace grf {
 
 using grf_rev::Rev;
 
-// leaves of the pointwise map: values, first derivatives (24 slots x 3), second derivatives
-// (12 slots x 6), KO sums, u_n, acc, lambda, g2
-enum : int { kLV = 0, kLD1 = 27, kLD2 = 99, kLKO = 171, kLUN = 198, kLACC = 225, kLLAM = 252, kLG2 = 253, kNLeaf = 254 };
-// tape entries per point and stage: the pointwise RHS records about 2,250, the stage update and
-// enforcement about 130 more; an overflow is detected and reported
-constexpr int kTapeCap = 5120;
-constexpr int kAdjThreads = 128;
-// tape columns (points per wave): 1024 per SM of a GB300, so that the sweep (at most 64 registers)
-// has 32 warps per SM to hide its dependent memory operations; the taping kernel is held to 128
-// registers for 16 warps per SM (more spills, but it ran faster than at 255 registers with 8)
-constexpr long long kAdjCols = 152LL * 1024;
-constexpr int kSweepThreads = 256;
-// derivative and dissipation adjoints per point (slots of the G buffer): d1 72, d2 72, KO 27
-constexpr int kGD2 = 72, kGKO = 144, kGSlots = 171;
-
-struct AdjArgs {
-    const double* src;    // u_{s-1} (ghosts valid)
-    const double* un;     // u_n
-    const double* acc;    // k_1 + 2 k_2 + 2 k_3 (stage 3)
-    const double* ubar;   // adjoint of the stage output u_s
-    double* abar;         // adjoint of the accumulator: written by stage 3, read by stages 0..2
-    double* vbar;         // adjoint of the values of u_{s-1} (stages 1..3, written)
-    double* unbar;        // adjoint of u_n (stage 3 writes it, stages 2..0 add)
-    double* G;            // kGSlots derivative / KO adjoints, with periodic images
-    double* pbar;         // per-column sums of the lambda and g2 adjoints
-    int* count;           // tape entries of each column (written by the taping kernel)
-    double dt, ko, min_chi, min_lapse;
-    int enforce;
-    int* status;
-    long long npts;
-};
-
 template <typename T>
 __device__ __forceinline__ void enforce_point_t(T u[NFIELDS], double min_chi, double min_lapse) {
     T hh[6], hi[6], id;
@@ -94,36 +62,6 @@ __device__ __forceinline__ void enforce_point_t(T u[NFIELDS], double min_chi, do
     for (int m = 0; m < 6; ++m) u[F_A + m] = fnma(hh[m], tr3, u[F_A + m]);
     u[F_CHI] = fmax(u[F_CHI], T(min_chi));
     u[F_LAPSE] = fmax(u[F_LAPSE], T(min_lapse));
-}
-
-// Reverse sweep of this column's tape: node adjoints are consumed (reset to zero) as they are
-// propagated, so the column is clean for its next point.
-// The tape entries do not depend on the adjoints, so the next entry is loaded while the current
-// one is applied.
-__device__ __forceinline__ void rev_sweep(int entries, long long col) {
-    const long long S = grf_rev::c_tape.stride;
-    double* __restrict__ adj = grf_rev::c_tape.adj;
-    const double2* __restrict__ w = grf_rev::c_tape.w;
-    const ushort4* __restrict__ ix = grf_rev::c_tape.ix;
-    if (entries <= 0) return;
-    double2 pw = __ldcs(&w[(long long)(entries - 1) * S + col]);
-    ushort4 o = __ldcs(&ix[(long long)(entries - 1) * S + col]);
-#pragma unroll 1
-    for (int n = entries - 1; n >= 0; --n) {
-        const double2 pc = pw;
-        const ushort4 oc = o;
-        if (n > 0) {
-            pw = __ldcs(&w[(long long)(n - 1) * S + col]);
-            o = __ldcs(&ix[(long long)(n - 1) * S + col]);
-        }
-        const long long node = (long long)(kNLeaf + n) * S + col;
-        const double g = adj[node];
-        if (g == 0.0) continue;
-        adj[node] = 0.0;
-        if (oc.x != grf_rev::kNone) adj[(long long)oc.x * S + col] = fma(pc.x, g, adj[(long long)oc.x * S + col]);
-        if (oc.y != grf_rev::kNone) adj[(long long)oc.y * S + col] = fma(pc.y, g, adj[(long long)oc.y * S + col]);
-        if (oc.z != grf_rev::kNone) adj[(long long)oc.z * S + col] += g;
-    }
 }
 
 // STAGE (0..3) is a run-time argument: one instantiation of the large pointwise map keeps the
@@ -189,50 +127,6 @@ __global__ void __launch_bounds__(kAdjThreads, 4) adj_tape_kernel(Geom g, Coeffs
         }
     }
     a.count[col] = min(grf_rev::s_count[threadIdx.x], grf_rev::c_tape.cap);
-}
-
-// Sweeps tape column col (point q0 + col) and hands the leaves' adjoints to the stage's outputs:
-// the values' to vbar / unbar / abar, the derivative and KO sums' to G (with periodic images),
-// lambda's and g2's to the column's sums.
-__global__ void __launch_bounds__(kSweepThreads, 4) adj_sweep_kernel(Geom g, AdjArgs a, int STAGE, long long q0) {
-    const long long col = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long q = q0 + col;
-    if (col >= grf_rev::c_tape.stride || q >= a.npts) return;
-    const long long S = grf_rev::c_tape.stride;
-    double* adj = grf_rev::c_tape.adj;
-    auto take = [&](int leaf) {
-        const long long o = (long long)leaf * S + col;
-        const double x = adj[o];
-        adj[o] = 0.0;
-        return x;
-    };
-    rev_sweep(a.count[col], col);
-    const long long nxy = (long long)g.nx * g.ny;
-    const int k = (int)(q / nxy);
-    const long long rem = q - (long long)k * nxy;
-    const int j = (int)(rem / g.nx), i = (int)(rem - (long long)j * g.nx);
-    const long long p = gidx(g, i + NG, j + NG, k + NG);
-#pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) {
-        const long long o = f * g.fstride + p;
-        const double vb = take(kLV + f);
-        if (STAGE == 0) {
-            a.unbar[o] += vb;
-        } else {
-            a.vbar[o] = vb;
-            const double ub = take(kLUN + f);
-            if (STAGE == 3) a.unbar[o] = ub;
-            else a.unbar[o] += ub;
-        }
-        if (STAGE == 3) a.abar[o] = take(kLACC + f);
-        store_with_images(g, a.G, kGKO + f, i, j, k, take(kLKO + f));
-    }
-#pragma unroll 1
-    for (int m = 0; m < 72; ++m) store_with_images(g, a.G, m, i, j, k, take(kLD1 + m));
-#pragma unroll 1
-    for (int m = 0; m < 72; ++m) store_with_images(g, a.G, kGD2 + m, i, j, k, take(kLD2 + m));
-    a.pbar[2 * col] += take(kLLAM);
-    a.pbar[2 * col + 1] += take(kLG2);
 }
 
 // X(q) += transposed stencils of the derivative / KO adjoints at interior q:
@@ -596,12 +490,11 @@ int grf_adjoint_rk4(const grf_box* box, const grf_params* params, const double* 
     a.count = (int*)(base + L.count);
     const dim3 tgrd((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz), tblk(32, 4, 1);
     const int tblocks = (int)((cols + kAdjThreads - 1) / kAdjThreads);
-    const int sblocks = (int)((cols + kSweepThreads - 1) / kSweepThreads);
     // one reversed stage: waves of `cols` points, each taped, then swept
     auto reverse_stage = [&](int stage) {
         for (long long q0 = 0; q0 < a.npts; q0 += cols) {
             adj_tape_kernel<<<tblocks, kAdjThreads, 0, st>>>(g, c, a, stage, q0);
-            adj_sweep_kernel<<<sblocks, kSweepThreads, 0, st>>>(g, a, stage, q0);
+            launch_adj_sweep(g, a, tape, stage, q0, st);
         }
     };
     const double sx0 = box->x0, sy0 = box->y0, sz0 = box->z0;

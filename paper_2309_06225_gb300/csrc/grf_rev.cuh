@@ -42,12 +42,12 @@ struct Tape {
 };
 
 // The tape of the current launch, and each thread's entry count (blocks of up to 256 threads).
-__constant__ Tape c_tape;
-__shared__ int s_count[256];
+static __constant__ Tape c_tape;
+static __shared__ int s_count[256];
 
 __device__ __forceinline__ long long rev_col() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
 
-__device__ __noinline__ int rev_record(int a, double pa, int b, double pb, int c) {
+static __device__ __noinline__ int rev_record(int a, double pa, int b, double pb, int c) {
     const int t = threadIdx.x;
     int n = s_count[t];
     s_count[t] = n + 1;
