@@ -290,7 +290,7 @@ Geom adj_geom(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    set_spacing(g, b->dx);
+    set_spacing(g, b->dx, NG);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;
     return g;

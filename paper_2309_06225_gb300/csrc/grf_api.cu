@@ -28,11 +28,17 @@ __global__ void __launch_bounds__(128) ko_kernel(Geom g, const double* __restric
 }
 
 // The 6th-order scheme's dissipation: rhs += ko sum_d Delta^8_d u (ko = -sigma / (256 dx)).
-__global__ void ko8_kernel(Geom g, const double* __restrict__ s, double* __restrict__ rhs, double ko) {
+__global__ void __launch_bounds__(128) ko8_kernel(Geom g, const double* __restrict__ s, double* __restrict__ rhs, double ko) {
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long long)g.nx * g.ny * g.nz) return;
     int i, j, k;
-    if (!interior_thread(g, i, j, k)) return;
-    const long long p = gidx(g, i + NG6, j + NG6, k + NG6);
-    for (int f = 0; f < NFIELDS; ++f) rhs[f * g.fstride + p] = fma(ko, ko8(s + f * g.fstride, p, g.pitch, g.plane), rhs[f * g.fstride + p]);
+    point_of(g, q, i, j, k);
+    const long long p = (long long)blockIdx.y * g.fstride + gidx(g, i + NG6, j + NG6, k + NG6);
+    AxisValues6 v;
+    load_axes6(g, s + p, v);
+    FieldDiffs r;
+    if (axis_diffs6<0>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko8(s + p, 0, g.pitch, g.plane);
+    rhs[p] = fma(ko, r.ko, rhs[p]);
 }
 
 // Periodic ghost fill: one thread per ghosted (i, j) column and field; walks k.
@@ -215,7 +221,7 @@ Geom make_geom(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    set_spacing(g, b->dx);
+    set_spacing(g, b->dx, b->ng);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = (b->bc == GRF_BC_REFLECT_LOW || b->bc == GRF_BC_REFLECT_LOW_SOMMERFELD);
     return g;
@@ -445,11 +451,9 @@ int grf_rhs(const grf_box* box, const grf_params* params, double* state, double*
 int grf_ko_dissipation(const grf_box* box, double sigma, const double* state, double* rhs_accum, grf_stream_t stream) {
     if (!box_ok(box) || !state || !rhs_accum) return GRF_EINVAL;
     Geom g = make_geom(box);
-    if (g.ng == NG6)
-        ko8_kernel<<<interior_grid(g), kBlock, 0, (cudaStream_t)stream>>>(g, state, rhs_accum, ko_factor(g, sigma));
-    else
-        ko_kernel<<<dim3(point_blocks((long long)g.nx * g.ny * g.nz, 128), NFIELDS), 128, 0, (cudaStream_t)stream>>>(
-            g, state, rhs_accum, ko_factor(g, sigma));
+    const dim3 grid(point_blocks((long long)g.nx * g.ny * g.nz, 128), NFIELDS);
+    if (g.ng == NG6) ko8_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(g, state, rhs_accum, ko_factor(g, sigma));
+    else ko_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(g, state, rhs_accum, ko_factor(g, sigma));
     return check_launch();
 }
 

@@ -71,7 +71,7 @@ void batch_box_desc(BoxDesc& d, const grf_box* b, const grf_params* p, double dt
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    set_spacing(g, b->dx);
+    set_spacing(g, b->dx, NG);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;  // mirror boxes are not accepted here
     d.c = make_coeffs(p);

@@ -9,7 +9,7 @@ namespace grf {
 // part[block][8] = {sum H^2, max|H|, sum M1^2, max|M1|, ...}
 // out4 (H, M_i; with the per-block norm partials in `part`) and dens (the energy densities of the
 // three scalar terms) are each written when non-null.
-// ORD = 4: as rhs_kernel; ORD = 6: the 6th-order per-thread gather.
+// ORD: the order of the scheme.
 // psi4 (2 fields, re and im) receives the Weyl scalar with the triad about the origin; o = the
 // coordinates of interior point (0, 0, 0); hyp (4 fields) the hyperbolicity diagnostics of the
 // coupled system (PointExtraT::hyp). PSI4 = 1 compiles those outputs in (they need the assembled
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, cons
         point_of(g, q, i, j, k);
         p = gidx(g, i + g.ng, j + g.ng, k + g.ng);
         if constexpr (ORD == 4) gather<0, PSI4>(g, s, p, in, kos);
-        else gather6<0>(g, s, p, in, kos, nullptr);
+        else gather6<0, PSI4>(g, s, p, in, kos);
     }
     double vals[4] = {0.0, 0.0, 0.0, 0.0};
     if (live) {

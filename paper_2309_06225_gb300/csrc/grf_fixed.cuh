@@ -28,7 +28,7 @@ namespace grf {
 // A positive finite constant c = m 2^(e - 63), m with its top bit set.
 struct FxScale {
     unsigned long long m;
-    int e;
+    int e, zero;  // (no padding: descriptors that hold it are compared bytewise)
 };
 
 inline FxScale fx_scale_of(double c) {
@@ -36,20 +36,21 @@ inline FxScale fx_scale_of(double c) {
     std::memcpy(&b, &c, sizeof b);
     FxScale s;
     s.e = (int)(b >> 52) - 1023;
+    s.zero = 0;
     s.m = (b << 11) | 0x8000000000000000ull;
     return s;
 }
 
-// Block exponents whose results (sums of magnitude 2^0 .. 2^63 units, times constants of exponents lo .. hi
-// or 1) are normal doubles.
+// Block exponents whose results (sums of magnitude 2^0 .. 2^63 units, or of 2^shift units where fx_room
+// coarsens them, times constants of exponents lo .. hi or 1) are normal doubles.
 struct FxRange {
     int emin, emax;
 };
 
-inline FxRange fx_range(int lo, int hi) {
+inline FxRange fx_range(int lo, int hi, int shift = 0) {
     FxRange r;
     r.emin = 66 - (lo < 0 ? lo : 0);
-    r.emax = 2046 - 13 - (hi > 0 ? hi : 0);
+    r.emax = 2046 - 13 - shift - (hi > 0 ? hi : 0);
     if (r.emin > r.emax) r.emax = -1;  // no block qualifies
     return r;
 }
@@ -108,6 +109,19 @@ GRF_HD unsigned long long fx_normal(long long I, int& z) {
     z = u ? __builtin_clzll(u) : 64;
     return u ? u << z : 0;
 #endif
+}
+
+// The right shift that leaves `bits` clear bits (and the sign) above the values whose magnitudes are OR-ed in
+// mag: sums of larger total weight stay exact while the values are small, and keep 62 - bits bits of the
+// largest one otherwise.
+GRF_HD unsigned long long fx_abs(long long x) { return (unsigned long long)(x < 0 ? -x : x); }
+GRF_HD int fx_room(unsigned long long mag, int bits) {
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)mag);
+#else
+    const int z = mag ? __builtin_clzll(mag) : 64;
+#endif
+    return z > bits ? 0 : bits + 1 - z;
 }
 
 // The double of mantissa p (64 bits, top bit set; rounded to nearest) and biased exponent E in the normal

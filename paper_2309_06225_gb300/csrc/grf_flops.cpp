@@ -187,6 +187,21 @@ int grf_host_point_hyp(const grf_params* p, const double* v, const double* d1, c
     return ok ? 0 : -5;
 }
 
+// The 6th-order second difference 2 (x6 + x0) - 27 (x5 + x1) + 270 (x4 + x2) - 490 x3 of 7 values, as
+// axis_diffs6 takes it.
+double grf_host_fixed_second6(const double* x) {
+    int mag = 0;
+    for (int i = 0; i < 7; ++i) mag = grf::fx_max(mag, grf::fx_mag(x[i]));
+    const grf::FxRange range = grf::fx_range(0, 0, 10);
+    const int e = grf::fx_max(mag >> 20, range.emin), lim = grf::fx_lim<2>(e);
+    if (e > range.emax) return std::nan("");
+    long long v[7];
+    for (int i = 0; i < 7; ++i) v[i] = grf::fx_int(x[i], lim);
+    const long long c2 = v[3] + v[3], p1 = v[4] + v[2] - c2, p2 = v[5] + v[1] - c2, p3 = v[6] + v[0] - c2;
+    const int sh = grf::fx_room(grf::fx_abs(p1) | grf::fx_abs(p2) | grf::fx_abs(p3), 9);
+    return grf::fx_value<2>(270 * (p1 >> sh) - 27 * (p2 >> sh) + 2 * (p3 >> sh), e + sh);
+}
+
 // sum_i w[i] x[i] in block fixed point with `guard` (1 or 2) guard bits, times c when c > 0; NaN above the range.
 double grf_host_fixed_sum(const double* x, const int* w, int n, int guard, double c) {
     int mag = 0;

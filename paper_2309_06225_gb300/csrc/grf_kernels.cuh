@@ -30,17 +30,21 @@ struct Geom {
     int periodic;            // ghosts are periodic images (written by the owner of each value)
     int reflect;             // the three low faces are mirror planes (images written by the owner)
     int ng;                  // ghost layers: 3 (4th-order scheme) or 4 (6th-order scheme)
-    FxScale i12, i12s, i144s;  // 1/(12 dx), 1/(12 dx^2), 1/(144 dx^2) (4th-order scheme)
-    FxRange fx;                // block exponents of the fixed-point sums
+    // the scheme's factors of first, second and mixed differences (4th order: 1/(12 dx), 1/(12 dx^2),
+    // 1/(144 dx^2); 6th order: 1/(60 dx), 1/(180 dx^2), 1/(3600 dx^2)), and the fixed-point sums' range
+    FxScale f1, f2, f11;
+    FxRange fx;
 };
 
-inline void set_spacing(Geom& g, double dx) {
+inline void set_spacing(Geom& g, double dx, int ng) {
+    const double d1 = ng == 4 ? 60.0 : 12.0, d2 = ng == 4 ? 180.0 : 12.0;
+    g.ng = ng;
     g.dx = dx;
-    g.i12 = fx_scale_of(1.0 / (12.0 * dx));
-    g.i12s = fx_scale_of(1.0 / (12.0 * dx * dx));
-    g.i144s = fx_scale_of(1.0 / (144.0 * dx * dx));
-    const int lo = g.i144s.e < g.i12.e ? g.i144s.e : g.i12.e, hi = g.i12s.e > g.i12.e ? g.i12s.e : g.i12.e;
-    g.fx = fx_range(lo, hi);
+    g.f1 = fx_scale_of(1.0 / (d1 * dx));
+    g.f2 = fx_scale_of(1.0 / (d2 * dx * dx));
+    g.f11 = fx_scale_of(1.0 / (d1 * d1 * dx * dx));
+    const int lo = g.f11.e < g.f1.e ? g.f11.e : g.f1.e, hi = g.f2.e > g.f1.e ? g.f2.e : g.f1.e;
+    g.fx = fx_range(lo, hi, ng == 4 ? 10 : 0);
 }
 
 constexpr int NG = 3;        // ghost layers of the 4th-order kernels (those of this header)
@@ -142,12 +146,12 @@ __device__ __forceinline__ int axis_diffs(const Geom& g, const AxisValues& v, bo
         const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
         const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
         const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2;  // pair sums less 2 u0
-        if (first) r.d1[d] = fx_value<2>(((q1 - m1) << 3) + (m2 - q2), e, g.i12);
-        if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<2>((p1 << 4) - p2, e, g.i12s);
+        if (first) r.d1[d] = fx_value<2>(((q1 - m1) << 3) + (m2 - q2), e, g.f1);
+        if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<2>((p1 << 4) - p2, e, g.f2);
         if (LOP) {
             const bool fw = bet[d] >= 0.0;
             const long long a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, b1 = fw ? m1 : q1;
-            r.up[d] = fx_value<2>(18 * a1 - 6 * a2 + a3 - 3 * b1 - 5 * c2, e, g.i12);
+            r.up[d] = fx_value<2>(18 * a1 - 6 * a2 + a3 - 3 * b1 - 5 * c2, e, g.f1);
         }
         t1 += p1;
         t2 += p2;
@@ -172,14 +176,29 @@ __device__ __forceinline__ double plane_diff(const Geom& g, const PlaneValues& v
 #pragma unroll
     for (int a = 0; a < 4; ++a)
         d[a] = ((fx_int(v.x[a][2], lim) - fx_int(v.x[a][1], lim)) << 3) + (fx_int(v.x[a][0], lim) - fx_int(v.x[a][3], lim));
-    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, g.i144s);
+    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, g.f11);
 }
+
+// The fields that the constraints take derivatives of: all but Theta, Gamma-hat, the lapse, the shift and B.
+constexpr unsigned kMetricScalarFields = ((1u << F_TH) - 1) | 1u << F_PHI | 1u << F_PI;
+
+// Where a gather's results go: a point's data, dissipation sums and (LOP) advection terms.
+struct PointSink {
+    PointIn& in;
+    double* kos;
+    double* adv;
+    __device__ __forceinline__ void value(int f, double x) const { in.v[f] = x; }
+    __device__ __forceinline__ void first(int slot, int d, double x) const { in.d1[slot][d] = x; }
+    __device__ __forceinline__ void second(int slot, int m, double x) const { in.d2[slot][m] = x; }
+    __device__ __forceinline__ void dissipation(int f, double x) const { kos[f] = x; }
+    __device__ __forceinline__ void advection(int f, double x) const { adv[f] = x; }
+};
 
 // The differences in FP64, for a point whose fields leave the fixed-point range (values near overflow,
 // infinities, NaNs): rewrites what gather() took.
-template <int LOP>
-__device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                         double* kos, double* adv, unsigned fields) {
+template <int LOP, typename Sink>
+__device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict__ s, long long p, const Sink& out,
+                                         unsigned fields) {
     const double i12 = 1.0 / (12.0 * g.dx), i12s = 1.0 / (12.0 * g.dx * g.dx);
     const long long st[3] = {1, g.pitch, g.plane};
 #pragma unroll 1
@@ -188,13 +207,13 @@ __device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict
         const double* u = s + f * g.fstride + p;
         const double u0 = GRF_LDG(u);
         double av = 0.0;
-        kos[f] = ko6(u, 0, g.pitch, g.plane);
+        out.dissipation(f, ko6(u, 0, g.pitch, g.plane));
 #pragma unroll 1
         for (int d = 0; d < 3; ++d) {
-            if (has_d1(f)) in.d1[d1slot(f)][d] = fd1(u, 0, st[d], i12);
+            if (has_d1(f)) out.first(d1slot(f), d, fd1(u, 0, st[d], i12));
             if (has_d2(f)) {
-                in.d2[d2slot(f)][d == 0 ? 0 : (d == 1 ? 3 : 5)] = fd2(u, 0, st[d], u0, i12s);
-                in.d2[d2slot(f)][d == 2 ? 4 : d + 1] = mixed_local(u, 0, st[d == 2], st[d == 0 ? 1 : 2], i12);
+                out.second(d2slot(f), d == 0 ? 0 : (d == 1 ? 3 : 5), fd2(u, 0, st[d], u0, i12s));
+                out.second(d2slot(f), d == 2 ? 4 : d + 1, mixed_local(u, 0, st[d == 2], st[d == 0 ? 1 : 2], i12));
             }
             if (LOP) {
                 const double b = GRF_LDG(s + (F_SHIFT + d) * g.fstride + p);
@@ -204,7 +223,7 @@ __device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict
                 av = fma(fabs(b), x * i12, av);
             }
         }
-        if (LOP) adv[f] = av;
+        if (LOP) out.advection(f, av);
     }
 }
 
@@ -216,14 +235,14 @@ __host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? 
 // Values, first derivatives and second derivatives of all fields at ghosted offset p, and each field's
 // Kreiss-Oliger sum sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3).
 //   LOP = 1: also the lopsided advection terms adv[f] = sum_d |beta^d| D_d u_f.
-//   ALL = 0: only the fields that the constraints take derivatives of (all but Theta, Gamma-hat, the lapse,
-//   the shift and B; the others' entries are left alone).
+//   ALL = 0: only the kMetricScalarFields (the others' entries are left alone).
 // Two rolled loops (the 12 fields with second derivatives, the 15 without): unrolled threefold, the integer
 // code of a field no longer stays in the instruction cache (128^3 step 44 -> 50 ms). Each block's values are
 // loaded one block ahead of their use, so that the loads' latency lies under the previous block's arithmetic.
-template <int LOP = 0, int ALL = 1>
-__device__ __forceinline__ void gather(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                       double kos[NFIELDS], double* adv = nullptr) {
+//   TEAM > 1: the point's fields are shared out over TEAM consecutive lanes, of which this is lane t (every
+//   lane of the warp calls this; in, kos and adv are the team's).
+template <int LOP, int ALL, int TEAM, typename Sink>
+__device__ __forceinline__ void gather_to(const Geom& g, const double* __restrict__ s, long long p, const Sink& out, int t) {
     const long long st[3] = {1, g.pitch, g.plane};
     double bet[3] = {0.0, 0.0, 0.0};
     if (LOP) {
@@ -232,50 +251,67 @@ __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__
     }
     // slots 0..6 (chi, h) and phi; with ALL also lapse and shift (slots 7..10); K, A; with ALL the rest
     constexpr int kLastSecond = ALL ? 10 : 6, kLastPlain = ALL ? 13 : 6;
-    const double* u = s + p;
+    auto next_second = [](int b) { return TEAM > 1 ? b + TEAM : (b == kLastSecond ? 11 : b + 1); };
+    auto next_plain = [](int b) { return TEAM > 1 ? b + TEAM : (b == kLastPlain ? 14 : b + 1); };
+    const double* u = s + d2field(t) * g.fstride + p;
     AxisValues ax;
     load_axes(g, u, ax);
     int mag = 0;
 #pragma unroll 1
-    for (int b = 0; b < 12; b = (b == kLastSecond ? 11 : b + 1)) {
+    for (int b = t; b < 12; b = next_second(b)) {
         FieldDiffs r;
         const int f = d2field(b);
-        in.v[f] = ax.c;
+        out.value(f, ax.c);
         mag = fx_max(mag, axis_diffs<LOP>(g, ax, true, true, bet, r));
-        in.d2[b][0] = r.d2[0]; in.d2[b][3] = r.d2[3]; in.d2[b][5] = r.d2[5];
+        out.second(b, 0, r.d2[0]);
+        out.second(b, 3, r.d2[3]);
+        out.second(b, 5, r.d2[5]);
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
             PlaneValues pl;
             load_plane(u, c < 2 ? 1 : st[1], c == 0 ? st[1] : st[2], pl);
-            in.d2[b][c < 2 ? c + 1 : 4] = plane_diff(g, pl, mag);
+            out.second(b, c < 2 ? c + 1 : 4, plane_diff(g, pl, mag));
         }
-        const int next = b == 11 ? F_K : d2field(b == kLastSecond ? 11 : b + 1);
+        const int nb = next_second(b), next = nb < 12 ? d2field(nb) : plainfield(t);
         u = s + next * g.fstride + p;
         load_axes(g, u, ax);
-        kos[f] = r.ko;
+        out.dissipation(f, r.ko);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
-        if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
+        for (int d = 0; d < 3; ++d) out.first(d1slot(f), d, r.d1[d]);
+        if (LOP) out.advection(f, fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0])));
     }
 #pragma unroll 1
-    for (int b = 0; b < 15; b = (b == kLastPlain ? 14 : b + 1)) {
+    for (int b = t; b < 15; b = next_plain(b)) {
         FieldDiffs r;
         const AxisValues now = ax;
-        if (b < 14) load_axes(g, s + plainfield(b == kLastPlain ? 14 : b + 1) * g.fstride + p, ax);
+        if (next_plain(b) < 15) load_axes(g, s + plainfield(next_plain(b)) * g.fstride + p, ax);
         const int f = plainfield(b);
-        in.v[f] = now.c;
+        out.value(f, now.c);
         mag = fx_max(mag, axis_diffs<LOP>(g, now, has_d1(f), false, bet, r));
-        kos[f] = r.ko;
+        out.dissipation(f, r.ko);
         if (has_d1(f)) {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
+            for (int d = 0; d < 3; ++d) out.first(d1slot(f), d, r.d1[d]);
         }
-        if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
+        if (LOP) out.advection(f, fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0])));
+    }
+    unsigned fields = ALL ? (1u << NFIELDS) - 1 : kMetricScalarFields;
+    if (TEAM > 1) {
+#pragma unroll
+        for (int o = 1; o < TEAM; o *= 2) mag = fx_max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+        fields = 0;
+        for (int b = t; b < 12; b += TEAM) fields |= 1u << d2field(b);
+        for (int b = t; b < 15; b += TEAM) fields |= 1u << plainfield(b);
     }
     if (mag >> 20 > g.fx.emax) {
-        constexpr unsigned kMetricScalar = ((1u << F_TH) - 1) | 1u << F_PHI | 1u << F_PI;
-        gather_fp64<LOP>(g, s, p, in, kos, adv, ALL ? (1u << NFIELDS) - 1 : kMetricScalar);
+        gather_fp64<LOP>(g, s, p, out, fields);
     }
+}
+
+template <int LOP = 0, int ALL = 1, int TEAM = 1>
+__device__ __forceinline__ void gather(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
+                                       double kos[NFIELDS], double* adv = nullptr, int t = 0) {
+    gather_to<LOP, ALL, TEAM>(g, s, p, PointSink{in, kos, adv}, t);
 }
 
 __device__ __forceinline__ bool interior_thread(const Geom& g, int& i, int& j, int& k) {

@@ -1,7 +1,7 @@
 // 6th-order scheme ("Accuracy": 4th- and 6th-order finite differences) on boxes with 4 ghost
 // layers: centred 6th-order first, second and mixed differences, Kreiss-Oliger dissipation with
 // the 8th difference, and the 6th-order lopsided advection stencil (offsets -2..4 towards the
-// side the shift points to). Each thread gathers its own point (no shuffles or shared rows).
+// side the shift points to). The sums are in block fixed point as the 4th-order ones.
 #pragma once
 
 #include "grf_kernels.cuh"
@@ -26,9 +26,10 @@ __device__ __forceinline__ double fd1_6(const double* __restrict__ u, long long 
 //   lopsided, beta^d >= 0 (mirrored for beta^d < 0; a_n = u at n points towards the side beta^d
 //   points to, b_n = u at n points away from it):
 //           beta^d D_d u = |beta^d| (2 b_2 - 24 b_1 - 35 u_0 + 80 a_1 - 30 a_2 + 8 a_3 - a_4) / (60 dx)
+// In FP64, for points whose fields leave the fixed-point range. `fields` as for gather_fp64.
 template <int LOP>
-__device__ __forceinline__ void gather6(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                        double kos[NFIELDS], double* adv) {
+__device__ __noinline__ void gather6_fp64(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
+                                          double* kos, double* adv, unsigned fields) {
     const double i60 = 1.0 / (60.0 * g.dx), i180s = 1.0 / (180.0 * g.dx * g.dx);
     const long long st[3] = {1, g.pitch, g.plane};
     double bet[3] = {0.0, 0.0, 0.0};
@@ -38,6 +39,7 @@ __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict_
     }
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
+        if (!(fields >> f & 1u)) continue;
         const double* u = s + f * g.fstride;
         const double u0 = __ldg(u + p);
         in.v[f] = u0;
@@ -86,193 +88,164 @@ __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict_
     }
 }
 
-// ---- block gather of the 6th-order scheme: blocks of 32 x 4 threads, each warp one x-row of
-// 32 consecutive points, the 4 warps consecutive y-rows. A mixed derivative d_s d_t u is the
-// 6th-order s-stencil applied to the first t-derivatives D_t u at s-offsets +-1..3; along x those
-// are the neighbouring lanes' own first derivatives (shuffles), plus a halo of 3 points beyond each
-// end of the row; d_y d_z takes the first z-derivatives of the rows y0-3 .. y0+6 from shared
-// memory. Threads past the interior take part at the last ghost column / row needed by interior
-// points (x, y <= n + 2), so every load stays inside the ghosted box.
+// ---- the gather in block fixed point
 
-// Halo of a warp's row: D_t (t = y, z) of the 12 fields with second derivatives at x0-3 .. x0-1
-// and x0+32 .. x0+34 (q = 0 .. 5). Combination c = 2 b + t (0 .. 23) lives in register c / 5 at
-// lanes 6 (c % 5) + q, so the register is the same for every lane of a shuffle.
-struct WarpRow6 {
-    int lane;
-    double hv[5];
+struct AxisValues6 {
+    double c, m[3][4], q[3][4];  // the point; at -(k+1) and +(k+1) along axis d
 };
 
-__device__ __forceinline__ double fd1_6r(const double* __restrict__ u, long long p, long long t, double i60) {
-    return __dmul_rn(fd1_6(u, p, t), i60);
-}
-
-__device__ __forceinline__ void warp_row_halo6(const Geom& g, const double* __restrict__ s, int x0, int j, int k, int lane,
-                                               WarpRow6& wr) {
-    const double i60 = 1.0 / (60.0 * g.dx);
-    wr.lane = lane;
-    const int q = lane % 6, cl = lane / 6;  // lanes 30, 31 hold nothing
-    const int hx = min(q < 3 ? x0 - 3 + q : x0 + 29 + q, g.nx + 2);
-    const long long ph = gidx(g, hx + NG6, j + NG6, k + NG6);
-#pragma unroll
-    for (int r = 0; r < 5; ++r) {
-        const int c = 5 * r + cl;
-        double v = 0.0;
-        if (lane < 30 && c < 24) {
-            const int b = c >> 1, t = c & 1;
-            v = fd1_6r(s + (long long)d2field(b) * g.fstride, ph, t ? g.plane : g.pitch, i60);
-        }
-        wr.hv[r] = v;
-    }
-}
-
-// d_x d_t u of d2 slot b from this lane's own D = D_t u and its neighbours'.
-__device__ __forceinline__ double mixed_x_warp6(const WarpRow6& wr, int b, int t, double own, double i60) {
-    const unsigned full = 0xffffffffu;
-    const int c = 2 * b + t, r = c / 5, base = 6 * (c % 5);
-    const int L = wr.lane;
-    double m[4], pl[4];
-    const double dn1 = __shfl_up_sync(full, own, 1), dn2 = __shfl_up_sync(full, own, 2), dn3 = __shfl_up_sync(full, own, 3);
-    const double up1 = __shfl_down_sync(full, own, 1), up2 = __shfl_down_sync(full, own, 2), up3 = __shfl_down_sync(full, own, 3);
-#pragma unroll
-    for (int o = 1; o <= 3; ++o) {
-        // a lane needs the halo on at most one side for offset o: below x0 (q = L - o + 3) or
-        // beyond x0 + 31 (q = L + o - 29)
-        const int qh = (L - o < 0) ? L - o + 3 : (L + o > 31 ? L + o - 29 : 0);
-        const double h = __shfl_sync(full, wr.hv[r], base + qh);
-        const double nm = o == 1 ? dn1 : (o == 2 ? dn2 : dn3);
-        const double np = o == 1 ? up1 : (o == 2 ? up2 : up3);
-        m[o] = (L - o < 0) ? h : nm;
-        pl[o] = (L + o > 31) ? h : np;
-    }
-    return __dmul_rn(fma(45.0, pl[1] - m[1], fma(-9.0, pl[2] - m[2], pl[3] - m[3])), i60);
-}
-
-struct YzRows6 {
-    double dz[12][10][32];  // rounded first z-derivatives on rows y0-3 .. y0+6 (row index y - y0 + 3)
-};
-
-// Every thread of the block calls this, then __syncthreads(). Warp wy fills its own row (y0+wy)
-// and, for wy < 3, the halo rows y0-3+wy and y0+4+wy.
-__device__ __forceinline__ void yz_rows_fill6(const Geom& g, const double* __restrict__ s, int x, int y0, int wy, int k,
-                                              int lane, YzRows6& sh) {
-    const double i60 = 1.0 / (60.0 * g.dx);
-    const int xc = min(x, g.nx + 2);
-    const int rows[3] = {wy + 3, wy, wy + 7};
-    const int nr = wy < 3 ? 3 : 1;
-    for (int q = 0; q < nr; ++q) {
-        const int ry = min(y0 - 3 + rows[q], g.ny + 2);
-        const long long po = gidx(g, xc + NG6, ry + NG6, k + NG6);
-#pragma unroll
-        for (int b = 0; b < 12; ++b) sh.dz[b][rows[q]][lane] = fd1_6r(s + (long long)d2field(b) * g.fstride, po, g.plane, i60);
-    }
-}
-
-// gather6 in block mode (all 128 threads of the block take part): as gather6, the x-mixed and
-// d_y d_z derivatives from the neighbours, the first z-derivatives of the 12 fields with second
-// derivatives from the shared rows.
-template <int LOP>
-__device__ __forceinline__ void gather6_block(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
-                                              double kos[NFIELDS], double* adv, const WarpRow6& wr, const YzRows6& sh,
-                                              int wy) {
-    const double i60 = 1.0 / (60.0 * g.dx), i180s = 1.0 / (180.0 * g.dx * g.dx);
+__device__ __forceinline__ void load_axes6(const Geom& g, const double* __restrict__ u, AxisValues6& v) {
     const long long st[3] = {1, g.pitch, g.plane};
-    const int lane = threadIdx.x & 31;
+    v.c = __ldg(u);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v.m[d][k] = __ldg(u - (k + 1) * st[d]);
+            v.q[d][k] = __ldg(u + (k + 1) * st[d]);
+        }
+}
+
+// As axis_diffs, 6th order. The weights of the second derivative (total 1,100) and of the dissipation (768)
+// exceed the room above two guard bits, so those sums are taken of second differences, shifted right only
+// where these are large (fx_room).
+template <int LOP>
+__device__ __forceinline__ int axis_diffs6(const Geom& g, const AxisValues6& v, bool first, bool second,
+                                           const double* bet, FieldDiffs& r) {
+    int mag = fx_mag(v.c);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mag = fx_max(mag, fx_max(fx_mag(v.m[d][k]), fx_mag(v.q[d][k])));
+    const int e = fx_max(mag >> 20, g.fx.emin), lim = fx_lim<2>(e);
+    const long long c0 = fx_int(v.c, lim), c2 = c0 + c0;
+    long long t1 = 0, t2 = 0, t3 = 0, t4 = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const long long m1 = fx_int(v.m[d][0], lim), q1 = fx_int(v.q[d][0], lim);
+        const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
+        const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
+        const long long m4 = fx_int(v.m[d][3], lim), q4 = fx_int(v.q[d][3], lim);
+        const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2, p3 = q3 + m3 - c2;  // pair sums less 2 u0
+        if (first) r.d1[d] = fx_value<2>(45 * (q1 - m1) - 9 * (q2 - m2) + (q3 - m3), e, g.f1);
+        if (second) {
+            const int sh = fx_room(fx_abs(p1) | fx_abs(p2) | fx_abs(p3), 9);
+            r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] =
+                fx_value<2>(270 * (p1 >> sh) - 27 * (p2 >> sh) + 2 * (p3 >> sh), e + sh, g.f2);
+        }
+        if (LOP) {
+            const bool fw = bet[d] >= 0.0;
+            const long long a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, a4 = fw ? q4 : m4;
+            const long long b1 = fw ? m1 : q1, b2 = fw ? m2 : q2;
+            r.up[d] = fx_value<2>(80 * a1 - 30 * a2 + 8 * a3 - a4 - 24 * b1 + 2 * b2 - 35 * c0, e, g.f1);
+        }
+        t1 += p1;
+        t2 += p2;
+        t3 += p3;
+        t4 += q4 + m4 - c2;
+    }
+    const int sh = fx_room(fx_abs(t1) | fx_abs(t2) | fx_abs(t3) | fx_abs(t4), 7);
+    r.ko = fx_value<2>(28 * (t2 >> sh) - 56 * (t1 >> sh) - 8 * (t3 >> sh) + (t4 >> sh), e + sh);
+    return mag;
+}
+
+// A mixed derivative: the tensor product of the first-difference weights (-1, 9, -45, 45, -9, 1) on its 36
+// points, first differences along b of the six rows, then along a, with their own block exponent.
+__device__ __forceinline__ double plane_diff6(const Geom& g, const double* __restrict__ u, long long sa, long long sb,
+                                              int& mag) {
+    double x[6][6];
+    int top = 0;
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+#pragma unroll
+        for (int b = 0; b < 6; ++b) {
+            x[a][b] = __ldg(u + (a < 3 ? a - 3 : a - 2) * sa + (b < 3 ? b - 3 : b - 2) * sb);
+            top = fx_max(top, fx_mag(x[a][b]));
+        }
+    mag = fx_max(mag, top);
+    const int e = fx_max(top >> 20, g.fx.emin), lim = fx_lim<2>(e);
+    long long d[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+        d[a] = 45 * (fx_int(x[a][3], lim) - fx_int(x[a][2], lim)) - 9 * (fx_int(x[a][4], lim) - fx_int(x[a][1], lim)) +
+               (fx_int(x[a][5], lim) - fx_int(x[a][0], lim));
+    const long long d1 = d[3] - d[2], d2 = d[4] - d[1], d3 = d[5] - d[0];
+    const int sh = fx_room(fx_abs(d1) | fx_abs(d2) | fx_abs(d3), 6);
+    return fx_value<2>(45 * (d1 >> sh) - 9 * (d2 >> sh) + (d3 >> sh), e + sh, g.f11);
+}
+
+// As gather() (LOP and ALL likewise), 6th order; kos[f] = sum_d Delta^8_d u. Rolled loops over the fields and
+// over the three planes of a field.
+template <int LOP = 0, int ALL = 1>
+__device__ __forceinline__ void gather6(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
+                                        double kos[NFIELDS], double* adv = nullptr) {
+    const long long st[3] = {1, g.pitch, g.plane};
+    constexpr unsigned kFields = ALL ? (1u << NFIELDS) - 1 : kMetricScalarFields;
     double bet[3] = {0.0, 0.0, 0.0};
     if (LOP) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) bet[d] = __ldg(s + (F_SHIFT + d) * g.fstride + p);
     }
+    int mag = 0;
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
-        const double* u = s + f * g.fstride;
-        const double u0 = __ldg(u + p);
-        in.v[f] = u0;
-        double pr[3][5], d1[3];
-        double av = 0.0;
+        if (!(kFields >> f & 1u)) continue;
+        const double* u = s + f * g.fstride + p;
+        const bool first = has_d1(f), second = has_d2(f);
+        AxisValues6 ax;
+        load_axes6(g, u, ax);
+        FieldDiffs r;
+        in.v[f] = ax.c;
+        mag = fx_max(mag, axis_diffs6<LOP>(g, ax, first, second, bet, r));
+        kos[f] = r.ko;
+        if (first) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            double m[5], q[5];
-#pragma unroll
-            for (int r = 1; r <= 4; ++r) {
-                m[r] = __ldg(u + p - r * st[d]);
-                q[r] = __ldg(u + p + r * st[d]);
-                pr[d][r] = m[r] + q[r];
-            }
-            const double x = fma(45.0, q[1] - m[1], fma(-9.0, q[2] - m[2], q[3] - m[3]));
-            if (d == 1 && has_d2(f)) d1[d] = __dmul_rn(x, i60);      // shared with the neighbours' d_x d_y
-            else if (d == 2 && has_d2(f)) d1[d] = sh.dz[d2slot(f)][wy + 3][lane];
-            else d1[d] = x * i60;
-            if (!(f >= F_B && f < F_B + 3)) in.d1[d1slot(f)][d] = d1[d];
-            if (LOP) {
-                const bool fw = bet[d] >= 0.0;
-                const double a1 = fw ? q[1] : m[1], a2 = fw ? q[2] : m[2], a3 = fw ? q[3] : m[3], a4 = fw ? q[4] : m[4];
-                const double b1 = fw ? m[1] : q[1], b2 = fw ? m[2] : q[2];
-                const double y = fma(80.0, a1, fma(-30.0, a2, fma(8.0, a3, -a4))) + fma(2.0, b2, fma(-24.0, b1, -35.0 * u0));
-                av = fma(fabs(bet[d]), y * i60, av);
-            }
+            for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
         }
-        if (LOP) adv[f] = av;
-        if (has_d2(f)) {
+        if (second) {
             const int b = d2slot(f);
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                in.d2[b][d == 0 ? 0 : (d == 1 ? 3 : 5)] =
-                    fma(270.0, pr[d][1], fma(-27.0, pr[d][2], fma(2.0, pr[d][3], -490.0 * u0))) * i180s;
-            in.d2[b][1] = mixed_x_warp6(wr, b, 0, d1[1], i60);
-            in.d2[b][2] = mixed_x_warp6(wr, b, 1, d1[2], i60);
-            const double(*rz)[32] = sh.dz[b];
-            const int c = wy + 3;
-            in.d2[b][4] = __dmul_rn(fma(45.0, rz[c + 1][lane] - rz[c - 1][lane],
-                                        fma(-9.0, rz[c + 2][lane] - rz[c - 2][lane], rz[c + 3][lane] - rz[c - 3][lane])),
-                                    i60);
+            in.d2[b][0] = r.d2[0];
+            in.d2[b][3] = r.d2[3];
+            in.d2[b][5] = r.d2[5];
+#pragma unroll 1
+            for (int c = 0; c < 3; ++c)
+                in.d2[b][c < 2 ? c + 1 : 4] = plane_diff6(g, u, c < 2 ? 1 : st[1], c == 0 ? st[1] : st[2], mag);
         }
-        double t[5];
-#pragma unroll
-        for (int r = 1; r <= 4; ++r) t[r] = (pr[0][r] + pr[1][r]) + pr[2][r];
-        kos[f] = fma(210.0, u0, fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
+        if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
     }
+    if (mag >> 20 > g.fx.emax) gather6_fp64<LOP>(g, s, p, in, kos, adv, kFields);
 }
 
 // One RK4 stage at one point of a 6th-order box, as stage_point (a.ko = -sigma/(256 dx)).
 template <int STAGE, int LOP>
-__device__ __forceinline__ void stage_point6(const Geom& g, const Coeffs& c, const StageArgs& a, int i, int j, int k,
-                                             const YzRows6& sh) {
-    const int lane = threadIdx.x & 31;
-    const int ic = min(i, g.nx + 2), jc = min(j, g.ny + 2);
-    const long long p = gidx(g, ic + NG6, jc + NG6, k + NG6);
+__device__ __forceinline__ void stage_point6(const Geom& g, const Coeffs& c, const StageArgs& a, int i, int j, int k) {
+    const long long p = gidx(g, i + NG6, j + NG6, k + NG6);
     PointIn in;
     double kos[NFIELDS], adv[LOP ? NFIELDS : 1];
-    WarpRow6 wr;
-    warp_row_halo6(g, a.src, i - lane, jc, k, lane, wr);
-    gather6_block<LOP>(g, a.src, p, in, kos, adv, wr, sh, threadIdx.y);
-    if (i >= g.nx || j >= g.ny) return;
+    gather6<LOP>(g, a.src, p, in, kos, adv);
     double r[NFIELDS];
     bool ok = true;
     point_rhs<double, double, -1, LOP>(c, in, r, nullptr, ok, adv);
     if (!ok) atomicOr(a.status, 1);
-    double out[NFIELDS];
 #pragma unroll 1
     for (int f = 0; f < NFIELDS; ++f) {
         const double kf = fma(a.ko, kos[f], r[f]);
         const double unf = (STAGE == 0) ? in.v[f] : a.un[f * g.fstride + p];
-        out[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
+        r[f] = rk4_value<STAGE>(a, f * g.fstride + p, kf, unf);
     }
-    if (a.enforce) enforce_point(out, a.min_chi, a.min_lapse);
+    if (a.enforce) enforce_point(r, a.min_chi, a.min_lapse);
 #pragma unroll 1
-    for (int f = 0; f < NFIELDS; ++f) store_with_images<NG6>(g, a.dst, f, i, j, k, out[f]);
+    for (int f = 0; f < NFIELDS; ++f) store_with_images<NG6>(g, a.dst, f, i, j, k, r[f]);
 }
 
-// Blocks of (32, 4, 1) threads (block gather); one plane per grid.z. The decoupled mode is read
-// from c at run time.
+// One thread per interior point of [q0, q1), as rk4_stage_kernel. The decoupled mode is read from c.
 template <int STAGE, int LOP>
 __global__ void __launch_bounds__(128, 3) rk4_stage6_kernel(Geom g, Coeffs c, StageArgs a) {
-    __shared__ YzRows6 sh;
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    const int j = blockIdx.y * 4 + threadIdx.y;
-    const int k = blockIdx.z;
-    yz_rows_fill6(g, a.src, i, blockIdx.y * 4, threadIdx.y, k, threadIdx.x, sh);
-    __syncthreads();
-    stage_point6<STAGE, LOP>(g, c, a, i, j, k, sh);
+    const long long q = a.q0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= a.q1) return;
+    int i, j, k;
+    point_of(g, q, i, j, k);
+    stage_point6<STAGE, LOP>(g, c, a, i, j, k);
 }
 
 // sum_d Delta^8_d u at ghosted offset p (pair sums added x, y, z)

@@ -38,8 +38,9 @@ void launch_stage_lopsided(int stage, unsigned blocks, unsigned threads, cudaStr
                            const StageArgs& a);
 void launch_stage_general(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                           const StageArgs& a);
-void launch_stage6(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a);
-void launch_stage6_lopsided(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
+void launch_stage6(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
+                   const StageArgs& a);
+void launch_stage6_lopsided(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                             const StageArgs& a);
 // Threads per block of a launch with one thread per point: 128, or 32 while a whole launch is less than
 // one wave of warps (12 a SM), where single-warp blocks spread evenly over the SMs.

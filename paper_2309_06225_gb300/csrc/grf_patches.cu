@@ -41,7 +41,7 @@ __host__ __device__ __forceinline__ Geom patch_geom(const PatchTable& t, int a, 
     g.plane = g.pitch * g.NY;
     g.fstride = g.plane * g.NZ;
     g.dx = 0.0;  // the spacing is not used by the copies
-    g.i12 = g.i12s = g.i144s = FxScale{0, 0};
+    g.f1 = g.f2 = g.f11 = FxScale{0, 0, 0};
     g.fx = FxRange{0, -1};
     g.periodic = 0;
     g.reflect = 0;
@@ -216,7 +216,7 @@ int grf_patch_copy(const grf_patch_level* level, double* box_state, double* cons
     box.pitch = B.pitch;
     box.plane = B.pitch * box.NY;
     box.fstride = box.plane * box.NZ;
-    set_spacing(box, B.dx);
+    set_spacing(box, B.dx, NG);
     box.periodic = 1;
     box.reflect = 0;
     const int h = direction == 0 ? 2 * NG : 0;

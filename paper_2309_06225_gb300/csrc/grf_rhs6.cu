@@ -4,25 +4,18 @@
 
 namespace grf {
 
-// Blocks of (32, 4, 1) threads (block gather, as rk4_stage6_kernel). LOP: lopsided advection.
+// One thread per interior point. LOP: lopsided advection.
 template <int LOP>
 __global__ void __launch_bounds__(128) rhs6_kernel(Geom g, Coeffs c, const double* __restrict__ s,
                                                    double* __restrict__ rhs, double ko, int* status) {
-    __shared__ YzRows6 sh;
-    const int lane = threadIdx.x;
-    const int i = blockIdx.x * 32 + lane;
-    const int j = blockIdx.y * 4 + threadIdx.y;
-    const int k = blockIdx.z;
-    yz_rows_fill6(g, s, i, blockIdx.y * 4, threadIdx.y, k, lane, sh);
-    __syncthreads();
-    const int jc = min(j, g.ny + 2);
-    const long long p = gidx(g, min(i, g.nx + 2) + NG6, jc + NG6, k + NG6);
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long long)g.nx * g.ny * g.nz) return;
+    int i, j, k;
+    point_of(g, q, i, j, k);
+    const long long p = gidx(g, i + NG6, j + NG6, k + NG6);
     PointIn in;
     double kos[NFIELDS], adv[LOP ? NFIELDS : 1];
-    WarpRow6 wr;
-    warp_row_halo6(g, s, i - lane, jc, k, lane, wr);
-    gather6_block<LOP>(g, s, p, in, kos, adv, wr, sh, threadIdx.y);
-    if (i >= g.nx || j >= g.ny) return;
+    gather6<LOP>(g, s, p, in, kos, adv);
     double r[NFIELDS];
     bool ok = true;
     point_rhs<double, double, -1, LOP>(c, in, r, nullptr, ok, adv);
@@ -32,9 +25,10 @@ __global__ void __launch_bounds__(128) rhs6_kernel(Geom g, Coeffs c, const doubl
 }
 
 void launch_rhs6(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs, double ko, int* status) {
-    const dim3 block(32, 4, 1), grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
-    if (c.advection) rhs6_kernel<kLopsided><<<grid, block, 0, st>>>(g, c, s, rhs, ko, status);
-    else rhs6_kernel<0><<<grid, block, 0, st>>>(g, c, s, rhs, ko, status);
+    const long long n = (long long)g.nx * g.ny * g.nz;
+    const unsigned threads = point_threads(n), blocks = point_blocks(n, threads);
+    if (c.advection) rhs6_kernel<kLopsided><<<blocks, threads, 0, st>>>(g, c, s, rhs, ko, status);
+    else rhs6_kernel<0><<<blocks, threads, 0, st>>>(g, c, s, rhs, ko, status);
 }
 
 void launch_constraints6(dim3 grid, cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* out4,

@@ -5,14 +5,14 @@
 
 namespace grf {
 void launch_stage(int stage, int k0, int planes, cudaStream_t st, const Geom& g, const Coeffs& c, StageArgs a) {
-    if (g.ng != NG) {
-        launch_stage6(stage, st, g, c, a);
-        return;
-    }
     const long long nxy = (long long)g.nx * g.ny;
     a.q0 = k0 * nxy;
     a.q1 = (k0 + planes) * nxy;
     const unsigned threads = point_threads(a.q1 - a.q0), blocks = point_blocks(a.q1 - a.q0, threads);
+    if (g.ng != NG) {
+        launch_stage6(stage, blocks, threads, st, g, c, a);
+        return;
+    }
     if (c.advection) {
         launch_stage_lopsided(stage, blocks, threads, st, g, c, a);
         return;

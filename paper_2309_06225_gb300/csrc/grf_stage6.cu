@@ -4,17 +4,17 @@
 #include "grf_launch.h"
 
 namespace grf {
-void launch_stage6(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a) {
-    const dim3 block(32, 4, 1), grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+void launch_stage6(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
+                   const StageArgs& a) {
     if (c.advection) {
-        launch_stage6_lopsided(stage, grid, block, st, g, c, a);
+        launch_stage6_lopsided(stage, blocks, threads, st, g, c, a);
         return;
     }
     switch (stage) {
-        case 0: rk4_stage6_kernel<0, 0><<<grid, block, 0, st>>>(g, c, a); break;
-        case 1: rk4_stage6_kernel<1, 0><<<grid, block, 0, st>>>(g, c, a); break;
-        case 2: rk4_stage6_kernel<2, 0><<<grid, block, 0, st>>>(g, c, a); break;
-        default: rk4_stage6_kernel<3, 0><<<grid, block, 0, st>>>(g, c, a); break;
+        case 0: rk4_stage6_kernel<0, 0><<<blocks, threads, 0, st>>>(g, c, a); break;
+        case 1: rk4_stage6_kernel<1, 0><<<blocks, threads, 0, st>>>(g, c, a); break;
+        case 2: rk4_stage6_kernel<2, 0><<<blocks, threads, 0, st>>>(g, c, a); break;
+        default: rk4_stage6_kernel<3, 0><<<blocks, threads, 0, st>>>(g, c, a); break;
     }
 }
 }  // namespace grf

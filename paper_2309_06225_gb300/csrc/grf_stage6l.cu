@@ -3,13 +3,13 @@
 #include "grf_launch.h"
 
 namespace grf {
-void launch_stage6_lopsided(int stage, dim3 grid, dim3 block, cudaStream_t st, const Geom& g, const Coeffs& c,
+void launch_stage6_lopsided(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                             const StageArgs& a) {
     switch (stage) {
-        case 0: rk4_stage6_kernel<0, kLopsided><<<grid, block, 0, st>>>(g, c, a); break;
-        case 1: rk4_stage6_kernel<1, kLopsided><<<grid, block, 0, st>>>(g, c, a); break;
-        case 2: rk4_stage6_kernel<2, kLopsided><<<grid, block, 0, st>>>(g, c, a); break;
-        default: rk4_stage6_kernel<3, kLopsided><<<grid, block, 0, st>>>(g, c, a); break;
+        case 0: rk4_stage6_kernel<0, kLopsided><<<blocks, threads, 0, st>>>(g, c, a); break;
+        case 1: rk4_stage6_kernel<1, kLopsided><<<blocks, threads, 0, st>>>(g, c, a); break;
+        case 2: rk4_stage6_kernel<2, kLopsided><<<blocks, threads, 0, st>>>(g, c, a); break;
+        default: rk4_stage6_kernel<3, kLopsided><<<blocks, threads, 0, st>>>(g, c, a); break;
     }
 }
 }  // namespace grf

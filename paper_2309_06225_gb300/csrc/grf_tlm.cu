@@ -45,26 +45,17 @@ struct TlmArgs {
 
 __device__ __forceinline__ double& comp(D3& x, int c) { return (&x.v)[c]; }
 
-// gather() for the value and its three tangents, each a state of its own.
-__device__ __forceinline__ void gather_d3(const Geom& g, const double* const* s, long long p, PointInT<D3>& in,
-                                          D3 kos[NFIELDS]) {
-    PointIn one;
-    double ko[NFIELDS];
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-        gather<0>(g, s[c], p, one, ko);
-#pragma unroll 1
-        for (int f = 0; f < NFIELDS; ++f) {
-            comp(in.v[f], c) = one.v[f];
-            comp(kos[f], c) = ko[f];
-        }
-#pragma unroll 1
-        for (int m = 0; m < 72; ++m) {
-            comp((&in.d1[0][0])[m], c) = (&one.d1[0][0])[m];
-            comp((&in.d2[0][0])[m], c) = (&one.d2[0][0])[m];
-        }
-    }
-}
+// One component (0: the value, 1..3: the tangents) of a dual point.
+struct DualSink {
+    PointInT<D3>& in;
+    D3* kos;
+    int c;
+    __device__ __forceinline__ void value(int f, double x) const { comp(in.v[f], c) = x; }
+    __device__ __forceinline__ void first(int slot, int d, double x) const { comp(in.d1[slot][d], c) = x; }
+    __device__ __forceinline__ void second(int slot, int m, double x) const { comp(in.d2[slot][m], c) = x; }
+    __device__ __forceinline__ void dissipation(int f, double x) const { comp(kos[f], c) = x; }
+    __device__ __forceinline__ void advection(int, double) const {}
+};
 
 __device__ __forceinline__ void enforce_point_d3(D3 u[NFIELDS], double min_chi, double min_lapse) {
     D3 hh[6], hi[6], id;
@@ -88,7 +79,8 @@ __global__ void __launch_bounds__(128) tlm_stage_kernel(Geom g, CoeffsT<D3> c, T
     const long long p = gidx(g, i + NG, j + NG, k + NG);
     PointInT<D3> in;
     D3 kos[NFIELDS];
-    gather_d3(g, a.src, p, in, kos);
+#pragma unroll 1
+    for (int cmp = 0; cmp < 4; ++cmp) gather_to<0, 1, 1>(g, a.src[cmp], p, DualSink{in, kos, cmp}, 0);
     D3 r[NFIELDS];
     bool ok = true;
     point_rhs<D3, D3>(c, in, r, nullptr, ok);
@@ -195,7 +187,7 @@ Geom geom_from(const grf_box* b) {
     g.pitch = b->pitch;
     g.plane = b->pitch * g.NY;
     g.fstride = g.plane * g.NZ;
-    set_spacing(g, b->dx);
+    set_spacing(g, b->dx, NG);
     g.periodic = (b->bc == GRF_BC_PERIODIC);
     g.reflect = 0;  // mirror boxes are not accepted here
     return g;

@@ -53,6 +53,30 @@ def test_sums_against_exact(fixed_sum, weights, guard, spread):
             assert abs(got - exact) <= bound, (x, c, float(got), float(exact))
 
 
+@pytest.mark.parametrize("rough", [0.0, 1e-12, 1e-3, 1.0])
+def test_sixth_order_second_difference_against_exact(rough):
+    """The sums whose weights exceed the room above the values: exact while the second differences are small,
+    else with them cut to 53 bits (a unit of 2^-53 of the largest one, times the weights 299, at most)."""
+    from paper_2309_06225_gb300 import build
+    L = C.CDLL(build.build_flops())
+    L.grf_host_fixed_second6.restype = C.c_double
+    L.grf_host_fixed_second6.argtypes = [C.POINTER(C.c_double)]
+    w = [2, -27, 270, -490, 270, -27, 2]
+    rng = np.random.default_rng(3)
+    for t in range(2000):
+        x = (1.0 + rough * rng.uniform(-1, 1, 7)) * 2.0 ** int(rng.integers(-100, 100)) * rng.choice([-1.0, 1.0])
+        if rough == 1.0:
+            x *= rng.choice([-1.0, 1.0], 7)             # alternating signs: the largest second differences
+        f = [Fraction(float(v)) for v in x]
+        exact = sum(a * b for a, b in zip(w, f))
+        top = Fraction(2) ** (int(np.frexp(np.max(np.abs(x)))[1]) - 1)
+        second = max(abs(f[3 + r] + f[3 - r] - 2 * f[3]) for r in (1, 2, 3))
+        bound = 299 * (second / 2 ** 53 if second > top / 2 ** 2 else 0) + 1098 * top / 2 ** 54 * any(
+            v != 0 and abs(v) * 4 < top for v in f) + abs(exact) * Fraction(1, 2 ** 53)
+        got = Fraction(L.grf_host_fixed_second6(x.ctypes.data_as(C.POINTER(C.c_double))))
+        assert abs(got - exact) <= bound, (list(x), float(got), float(exact))
+
+
 @pytest.mark.parametrize("guard", [1, 2])
 def test_special_values(fixed_sum, guard):
     w = MIXED
