@@ -30,8 +30,11 @@ inline Coeffs make_coeffs(const grf_params* p) {
 // One stage on the interior z-planes [k0, k0 + planes) of a box: picks the instantiation and the launch
 // shape (grf_stage.cu).
 void launch_stage(int stage, int k0, int planes, cudaStream_t st, const Geom& g, const Coeffs& c, StageArgs a);
-// Its instantiations, each in its own translation unit: without backreaction; lopsided advection; every
+// Its instantiations, each in its own translation unit: small boxes (a team of 4 or 2 lanes per
+// point); without backreaction; lopsided advection; every
 // coupling (both decoupled modes compiled in); the 6th-order scheme, centred and lopsided.
+void launch_stage_team4(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a);
+void launch_stage_team2(int stage, cudaStream_t st, const Geom& g, const Coeffs& c, const StageArgs& a);
 void launch_stage_decoupled(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
                             const StageArgs& a);
 void launch_stage_lopsided(int stage, unsigned blocks, unsigned threads, cudaStream_t st, const Geom& g, const Coeffs& c,
@@ -45,6 +48,9 @@ void launch_stage6_lopsided(int stage, unsigned blocks, unsigned threads, cudaSt
 // Threads per block of a launch with one thread per point: 128, or 32 while a whole launch is less than
 // one wave of warps (12 a SM), where single-warp blocks spread evenly over the SMs.
 inline unsigned point_threads(long long npts) { return npts <= 152LL * 12 * 32 ? 32u : 128u; }
+// Whether a launch takes teams of `team` lanes per point: while that leaves each of the 4 schedulers of an SM
+// one warp at most.
+inline bool team_fits(long long npts, int team) { return npts * team <= 152LL * 4 * 32; }
 inline unsigned point_blocks(long long npts, unsigned threads) { return (unsigned)((npts + threads - 1) / threads); }
 void launch_rhs6(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s, double* rhs,
                  double ko, int* status);

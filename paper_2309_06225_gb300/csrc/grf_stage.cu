@@ -13,6 +13,14 @@ void launch_stage(int stage, int k0, int planes, cudaStream_t st, const Geom& g,
         launch_stage6(stage, blocks, threads, st, g, c, a);
         return;
     }
+    if (team_fits(a.q1 - a.q0, 4)) {
+        launch_stage_team4(stage, st, g, c, a);
+        return;
+    }
+    if (team_fits(a.q1 - a.q0, 2)) {
+        launch_stage_team2(stage, st, g, c, a);
+        return;
+    }
     if (c.advection) {
         launch_stage_lopsided(stage, blocks, threads, st, g, c, a);
         return;
