@@ -10,7 +10,7 @@
 // 4-point Lagrange polynomials (cubic, 4th order) on the points i0-1 .. i0+2 around the sample.
 // Three launches, all sums in a fixed order: the Gauss-Legendre rule (one thread per node), the
 // ring sums (one block per ring: the ring's samples into shared memory, then one thread per m),
-// the modes (one thread per (l, m)).
+// the modes (one block per (l, m)).
 #include <cstdint>
 
 #include <math_constants.h>
@@ -87,16 +87,26 @@ __device__ __forceinline__ double interp4(const Geom& g, const double* __restric
 }
 
 // One block per ring theta_i: its nphi samples into shared memory, then F_m for m = -lmax .. lmax
-// (thread lmax + m), written to F[i][lmax + m] (re, im).
+// (thread lmax + m), written to F[i][lmax + m] (re, im). Up to kTablePhi samples the phases e^{2 pi i k/nphi}
+// are tabulated too, by all threads: taken one by one inside the sum, a sincospi is most of its time
+// (24 rings of 48 samples now 29 us).
+constexpr int kTablePhi = 1024;
+
+template <bool TABLE>
 __global__ void __launch_bounds__(256) ring_sums_kernel(Geom g, const double* __restrict__ fre,
                                                         const double* __restrict__ fim, SphereArgs s,
                                                         const double* __restrict__ mu, double* __restrict__ F) {
-    __shared__ double sre[kMaxNphi], sim[kMaxNphi];
+    constexpr int N = TABLE ? kTablePhi : kMaxNphi;
+    __shared__ double sre[N], sim[N], tc[TABLE ? N : 1], ts[TABLE ? N : 1];
     const int i = blockIdx.x;
     const double ct = mu[i], st = sqrt(fmax(0.0, 1.0 - ct * ct));
     for (int j = threadIdx.x; j < s.nphi; j += blockDim.x) {
         double sp, cp;
         sincospi(2.0 * j / s.nphi, &sp, &cp);
+        if (TABLE) {
+            tc[j] = cp;
+            ts[j] = sp;
+        }
         const double x = s.cx + s.R * st * cp, y = s.cy + s.R * st * sp, z = s.cz + s.R * ct;
         sre[j] = interp4(g, fre, s, x, y, z);
         sim[j] = fim ? interp4(g, fim, s, x, y, z) : 0.0;
@@ -104,11 +114,19 @@ __global__ void __launch_bounds__(256) ring_sums_kernel(Geom g, const double* __
     __syncthreads();
     const int nm = 2 * s.lmax + 1;
     if ((int)threadIdx.x >= nm) return;
-    const int m = (int)threadIdx.x - s.lmax;
+    const int m = (int)threadIdx.x - s.lmax, step = m < 0 ? (m % s.nphi + s.nphi) % s.nphi : m % s.nphi;
     double ar = 0.0, ai = 0.0;
+    int k = 0;  // m j modulo nphi
     for (int j = 0; j < s.nphi; ++j) {
-        double sp, cp;
-        sincospi(2.0 * m * j / s.nphi, &sp, &cp);  // e^{-i m phi_j} = cp - i sp
+        double sp, cp;  // e^{-i m phi_j} = cp - i sp
+        if (TABLE) {
+            cp = tc[k];
+            sp = ts[k];
+            k += step;
+            if (k >= s.nphi) k -= s.nphi;
+        } else {
+            sincospi(2.0 * m * j / s.nphi, &sp, &cp);
+        }
         ar = fma(sre[j], cp, fma(sim[j], sp, ar));
         ai = fma(sim[j], cp, fma(-sre[j], sp, ai));
     }
@@ -117,40 +135,50 @@ __global__ void __launch_bounds__(256) ring_sums_kernel(Geom g, const double* __
     F[2 * ((long long)i * nm + m + s.lmax) + 1] = ai * dphi;
 }
 
-// A_lm(theta) of sY_lm = A_lm(theta) e^{i m phi} (Goldberg et al.'s sum, Condon-Shortley phase).
+// A_lm(theta) of sY_lm = A_lm(theta) e^{i m phi} (Goldberg et al.'s sum, Condon-Shortley phase):
+//   sin^2l(theta/2) sum_r c_r cot^k(theta/2) = sum_r c_r cos^k(theta/2) sin^(2l - k)(theta/2), k = 2r + s - m
+// in integer powers of non-negative exponent (c_r vanishes for the others).
 __device__ double sylm_theta(int s, int l, int m, double ct) {
     if (l < abs(s) || abs(m) > l) return 0.0;
     auto fact = [](int n) { double f = 1.0; for (int k = 2; k <= n; ++k) f *= k; return f; };
     auto binom = [&](int n, int k) { return (k < 0 || k > n) ? 0.0 : fact(n) / (fact(k) * fact(n - k)); };
+    auto power = [](double x, int n) {
+        double p = 1.0;
+        for (; n > 0; n >>= 1, x *= x)
+            if (n & 1) p *= x;
+        return p;
+    };
     const double pre = ((m & 1) ? -1.0 : 1.0) *
                        sqrt(fact(l + m) * fact(l - m) * (2 * l + 1) / (4.0 * CUDART_PI * fact(l + s) * fact(l - s)));
-    // sin^2(theta/2) = (1 - cos theta)/2, cot(theta/2) = sqrt((1 + cos theta)/(1 - cos theta))
-    const double s2 = 0.5 * (1.0 - ct), cot = sqrt((1.0 + ct) / (1.0 - ct));
+    const double sh = sqrt(0.5 * (1.0 - ct)), ch = sqrt(0.5 * (1.0 + ct));
     double sum = 0.0;
     for (int r = 0; r <= l - s; ++r) {
         const double c = binom(l - s, r) * binom(l + s, r + s - m);
         if (c == 0.0) continue;
-        sum += c * (((l - r - s) & 1) ? -1.0 : 1.0) * pow(cot, (double)(2 * r + s - m));
+        const int k = 2 * r + s - m;
+        sum += c * (((l - r - s) & 1) ? -1.0 : 1.0) * power(ch, k) * power(sh, 2 * l - k);
     }
-    return pre * pow(s2, (double)l) * sum;
+    return pre * sum;
 }
 
-// a_lm = sum_i w_i A_lm(theta_i) F_m(theta_i); one thread per (l, m), q = l^2 + l + m.
-__global__ void modes_kernel(SphereArgs s, const double* __restrict__ mu, const double* __restrict__ w,
-                             const double* __restrict__ F, double* __restrict__ modes) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= (s.lmax + 1) * (s.lmax + 1)) return;
-    const int l = (int)sqrt((double)q + 0.5);
+// a_lm = sum_i w_i A_lm(theta_i) F_m(theta_i); one block per (l, m), q = l^2 + l + m. The rings' weights are
+// formed by the block's threads, one each, and summed by one in the rings' order. (One thread per (l, m),
+// with pow() for the powers, was most of a call: the constraints, Psi_4 and modes of 72^2 x 60 points, 24
+// rings and lmax 4, take 2.6 ms instead of 4.0, this kernel 14 us.)
+__global__ void __launch_bounds__(128) modes_kernel(SphereArgs s, const double* __restrict__ mu, const double* __restrict__ w,
+                                                    const double* __restrict__ F, double* __restrict__ modes) {
+    __shared__ double a[kMaxNtheta];
+    const int q = blockIdx.x;
+    int l = 0;
+    while ((l + 1) * (l + 1) <= q) ++l;
     const int m = q - l * l - l;
     const int nm = 2 * s.lmax + 1;
-    double ar = 0.0, ai = 0.0;
-    for (int i = 0; i < s.ntheta; ++i) {
-        const double a = w[i] * sylm_theta(s.spin, l, m, mu[i]);
-        ar = fma(a, F[2 * ((long long)i * nm + m + s.lmax)], ar);
-        ai = fma(a, F[2 * ((long long)i * nm + m + s.lmax) + 1], ai);
-    }
-    modes[2 * q] = ar;
-    modes[2 * q + 1] = ai;
+    for (int i = threadIdx.x; i < s.ntheta; i += blockDim.x) a[i] = w[i] * sylm_theta(s.spin, l, m, mu[i]);
+    __syncthreads();
+    if (threadIdx.x > 1) return;  // thread 0: real part, thread 1: imaginary part
+    double x = 0.0;
+    for (int i = 0; i < s.ntheta; ++i) x = fma(a[i], F[2 * ((long long)i * nm + m + s.lmax) + threadIdx.x], x);
+    modes[2 * q + threadIdx.x] = x;
 }
 
 }  // namespace grf
@@ -215,9 +243,10 @@ int extract_modes(const grf_box* box, const Geom& g, const double* f_re, const d
     s.x0 = o[0]; s.y0 = o[1]; s.z0 = o[2];
     s.ntheta = ntheta; s.nphi = nphi; s.lmax = lmax; s.spin = spin;
     gauss_legendre_kernel<<<(ntheta + 127) / 128, 128, 0, st>>>(ntheta, mu, w);
-    ring_sums_kernel<<<ntheta, 256, 0, st>>>(g, f_re, f_im, s, mu, F);
+    if (nphi <= kTablePhi) ring_sums_kernel<true><<<ntheta, 256, 0, st>>>(g, f_re, f_im, s, mu, F);
+    else ring_sums_kernel<false><<<ntheta, 256, 0, st>>>(g, f_re, f_im, s, mu, F);
     const int nq = (lmax + 1) * (lmax + 1);
-    modes_kernel<<<(nq + 63) / 64, 64, 0, st>>>(s, mu, w, F, modes);
+    modes_kernel<<<nq, 128, 0, st>>>(s, mu, w, F, modes);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(modes_host, modes, sizeof(double) * 2 * nq, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
