@@ -14,12 +14,13 @@ namespace grf {
 // coordinates of interior point (0, 0, 0); hyp (4 fields) the hyperbolicity diagnostics of the
 // coupled system (PointExtraT::hyp). PSI4 = 1 compiles those outputs in (they need the assembled
 // or solved coupled system); with PSI4 = 0 the compiler drops the coupled solve, which H, M_i and
-// the densities do not use.
+// the densities do not use. Bound by the FP64 pipe, held to 168 registers for 3 blocks per SM (constraints,
+// Psi_4 and modes of 72^2 x 60 points: 2.93 -> 2.61 ms a call against 255 and 2).
 template <int ORD, int PSI4>
-__global__ void __launch_bounds__(128) constraints_kernel(Geom g, Coeffs c, const double* __restrict__ s,
-                                                          double* __restrict__ out4, double* __restrict__ part,
-                                                          double* __restrict__ dens, double* __restrict__ psi4,
-                                                          double3 o, double* __restrict__ hyp) {
+__global__ void __launch_bounds__(128, 3) constraints_kernel(Geom g, Coeffs c, const double* __restrict__ s,
+                                                             double* __restrict__ out4, double* __restrict__ part,
+                                                             double* __restrict__ dens, double* __restrict__ psi4,
+                                                             double3 o, double* __restrict__ hyp) {
     // 128 consecutive points a block; every thread stays to the reduction
     __shared__ double red[8][128];
     const long long q = (long long)blockIdx.x * 128 + threadIdx.x;

@@ -4,10 +4,10 @@
 
 namespace grf {
 
-// One thread per interior point. LOP: lopsided advection.
+// One thread per interior point, held to 168 registers as rhs_kernel. LOP: lopsided advection.
 template <int LOP>
-__global__ void __launch_bounds__(128) rhs6_kernel(Geom g, Coeffs c, const double* __restrict__ s,
-                                                   double* __restrict__ rhs, double ko, int* status) {
+__global__ void __launch_bounds__(128, 3) rhs6_kernel(Geom g, Coeffs c, const double* __restrict__ s,
+                                                      double* __restrict__ rhs, double ko, int* status) {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= (long long)g.nx * g.ny * g.nz) return;
     int i, j, k;
