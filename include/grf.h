@@ -164,9 +164,9 @@ int grf_rk4_step(const grf_box* box, const grf_params* params, double* state, do
  *   state:    device buffer of the same size; overwritten, and on completion it holds the
  *             same result as host_out.
  *   ws:       as for grf_rk4_step.
- * The state is copied in slabs of z-planes (at most 16) on a high-priority copy stream owned by
- * the library; each slab's first-stage launch waits only for the planes its stencils read. The
- * last stage runs slab by slab and each finished slab is copied to host_out while the next is
+ * The state is copied in slabs of z-planes (at most 16, of 290,000 points or more) on a
+ * high-priority copy stream owned by the library; each slab's first-stage launch waits only for
+ * the planes its stencils read. The last stage runs slab by slab and each finished slab is copied to host_out while the next is
  * computed. Page-locked buffers are copied by a small kernel (48 blocks) that reads or writes
  * host memory directly, which keeps the full host-link rate while the stages run; pageable
  * buffers are copied with cudaMemcpyAsync. Results are bit-identical to: copy host_in to state,

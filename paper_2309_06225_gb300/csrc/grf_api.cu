@@ -283,6 +283,7 @@ size_t constraint_partials(const Geom& g) {
 
 // ---- host-to-host stepping (grf_rk4_step_host): per-device copy stream and events
 constexpr int kMaxSlabs = 16;
+constexpr long long kSlabPoints = 5LL * 152 * 12 * 32;
 constexpr int kMaxDevices = 64;
 
 struct CopyPipe {
@@ -569,8 +570,12 @@ int grf_rk4_step_host(const grf_box* box, const grf_params* params, const double
     double* acc = (double*)((char*)ws + 2 * sb);
     // Slab s = interior planes [lo(s), hi(s)); its copy chunk = ghosted planes [clo(s), chi(s)), the
     // first and last chunks also holding the z-ghost planes. Q >= 4 planes, so the planes a slab's
-    // stencils read (up to interior plane hi + 2) lie in chunks s-1, s and s+1.
-    const int Q = std::max(4, (g.nz + kMaxSlabs - 1) / kMaxSlabs);
+    // stencils read (up to interior plane hi + 2) lie in chunks s-1, s and s+1; and enough planes for
+    // kSlabPoints points, five waves of warps, since a slab's launch ends before the next one's begins
+    // (48^3 in 12 slabs: 4.68 ms a step, in one: 2.86; 96^3 in 16: 18.7, in 3: 18.1; 160^3 in 16: 79.3, in 14: 77.7).
+    const long long nxy = (long long)g.nx * g.ny;
+    const int Q = (int)std::min((long long)std::max(g.nz, 4),
+                                std::max((long long)std::max(4, (g.nz + kMaxSlabs - 1) / kMaxSlabs), (kSlabPoints + nxy - 1) / nxy));
     const int S = (g.nz + Q - 1) / Q;
     auto lo = [&](int s) { return s * Q; };
     auto hi = [&](int s) { return std::min(g.nz, (s + 1) * Q); };
