@@ -62,6 +62,8 @@ void launch_rhs(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s
 void launch_constraints(cudaStream_t st, const Geom& g, const Coeffs& c, const double* s,
                         double* out4, double* part, double* dens, double* psi4, double3 origin,
                          double* hyp = nullptr);
+// Periodic ghost fill of a state.
+void launch_periodic_fill(const Geom& g, double* s, cudaStream_t st);
 // Outer boundaries (grf_boundary.cu): the extrapolation fill of all ghosts of s, and the
 // Sommerfeld ghost update of one RK4 stage (stage 0..3) or, with stage -1, the ghosts' right-hand
 // side written to out (a.src the state).

@@ -195,22 +195,6 @@ Geom geom_from(const grf_box* b) {
 
 size_t sbytes(const Geom& g) { return sizeof(double) * (size_t)NFIELDS * (size_t)g.fstride; }
 
-__global__ void tlm_ghost_fill_kernel(Geom g, double* __restrict__ s) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int f = blockIdx.z;
-    if (i >= g.NX || j >= g.NY) return;
-    auto wrap = [](int a, int n) { int x = (a - NG) % n; if (x < 0) x += n; return x + NG; };
-    const int wi = wrap(i, g.nx), wj = wrap(j, g.ny);
-    const bool ghost_ij = (wi != i) || (wj != j);
-    double* u = s + f * g.fstride;
-    for (int k = 0; k < g.NZ; ++k) {
-        const int wk = wrap(k, g.nz);
-        if (!ghost_ij && wk == k) continue;
-        u[gidx(g, i, j, k)] = u[gidx(g, wi, wj, wk)];
-    }
-}
-
 }  // namespace
 
 extern "C" {
@@ -246,8 +230,7 @@ int grf_tlm_rk4(const grf_box* box, const grf_params* params, const double* dpar
     if (e != cudaSuccess) return record_cuda_error(e);
     for (int c = 0; c < 4; ++c) {
         if (g.periodic) {
-            dim3 blk(32, 8, 1), grd((g.NX + 31) / 32, (g.NY + 7) / 8, NFIELDS);
-            tlm_ghost_fill_kernel<<<grd, blk, 0, st>>>(g, un[c]);
+            launch_periodic_fill(g, un[c], st);
         } else {
             e = cudaMemcpyAsync(buf(0, c), un[c], sb, cudaMemcpyDeviceToDevice, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(buf(1, c), un[c], sb, cudaMemcpyDeviceToDevice, st);
