@@ -25,7 +25,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-fmad=false", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INC, "-I" + CSRC]
 # Per-source ptxas flags. The dual-number (tangent) kernels are very large functions on which
 # ptxas -O2/-O3 settles for 32 registers and an 87 KB stack; -O1 keeps 255 registers and a
-# 36 KB stack. The reverse-mode stage (about 4,300 recording calls) takes ptxas 10 minutes at
+# 36 KB stack. The reverse-mode stage (about 2,400 recording calls, 4,300 when this was measured) takes ptxas 10 minutes at
 # -O3 and under 2 at -O1, with the same 255 registers and 7 KB stack.
 SOURCE_FLAGS = {"grf_tlm.cu": ["-Xptxas", "-O1"], "grf_adjoint.cu": ["-Xptxas", "-O1"]}
 

@@ -13,8 +13,8 @@ enum : int { kLV = 0, kLD1 = 27, kLD2 = 99, kLKO = 171, kLUN = 198, kLACC = 225,
 // enforcement about 130 more; an overflow is detected and reported
 constexpr int kTapeCap = 5120;
 constexpr int kAdjThreads = 128;
-// tape columns (points per wave): 1024 per SM of a GB300, so that the sweep (at most 64 registers)
-// has 32 warps per SM to hide its dependent memory operations; the taping kernel is held to 128
+// tape columns (points per wave): 1024 per SM of a GB300, so that the sweep (28 warps per SM at 72
+// registers) has warps to hide its dependent memory operations; the taping kernel is held to 128
 // registers for 16 warps per SM (more spills, but it ran faster than at 255 registers with 8)
 constexpr long long kAdjCols = 152LL * 1024;
 constexpr int kSweepThreads = 128;
@@ -38,7 +38,7 @@ struct AdjArgs {
     long long npts;
 };
 
-// Sweeps the wave's tape columns (points q0 ..); `cols` columns.
+// Sweeps the wave's tape columns (points q0 ..).
 void launch_adj_sweep(const Geom& g, const AdjArgs& a, const grf_rev::Tape& tape, int stage, long long q0, cudaStream_t st);
 
 }  // namespace grf

@@ -24,9 +24,9 @@
 // chosen by their instruction count. The curvature goes through the six components of the 3D Riemann
 // tensor (its double dual is the raised Einstein tensor), the derivatives of Gt^k that cancel between
 // R_ij and D_(i Z_j) are never formed, and C_ij and H_nn are the unknowns, in which the lapse's
-// derivatives and the shift terms cancel. About 2,100 FP64 instructions where the forms through
-// d_m (h^ij Gt_lij) and d_t K_ij took 2,900: 256^3 step 506 -> 412 ms, 36 x 32 x 30 gradient (whose tape
-// has one entry per operation) 76.9 -> 52.7 ms, 72^2 x 60 diagnostics 6.57 -> 4.97 ms.
+// derivatives and the shift terms cancel. About 2,000 FP64 instructions where the forms through
+// d_m (h^ij Gt_lij) and d_t K_ij took 2,900: by itself 256^3 step 506 -> 412 ms, 36 x 32 x 30 gradient (whose
+// tape has one entry per operation) 76.9 -> 52.7 ms, 72^2 x 60 diagnostics 6.57 -> 4.97 ms.
 // Products and sums are fused only where fma is written (-fmad=false), so all instantiations round alike.
 //
 // The cubic Horndeski term (1/16 pi) g3 X box(phi) (general instantiation, COUP = 1) adds, with

@@ -1,17 +1,15 @@
 """FP64 operation counts of the kernels' formulation (host build of the kernel source).
 
 The pointwise part (RHS + 7x7 solve) is counted by running the kernel's own source with an
-operation-counting scalar (libgrf_flops.so). The stencil gather, KO dissipation and stage
-update are fixed expressions in grf_kernels.cuh and are counted here from their code:
+operation-counting scalar (libgrf_flops.so). The stencils, KO dissipation and stage update are
+counted as the FP64 operations of their definitions (the kernels form the stencil sums in 64-bit
+integers, grf_fixed.cuh, and execute fewer FP64 instructions than this):
   fd1  (u-2 - u+2) + 8 (u+1 - u-1), * 1/(12dx)            : 2 add, 1 fma, 1 mul
   fd2  16 (u+1 + u-1) - (u+2 + u-2) - 30 u0, * 1/(12dx^2)  : 2 fma, 1 mul (the two pair sums
        are shared with the KO sum of the same field)
-  d_x d_y, d_x d_z, d_y d_z: the first-derivative stencil applied to the rounded first
-       derivatives of the four neighbours (neighbouring lanes of the warp for x, the block's
-       shared rows for y)                                              : 2 add, 1 fma, 1 mul
-  halos: 3 first derivatives per point for the warp's row ends (the y / z derivatives at the 4
-       points past the ends of a 32-point row, 12 fields) and 12 per point for the block's 4 halo
-       rows of z-derivatives                                          : 15 x (2 add, 1 fma, 1 mul)
+  d_x d_y, d_x d_z, d_y d_z: the first-derivative stencil applied to first derivatives that
+       neighbouring points share                                       : 2 add, 1 fma, 1 mul
+  15 first derivatives per point that a 32 x 4 tile computes past its edges : 15 x (2 add, 1 fma, 1 mul)
   ko6  3 x (3 pair sums + 3 accumulations) - 3, 3 fma; + ko*value into the RHS: 15 add, 4 fma
   stage update (per field): 1-2 fma (+1 add on the last stage)
 Counting convention: add/sub/mul = 1 flop, fma = 2, division = 1.
