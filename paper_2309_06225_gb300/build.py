@@ -23,11 +23,6 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: products and sums fuse only where the source writes fma, so that every instantiation of
 # the pointwise equations (coupling kinds, batched boxes, tangents) gives the same bits.
 FLAGS = ["-O3", "-lineinfo", "-fmad=false", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INC, "-I" + CSRC]
-# Per-source ptxas flags. The dual-number (tangent) kernels are very large functions on which
-# ptxas -O2/-O3 settles for 32 registers and an 87 KB stack; -O1 keeps 255 registers and a
-# 36 KB stack. The reverse-mode stage (about 2,400 recording calls, 4,300 when this was measured) takes ptxas 10 minutes at
-# -O3 and under 2 at -O1, with the same 255 registers and 7 KB stack.
-SOURCE_FLAGS = {"grf_tlm.cu": ["-Xptxas", "-O1"], "grf_adjoint.cu": ["-Xptxas", "-O1"]}
 
 
 def _deps():
@@ -61,7 +56,7 @@ def build(force=False, verbose=False, ptxas_verbose=False):
 
     def compile_one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [NVCC] + ARCH + FLAGS + SOURCE_FLAGS.get(src, []) + extra + ["-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [NVCC] + ARCH + FLAGS + extra + ["-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), flush=True)
         res = subprocess.run(cmd, capture_output=True, text=True)

@@ -1,5 +1,4 @@
-// Reverse mode: the sweep over the tapes (see grf_adjoint.cu), in its own translation unit because the taping
-// kernel's is compiled at -O1.
+// Reverse mode: the sweep over the tapes (see grf_adjoint.cu), in a translation unit of its own.
 #include "grf_adjoint.cuh"
 
 namespace grf {
