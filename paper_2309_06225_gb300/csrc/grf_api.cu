@@ -22,9 +22,9 @@ __global__ void __launch_bounds__(128) ko_kernel(Geom g, const double* __restric
     point_of(g, q, i, j, k);
     const long long p = (long long)blockIdx.y * g.fstride + gidx(g, i + NG, j + NG, k + NG);
     AxisValues v;
-    load_axes(g, s + p, v);
+    load_axes<1>(g, s + p, v);
     FieldDiffs r;
-    if (axis_diffs<0>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko6(s + p, 0, g.pitch, g.plane);
+    if (axis_diffs<0, 1>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko6(s + p, 0, g.pitch, g.plane);
     rhs[p] = fma(ko, r.ko, rhs[p]);
 }
 
@@ -36,9 +36,9 @@ __global__ void __launch_bounds__(128) ko8_kernel(Geom g, const double* __restri
     point_of(g, q, i, j, k);
     const long long p = (long long)blockIdx.y * g.fstride + gidx(g, i + NG6, j + NG6, k + NG6);
     AxisValues6 v;
-    load_axes6(g, s + p, v);
+    load_axes6<1>(g, s + p, v);
     FieldDiffs r;
-    if (axis_diffs6<0>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko8(s + p, 0, g.pitch, g.plane);
+    if (axis_diffs6<0, 1>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax) r.ko = ko8(s + p, 0, g.pitch, g.plane);
     rhs[p] = fma(ko, r.ko, rhs[p]);
 }
 

@@ -8,13 +8,16 @@
 //   * every value x of the block becomes the two's complement integer x / 2^(emax - 1075 - G), emax the
 //     largest biased exponent of the block and G guard bits below the largest value's last bit. Values
 //     down to 2^-G of the largest keep all their bits; of smaller ones the bits below 2^-(52 + G) of the
-//     largest are dropped, where an FP64 sum would round at 2^-53 of its partial sums;
-//   * sums with weights of total magnitude below 2^(10 - G) cannot overflow, and are exact and
-//     independent of their order, so every caller gets the same bits;
+//     largest are dropped, where an FP64 sum would round at 2^-53 of its partial sums. A block is one
+//     sum's points along one grid line (grf_diffs.cuh), since across lines the magnitudes may differ by
+//     more than that: what a derivative keeps depends on no point that it does not read;
+//   * where the weights leave no room above G guard bits, the differences that are weighted are shifted right
+//     by what their own magnitude asks for (fx_room), which drops less than 2^-55 of the largest of them;
+//   * the integer sums are independent of their order, so every caller gets the same bits;
 //   * the sum times a positive constant (the grid-spacing factor, as a 64-bit mantissa) is rounded once to
 //     double.
 // Range: the caller bounds the block exponent (FxRange), so that no result leaves the normal doubles and no
-// result has to be checked: blocks below the range count as their values' multiples of a tiny unit (2^-1000
+// result has to be checked: blocks below the range count as their values' multiples of a tiny unit (2^-900
 // and less at common spacings), blocks above it, with infinities and NaNs among them, take the FP64 sums.
 // The functions compile for the host too, where tests compare them with exact arithmetic.
 #pragma once
@@ -41,15 +44,16 @@ inline FxScale fx_scale_of(double c) {
     return s;
 }
 
-// Block exponents whose results (sums of magnitude 2^0 .. 2^63 units, or of 2^shift units where fx_room
-// coarsens them, times constants of exponents lo .. hi or 1) are normal doubles.
+// Block exponents whose results (sums of magnitude 2^0 .. 2^63 units, of 2^shift units where fx_room coarsens
+// them, of 2^-25 units where fx_aligned refines them, times constants of exponents lo .. hi or 1) are normal
+// doubles.
 struct FxRange {
     int emin, emax;
 };
 
 inline FxRange fx_range(int lo, int hi, int shift = 0) {
     FxRange r;
-    r.emin = 66 - (lo < 0 ? lo : 0);
+    r.emin = 96 - (lo < 0 ? lo : 0);
     r.emax = 2046 - 13 - shift - (hi > 0 ? hi : 0);
     if (r.emin > r.emax) r.emax = -1;  // no block qualifies
     return r;
@@ -111,17 +115,50 @@ GRF_HD unsigned long long fx_normal(long long I, int& z) {
 #endif
 }
 
-// The right shift that leaves `bits` clear bits (and the sign) above the values whose magnitudes are OR-ed in
-// mag: sums of larger total weight stay exact while the values are small, and keep 62 - bits bits of the
-// largest one otherwise.
-GRF_HD unsigned long long fx_abs(long long x) { return (unsigned long long)(x < 0 ? -x : x); }
-GRF_HD int fx_room(unsigned long long mag, int bits) {
+// The top word of |x|, for x < 0 of |x| - 1: enough to bound |x|.
+GRF_HD unsigned fx_top(long long x) {
+    const int hi = (int)(x >> 32);
+    return (unsigned)(hi ^ (hi >> 31));
+}
+GRF_HD int fx_clz32(unsigned x) {
 #ifdef __CUDA_ARCH__
-    const int z = __clzll((long long)mag);
+    return __clz((int)x);
 #else
-    const int z = mag ? __builtin_clzll(mag) : 64;
+    return x ? __builtin_clz(x) : 32;
 #endif
-    return z > bits ? 0 : bits + 1 - z;
+}
+// The right shift (below 32) after which integers whose top words are OR-ed in `top` are below 2^bits.
+GRF_HD int fx_room(unsigned top, int bits) { return fx_max(0, 64 - bits - fx_clz32(top)); }
+
+// x >> s: for 0 <= s < 32, and for any s >= 0.
+GRF_HD long long fx_sar(long long x, int s) {
+#ifdef __CUDA_ARCH__
+    const int hi = (int)(x >> 32);
+    return ((long long)(hi >> s) << 32) | __funnelshift_r((unsigned)x, (unsigned)hi, (unsigned)s);
+#else
+    return x >> s;
+#endif
+}
+GRF_HD long long fx_sar_any(long long x, int s) {
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));  // (clamped at 64)
+    return r;
+#else
+    return x >> (s > 63 ? 63 : s);
+#endif
+}
+// x in units of 2^e as an integer in units of 2^(E - left), e <= E, left <= 31: for n = left - (E - e), x << n or
+// x >> -n.
+GRF_HD long long fx_aligned(long long x, int n) {
+#ifdef __CUDA_ARCH__
+    const int l = fx_max(n, 0);
+    const unsigned hi = __funnelshift_l((unsigned)x, (unsigned)((unsigned long long)x >> 32), (unsigned)l);
+    x = (long long)(((unsigned long long)hi << 32) | ((unsigned)x << l));
+    return fx_sar_any(x, fx_max(-n, 0));
+#else
+    return n >= 0 ? (long long)((unsigned long long)x << n) : fx_sar_any(x, -n);
+#endif
 }
 
 // The double of mantissa p (64 bits, top bit set; rounded to nearest) and biased exponent E in the normal

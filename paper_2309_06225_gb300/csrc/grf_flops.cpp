@@ -80,7 +80,7 @@ inline void opaque(double&) {}
 
 #define GRF_SECTION(id) (grfc::g_sec = (id))
 #define GRF_OPAQUE(x) grfc::opaque(x)
-#include "grf_fixed.cuh"
+#include "grf_diffs.cuh"
 #include "grf_point.cuh"
 #include "grf.h"
 
@@ -108,6 +108,18 @@ grf::PointInT<double> host_point(const double* v, const double* d1, const double
     for (int b = 0; b < 12; ++b)
         for (int m = 0; m < 6; ++m) in.d2[b][m] = d2[b * 6 + m];
     return in;
+}
+
+// What the differences read of a box's geometry (Geom in grf_kernels.cuh).
+struct HostSpacing {
+    grf::FxScale f1, f2, f11;
+    grf::FxRange fx;
+};
+
+HostSpacing host_spacing(double dx, int ng) {
+    HostSpacing g;
+    grf::spacing_factors(g, dx, ng);
+    return g;
 }
 
 }  // namespace
@@ -187,23 +199,83 @@ int grf_host_point_hyp(const grf_params* p, const double* v, const double* d1, c
     return ok ? 0 : -5;
 }
 
+// The differences of one field at one point, as the kernels take them, at spacing dx. ng: 3 (4th order) or 4
+// (6th order). axes: the point, then along each axis the values at -1, .., -ng and 1, .., ng; planes: the values
+// of the coordinate planes xy, xz, yz at offsets -(ng - 1) .. ng - 1 but 0 along both axes (the second one
+// fastest); beta: the side of the lopsided differences along each axis. out: d1[3], d2[6], the dissipation's
+// sum, the lopsided d1[3]. Without outer, the points at +-ng are not read and those last four are not formed.
+// Returns 1, and sets nothing, where the kernels would take the sums in FP64.
+int grf_host_diffs(int ng, double dx, int outer, const double* axes, const double* planes, const double* beta, double* out) {
+    const HostSpacing g = host_spacing(dx, ng);
+    grf::FieldDiffs r = {};
+    const int n = outer ? ng : ng - 1;
+    int mag;
+    const auto at = [&](int d, int side, int k) { return axes[1 + (2 * d + side) * ng + k]; };
+    if (ng == 3) {
+        grf::AxisValues v = {};
+        v.c = axes[0];
+        for (int d = 0; d < 3; ++d)
+            for (int k = 0; k < n; ++k) { v.m[d][k] = at(d, 0, k); v.q[d][k] = at(d, 1, k); }
+        mag = outer ? grf::axis_diffs<1, 1>(g, v, true, true, beta, r) : grf::axis_diffs<0, 0>(g, v, true, true, beta, r);
+    } else {
+        grf::AxisValues6 v = {};
+        v.c = axes[0];
+        for (int d = 0; d < 3; ++d)
+            for (int k = 0; k < n; ++k) { v.m[d][k] = at(d, 0, k); v.q[d][k] = at(d, 1, k); }
+        mag = outer ? grf::axis_diffs6<1, 1>(g, v, true, true, beta, r) : grf::axis_diffs6<0, 0>(g, v, true, true, beta, r);
+    }
+    const int w = 2 * (ng - 1);
+    for (int c = 0; c < 3; ++c) {
+        const double* x = planes + c * w * w;
+        double& mixed = r.d2[c < 2 ? c + 1 : 4];
+        if (ng == 3) {
+            grf::PlaneValues v;
+            std::memcpy(v.x, x, sizeof v.x);
+            mixed = grf::plane_diff(g, v, mag);
+        } else {
+            grf::PlaneValues6 v;
+            std::memcpy(v.x, x, sizeof v.x);
+            mixed = grf::plane_diff6(g, v, mag);
+        }
+    }
+    if (mag >> 20 > g.fx.emax) return 1;
+    std::memcpy(out, r.d1, sizeof r.d1);
+    std::memcpy(out + 3, r.d2, sizeof r.d2);
+    out[9] = r.ko;
+    std::memcpy(out + 10, r.up, sizeof r.up);
+    return 0;
+}
+
 // The 6th-order second difference 2 (x6 + x0) - 27 (x5 + x1) + 270 (x4 + x2) - 490 x3 of 7 values, as
 // axis_diffs6 takes it.
 double grf_host_fixed_second6(const double* x) {
-    int mag = 0;
-    for (int i = 0; i < 7; ++i) mag = grf::fx_max(mag, grf::fx_mag(x[i]));
-    const grf::FxRange range = grf::fx_range(0, 0, 10);
-    const int e = grf::fx_max(mag >> 20, range.emin), lim = grf::fx_lim<2>(e);
-    if (e > range.emax) return std::nan("");
-    long long v[7];
-    for (int i = 0; i < 7; ++i) v[i] = grf::fx_int(x[i], lim);
-    const long long c2 = v[3] + v[3], p1 = v[4] + v[2] - c2, p2 = v[5] + v[1] - c2, p3 = v[6] + v[0] - c2;
-    const int sh = grf::fx_room(grf::fx_abs(p1) | grf::fx_abs(p2) | grf::fx_abs(p3), 9);
-    return grf::fx_value<2>(270 * (p1 >> sh) - 27 * (p2 >> sh) + 2 * (p3 >> sh), e + sh);
+    HostSpacing g;
+    g.f1 = g.f2 = g.f11 = grf::fx_scale_of(1.0);
+    g.fx = grf::fx_range(0, 0, 10);
+    grf::AxisValues6 v = {};
+    v.c = x[3];
+    for (int d = 0; d < 3; ++d)
+        for (int k = 0; k < 3; ++k) { v.m[d][k] = x[2 - k]; v.q[d][k] = x[4 + k]; }
+    grf::FieldDiffs r = {};
+    return grf::axis_diffs6<0, 0>(g, v, false, true, nullptr, r) >> 20 > g.fx.emax ? std::nan("") : r.d2[0];
 }
 
 // sum_i w[i] x[i] in block fixed point with `guard` (1 or 2) guard bits, times c when c > 0; NaN above the range.
+// One block, but for the dissipation's sum of a point (19 values: the point, then by axis and distance the pairs),
+// which is taken line by line as the kernels do.
 double grf_host_fixed_sum(const double* x, const int* w, int n, int guard, double c) {
+    const int ko[19] = {-60, 15, 15, -6, -6, 1, 1, 15, 15, -6, -6, 1, 1, 15, 15, -6, -6, 1, 1};
+    if (n == 19 && guard == 2 && c <= 0.0 && std::memcmp(w, ko, sizeof ko) == 0) {
+        HostSpacing g;
+        g.f1 = g.f2 = g.f11 = grf::fx_scale_of(1.0);
+        g.fx = grf::fx_range(0, 0);
+        grf::AxisValues v;
+        v.c = x[0];
+        for (int d = 0; d < 3; ++d)
+            for (int k = 0; k < 3; ++k) { v.m[d][k] = x[1 + 6 * d + 2 * k]; v.q[d][k] = x[2 + 6 * d + 2 * k]; }
+        grf::FieldDiffs r = {};
+        return grf::axis_diffs<0, 1>(g, v, false, false, nullptr, r) >> 20 > g.fx.emax ? std::nan("") : r.ko;
+    }
     int mag = 0;
     for (int i = 0; i < n; ++i) mag = grf::fx_max(mag, grf::fx_mag(x[i]));
     const grf::FxScale k = grf::fx_scale_of(c > 0.0 ? c : 1.0);

@@ -4,7 +4,7 @@
 
 #include <cuda_runtime.h>
 
-#include "grf_fixed.cuh"
+#include "grf_diffs.cuh"
 #include "grf_point.cuh"
 
 // Loads of stencil sources. By default the read-only, non-coherent path (__ldg): every kernel
@@ -37,14 +37,9 @@ struct Geom {
 };
 
 inline void set_spacing(Geom& g, double dx, int ng) {
-    const double d1 = ng == 4 ? 60.0 : 12.0, d2 = ng == 4 ? 180.0 : 12.0;
     g.ng = ng;
     g.dx = dx;
-    g.f1 = fx_scale_of(1.0 / (d1 * dx));
-    g.f2 = fx_scale_of(1.0 / (d2 * dx * dx));
-    g.f11 = fx_scale_of(1.0 / (d1 * d1 * dx * dx));
-    const int lo = g.f11.e < g.f1.e ? g.f11.e : g.f1.e, hi = g.f2.e > g.f1.e ? g.f2.e : g.f1.e;
-    g.fx = fx_range(lo, hi, ng == 4 ? 10 : 0);
+    spacing_factors(g, dx, ng);
 }
 
 constexpr int NG = 3;        // ghost layers of the 4th-order kernels (those of this header)
@@ -90,21 +85,15 @@ __device__ __forceinline__ bool has_d1(int f) { return !(f >= F_B && f < F_B + 3
 
 // ---- the gather: differences of the fields at one point, the sums in block fixed point (grf_fixed.cuh)
 
-// One field on the three axes through the point (19 values), and on one coordinate plane (16).
-struct AxisValues {
-    double c, m[3][3], q[3][3];  // the point; at -(k+1) and +(k+1) along axis d
-};
-struct PlaneValues {
-    double x[4][4];  // at offsets -2, -1, 1, 2 along both axes
-};
-
+// The values axis_diffs reads; the outermost ones only where they count (KO, LOP).
+template <int OUTER>
 __device__ __forceinline__ void load_axes(const Geom& g, const double* __restrict__ u, AxisValues& v) {
     const long long st[3] = {1, g.pitch, g.plane};
     v.c = GRF_LDG(u);
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < (OUTER ? 3 : 2); ++k) {
             v.m[d][k] = GRF_LDG(u - (k + 1) * st[d]);
             v.q[d][k] = GRF_LDG(u + (k + 1) * st[d]);
         }
@@ -115,68 +104,6 @@ __device__ __forceinline__ void load_plane(const double* __restrict__ u, long lo
 #pragma unroll
         for (int b = 0; b < 4; ++b)
             v.x[a][b] = GRF_LDG(u + (a < 2 ? a - 2 : a - 1) * sa + (b < 2 ? b - 2 : b - 1) * sb);
-}
-
-// Differences of one field at one point.
-struct FieldDiffs {
-    double d1[3], d2[6], ko;  // first and second derivatives, Kreiss-Oliger sum
-    double up[3];             // lopsided first differences (LOP)
-};
-
-// The axis part: first derivatives, unmixed second derivatives and the Kreiss-Oliger sum. The 19 points take
-// one block exponent; weights of total magnitude up to 192 leave room for two guard bits. Returns the
-// block's largest magnitude word.
-//   LOP = 1: also the differences biased towards the side the shift component bet[d] points to (offsets
-//   -1..3, mirrored for bet[d] < 0): (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx) with a_n = u at n
-//   points towards that side, b1 = u one point away from it.
-template <int LOP>
-__device__ __forceinline__ int axis_diffs(const Geom& g, const AxisValues& v, bool first, bool second, const double* bet,
-                                          FieldDiffs& r) {
-    int mag = fx_mag(v.c);
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) mag = fx_max(mag, fx_max(fx_mag(v.m[d][k]), fx_mag(v.q[d][k])));
-    const int e = fx_max(mag >> 20, g.fx.emin), lim = fx_lim<2>(e);
-    const long long c0 = fx_int(v.c, lim), c2 = c0 + c0;
-    long long t1 = 0, t2 = 0, t3 = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const long long m1 = fx_int(v.m[d][0], lim), q1 = fx_int(v.q[d][0], lim);
-        const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
-        const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
-        const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2;  // pair sums less 2 u0
-        if (first) r.d1[d] = fx_value<2>(((q1 - m1) << 3) + (m2 - q2), e, g.f1);
-        if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<2>((p1 << 4) - p2, e, g.f2);
-        if (LOP) {
-            const bool fw = bet[d] >= 0.0;
-            const long long a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, b1 = fw ? m1 : q1;
-            r.up[d] = fx_value<2>(18 * a1 - 6 * a2 + a3 - 3 * b1 - 5 * c2, e, g.f1);
-        }
-        t1 += p1;
-        t2 += p2;
-        t3 += q3 + m3 - c2;
-    }
-    r.ko = fx_value<2>((t1 << 4) - t1 - 6 * t2 + t3, e);
-    return mag;
-}
-
-// A mixed derivative: the tensor product of the first-difference weights (1, -8, 8, -1) on its 16 points,
-// with their own block exponent. Weights of total magnitude 18^2 leave room for one guard bit. mag collects
-// the largest magnitude word.
-__device__ __forceinline__ double plane_diff(const Geom& g, const PlaneValues& v, int& mag) {
-    int top = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) top = fx_max(top, fx_mag(v.x[a][b]));
-    mag = fx_max(mag, top);
-    const int e = fx_max(top >> 20, g.fx.emin), lim = fx_lim<1>(e);
-    long long d[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-        d[a] = ((fx_int(v.x[a][2], lim) - fx_int(v.x[a][1], lim)) << 3) + (fx_int(v.x[a][0], lim) - fx_int(v.x[a][3], lim));
-    return fx_value<1>(((d[2] - d[1]) << 3) + (d[0] - d[3]), e, g.f11);
 }
 
 // The fields that the constraints take derivatives of: all but Theta, Gamma-hat, the lapse, the shift and B.
@@ -196,7 +123,7 @@ struct PointSink {
 
 // The differences in FP64, for a point whose fields leave the fixed-point range (values near overflow,
 // infinities, NaNs): rewrites what gather() took.
-template <int LOP, typename Sink>
+template <int LOP, int KO, typename Sink>
 __device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict__ s, long long p, const Sink& out,
                                          unsigned fields) {
     const double i12 = 1.0 / (12.0 * g.dx), i12s = 1.0 / (12.0 * g.dx * g.dx);
@@ -207,7 +134,7 @@ __device__ __noinline__ void gather_fp64(const Geom& g, const double* __restrict
         const double* u = s + f * g.fstride + p;
         const double u0 = GRF_LDG(u);
         double av = 0.0;
-        out.dissipation(f, ko6(u, 0, g.pitch, g.plane));
+        if (KO) out.dissipation(f, ko6(u, 0, g.pitch, g.plane));
 #pragma unroll 1
         for (int d = 0; d < 3; ++d) {
             if (has_d1(f)) out.first(d1slot(f), d, fd1(u, 0, st[d], i12));
@@ -236,12 +163,13 @@ __host__ __device__ constexpr int d2field(int b) { return b < 7 ? b : (b == 7 ? 
 // Kreiss-Oliger sum sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_+1 - 6 u_+2 + u_+3).
 //   LOP = 1: also the lopsided advection terms adv[f] = sum_d |beta^d| D_d u_f.
 //   ALL = 0: only the kMetricScalarFields (the others' entries are left alone).
+//   KO = 0: no Kreiss-Oliger sums; the outermost points, at +-3, are then read for LOP only.
 // Two rolled loops (the 12 fields with second derivatives, the 15 without): unrolled threefold, the integer
 // code of a field no longer stays in the instruction cache (128^3 step 44 -> 50 ms). Each block's values are
 // loaded one block ahead of their use, so that the loads' latency lies under the previous block's arithmetic.
 //   TEAM > 1: the point's fields are shared out over TEAM consecutive lanes, of which this is lane t (every
 //   lane of the warp calls this; in, kos and adv are the team's).
-template <int LOP, int ALL, int TEAM, typename Sink>
+template <int LOP, int ALL, int TEAM, int KO, typename Sink>
 __device__ __forceinline__ void gather_to(const Geom& g, const double* __restrict__ s, long long p, const Sink& out, int t) {
     const long long st[3] = {1, g.pitch, g.plane};
     double bet[3] = {0.0, 0.0, 0.0};
@@ -255,14 +183,14 @@ __device__ __forceinline__ void gather_to(const Geom& g, const double* __restric
     auto next_plain = [](int b) { return TEAM > 1 ? b + TEAM : (b == kLastPlain ? 14 : b + 1); };
     const double* u = s + d2field(t) * g.fstride + p;
     AxisValues ax;
-    load_axes(g, u, ax);
+    load_axes<LOP || KO>(g, u, ax);
     int mag = 0;
 #pragma unroll 1
     for (int b = t; b < 12; b = next_second(b)) {
         FieldDiffs r;
         const int f = d2field(b);
         out.value(f, ax.c);
-        mag = fx_max(mag, axis_diffs<LOP>(g, ax, true, true, bet, r));
+        mag = fx_max(mag, axis_diffs<LOP, KO>(g, ax, true, true, bet, r));
         out.second(b, 0, r.d2[0]);
         out.second(b, 3, r.d2[3]);
         out.second(b, 5, r.d2[5]);
@@ -274,8 +202,8 @@ __device__ __forceinline__ void gather_to(const Geom& g, const double* __restric
         }
         const int nb = next_second(b), next = nb < 12 ? d2field(nb) : plainfield(t);
         u = s + next * g.fstride + p;
-        load_axes(g, u, ax);
-        out.dissipation(f, r.ko);
+        load_axes<LOP || KO>(g, u, ax);
+        if (KO) out.dissipation(f, r.ko);
 #pragma unroll
         for (int d = 0; d < 3; ++d) out.first(d1slot(f), d, r.d1[d]);
         if (LOP) out.advection(f, fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0])));
@@ -284,11 +212,11 @@ __device__ __forceinline__ void gather_to(const Geom& g, const double* __restric
     for (int b = t; b < 15; b = next_plain(b)) {
         FieldDiffs r;
         const AxisValues now = ax;
-        if (next_plain(b) < 15) load_axes(g, s + plainfield(next_plain(b)) * g.fstride + p, ax);
+        if (next_plain(b) < 15) load_axes<LOP || KO>(g, s + plainfield(next_plain(b)) * g.fstride + p, ax);
         const int f = plainfield(b);
         out.value(f, now.c);
-        mag = fx_max(mag, axis_diffs<LOP>(g, now, has_d1(f), false, bet, r));
-        out.dissipation(f, r.ko);
+        mag = fx_max(mag, axis_diffs<LOP, KO>(g, now, has_d1(f), false, bet, r));
+        if (KO) out.dissipation(f, r.ko);
         if (has_d1(f)) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) out.first(d1slot(f), d, r.d1[d]);
@@ -304,14 +232,14 @@ __device__ __forceinline__ void gather_to(const Geom& g, const double* __restric
         for (int b = t; b < 15; b += TEAM) fields |= 1u << plainfield(b);
     }
     if (mag >> 20 > g.fx.emax) {
-        gather_fp64<LOP>(g, s, p, out, fields);
+        gather_fp64<LOP, KO>(g, s, p, out, fields);
     }
 }
 
-template <int LOP = 0, int ALL = 1, int TEAM = 1>
+template <int LOP = 0, int ALL = 1, int TEAM = 1, int KO = 1>
 __device__ __forceinline__ void gather(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
                                        double kos[NFIELDS], double* adv = nullptr, int t = 0) {
-    gather_to<LOP, ALL, TEAM>(g, s, p, PointSink{in, kos, adv}, t);
+    gather_to<LOP, ALL, TEAM, KO>(g, s, p, PointSink{in, kos, adv}, t);
 }
 
 __device__ __forceinline__ bool interior_thread(const Geom& g, int& i, int& j, int& k) {
@@ -457,7 +385,7 @@ __device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, cons
 
 // One thread per interior point of [q0, q1), consecutive threads consecutive points in x-fastest order,
 // so that every lane of every warp but the last works whatever the box's extents (no derivative is
-// exchanged between lanes, so the mapping is free). Blocks of stage_threads() threads.
+// exchanged between lanes, so the mapping is free). Blocks of point_threads() threads (grf_launch.h).
 // What bounds it: the FP64 pipe (79% of its issue slots), 2,212 instructions a point and stage. 12 resident
 // warps per SM (168 registers a thread) hide its latency; more would spill more: 128^3 step 51.8 ms with 8
 // warps, 36.5 with 12, 39.2 with 16, 43.8 with 20. (256^3 step 506 -> 296 ms since the stencils are summed in

@@ -27,7 +27,7 @@ __device__ __forceinline__ double fd1_6(const double* __restrict__ u, long long 
 //   points to, b_n = u at n points away from it):
 //           beta^d D_d u = |beta^d| (2 b_2 - 24 b_1 - 35 u_0 + 80 a_1 - 30 a_2 + 8 a_3 - a_4) / (60 dx)
 // In FP64, for points whose fields leave the fixed-point range. `fields` as for gather_fp64.
-template <int LOP>
+template <int LOP, int KO>
 __device__ __noinline__ void gather6_fp64(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
                                           double* kos, double* adv, unsigned fields) {
     const double i60 = 1.0 / (60.0 * g.dx), i180s = 1.0 / (180.0 * g.dx * g.dx);
@@ -84,99 +84,36 @@ __device__ __noinline__ void gather6_fp64(const Geom& g, const double* __restric
         }
 #pragma unroll
         for (int r = 1; r <= 4; ++r) t[r] = (pr[0][r] + pr[1][r]) + pr[2][r];
-        kos[f] = fma(210.0, u0, fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
+        if (KO) kos[f] = fma(210.0, u0, fma(-56.0, t[1], fma(28.0, t[2], fma(-8.0, t[3], t[4]))));
     }
 }
 
 // ---- the gather in block fixed point
 
-struct AxisValues6 {
-    double c, m[3][4], q[3][4];  // the point; at -(k+1) and +(k+1) along axis d
-};
-
+// The values axis_diffs6 reads; the outermost ones only where they count (KO, LOP).
+template <int OUTER>
 __device__ __forceinline__ void load_axes6(const Geom& g, const double* __restrict__ u, AxisValues6& v) {
     const long long st[3] = {1, g.pitch, g.plane};
     v.c = __ldg(u);
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < (OUTER ? 4 : 3); ++k) {
             v.m[d][k] = __ldg(u - (k + 1) * st[d]);
             v.q[d][k] = __ldg(u + (k + 1) * st[d]);
         }
 }
 
-// As axis_diffs, 6th order. The weights of the second derivative (total 1,100) and of the dissipation (768)
-// exceed the room above two guard bits, so those sums are taken of second differences, shifted right only
-// where these are large (fx_room).
-template <int LOP>
-__device__ __forceinline__ int axis_diffs6(const Geom& g, const AxisValues6& v, bool first, bool second,
-                                           const double* bet, FieldDiffs& r) {
-    int mag = fx_mag(v.c);
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) mag = fx_max(mag, fx_max(fx_mag(v.m[d][k]), fx_mag(v.q[d][k])));
-    const int e = fx_max(mag >> 20, g.fx.emin), lim = fx_lim<2>(e);
-    const long long c0 = fx_int(v.c, lim), c2 = c0 + c0;
-    long long t1 = 0, t2 = 0, t3 = 0, t4 = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const long long m1 = fx_int(v.m[d][0], lim), q1 = fx_int(v.q[d][0], lim);
-        const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
-        const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
-        const long long m4 = fx_int(v.m[d][3], lim), q4 = fx_int(v.q[d][3], lim);
-        const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2, p3 = q3 + m3 - c2;  // pair sums less 2 u0
-        if (first) r.d1[d] = fx_value<2>(45 * (q1 - m1) - 9 * (q2 - m2) + (q3 - m3), e, g.f1);
-        if (second) {
-            const int sh = fx_room(fx_abs(p1) | fx_abs(p2) | fx_abs(p3), 9);
-            r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] =
-                fx_value<2>(270 * (p1 >> sh) - 27 * (p2 >> sh) + 2 * (p3 >> sh), e + sh, g.f2);
-        }
-        if (LOP) {
-            const bool fw = bet[d] >= 0.0;
-            const long long a1 = fw ? q1 : m1, a2 = fw ? q2 : m2, a3 = fw ? q3 : m3, a4 = fw ? q4 : m4;
-            const long long b1 = fw ? m1 : q1, b2 = fw ? m2 : q2;
-            r.up[d] = fx_value<2>(80 * a1 - 30 * a2 + 8 * a3 - a4 - 24 * b1 + 2 * b2 - 35 * c0, e, g.f1);
-        }
-        t1 += p1;
-        t2 += p2;
-        t3 += p3;
-        t4 += q4 + m4 - c2;
-    }
-    const int sh = fx_room(fx_abs(t1) | fx_abs(t2) | fx_abs(t3) | fx_abs(t4), 7);
-    r.ko = fx_value<2>(28 * (t2 >> sh) - 56 * (t1 >> sh) - 8 * (t3 >> sh) + (t4 >> sh), e + sh);
-    return mag;
-}
-
-// A mixed derivative: the tensor product of the first-difference weights (-1, 9, -45, 45, -9, 1) on its 36
-// points, first differences along b of the six rows, then along a, with their own block exponent.
-__device__ __forceinline__ double plane_diff6(const Geom& g, const double* __restrict__ u, long long sa, long long sb,
-                                              int& mag) {
-    double x[6][6];
-    int top = 0;
+__device__ __forceinline__ void load_plane6(const double* __restrict__ u, long long sa, long long sb, PlaneValues6& v) {
 #pragma unroll
     for (int a = 0; a < 6; ++a)
 #pragma unroll
-        for (int b = 0; b < 6; ++b) {
-            x[a][b] = __ldg(u + (a < 3 ? a - 3 : a - 2) * sa + (b < 3 ? b - 3 : b - 2) * sb);
-            top = fx_max(top, fx_mag(x[a][b]));
-        }
-    mag = fx_max(mag, top);
-    const int e = fx_max(top >> 20, g.fx.emin), lim = fx_lim<2>(e);
-    long long d[6];
-#pragma unroll
-    for (int a = 0; a < 6; ++a)
-        d[a] = 45 * (fx_int(x[a][3], lim) - fx_int(x[a][2], lim)) - 9 * (fx_int(x[a][4], lim) - fx_int(x[a][1], lim)) +
-               (fx_int(x[a][5], lim) - fx_int(x[a][0], lim));
-    const long long d1 = d[3] - d[2], d2 = d[4] - d[1], d3 = d[5] - d[0];
-    const int sh = fx_room(fx_abs(d1) | fx_abs(d2) | fx_abs(d3), 6);
-    return fx_value<2>(45 * (d1 >> sh) - 9 * (d2 >> sh) + (d3 >> sh), e + sh, g.f11);
+        for (int b = 0; b < 6; ++b) v.x[a][b] = __ldg(u + (a < 3 ? a - 3 : a - 2) * sa + (b < 3 ? b - 3 : b - 2) * sb);
 }
 
-// As gather() (LOP and ALL likewise), 6th order; kos[f] = sum_d Delta^8_d u. Rolled loops over the fields and
+// As gather() (LOP, ALL and KO likewise), 6th order; kos[f] = sum_d Delta^8_d u. Rolled loops over the fields and
 // over the three planes of a field.
-template <int LOP = 0, int ALL = 1>
+template <int LOP = 0, int ALL = 1, int KO = 1>
 __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict__ s, long long p, PointIn& in,
                                         double kos[NFIELDS], double* adv = nullptr) {
     const long long st[3] = {1, g.pitch, g.plane};
@@ -193,11 +130,11 @@ __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict_
         const double* u = s + f * g.fstride + p;
         const bool first = has_d1(f), second = has_d2(f);
         AxisValues6 ax;
-        load_axes6(g, u, ax);
+        load_axes6<LOP || KO>(g, u, ax);
         FieldDiffs r;
         in.v[f] = ax.c;
-        mag = fx_max(mag, axis_diffs6<LOP>(g, ax, first, second, bet, r));
-        kos[f] = r.ko;
+        mag = fx_max(mag, axis_diffs6<LOP, KO>(g, ax, first, second, bet, r));
+        if (KO) kos[f] = r.ko;
         if (first) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) in.d1[d1slot(f)][d] = r.d1[d];
@@ -208,12 +145,15 @@ __device__ __forceinline__ void gather6(const Geom& g, const double* __restrict_
             in.d2[b][3] = r.d2[3];
             in.d2[b][5] = r.d2[5];
 #pragma unroll 1
-            for (int c = 0; c < 3; ++c)
-                in.d2[b][c < 2 ? c + 1 : 4] = plane_diff6(g, u, c < 2 ? 1 : st[1], c == 0 ? st[1] : st[2], mag);
+            for (int c = 0; c < 3; ++c) {
+                PlaneValues6 pl;
+                load_plane6(u, c < 2 ? 1 : st[1], c == 0 ? st[1] : st[2], pl);
+                in.d2[b][c < 2 ? c + 1 : 4] = plane_diff6(g, pl, mag);
+            }
         }
         if (LOP) adv[f] = fma(fabs(bet[2]), r.up[2], fma(fabs(bet[1]), r.up[1], fabs(bet[0]) * r.up[0]));
     }
-    if (mag >> 20 > g.fx.emax) gather6_fp64<LOP>(g, s, p, in, kos, adv, kFields);
+    if (mag >> 20 > g.fx.emax) gather6_fp64<LOP, KO>(g, s, p, in, kos, adv, kFields);
 }
 
 // One RK4 stage at one point of a 6th-order box, as stage_point (a.ko = -sigma/(256 dx)).

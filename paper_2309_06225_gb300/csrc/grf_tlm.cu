@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(128, 2) tlm_stage_kernel(Geom g, CoeffsT<D3> c
     PointInT<D3> in;
     D3 kos[NFIELDS];
 #pragma unroll 1
-    for (int cmp = 0; cmp < 4; ++cmp) gather_to<0, 1, 1>(g, a.src[cmp], p, DualSink{in, kos, cmp}, 0);
+    for (int cmp = 0; cmp < 4; ++cmp) gather_to<0, 1, 1, 1>(g, a.src[cmp], p, DualSink{in, kos, cmp}, 0);
     D3 r[NFIELDS];
     bool ok = true;
     point_rhs<D3, D3>(c, in, r, nullptr, ok);
