@@ -28,12 +28,11 @@ __global__ void __launch_bounds__(128, 3) constraints_kernel(Geom g, Coeffs c, c
     int i = 0, j = 0, k = 0;
     long long p = 0;
     PointIn in;
-    double kos[NFIELDS];
     if (live) {
         point_of(g, q, i, j, k);
         p = gidx(g, i + g.ng, j + g.ng, k + g.ng);
-        if constexpr (ORD == 4) gather<0, PSI4>(g, s, p, in, kos);
-        else gather6<0, PSI4>(g, s, p, in, kos);
+        if constexpr (ORD == 4) gather<0, PSI4, 1, 0>(g, s, p, in, nullptr);
+        else gather6<0, PSI4, 0>(g, s, p, in, nullptr);
     }
     double vals[4] = {0.0, 0.0, 0.0, 0.0};
     if (live) {
