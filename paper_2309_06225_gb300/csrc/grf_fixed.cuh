@@ -55,7 +55,9 @@ inline FxRange fx_range(int lo, int hi, int shift = 0) {
     FxRange r;
     r.emin = 96 - (lo < 0 ? lo : 0);
     r.emax = 2046 - 13 - shift - (hi > 0 ? hi : 0);
-    if (r.emin > r.emax) r.emax = -1;  // no block qualifies
+    // no block qualifies: no exponent is left, or a constant is itself zero, subnormal or infinite (fx_scale_of holds
+    // normal ones only)
+    if (r.emin > r.emax || lo <= -1023 || hi >= 1024) r.emax = -1;
     return r;
 }
 

@@ -139,3 +139,14 @@ def test_derivatives_keep_clear_of_the_outermost_points(host, ng, garbage):
             assert np.array_equal(got[:9], want[:9]), (name, ng, garbage)
         else:
             assert not abs(garbage) < 1e300
+
+
+@pytest.mark.parametrize("ng", [3, 4])
+def test_spacings_whose_factors_are_not_normal_take_fp64(host, ng):
+    """1 / dx^2 beyond the doubles, or below the normal ones: the FP64 sums give what their division gives."""
+    c, line, planes = stencil(fields(np.random.default_rng(2))["smooth"], ng)
+    axes = [c] + [x for d in range(3) for s in range(2) for x in line[d][s]]
+    for dx in (1e-160, 1e-200, 1e153, 1e160, 1e300):
+        assert host(ng, axes, planes, np.ones(3), dx=dx) is None
+    for dx in (1e-100, 1.0, 1e100):
+        assert np.all(np.isfinite(host(ng, axes, planes, np.ones(3), dx=dx)))
