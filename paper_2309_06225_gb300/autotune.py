@@ -2,10 +2,10 @@
 
 For a batch signature (the multiset of box shapes and boundary types, together with the
 kernel variants the boxes' parameters select: coupling kind, backreaction and advection
-stencil), each candidate configuration (launch variant x tile shape) is timed on scratch
+stencil), each candidate configuration (launch variant x tile size) is timed on scratch
 copies of the states with CUDA events: one untimed step, then the median of REPEATS timed
-steps. The fastest is returned and cached in a JSON file keyed by the signature and the GPU
-name. The states passed in are not modified.
+steps. The fastest is returned and cached in a JSON file keyed by the signature, the GPU name
+and KERNELS. The states passed in are not modified.
 """
 from __future__ import annotations
 
@@ -16,15 +16,16 @@ import statistics
 from . import (GRF_BATCH_GRAPH, GRF_BATCH_PERSISTENT, alloc_workspace, batch_config, batch_items,
                grf_batched_rk4, grf_batched_workspace_bytes)
 
+# A tile is tile_x * tile_y * tile_z consecutive points, one per thread of a block: the product alone counts.
 CANDIDATES = [
     (GRF_BATCH_GRAPH, (32, 4, 1)),
-    (GRF_BATCH_GRAPH, (64, 2, 1)),
-    (GRF_BATCH_GRAPH, (32, 2, 2)),
-    (GRF_BATCH_GRAPH, (16, 8, 1)),
-    (GRF_BATCH_GRAPH, (16, 4, 2)),
+    (GRF_BATCH_GRAPH, (32, 2, 1)),
+    (GRF_BATCH_GRAPH, (32, 1, 1)),
     (GRF_BATCH_PERSISTENT, (32, 4, 1)),
-    (GRF_BATCH_PERSISTENT, (64, 2, 1)),
+    (GRF_BATCH_PERSISTENT, (32, 2, 1)),
 ]
+# Names the batched kernels whose times a cache entry holds; changed with them or with the candidates.
+KERNELS = "consecutive-points"
 REPEATS = 3
 
 
@@ -49,6 +50,11 @@ def signature(boxes, params=None, params_index=None):
     return ";".join(f"{k[0]}x{k[1]}x{k[2]}/{k[3]}{k[4]}:{v}" for k, v in sorted(counts.items()))
 
 
+def cache_key(gpu, boxes, params=None, params_index=None):
+    """The entry of a batch in the cache."""
+    return f"{gpu}|{KERNELS}|{signature(boxes, params, params_index)}"
+
+
 def _load(path):
     try:
         with open(path) as f:
@@ -62,7 +68,7 @@ def tune(boxes, states, params_index, dts, params, cache_path=None, use_cache=Tr
     cache when the signature was tuned before on this GPU."""
     import torch
     path = cache_path or default_cache_path()
-    key = f"{torch.cuda.get_device_name()}|{signature(boxes, params, params_index)}"
+    key = cache_key(torch.cuda.get_device_name(), boxes, params, params_index)
     cache = _load(path) if use_cache else {}
     if key in cache:
         c = cache[key]
