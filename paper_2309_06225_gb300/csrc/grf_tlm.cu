@@ -43,7 +43,9 @@ struct TlmArgs {
     int* status;
 };
 
-__device__ __forceinline__ double& comp(D3& x, int c) { return (&x.v)[c]; }
+__device__ __forceinline__ double& comp(D3& x, int c) {
+    return c == 0 ? x.v : (c == 1 ? x.d0 : (c == 2 ? x.d1 : x.d2));
+}
 
 // One component (0: the value, 1..3: the tangents) of a dual point.
 struct DualSink {
