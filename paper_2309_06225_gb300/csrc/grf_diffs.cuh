@@ -3,9 +3,10 @@
 //
 // Blocks: the points of one difference along one grid line. A difference across a line's neighbours (a mixed
 // derivative, the dissipation's sum over the axes) is taken of the lines' sums, brought to a common unit that
-// the largest of them fills. So a sum's error is bounded by its own points' magnitudes, as an FP64 sum's is,
-// and it is the smaller of the two (1e-2 exp(-r^2), 10 cells out: first derivatives across the gradient 2e-17
-// relative, mixed ones 3e-16 against 1.7e-15; 1e-10 and 3e-14 with one unit for the lines of all three axes).
+// the largest of them fills. So a sum's error is bounded by its own points' magnitudes, as an FP64 sum's is, and
+// it is the smaller of the two: in the tail of 1e-2 exp(-r^2), 8 to 16 cells out, mean relative errors of first
+// and mixed derivatives 1.2e-16 and 4.4e-16 where FP64 has 2.4e-16 and 1.9e-15 (one exponent for the lines of all
+// three axes left 2e-10 at r = 6, and took 3% of a 256^3 step less).
 #pragma once
 
 #include "grf_fixed.cuh"
@@ -49,8 +50,8 @@ struct PlaneValues {
 //   LOP = 1: also the differences biased towards the side the shift component bet[d] points to (offsets
 //   -1..3, mirrored for bet[d] < 0): (-3 b1 - 10 u0 + 18 a1 - 6 a2 + a3) / (12 dx) with a_n = u at n
 //   points towards that side, b1 = u one point away from it.
-// The bounds in units, values below 2^58: first 18 x 2^58; second |p1| < 2^58, |p2| < 2^60 (16 + 4) x 2^58; the
-// dissipation's |p1| < 2^58, |p2| < 2^59 (15 + 12 + 2) x 2^58; lopsided (18 + 6 + 6 + 1) x 2^58: all below 2^63.
+// The bounds, of values below 2^58: first 18 x 2^58; a quarter of the second 16 x 2^58 and of the dissipation's
+// 15.5 x 2^58; half the lopsided sum 18.5 x 2^58: all below 2^63.
 template <int LOP, int KO, typename Spacing>
 GRF_HD int axis_diffs(const Spacing& g, const AxisValues& v, bool first, bool second, const double* bet, FieldDiffs& r) {
     constexpr int G = kGuard4;
@@ -68,11 +69,11 @@ GRF_HD int axis_diffs(const Spacing& g, const AxisValues& v, bool first, bool se
         if (first) r.d1[d] = fx_value<G>(((q1 - m1) << 3) + (m2 - q2), ed, g.f1);
         if (second || KO) {
             const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2;  // pair sums less 2 u0
-            const int sh = fx_room(fx_top(p1) | fx_top(p2) >> 1, 58);
-            const long long s1 = fx_sar(p1, sh), s2 = fx_sar(p2, sh);
-            if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<G>((s1 << 4) - s2, ed + sh, g.f2);
-            inner[d] = (s1 << 4) - s1 - 6 * s2 - fx_sar(c2, sh);  // the dissipation's sum without u_-3 + u_3
-            e[d] = ed + sh;
+            // a quarter of the sums: what their constant shifts drop is below 2^-57 of the largest value
+            if (second) r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = fx_value<G - 2>((p1 << 2) - (p2 >> 2), ed, g.f2);
+            // the dissipation's 15 p1 - 6 p2 - 2 u0, without u_-3 + u_3
+            inner[d] = (p1 << 2) - (p1 >> 2) - p2 - (p2 >> 1) - (c0 >> 1);
+            e[d] = ed;
         }
         if (LOP) {
             const bool fw = bet[d] >= 0.0;
@@ -88,13 +89,9 @@ GRF_HD int axis_diffs(const Spacing& g, const AxisValues& v, bool first, bool se
             } else {
                 eb = ed;
             }
-            a1 -= u0;
-            a2 -= u0;
-            b1 -= u0;
-            const int sh = fx_room(fx_top(a1) | fx_top(a2), 58);
-            const long long x = 18 * fx_sar(a1, sh) - 6 * fx_sar(a2, sh) - 3 * fx_sar(b1, sh) - fx_sar(u0, sh);
+            const long long x = 9 * a1 - 3 * a2 - 5 * u0 - b1 - (b1 >> 1);  // half the sum without the far point
             const int eu = fx_max(eb, fx_mag(far) >> 20);  // the unit of the far point, three guard bits: 38 x 2^56
-            r.up[d] = fx_value<3>(fx_sar_round(x, eu - (eb + sh) + 2) + fx_int(far, fx_lim<3>(eu)), eu, g.f1);
+            r.up[d] = fx_value<3>(fx_sar_round(x, eu - eb + 1) + fx_int(far, fx_lim<3>(eu)), eu, g.f1);
             mag = fx_max(mag, fx_mag(far));
         }
     }
@@ -105,7 +102,7 @@ GRF_HD int axis_diffs(const Spacing& g, const AxisValues& v, bool first, bool se
         long long t = 0;
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            t += fx_int(v.m[d][2], lim) + fx_int(v.q[d][2], lim) + fx_sar_round(inner[d], E - e[d] + 3);
+            t += fx_int(v.m[d][2], lim) + fx_int(v.q[d][2], lim) + fx_sar_round(inner[d], E - e[d] + 1);
         r.ko = fx_value<2>(t, E);
     }
     return mag;
