@@ -156,16 +156,14 @@ struct PlaneValues6 {
     double x[6][6];  // at offsets -3, -2, -1, 1, 2, 3 along both axes
 };
 
-// 45 d1 - 9 d2 + d3 in units of 2^sh: 45 x 2^57 + 9 x 2^57 + 2^60 < 2^63.
-GRF_HD long long first6(long long d1, long long d2, long long d3, int& sh) {
-    sh = fx_room(fx_top(d1) | fx_top(d2) | fx_top(d3) >> 3, 57);
-    return 45 * fx_sar(d1, sh) - 9 * fx_sar(d2, sh) + fx_sar(d3, sh);
+// A 32nd of 45 d1 - 9 d2 + d3 of differences below 2^62 (110/32 x 2^61 < 2^63).
+GRF_HD long long first6(long long d1, long long d2, long long d3) {
+    return d1 + (d1 >> 2) + (d1 >> 3) + (d1 >> 5) - (d2 >> 2) - (d2 >> 5) + (d3 >> 5);
 }
 
 // As axis_diffs, 6th order; the outermost values are those at +-4.
 //   second: |p1| < 2^54, |p2| < 2^56, |p3| < 2^59: 270 x 2^54 + 27 x 2^56 + 2^60 < 2^63;
-//   dissipation: |p1| < 2^55, |p2| < 2^56, |p3| < 2^58, 2 |u0| < 2^59: 2^60.9 + 2^60.9 + 2^61 + 2^59 < 2^63;
-//   lopsided: |a1| < 2^54, |a2|, |b1| < 2^56, |a3| < 2^57, |u0| < 2^58, |b2| < 2^59: 2^62.8.
+//   a 64th of the dissipation's line sum 254/64 x 2^61, of the lopsided sum 179/64 x 2^61: below 2^63.
 template <int LOP, int KO, typename Spacing>
 GRF_HD int axis_diffs6(const Spacing& g, const AxisValues6& v, bool first, bool second, const double* bet, FieldDiffs& r) {
     constexpr int G = kGuard6;
@@ -184,20 +182,16 @@ GRF_HD int axis_diffs6(const Spacing& g, const AxisValues6& v, bool first, bool 
         const long long m2 = fx_int(v.m[d][1], lim), q2 = fx_int(v.q[d][1], lim);
         const long long m3 = fx_int(v.m[d][2], lim), q3 = fx_int(v.q[d][2], lim);
         const long long p1 = q1 + m1 - c2, p2 = q2 + m2 - c2, p3 = q3 + m3 - c2;  // pair sums less 2 u0
-        if (first) {
-            int sh;
-            const long long x = first6(q1 - m1, q2 - m2, q3 - m3, sh);
-            r.d1[d] = fx_value<G>(x, ed + sh, g.f1);
-        }
+        if (first) r.d1[d] = fx_value<G - 5>(first6(q1 - m1, q2 - m2, q3 - m3), ed, g.f1);
         if (second) {
             const int sh = fx_room(fx_top(p1) | fx_top(p2) >> 2 | fx_top(p3) >> 5, 54);
             r.d2[d == 0 ? 0 : (d == 1 ? 3 : 5)] =
                 fx_value<G>(270 * fx_sar(p1, sh) - 27 * fx_sar(p2, sh) + 2 * fx_sar(p3, sh), ed + sh, g.f2);
         }
         if (KO) {
-            const int sh = fx_room(fx_top(p1) | fx_top(p2) >> 1 | fx_top(p3) >> 3 | fx_top(c2) >> 4, 55);
-            inner[d] = 28 * fx_sar(p2, sh) - 56 * fx_sar(p1, sh) - 8 * fx_sar(p3, sh) - fx_sar(c2, sh);
-            e[d] = ed + sh;
+            // a 64th of 28 p2 - 56 p1 - 8 p3 - 2 u0, the dissipation without u_-4 + u_4
+            inner[d] = (p2 >> 1) - (p2 >> 4) - p1 + (p1 >> 3) - (p3 >> 3) - (c0 >> 5);
+            e[d] = ed + 6;
         }
         if (LOP) {
             const bool fw = bet[d] >= 0.0;
@@ -218,21 +212,11 @@ GRF_HD int axis_diffs6(const Spacing& g, const AxisValues6& v, bool first, bool 
             } else {
                 eb = ed;
             }
-            a1 -= u0;
-            a2 -= u0;
-            a3 -= u0;
-            b1 -= u0;
-            b2 -= u0;
-            const int sh = fx_room(fx_top(a1) | (fx_top(a2) | fx_top(b1)) >> 2 | fx_top(a3) >> 3 | fx_top(u0) >> 4 | fx_top(b2) >> 5, 54);
-            long long x[2] = {80 * fx_sar(a1, sh) - 30 * fx_sar(a2, sh) + 8 * fx_sar(a3, sh) - 24 * fx_sar(b1, sh) +
-                                  2 * fx_sar(b2, sh) + fx_sar(u0, sh),
-                              0};
-            const int ef = fx_max(fx_mag(far) >> 20, g.fx.emin), ex[2] = {eb + sh, ef};
-            x[1] = fx_int(far, fx_lim<G>(ef));
-            int eu;
-            const int bits[2] = {61, 61};
-            align_lines(x, ex, bits, eu);
-            r.up[d] = fx_value<G>(x[0] - x[1], eu, g.f1);
+            // a 64th of 80 a1 - 30 a2 + 8 a3 - 24 b1 + 2 b2 - 35 u0
+            const long long x = (a1 + (a1 >> 2)) - ((a2 >> 1) - (a2 >> 5)) + (a3 >> 3) - ((b1 >> 2) + (b1 >> 3)) + (b2 >> 5) -
+                                ((u0 >> 1) + (u0 >> 5) + (u0 >> 6));
+            const int eu = fx_max(eb, fx_mag(far) >> 20);  // the unit of the far point, one guard bit: 180 x 2^54
+            r.up[d] = fx_value<1>(fx_sar_round(x, eu - eb + 1) - fx_int(far, fx_lim<1>(eu)), eu, g.f1);
             mag = fx_max(mag, fx_mag(far));
         }
     }
@@ -268,14 +252,13 @@ GRF_HD double plane_diff6(const Spacing& g, const PlaneValues6& v, int& mag) {
         for (int b = 0; b < 6; ++b) top = fx_max(top, fx_mag(v.x[a][b]));
         mag = fx_max(mag, top);
         const int ed = fx_max(top >> 20, g.fx.emin), lim = fx_lim<G>(ed);
-        int sh;
         d[a] = first6(fx_int(v.x[a][3], lim) - fx_int(v.x[a][2], lim), fx_int(v.x[a][4], lim) - fx_int(v.x[a][1], lim),
-                      fx_int(v.x[a][5], lim) - fx_int(v.x[a][0], lim), sh);
-        e[a] = ed + sh;
+                      fx_int(v.x[a][5], lim) - fx_int(v.x[a][0], lim));
+        e[a] = ed;
     }
     const int bits[6] = {60, 57, 55, 55, 57, 60};
     align_lines(d, e, bits, E);
-    return fx_value<G>(45 * (d[3] - d[2]) - 9 * (d[4] - d[1]) + (d[5] - d[0]), E, g.f11);
+    return fx_value<G - 5>(45 * (d[3] - d[2]) - 9 * (d[4] - d[1]) + (d[5] - d[0]), E, g.f11);
 }
 
 }  // namespace grf

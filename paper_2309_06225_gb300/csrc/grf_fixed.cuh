@@ -11,8 +11,9 @@
 //     largest are dropped, where an FP64 sum would round at 2^-53 of its partial sums. A block is one
 //     sum's points along one grid line (grf_diffs.cuh), since across lines the magnitudes may differ by
 //     more than that: what a derivative keeps depends on no point that it does not read;
-//   * where the weights leave no room above G guard bits, the differences that are weighted are shifted right
-//     by what their own magnitude asks for (fx_room), which drops less than 2^-55 of the largest of them;
+//   * where the weights leave no room above G guard bits, sums are taken in halves, quarters and so on by constant
+//     shifts of the terms, or the differences that are weighted are shifted right by what their own magnitude asks
+//     for (fx_room): what that drops lies below 2^-53 of the largest term;
 //   * the integer sums are independent of their order, so every caller gets the same bits;
 //   * the sum times a positive constant (the grid-spacing factor, as a 64-bit mantissa) is rounded once to
 //     double.
