@@ -9,10 +9,11 @@ namespace grf {
 // What bounds it: each column is a chain of entries, 24 bytes and 2.5 operands each. A read-modify-write of an
 // operand's adjoint in global memory is a link of that chain. Contributions to the last kWindow entries (36% at
 // 16 entries, half at 100) go to a window in shared memory instead, and the others are added by the memory
-// (atomicAdd without a result: a column is one thread's, so the order is the program's). An entry's adjoint is
-// its window slot plus what farther entries left in global memory, which is final kWindow entries ahead, so
-// entries and those adjoints are loaded kAhead entries before they are used. Comparisons with zero are taken on
-// the integer pipe: the FP64 pipe, 16 clocks an instruction, is the next bound.
+// (atomicAdd without a result: a column is one thread's, so the order is the program's; the product is rounded
+// before the sum, 6-8% more rounding in the sweep than with fma, where plain read-modify-writes take 16% more time).
+// An entry's adjoint is its window slot plus what farther entries left in global memory, which is final kWindow
+// entries ahead, so entries and those adjoints are loaded kAhead entries before they are used. Comparisons with
+// zero are taken on the integer pipe: the FP64 pipe, 16 clocks an instruction, is the next bound.
 constexpr int kWindow = 16, kAhead = 4;
 
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }

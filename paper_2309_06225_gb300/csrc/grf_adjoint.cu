@@ -67,9 +67,9 @@ __device__ __forceinline__ void enforce_point_t(T u[NFIELDS], double min_chi, do
 // STAGE (0..3) is a run-time argument: one instantiation of the large pointwise map keeps the
 // library's build time down (its four stage variants differ only in a few scalars and leaves).
 // Thread col tapes point q0 + col of the wave into tape column col.
-// What bounds it: the FP64 pipe (53% of its slots, 8,720 instructions a point) beside 75 KB a point written, the
-// tape and spills. At -O3 it spills 19 KB of stores and 47 KB of loads a thread where -O1 spilled 24 and 83:
-// 36 x 32 x 30 gradient 37.1 -> 36.1 ms, 64^3 167.4 -> 162.3.
+// What bounds it: the FP64 pipe (43% of its slots, 6,640 instructions a point) beside 78 KB a point written, the
+// tape and spills. At -O3 it spills 18 KB of stores and 46 KB of loads a thread (at -O1, when the two were compared,
+// 24 and 83 against 19 and 47: 36 x 32 x 30 gradient 37.1 -> 36.1 ms, 64^3 167.4 -> 162.3).
 __global__ void __launch_bounds__(kAdjThreads, 4) adj_tape_kernel(Geom g, Coeffs c, AdjArgs a, int STAGE, long long q0) {
     const long long col = grf_rev::rev_col();
     const long long q = q0 + col;

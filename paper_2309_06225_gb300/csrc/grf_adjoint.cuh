@@ -9,7 +9,7 @@ namespace grf {
 // leaves of the pointwise map: values, first derivatives (24 slots x 3), second derivatives
 // (12 slots x 6), KO sums, u_n, acc, lambda, g2
 enum : int { kLV = 0, kLD1 = 27, kLD2 = 99, kLKO = 171, kLUN = 198, kLACC = 225, kLLAM = 252, kLG2 = 253, kNLeaf = 254 };
-// tape entries per point and stage: the pointwise RHS records about 2,250, the stage update and
+// tape entries per point and stage: the pointwise RHS records about 2,330, the stage update and
 // enforcement about 130 more; an overflow is detected and reported
 constexpr int kTapeCap = 5120;
 constexpr int kAdjThreads = 128;

@@ -580,7 +580,7 @@ int grf_rk4_step_host(const grf_box* box, const grf_params* params, const double
     // first and last chunks also holding the z-ghost planes. Q >= 4 planes, so the planes a slab's
     // stencils read (up to interior plane hi + 2) lie in chunks s-1, s and s+1; and enough planes for
     // kSlabPoints points, five waves of warps, since a slab's launch ends before the next one's begins
-    // (48^3 in 12 slabs: 4.68 ms a step, in one: 2.86; 96^3 in 16: 18.7, in 3: 18.1; 160^3 in 16: 79.3, in 14: 77.7).
+    // (48^3 in 12 slabs: 4.88 ms a step, in one: 2.97; 96^3 in 16: 19.7, in 3: 18.6; 160^3 in 16: 84.4, in 14: 83.1).
     const long long nxy = (long long)g.nx * g.ny;
     const int Q = (int)std::min((long long)std::max(g.nz, 4),
                                 std::max((long long)std::max(4, (g.nz + kMaxSlabs - 1) / kMaxSlabs), (kSlabPoints + nxy - 1) / nxy));

@@ -15,7 +15,7 @@ namespace grf {
 // coupled system (PointExtraT::hyp). PSI4 = 1 compiles those outputs in (they need the assembled
 // or solved coupled system); with PSI4 = 0 the compiler drops the coupled solve, which H, M_i and
 // the densities do not use. Bound by the FP64 pipe, held to 168 registers for 3 blocks per SM (constraints,
-// Psi_4 and modes of 72^2 x 60 points: 2.93 -> 2.61 ms a call against 255 and 2).
+// Psi_4 and modes of 72^2 x 60 points: 2.96 -> 2.61 ms a call against 255 and 2).
 template <int ORD, int PSI4>
 __global__ void __launch_bounds__(128, 3) constraints_kernel(Geom g, Coeffs c, const double* __restrict__ s,
                                                              double* __restrict__ out4, double* __restrict__ part,

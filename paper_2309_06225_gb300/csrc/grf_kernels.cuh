@@ -386,9 +386,9 @@ __device__ __forceinline__ void stage_point(const Geom& g, const Coeffs& c, cons
 // One thread per interior point of [q0, q1), consecutive threads consecutive points in x-fastest order,
 // so that every lane of every warp but the last works whatever the box's extents (no derivative is
 // exchanged between lanes, so the mapping is free). Blocks of point_threads() threads (grf_launch.h).
-// What bounds it: the FP64 pipe (79% of its issue slots), 2,212 instructions a point and stage. 12 resident
-// warps per SM (168 registers a thread) hide its latency; more would spill more: 128^3 step 51.8 ms with 8
-// warps, 36.5 with 12, 39.2 with 16, 43.8 with 20. (256^3 step 506 -> 296 ms since the stencils are summed in
+// What bounds it: the FP64 pipe (80% of its issue slots), 2,292 instructions a point and stage. 12 resident
+// warps per SM (168 registers a thread) hide its latency; more would spill more: 128^3 step 51.1 ms with 8
+// warps, 38.8 with 12, 42.0 with 16, 45.8 with 20. (256^3 step 506 -> 317 ms since the stencils are summed in
 // integers, grf_fixed.cuh, and the equations need fewer operations, grf_point.cuh.)
 // DEC: 0 full theory, 1 without backreaction (a separate instantiation each, so the full
 // theory's kernel carries no test of the mode), -1 the mode read from c. LOP: lopsided advection.

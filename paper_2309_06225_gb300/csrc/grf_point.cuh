@@ -35,7 +35,7 @@
 // side and the departure apart. Errors against long double, near one of two punctures, over those of the plain
 // formulation (Ricci tensor and D_i Z_j term by term, S_ij from the solution): off-diagonal d_t A_ij 1.0 (2.1 to 2.6
 // with the chi part summed first and A_ij from the eliminated C_ij), K 1.07 (1.4), Theta 1.03 (1.5), all fields 0.9.
-// It takes about 80 instructions more: 256^3 step 296 -> 306 ms.
+// It takes about 80 instructions more: 256^3 step 296 -> 306 ms when it came in.
 //
 // The cubic Horndeski term (1/16 pi) g3 X box(phi) (general instantiation, COUP = 1) adds, with
 // H = nabla nabla phi in the same basis (H_nn holding d_t Pi, H_ni, H_ij = D_i D_j phi + K_ij Pi),

@@ -5,7 +5,7 @@
 namespace grf {
 
 // One thread per interior point, as rk4_stage_kernel, and bound like it. LOP: lopsided advection.
-// Held to 168 registers for 3 blocks per SM (80 x 64 x 72: 2.26 -> 1.87 ms a call against 255 and 2).
+// Held to 168 registers for 3 blocks per SM (80 x 64 x 72 with its dissipation: 2.35 -> 1.97 ms against 255 and 2).
 template <int LOP>
 __global__ void __launch_bounds__(128, 3) rhs_kernel(Geom g, Coeffs c, const double* __restrict__ s, double* __restrict__ rhs,
                                                      double ko, int* status) {

@@ -4,7 +4,7 @@
 // the larger part of that. Here the lanes of a team each gather a share of the point's fields into shared
 // memory and then all evaluate the point's equations (the FP64 pipe is idle enough), so that the gather takes
 // a quarter or half of the time. The operations on each value are those of rk4_stage_kernel, and so are the bits.
-// 16^3 step: 0.61 ms with one lane a point, 0.50 with 2, 0.45 with 4; 20^3: 0.64, 0.53, 0.65 (the FP64 work of a
+// 16^3 step: 0.66 ms with one lane a point, 0.53 with 2, 0.46 with 4; 20^3: 0.69, 0.55, 0.68 (the FP64 work of a
 // point is done once a lane, so 4 lanes pay only while a scheduler has one warp at most).
 #pragma once
 

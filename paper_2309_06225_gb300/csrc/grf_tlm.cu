@@ -72,10 +72,10 @@ __device__ __forceinline__ void enforce_point_d3(D3 u[NFIELDS], double min_chi, 
     u[F_LAPSE] = grf_dual::fmax(u[F_LAPSE], min_lapse);
 }
 
-// What bounds it: the FP64 pipe (67% of its slots) at 8 warps per SM, 14,226 instructions a point and stage.
+// What bounds it: the FP64 pipe (68% of its slots) at 8 warps per SM, 14,546 instructions a point and stage.
 // 255 registers and 2 blocks per SM, named to ptxas, which otherwise settles for 32 registers and an 87 KB stack
-// (so it ran at -O1: 96^3 step 118.7 -> 111.6 ms, 40 x 32 x 36 9.17 -> 8.83). 3 blocks per SM take 130 ms at
-// 96^3, 4 take 128; they win only where 2 leave a nearly empty last wave (40 x 32 x 36: 7.2 ms).
+// (so it ran at -O1, 5% slower). 96^3 step 119 to 134 ms by run; 3 blocks per SM take 4% more there, and less only
+// where 2 leave a nearly empty last wave (40 x 32 x 36: 9.1 -> 8.5 ms).
 template <int STAGE>
 __global__ void __launch_bounds__(128, 2) tlm_stage_kernel(Geom g, CoeffsT<D3> c, TlmArgs a) {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
